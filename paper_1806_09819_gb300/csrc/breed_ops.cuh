@@ -153,4 +153,91 @@ __device__ __forceinline__ void mutate8_direct(float sigma, uint32_t gen, const 
     apply_mutation8(sigma, hit, z, v);
 }
 
+// ---- mask draws as words -------------------------------------------------------
+// A unit's eight 16-bit mask draws stay in the four words of their Philox
+// block: genes 8u + 2s and 8u + 2s + 1 draw the low and the high half of word
+// s.  With lim = (thr << 16) - 1 (0 < thr <= 65536) the high half is below thr
+// iff w <= lim and the low half iff (w << 16) <= lim, one comparison each and no
+// mask to assemble.
+__device__ __forceinline__ uint32_t mask_limit(uint32_t thr) { return (thr << 16) - 1u; }
+__device__ __forceinline__ bool hit_lo(uint32_t w, uint32_t lim) { return (w << 16) <= lim; }
+__device__ __forceinline__ bool hit_hi(uint32_t w, uint32_t lim) { return w <= lim; }
+__device__ __forceinline__ bool hit_any(uint32_t w, uint32_t lim) { return min(w, w << 16) <= lim; }
+
+// One lane's 8 genes after uniform crossover: parent 2's gene where its draw hits.
+__device__ __forceinline__ void cross8(const uint4& r, uint32_t lim, float (&v)[8], const float (&b)[8])
+{
+    const uint32_t w[4] = { r.x, r.y, r.z, r.w };
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        v[2 * s] = hit_lo(w[s], lim) ? b[2 * s] : v[2 * s];
+        v[2 * s + 1] = hit_hi(w[s], lim) ? b[2 * s + 1] : v[2 * s + 1];
+    }
+}
+
+// The masked Box-Muller pairs of a warp's U units per lane (unit i of lane l is
+// u0 + 32 i + l), gathered into one dense job list so that consecutive lanes
+// compute their normals.  The pair of slot s of unit i of lane l has the code
+// 4 (32 i + l) + s: pair code & 1 of NORMAL block 2 u0 + (code >> 1), the genes
+// 2 code and 2 code + 1 of the warp's chunk.  words[code] receives every slot's
+// mask word, codes[] the listed ones; returns how many.  w[i]: the unit's mask
+// words (all ones for a unit that does not exist).  Every lane of the warp
+// calls it.
+template <int U>
+__device__ __forceinline__ uint32_t list_masked_pairs(const uint32_t (&w)[U][4], uint32_t lim, int lane,
+                                                      uint32_t* words, uint8_t* codes)
+{
+    static_assert(U == 1 || U == 2, "a job code is one byte");
+    uint32_t need = 0;
+#pragma unroll
+    for (int i = 0; i < U; ++i)
+#pragma unroll
+        for (int s = 0; s < 4; ++s) need |= hit_any(w[i][s], lim) ? 1u << (4 * i + s) : 0u;
+    const uint32_t cnt = static_cast<uint32_t>(__popc(need));
+    // Exclusive prefix of the counts (0 .. 4 U) from the ballots of their bits.
+    const uint32_t lt = (1u << lane) - 1u;
+    uint32_t at = 0;
+#pragma unroll
+    for (int b = 0; b < (U == 1 ? 3 : 4); ++b)
+        at += static_cast<uint32_t>(__popc(__ballot_sync(0xFFFFFFFFu, (cnt >> b) & 1u) & lt)) << b;
+    const uint32_t total = __shfl_sync(0xFFFFFFFFu, at + cnt, 31);
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+        reinterpret_cast<uint4*>(words)[32 * i + lane] = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+            if (need & (1u << (4 * i + s))) codes[at++] = static_cast<uint8_t>(4 * (32 * i + lane) + s);
+    }
+    __syncwarp();
+    return total;
+}
+
+// The normals of one listed pair.
+template <typename Key>
+__device__ __forceinline__ float2 listed_normals(uint32_t code, uint32_t u0, uint32_t gen, const Key& key, uint32_t ent)
+{
+    const uint4 n = philox_keyed(make_uint4(2u * u0 + (code >> 1), ent, gen, kTagNormal), key);
+    return (code & 1u) ? box_muller(n.z, n.w) : box_muller(n.x, n.y);
+}
+
+// Mutation of one unit by its own lane, for high mutation rates: both NORMAL blocks
+// and all four pairs of the unit (each block serves two pairs, which the list
+// cannot share).  ALL: every gene mutates.
+template <bool ALL, typename Key>
+__device__ __forceinline__ void mutate8_dense(float sigma, uint32_t gen, const Key& key, uint32_t ent, uint32_t u,
+                                              const uint32_t (&w)[4], uint32_t lim, float (&v)[8])
+{
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const uint4 n = philox_keyed(make_uint4(2u * u + q, ent, gen, kTagNormal), key);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int s = 2 * q + h;
+            const float2 z = h ? box_muller(n.z, n.w) : box_muller(n.x, n.y);
+            if (ALL || hit_lo(w[s], lim)) v[2 * s] = fmaf(sigma, z.x, v[2 * s]);
+            if (ALL || hit_hi(w[s], lim)) v[2 * s + 1] = fmaf(sigma, z.y, v[2 * s + 1]);
+        }
+    }
+}
+
 }  // namespace leea

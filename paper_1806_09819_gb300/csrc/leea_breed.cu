@@ -1,34 +1,46 @@
 // leea_breed.cu -- crossover and mutation (Section 3.2) fused into one
 // streaming pass over every child's genes.
 //
-// The pass is HBM-bound: per gene it reads one (mutation, elite) or two
-// (crossover) parent floats and writes one child float.  To keep HBM busy
-// while the generator arithmetic runs, the kernel is persistent (one CTA per
-// SM) and decoupled:
-//   warp 0               streams parent chunks (6144 genes = 24 KB per parent
-//                        for one run, 4096 for many) into a ring of
-//                        shared-memory stages with cp.async.bulk, tracked by
-//                        transaction-count mbarriers;
-//   warps 1-24 (1-16)    take a stage, compute the child chunk and write it
-//                        with 128-bit stores, then release the stage.
-// Work items walk the children alternately from the front (elites, crossover
-// children) and the back (mutation children), so every SM mixes the
-// HBM-heavier crossover items with the arithmetic-heavier mutation items;
-// with one run they go chunk by chunk over all children, so that parents
-// shared by several children are read from HBM about once.  The producer
-// warp resolves 32 items' children and parents at a time.
-// With many runs each CTA takes a contiguous range of items, so that it
-// meets few run boundaries (each one reloads the run's arguments).
-// A consumer thread owns 8 consecutive genes of the chunk: one Philox block
-// of 16-bit mask draws (crossover or mutation mask) and two Philox blocks of
-// normals.  In mutation children only the Box-Muller pairs that hold a masked
-// gene are generated, and a warp first gathers them into a dense job list in
-// shared memory (one ballot per pair slot) so that normals are computed by
-// consecutive lanes instead of by whichever lane happens to own a masked
-// gene; the normals go back through the same list.  Every mbarrier
-// wait is bounded in time; on expiry the kernel sets kStatusBreedTimeout.
+// Per gene the pass reads one (mutation, elite) or two (crossover) parent
+// floats, draws the gene's random numbers and writes one child float.  What
+// bounds it at the usual rates is not memory but the generator: a Philox block
+// is 20 wide multiplies, four cycles each on one pipe (86 cycles a warp,
+// measured alone), a Box-Muller pair about 104.  So the kernel is built to keep
+// the arithmetic pipes fed and to spend few instructions on anything else.
+//
+// Every warp works for itself: an item is 64 units of one child (a unit: the 8
+// consecutive genes whose 16-bit mask draws share a Philox block), lane l owns
+// units l and l + 32.  No warp waits for another; twenty of them on an SM hide
+// each other's loads and arithmetic (24 gained 3 % at equal shares of
+// crossover and mutation and lost 10-20 % with more crossover or shadows).
+//   crossover        both parents by 32-byte loads, in flight while the masks
+//                    are drawn; 32-byte stores
+//   mutation, q < kDenseRate   the parent's chunk is copied into shared memory
+//                    asynchronously, one item ahead; meanwhile the masks are
+//                    drawn and the Box-Muller pairs that hold a masked gene are
+//                    gathered into a dense job list, so that consecutive lanes
+//                    compute their normals and change the chunk in place; an
+//                    asynchronous copy stores it.  The 90 % of genes that do not
+//                    change never pass through a register.
+//   mutation, else   every lane makes all pairs of its units, two pairs per
+//                    Philox block; at q = 1 without drawing any mask
+// Items go chunk by chunk over all children (all children's first chunk, then
+// all second chunks, ...), so a parent chunk shared by several children comes
+// from HBM about once.  Neighbouring items alternate between the front (elites,
+// crossover children) and the back (mutation children) of the population, so
+// that every SM mixes both kinds.  A warp resolves its next 32 items at a time,
+// one per lane, down to addresses.
+//
+// Measured (P = 1000, 784-112-10, half crossover, 10 % of genes mutating):
+// 97.5 us, 7.3 TB/s of one read and one write per gene (shared parents come
+// from L2), against 136.7 us for the block-wide ring of parent chunks with a
+// producer warp that it replaced; crossover alone 94 (104), mutation alone 129
+// (171); every gene mutating on 196-256-128-64-10: 117 (237); BF16 shadows at
+// P = 4096: 488 (684), FP8 492 (712); 64 runs together 3.15 ms (4.01).
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
+
+#include <type_traits>
 
 #include "breed_ops.cuh"
 #include "leea_internal.h"
@@ -39,150 +51,115 @@ namespace leea {
 
 namespace {
 
-// Shape of the kernel: one run takes 24 consumer warps (about six per
-// scheduler, to hide the Philox and Box-Muller dependency chains) over
-// 6144-gene chunks in a 4-deep ring; many runs keep 16 warps over 4096-gene
-// chunks in a 6-deep ring (their per-run state needs more registers).
-template <bool MULTI>
-struct BreedShape {
-    static constexpr int kConsumerWarps = MULTI ? 16 : 24;
-    static constexpr int kThreads = 32 * (1 + kConsumerWarps);
-    static constexpr int kChunk = 8 * 32 * kConsumerWarps;  // genes per work item: 8 per consumer thread
-    static constexpr int kStages = MULTI ? 6 : 4;           // ring depth (2 parent chunks per stage)
-    static constexpr uint32_t kChunkBytes = kChunk * 4;
-};
+constexpr int kWarps = 20;         // one CTA per SM
+constexpr int kUnitGenes = 8;
+constexpr int kUnits = 2;          // U: units per lane and item
+constexpr int kChunk = 32 * kUnits * kUnitGenes;  // genes per item
+constexpr int kJobSlots = 4 * 32 * kUnits;        // Box-Muller pairs of a warp's item
+// Rate from which a lane makes all its pairs itself: 16-bit threshold of
+// kDenseRate = 0.35.  Mutation children alone at P = 1000, 784-112-10: the list
+// takes 129 us at q = 0.1 and 196 at 0.3, all pairs 190 at any q.
+constexpr uint32_t kDenseThr = 22937;
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 constexpr uint64_t kDrainLimitNs = 200000000ull;
 constexpr int32_t kKindInvalid = -1;
 
-struct StageMeta {
-    int32_t j;       // child
-    int32_t kind;    // 0 elite, 1 crossover, 2 mutation, -1 invalid parent index
-    int32_t g0;      // first gene of the chunk
-    int32_t len;     // genes in the chunk (multiple of 32)
-    int32_t sexp;    // precision form, FP8: exponent of the child's scale
-    int32_t run;     // many runs: index of the child's run
-    float sigma;     // the child's mutation strength
-    int32_t pad;
-};
-
-constexpr int kJobSlots = 4 * 32;  // Box-Muller pairs of a warp's 32 units
-
-// An item's source as the producer warp resolves it, 32 items at a time.
-struct ItemSrc {
-    const float* p1;  // parent chunks (NULL for an invalid parent index)
-    const float* p2;
-    StageMeta m;
-};
-
-struct BreedSmem {
-    uint8_t* base;   // stage i: parent 1 at base + 2i chunks, parent 2 at base + (2i+1) chunks
-    StageMeta* meta;
-    ItemSrc* batch;  // [32]: the producer warp's next 32 items
-    float2* job_z;      // [consumer warps][kJobSlots]: normals of a warp's job list
-    uint8_t* job_code;  // [consumer warps][kJobSlots]: owner lane << 2 | pair slot
-    uint64_t* full;
-    uint64_t* empty;
-    volatile int* abort_flag;
-};
-
-template <bool MULTI>
-__device__ __forceinline__ BreedSmem carve(uint8_t* raw)
+// How mutation children draw their normals.
+enum MutMode { kMutNone, kMutSparse, kMutDense, kMutAll };
+MutMode mut_mode(uint32_t thr)
 {
-    using S = BreedShape<MULTI>;
-    constexpr int kStages = S::kStages, kConsumerWarps = S::kConsumerWarps;
-    constexpr uint32_t kChunkBytes = S::kChunkBytes;
-    BreedSmem s;
-    uint8_t* base = raw + ((128u - (ptx::smem_u32(raw) & 127u)) & 127u);
-    s.base = base;
-    uint8_t* p = base + 2 * kStages * kChunkBytes;
-    s.meta = reinterpret_cast<StageMeta*>(p);
-    p += sizeof(StageMeta) * kStages;
-    s.batch = reinterpret_cast<ItemSrc*>(p);
-    p += sizeof(ItemSrc) * 32;
-    s.job_z = reinterpret_cast<float2*>(p);
-    p += sizeof(float2) * kConsumerWarps * kJobSlots;
-    s.job_code = p;
-    p += kConsumerWarps * kJobSlots;
-    s.full = reinterpret_cast<uint64_t*>(p);
-    s.empty = s.full + kStages;
-    s.abort_flag = reinterpret_cast<volatile int*>(s.empty + kStages);
-    return s;
+    return thr == 0u ? kMutNone : (thr >= 65536u ? kMutAll : (thr >= kDenseThr ? kMutDense : kMutSparse));
 }
 
-template <bool MULTI>
-constexpr size_t breed_smem_bytes()
-{
-    using S = BreedShape<MULTI>;
-    return 128 + 2 * S::kStages * S::kChunkBytes + sizeof(StageMeta) * S::kStages + sizeof(ItemSrc) * 32 +
-           (sizeof(float2) + 1) * S::kConsumerWarps * kJobSlots + 16 * S::kStages + 16;
-}
-static_assert(breed_smem_bytes<false>() <= 227 * 1024 && breed_smem_bytes<true>() <= 227 * 1024,
-              "breed ring must fit in shared memory");
+// An item as its warp resolved it (one lane per item), so that the loop over
+// the items has no table look-ups or 64-bit products.
+struct __align__(16) Item {
+    const float *pa, *pb;  // the parents' chunks
+    float* child;          // the child's chunk
+    uint64_t seed;
+    uint32_t u0, n_units;  // the chunk's first unit, and the child's units from there on
+    uint32_t ent;          // Philox entity
+    int32_t kind;          // 0 elite, 1 crossover, 2 mutation, -1 invalid parent index
+    float sigma;           // the child's mutation strength
+    int32_t genes;         // genes below c in the chunk, at most kChunk (the rest is padding)
+    // precision form
+    float inv;             // FP8: 2^-e of the child's scale
+    uint32_t w1_units;     // units of W1 from u0 on
+    uint8_t* shadow;       // the child's shadow
+    float* amax;
+    int32_t sh_h, pad[3];
+};
 
-// The shadow of 8 child genes i0 .. i0+7 of W1: 8 BF16 (16 bytes) or 8 FP8-e4m3
-// of w / 2^sexp with saturation (8 bytes).  Returns max |w| of the 8 genes.
-__device__ __forceinline__ float write_shadow8(const BreedArgs& a, int32_t j, int32_t sexp, int64_t i0,
-                                               const float4 (&v)[2])
+// A warp's shared memory.
+struct __align__(128) WarpSmem {
+    float buf[2][kChunk];           // sparse mutation: the parent's chunk, changed in place into the child's
+    uint32_t words[kJobSlots];      // mask words by pair code
+    Item items[32];                 // the warp's next items
+    uint64_t full[2];               // a parent's chunk has landed in buf
+    int abort;                      // never set: the waits end by their limit
+    uint8_t codes[kJobSlots];       // the listed pairs
+};
+
+// 8 consecutive floats; W32: the address is 32-byte aligned.  Parents are read
+// once per child, so they are kept out of L1.
+template <bool W32>
+__device__ __forceinline__ void load8(const float* p, float (&v)[8])
 {
-    const float mx = fmaxf(fmaxf(fmaxf(fabsf(v[0].x), fabsf(v[0].y)), fmaxf(fabsf(v[0].z), fabsf(v[0].w))),
-                           fmaxf(fmaxf(fabsf(v[1].x), fabsf(v[1].y)), fmaxf(fabsf(v[1].z), fabsf(v[1].w))));
-    // Eight genes of one row: d_0 % 16 == 0 keeps them in one 16-byte (BF16)
-    // or 8-byte (FP8) piece of a chunk.
-    const int32_t i32 = static_cast<int32_t>(i0);  // a W1 gene: i0 < h d_0 < 2^31
-    const int32_t o = i32 / a.sh_k;
-    const int32_t k = i32 - o * a.sh_k;
-    uint8_t* dst = a.shadow + static_cast<int64_t>(j) * a.sh_stride +
-                   shadow_offset(a.sh_h, a.precision == 1 ? 2 : 1, o, k);
-    if (a.precision == 1) {
-        const __nv_bfloat162 b0 = __floats2bfloat162_rn(v[0].x, v[0].y);
-        const __nv_bfloat162 b1 = __floats2bfloat162_rn(v[0].z, v[0].w);
-        const __nv_bfloat162 b2 = __floats2bfloat162_rn(v[1].x, v[1].y);
-        const __nv_bfloat162 b3 = __floats2bfloat162_rn(v[1].z, v[1].w);
-        uint4 w;
-        w.x = *reinterpret_cast<const uint32_t*>(&b0);
-        w.y = *reinterpret_cast<const uint32_t*>(&b1);
-        w.z = *reinterpret_cast<const uint32_t*>(&b2);
-        w.w = *reinterpret_cast<const uint32_t*>(&b3);
-        *reinterpret_cast<uint4*>(dst) = w;
+    if (W32) {
+        asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                     : "l"(p));
     } else {
-        const float inv = ldexpf(1.0f, -sexp);  // exact: a power of two
-        const __nv_fp8x2_storage_t q0 =
-            __nv_cvt_float2_to_fp8x2(make_float2(v[0].x * inv, v[0].y * inv), __NV_SATFINITE, __NV_E4M3);
-        const __nv_fp8x2_storage_t q1 =
-            __nv_cvt_float2_to_fp8x2(make_float2(v[0].z * inv, v[0].w * inv), __NV_SATFINITE, __NV_E4M3);
-        const __nv_fp8x2_storage_t q2 =
-            __nv_cvt_float2_to_fp8x2(make_float2(v[1].x * inv, v[1].y * inv), __NV_SATFINITE, __NV_E4M3);
-        const __nv_fp8x2_storage_t q3 =
-            __nv_cvt_float2_to_fp8x2(make_float2(v[1].z * inv, v[1].w * inv), __NV_SATFINITE, __NV_E4M3);
-        uint2 w;
-        w.x = static_cast<uint32_t>(q0) | (static_cast<uint32_t>(q1) << 16);
-        w.y = static_cast<uint32_t>(q2) | (static_cast<uint32_t>(q3) << 16);
-        *reinterpret_cast<uint2*>(dst) = w;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                         : "=f"(v[4 * h]), "=f"(v[4 * h + 1]), "=f"(v[4 * h + 2]), "=f"(v[4 * h + 3])
+                         : "l"(p + 4 * h));
+    }
+}
+
+template <bool W32>
+__device__ __forceinline__ void store8(float* p, const float (&v)[8])
+{
+    if (W32) {
+        asm volatile("st.global.v8.f32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"f"(v[0]), "f"(v[1]), "f"(v[2]),
+                     "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "l"(p)
+                     : "memory");
+    } else {
+        reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
+    }
+}
+
+// The shadow of unit u of W1 (8 genes of one row, as d_0 % 16 == 0): 8 BF16
+// (16 bytes) or 8 FP8-e4m3 of w 2^-e (saturating; 8 bytes), inside one 16-byte
+// piece of a chunk.  Returns max |w| of the 8 genes (NaN ignored).
+__device__ __forceinline__ float write_shadow8(const BreedArgs& a, const Item& m, uint32_t u, const float (&v)[8])
+{
+    float mx = 0.0f;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) mx = fmaxf(mx, fabsf(v[t]));
+    const uint32_t o = __umulhi(u, a.sh_row_mul);  // u / (sh_k / 8)
+    const int32_t k = static_cast<int32_t>(8u * u - o * static_cast<uint32_t>(a.sh_k));
+    uint8_t* dst = m.shadow + shadow_offset(m.sh_h, a.precision == 1 ? 2 : 1, static_cast<int32_t>(o), k);
+    if (a.precision == 1) {
+        uint32_t w[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * t], v[2 * t + 1]);
+            w[t] = *reinterpret_cast<const uint32_t*>(&b);
+        }
+        *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+    } else {
+        uint32_t q[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+            q[t] = __nv_cvt_float2_to_fp8x2(make_float2(v[2 * t] * m.inv, v[2 * t + 1] * m.inv), __NV_SATFINITE,
+                                            __NV_E4M3);
+        *reinterpret_cast<uint2*>(dst) = make_uint2(q[0] | (q[1] << 16), q[2] | (q[3] << 16));
     }
     return mx;
 }
-
-__device__ __forceinline__ float* stage_a(const BreedSmem& s, uint32_t stage, uint32_t chunk_bytes)
-{
-    return reinterpret_cast<float*>(s.base + (2u * stage) * chunk_bytes);
-}
-
-__device__ __forceinline__ float* stage_b(const BreedSmem& s, uint32_t stage, uint32_t chunk_bytes)
-{
-    return reinterpret_cast<float*>(s.base + (2u * stage + 1u) * chunk_bytes);
-}
-
-__device__ __forceinline__ void raise_abort(volatile int* abort_flag, unsigned int* status)
-{
-    *abort_flag = 1;
-    atomicOr(status, kStatusBreedTimeout);
-}
-
-constexpr int kGenesPerLane = 8;  // one Philox block of 16-bit mask draws per lane and chunk
-static_assert(BreedShape<false>::kChunk == kGenesPerLane * 32 * BreedShape<false>::kConsumerWarps &&
-                  BreedShape<true>::kChunk == kGenesPerLane * 32 * BreedShape<true>::kConsumerWarps,
-              "consumers must tile a chunk exactly");
 
 // The run owning global work item `it`: the last one whose first item is <= it.
 __device__ __forceinline__ int32_t run_of_item(const BreedRun* runs, int32_t n_runs, int64_t it)
@@ -196,208 +173,249 @@ __device__ __forceinline__ int32_t run_of_item(const BreedRun* runs, int32_t n_r
     return lo;
 }
 
-// MULTI = false: one run (run0), generation in run0.a.gen.  MULTI = true: the
-// runs of a device table, whose work items are numbered consecutively, and
-// the generation read from gen_dev.
-template <bool MULTI>
-__global__ void __launch_bounds__(BreedShape<MULTI>::kThreads, 1)
-breed_kernel(const __grid_constant__ BreedRun run0, const BreedRun* __restrict__ runs, int32_t n_runs,
-             int64_t n_items, const uint32_t* __restrict__ gen_dev, unsigned int* __restrict__ status)
+// Item `it` of run R.
+__device__ __forceinline__ void resolve_item(const BreedRun& R, int64_t it, Item* m)
 {
-    extern __shared__ uint8_t smem_raw[];
+    const BreedArgs& a = R.a;
+    const uint32_t li = static_cast<uint32_t>(it - R.item0);  // below 2^32: under 2^38 genes fit in memory, pop <= 2^24
+    const uint32_t pop = static_cast<uint32_t>(a.pop), ck = li / pop, ci = li - ck * pop;
+    // Front and back children alternate; odd chunks swap the two of a pair, so
+    // that a warp whose items keep one parity of ci still meets both.
+    uint32_t x = ci ^ (ck & 1u);
+    if (x >= pop) x = ci;
+    const int32_t j = static_cast<int32_t>((x & 1u) ? static_cast<uint32_t>(a.pop) - 1u - (x >> 1) : (x >> 1));
+    const int32_t p1 = R.par1[j], p2 = R.par2[j];
+    const int32_t n_par = a.n_parents > 0 ? a.n_parents : a.pop;
+    const int64_t g0 = static_cast<int64_t>(ck) * kChunk;
+    m->pa = R.parents + static_cast<int64_t>(p1) * a.c_pad + g0;
+    m->pb = R.parents + static_cast<int64_t>(p2) * a.c_pad + g0;
+    m->child = R.children + static_cast<int64_t>(j) * a.c_pad + g0;
+    m->seed = a.seed;
+    m->u0 = ck * (32u * kUnits);
+    m->n_units = static_cast<uint32_t>((a.c_pad - g0) >> 3);
+    m->ent = a.entity ? a.entity[j] : static_cast<uint32_t>(j);
+    m->kind = (p1 < 0 || p1 >= n_par || p2 < 0 || p2 >= n_par) ? kKindInvalid : R.kind[j];
+    m->sigma = a.sigma_child ? a.sigma_child[j] : a.sigma;
+    const int64_t genes = a.c - g0;
+    m->genes = genes < kChunk ? static_cast<int32_t>(genes) : kChunk;
+    if (a.precision > 0) {
+        m->inv = a.precision == 2 ? ldexpf(1.0f, -a.scale_exp[j]) : 1.0f;  // exact: a power of two
+        m->w1_units = g0 < a.n_w1 ? static_cast<uint32_t>((a.n_w1 - g0) >> 3) : 0u;
+        m->shadow = a.shadow + static_cast<int64_t>(j) * a.sh_stride;
+        m->amax = a.amax_out + j;
+        m->sh_h = a.sh_h;
+    }
+}
+
+template <bool MULTI>
+__device__ __forceinline__ auto item_key(uint64_t seed, const PhiloxKeys& keys0) ->
+    typename std::conditional<MULTI, PhiloxSeed, const PhiloxKeys&>::type
+{
+    if constexpr (MULTI) return PhiloxSeed{ static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32) };
+    else return keys0;
+}
+
+// MULTI = false: one run (run0), generation in run0.a.gen, the seed's round keys
+// in keys0.  MULTI = true: the runs of a device table, whose items are numbered
+// consecutively, the generation read from gen_dev, and what the runs have in
+// common (operators, precision, d_0) in run0.a.
+template <bool MULTI, bool W32, int MUT, bool SHADOW>
+__global__ void __launch_bounds__(32 * kWarps, 1)
+breed_kernel(const __grid_constant__ BreedRun run0, const __grid_constant__ PhiloxKeys keys0,
+             const BreedRun* __restrict__ runs, int32_t n_runs, int64_t n_items, const uint32_t* __restrict__ gen_dev,
+             unsigned int* __restrict__ status)
+{
+    extern __shared__ __align__(128) uint8_t smem_raw[];
     ptx::grid_dep_launch();  // the evaluation that follows may stage its batch meanwhile
     ptx::grid_dep_wait();    // the selection comes from the previous kernel
-    using S = BreedShape<MULTI>;
-    constexpr int kStages = S::kStages, kConsumerWarps = S::kConsumerWarps, kChunk = S::kChunk;
-    constexpr uint32_t kChunkBytes = S::kChunkBytes;
-    const BreedSmem s = carve<MULTI>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // Items of this CTA: many runs, a contiguous range; one run, every gridDim.x-th
-    // (neighbouring CTAs then work on neighbouring children, which share parents in L2).
-    const int64_t it_begin = MULTI ? n_items * blockIdx.x / gridDim.x : blockIdx.x;
-    const int64_t it_end = MULTI ? n_items * (blockIdx.x + 1) / gridDim.x : n_items;
-    const int64_t it_step = MULTI ? 1 : gridDim.x;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kStages; ++i) {
-            ptx::mbar_init(&s.full[i], 1);
-            ptx::mbar_init(&s.empty[i], kConsumerWarps);
-        }
-        *s.abort_flag = 0;
+    WarpSmem& s = reinterpret_cast<WarpSmem*>(smem_raw)[warp];
+    volatile int* abort_flag = &s.abort;
+    if (lane == 0) {
+        ptx::mbar_init(&s.full[0], 1);
+        ptx::mbar_init(&s.full[1], 1);
+        s.abort = 0;
         ptx::fence_mbar_init();
     }
-    __syncthreads();
-
-    if (warp == 0) {
-        // ------------------------------------------------------------ producer
-        // The warp resolves 32 items at a time (lane l: the item's child,
-        // kind, parents, scale and sigma; loads of all lanes in flight
-        // together), then lane 0 streams their parent chunks into the ring.
-        uint32_t stage = 0, phase = 0;
-        uint32_t issued_mask = 0, parity_mask = 0;  // per stage: issued at all / parity of the last issue
-        bool ok = true;
-        for (int64_t base = it_begin; ok && base < it_end; base += 32 * it_step) {
-            {
-                const int64_t it = base + lane * it_step;
-                ItemSrc src{};
-                src.m.kind = kKindInvalid;
-                src.m.len = 0;
-                if (it < it_end) {
-                    const int32_t ri = MULTI ? run_of_item(runs, n_runs, it) : 0;
-                    const BreedRun& R = MULTI ? runs[ri] : run0;
-                    const BreedArgs& a = R.a;
-                    const int64_t li = it - R.item0;
-                    // One run: chunk-major (all children's chunk 0, then chunk
-                    // 1, ...), so the parents' chunk (pool x 16 KB) stays in L2
-                    // while every child that reads it is made: each parent
-                    // chunk comes from HBM about once however many children
-                    // share it.  Many runs: child-major within each CTA's
-                    // contiguous range.
-                    const int32_t ci = MULTI ? static_cast<int32_t>(li / R.chunks) : static_cast<int32_t>(li % a.pop);
-                    const int32_t ck = MULTI ? static_cast<int32_t>(li - static_cast<int64_t>(ci) * R.chunks)
-                                             : static_cast<int32_t>(li / a.pop);
-                    // Front (elites, crossover) and back (mutation) children
-                    // alternate along a CTA's items; with an even grid a CTA's
-                    // ci keep one parity, so alternate rounds swap ci with its
-                    // pair partner (a bijection on each chunk's children).
-                    int32_t x = ci;
-                    if (!MULTI && (gridDim.x & 1u) == 0u) {
-                        const int32_t y = ci ^ static_cast<int32_t>((static_cast<uint32_t>(ci) / gridDim.x) & 1u);
-                        if (y < a.pop) x = y;
-                    }
-                    const int32_t j = (x & 1) ? a.pop - 1 - (x >> 1) : (x >> 1);
-                    int32_t kind = R.kind[j];
-                    const int32_t p1 = R.par1[j], p2 = R.par2[j];
-                    const int32_t n_par = a.n_parents > 0 ? a.n_parents : a.pop;
-                    if (p1 < 0 || p1 >= n_par || p2 < 0 || p2 >= n_par) kind = kKindInvalid;
-                    const int64_t g0 = static_cast<int64_t>(ck) * kChunk;
-                    const int32_t len = static_cast<int32_t>(a.c_pad - g0 < kChunk ? a.c_pad - g0 : kChunk);
-                    src.m = StageMeta{ j, kind, static_cast<int32_t>(g0), len,
-                                       (a.precision == 2) ? a.scale_exp[j] : 0, ri,
-                                       a.sigma_child ? a.sigma_child[j] : a.sigma, 0 };
-                    if (kind != kKindInvalid) {
-                        src.p1 = R.parents + static_cast<int64_t>(p1) * a.c_pad + g0;
-                        src.p2 = R.parents + static_cast<int64_t>(p2) * a.c_pad + g0;
-                    }
-                }
-                s.batch[lane] = src;
+    const BreedArgs& a = run0.a;
+    const int64_t it0 = static_cast<int64_t>(warp) * gridDim.x + blockIdx.x;
+    const int64_t step = static_cast<int64_t>(kWarps) * gridDim.x;
+    const uint32_t gen = MULTI ? *gen_dev : a.gen;
+    const uint32_t lim_mut = mask_limit(a.thr_mut), lim_xo = mask_limit(a.thr_xo);
+    uint32_t loads = 0, done = 0;  // sparse mutation items whose parent was asked for / that are finished
+    bool ok = true;
+    // Asks for the parent of item l of the batch, if it is a sparse mutation
+    // child, in the next of the two buffers (one thread; its earlier store
+    // from that buffer has been read by then).
+    auto load_ahead = [&](int l) {
+        const Item& m = s.items[l];
+        if (m.kind != 2) return;
+        const uint32_t bytes = 32u * min(m.n_units, 32u * kUnits), b = loads++ & 1u;
+        ptx::bulk_wait_read<0>();
+        ptx::mbar_arrive_expect_tx(&s.full[b], bytes);
+        ptx::bulk_load(s.buf[b], m.pa, bytes, &s.full[b]);
+    };
+    for (int64_t base = it0; ok && base < n_items; base += 32 * step) {
+        __syncwarp();
+        {
+            const int64_t it = base + lane * step;
+            if (it < n_items) {
+                if (MULTI) resolve_item(runs[run_of_item(runs, n_runs, it)], it, &s.items[lane]);
+                else resolve_item(run0, it, &s.items[lane]);
             }
-            __syncwarp();
-            if (lane == 0) {
-                for (int l = 0; l < 32 && base + l * it_step < it_end; ++l) {
-                    if (!ptx::mbar_wait_bounded(&s.empty[stage], phase ^ 1u, s.abort_flag, kWaitLimitNs)) {
-                        raise_abort(s.abort_flag, status);
-                        ok = false;
-                        break;
-                    }
-                    const ItemSrc src = s.batch[l];
-                    s.meta[stage] = src.m;
-                    const uint32_t bytes = static_cast<uint32_t>(src.m.len) * 4u;
-                    if (src.m.kind == kKindInvalid) {
-                        ptx::mbar_arrive(&s.full[stage]);
-                    } else {
-                        const bool two = (src.m.kind == 1);
-                        ptx::mbar_arrive_expect_tx(&s.full[stage], two ? 2u * bytes : bytes);
-                        ptx::bulk_load(stage_a(s, stage, kChunkBytes), src.p1, bytes, &s.full[stage]);
-                        if (two) ptx::bulk_load(stage_b(s, stage, kChunkBytes), src.p2, bytes, &s.full[stage]);
-                    }
-                    issued_mask |= 1u << stage;
-                    parity_mask = (parity_mask & ~(1u << stage)) | (phase << stage);
-                    if (++stage == kStages) { stage = 0; phase ^= 1u; }
-                }
-            }
-            ok = __shfl_sync(0xFFFFFFFFu, ok, 0);  // also: lane 0 is done with the batch
         }
-        if (!ok && lane == 0) {  // let copies in flight land before the CTA exits
-            volatile int never = 0;
-            for (int i = 0; i < kStages; ++i)
-                if (issued_mask & (1u << i))
-                    ptx::mbar_wait_bounded(&s.full[i], (parity_mask >> i) & 1u, &never, kDrainLimitNs);
-        }
-    } else {
-        // ------------------------------------------------------------ consumers
-        const int ct = threadIdx.x - 32;
-        const uint32_t gen = MULTI ? *gen_dev : run0.a.gen;
-        PhiloxKeys key = philox_keys(run0.a.seed);
-        // The current run's arguments and generator keys, held in registers
-        // while consecutive items belong to the same run (many runs: the
-        // table lives in global memory).
-        BreedArgs a = run0.a;
-        float* children = run0.children;
-        int32_t cur_run = MULTI ? -1 : 0;
-        uint32_t stage = 0, phase = 0;
-        for (int64_t it = it_begin; it < it_end; it += it_step) {
-            if (!ptx::mbar_wait_bounded(&s.full[stage], phase, s.abort_flag, kWaitLimitNs)) {
-                raise_abort(s.abort_flag, status);
-                break;
-            }
-            const StageMeta m = s.meta[stage];
-            if (MULTI && m.run != cur_run) {
-                a = runs[m.run].a;
-                children = runs[m.run].children;
-                key = philox_keys(a.seed);
-                cur_run = m.run;
-            }
-            const float4* A = reinterpret_cast<const float4*>(stage_a(s, stage, kChunkBytes));
-            const float4* B = reinterpret_cast<const float4*>(stage_b(s, stage, kChunkBytes));
-            float4* O = reinterpret_cast<float4*>(children + static_cast<int64_t>(m.j) * a.c_pad + m.g0);
-            const uint32_t j = a.entity ? a.entity[m.j] : static_cast<uint32_t>(m.j);  // Philox entity
-            const bool live = ct * kGenesPerLane < m.len;
-            const uint32_t u = (static_cast<uint32_t>(m.g0) >> 3) + static_cast<uint32_t>(ct);  // 8-gene unit
-            float4 v[2] = { make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f) };
-            if (live && m.kind >= 0) {
-                v[0] = A[2 * ct];
-                v[1] = A[2 * ct + 1];
-            }
-            if (m.kind == 2) {
-                // Lanes of a warp own consecutive units: lane o owns u - lane + o.
-                const int cw = warp - 1;  // consumer warp
-                const uint32_t hit = live ? mask8(philox_keyed(make_uint4(u, j, gen, kTagMutMask), key), a.thr_mut) : 0u;
-                mutate8(m.sigma, gen, key, j, hit, v, lane, s.job_z + cw * kJobSlots, s.job_code + cw * kJobSlots,
-                        [&](uint32_t o) { return u - static_cast<uint32_t>(lane) + o; });
-            } else if (live && m.kind == 1) {
-                const float4 b0 = B[2 * ct], b1 = B[2 * ct + 1];
-                if (a.xo_op == 0) {
-                    const uint32_t msk = mask8(philox_keyed(make_uint4(u, j, gen, kTagXo), key), a.thr_xo);
-                    v[0] = select4(msk, v[0], b0);
-                    v[1] = select4(msk >> 4, v[1], b1);
-                } else {
-                    v[0] = mean4(v[0], b0);
-                    v[1] = mean4(v[1], b1);
-                }
-            } else if (m.kind == kKindInvalid) {
-                const float nan = __int_as_float(0x7FC00000);
-                v[0] = v[1] = make_float4(nan, nan, nan, nan);
-            }
-            if (live) {
-                const int64_t i0 = static_cast<int64_t>(m.g0) + kGenesPerLane * ct;
-                if (i0 + kGenesPerLane > a.c) {  // only a child's last chunk holds padding
-                    v[0] = clear_padding(v[0], i0, a.c);
-                    v[1] = clear_padding(v[1], i0 + 4, a.c);
-                }
-                O[2 * ct] = v[0];
-                O[2 * ct + 1] = v[1];
-            }
-            if (a.precision > 0 && static_cast<int64_t>(m.g0) < a.n_w1) {  // warp-uniform
-                const int64_t i0 = static_cast<int64_t>(m.g0) + kGenesPerLane * ct;
-                float mx = 0.0f;
-                if (live && i0 < a.n_w1) mx = write_shadow8(a, m.j, m.sexp, i0, v);
+        __syncwarp();
+        const int64_t left = (n_items - base + step - 1) / step;
+        const int n_here = left < 32 ? static_cast<int>(left) : 32;
+        if (MUT == kMutSparse && lane == 0) load_ahead(0);
+        for (int l = 0; l < n_here; ++l) {
+            const Item& m = s.items[l];
+            // One run: the round keys are kernel parameters (constant operands);
+            // many: each item's run has its own seed.
+            typename std::conditional<MULTI, PhiloxSeed, const PhiloxKeys&>::type key = item_key<MULTI>(m.seed, keys0);
+            const uint32_t ent = m.ent, u0 = m.u0, n_units = m.n_units;
+            const int32_t kind = m.kind;
+            float mx = 0.0f;
+            if (MUT == kMutSparse && kind == 2) {
+                // The parent's chunk is on its way into shared memory; the listed
+                // pairs are changed there and the chunk is stored from there.
+                uint32_t w[kUnits][4];
 #pragma unroll
-                for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
-                if (lane == 0 && mx > 0.0f) atomicMax(reinterpret_cast<int*>(a.amax_out + m.j), __float_as_int(mx));
+                for (int i = 0; i < kUnits; ++i) {
+                    const uint32_t ui = 32u * i + lane;
+                    const uint4 r = philox_keyed(make_uint4(u0 + ui, ent, gen, kTagMutMask), key);
+                    const uint32_t none = ui < n_units ? 0u : ~0u;
+                    w[i][0] = r.x | none;
+                    w[i][1] = r.y | none;
+                    w[i][2] = r.z | none;
+                    w[i][3] = r.w | none;
+                }
+                const uint32_t total = list_masked_pairs<kUnits>(w, lim_mut, lane, s.words, s.codes);
+                if (lane == 0 && l + 1 < n_here) load_ahead(l + 1);
+                const uint32_t b = done & 1u;
+                ok = __all_sync(0xFFFFFFFFu,
+                                ptx::mbar_wait_bounded(&s.full[b], (done >> 1) & 1u, abort_flag, kWaitLimitNs));
+                if (!ok) break;
+                ++done;
+                float* buf = s.buf[b];
+                const float sigma = m.sigma;
+                for (uint32_t job = static_cast<uint32_t>(lane); job < total; job += 32) {
+                    const uint32_t code = s.codes[job];
+                    const float2 z = listed_normals(code, u0, gen, key, ent);
+                    const uint32_t wd = s.words[code];
+                    float2 v = reinterpret_cast<float2*>(buf)[code];
+                    if (hit_lo(wd, lim_mut)) v.x = fmaf(sigma, z.x, v.x);
+                    if (hit_hi(wd, lim_mut)) v.y = fmaf(sigma, z.y, v.y);
+                    reinterpret_cast<float2*>(buf)[code] = v;
+                }
+                __syncwarp();
+                if (m.genes < kChunk) {
+                    for (int g = m.genes + lane; g < kChunk; g += 32)
+                        if (g >= 0) buf[g] = 0.0f;
+                    __syncwarp();
+                }
+                if (SHADOW) {
+#pragma unroll
+                    for (int i = 0; i < kUnits; ++i) {
+                        const uint32_t ui = 32u * i + lane;
+                        if (ui < m.w1_units) {
+                            const float4 lo = reinterpret_cast<const float4*>(buf)[2 * ui];
+                            const float4 hi = reinterpret_cast<const float4*>(buf)[2 * ui + 1];
+                            const float v[8] = { lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w };
+                            mx = fmaxf(mx, write_shadow8(a, m, u0 + ui, v));
+                        }
+                    }
+                }
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    ptx::bulk_store(m.child, buf, 32u * min(n_units, 32u * kUnits));
+                    ptx::bulk_commit();
+                }
+            } else {
+                if (MUT == kMutSparse && lane == 0 && l + 1 < n_here) load_ahead(l + 1);
+                const float *pa = m.pa + 8 * lane, *pb = m.pb + 8 * lane;
+                float* child = m.child + 8 * lane;
+                const float sigma = m.sigma;
+                const int32_t genes = m.genes;
+                // Padding, the child's genes and their shadow, unit i.
+                auto finish = [&](int i, float (&v)[8]) {
+                    const uint32_t ui = 32u * i + lane;
+                    if (genes < kChunk) {
+#pragma unroll
+                        for (int t = 0; t < 8; ++t)
+                            if (static_cast<int32_t>(8u * ui) + t >= genes) v[t] = 0.0f;
+                    }
+                    store8<W32>(child + 256 * i, v);
+                    if (SHADOW && ui < m.w1_units) mx = fmaxf(mx, write_shadow8(a, m, u0 + ui, v));
+                };
+                if (kind == 1) {
+                    float v[kUnits][8], p2[kUnits][8];
+#pragma unroll
+                    for (int i = 0; i < kUnits; ++i) {
+                        if (32u * i + lane < n_units) {
+                            load8<W32>(pa + 256 * i, v[i]);
+                            load8<W32>(pb + 256 * i, p2[i]);
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < kUnits; ++i) {
+                        if (a.xo_op == 0) {
+                            const uint4 r = philox_keyed(make_uint4(u0 + 32u * i + lane, ent, gen, kTagXo), key);
+                            if (a.thr_xo > 0u) cross8(r, lim_xo, v[i], p2[i]);
+                        } else {
+#pragma unroll
+                            for (int t = 0; t < 8; ++t) v[i][t] = 0.5f * (v[i][t] + p2[i][t]);
+                        }
+                        if (32u * i + lane < n_units) finish(i, v[i]);
+                    }
+                } else {
+#pragma unroll 1
+                    for (int i = 0; i < kUnits; ++i) {
+                        const uint32_t ui = 32u * i + lane, u = u0 + ui;
+                        if (ui >= n_units) break;
+                        float v[8];
+                        if (kind < 0) {
+#pragma unroll
+                            for (int t = 0; t < 8; ++t) v[t] = kind == kKindInvalid ? __int_as_float(0x7FC00000) : 0.0f;
+                        } else {
+                            load8<W32>(pa + 256 * i, v);
+                        }
+                        if (kind == 2 && MUT != kMutNone) {
+                            uint32_t w[4] = { 0u, 0u, 0u, 0u };
+                            if (MUT == kMutDense) {
+                                const uint4 r = philox_keyed(make_uint4(u, ent, gen, kTagMutMask), key);
+                                w[0] = r.x; w[1] = r.y; w[2] = r.z; w[3] = r.w;
+                            }
+                            mutate8_dense<MUT == kMutAll>(sigma, gen, key, ent, u, w, lim_mut, v);
+                        }
+                        finish(i, v);
+                    }
+                }
             }
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&s.empty[stage]);
-            if (++stage == kStages) { stage = 0; phase ^= 1u; }
+            if (SHADOW && m.w1_units > 0u) {
+                // Non-negative floats order as their bits.
+                const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mx));
+                if (lane == 0 && top > 0u) atomicMax(reinterpret_cast<int*>(m.amax), static_cast<int>(top));
+            }
         }
     }
-    __syncthreads();
+    if (!ok && lane == 0) {  // let the parents on their way land before the CTA exits
+        atomicOr(status, kStatusBreedTimeout);
+        volatile int never = 0;
+        for (; done < loads; ++done) ptx::mbar_wait_bounded(&s.full[done & 1u], (done >> 1) & 1u, &never, kDrainLimitNs);
+    }
+    if (MUT == kMutSparse && lane == 0) ptx::bulk_wait<0>();  // the stores have left shared memory and are done
 }
 
 }  // namespace
 
-int32_t breed_chunks(int64_t c_pad)
+int32_t breed_chunks(int64_t c_pad) { return static_cast<int32_t>((c_pad + kChunk - 1) / kChunk); }
+
+uint32_t shadow_row_mul(int32_t k)
 {
-    return static_cast<int32_t>((c_pad + BreedShape<true>::kChunk - 1) / BreedShape<true>::kChunk);
+    // floor(u mul / 2^32) = u / (k / 8) for u < 2^32 / (k / 8): W1 has fewer units.
+    return static_cast<uint32_t>((uint64_t{1} << 32) / (static_cast<uint32_t>(k) / 8u)) + 1u;
 }
 
 namespace {
@@ -413,6 +431,35 @@ cudaError_t breed_grid(int64_t items, int* grid)
     return cudaSuccess;
 }
 
+typedef void (*BreedKernel)(const BreedRun, const PhiloxKeys, const BreedRun*, int32_t, int64_t, const uint32_t*,
+                            unsigned int*);
+
+template <bool MULTI, bool W32, bool SHADOW>
+BreedKernel breed_kernel_mut(MutMode mode)
+{
+    switch (mode) {
+    case kMutNone: return breed_kernel<MULTI, W32, kMutNone, SHADOW>;
+    case kMutSparse: return breed_kernel<MULTI, W32, kMutSparse, SHADOW>;
+    case kMutDense: return breed_kernel<MULTI, W32, kMutDense, SHADOW>;
+    default: return breed_kernel<MULTI, W32, kMutAll, SHADOW>;
+    }
+}
+
+PhiloxKeys host_philox_keys(uint64_t seed)
+{
+    PhiloxKeys k;
+    uint32_t a = static_cast<uint32_t>(seed), b = static_cast<uint32_t>(seed >> 32);
+    for (int r = 0; r < 10; ++r) {
+        k.k0[r] = a;
+        k.k1[r] = b;
+        a += kPhiloxW0;
+        b += kPhiloxW1;
+    }
+    return k;
+}
+
+constexpr size_t kBreedSmem = sizeof(WarpSmem) * kWarps;
+
 }  // namespace
 
 cudaError_t launch_breed(const BreedArgs& a, const float* parents, const int32_t* par1, const int32_t* par2,
@@ -425,32 +472,36 @@ cudaError_t launch_breed(const BreedArgs& a, const float* parents, const int32_t
     r.par2 = par2;
     r.kind = kind;
     r.children = children;
-    r.chunks = static_cast<int32_t>((a.c_pad + BreedShape<false>::kChunk - 1) / BreedShape<false>::kChunk);
+    r.chunks = breed_chunks(a.c_pad);
     r.item0 = 0;
     const int64_t items = static_cast<int64_t>(a.pop) * r.chunks;
     int grid = 0;
     cudaError_t err = breed_grid(items, &grid);
     if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(breed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(breed_smem_bytes<false>()));
+    const bool w32 = ((reinterpret_cast<uintptr_t>(parents) | reinterpret_cast<uintptr_t>(children)) & 31u) == 0;
+    const MutMode mode = mut_mode(a.thr_mut);
+    // Shadows belong to library-owned populations, which are 32-byte aligned.
+    const BreedKernel kernel = a.precision > 0 ? breed_kernel_mut<false, true, true>(mode)
+                                               : (w32 ? breed_kernel_mut<false, true, false>(mode)
+                                                      : breed_kernel_mut<false, false, false>(mode));
+    err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBreedSmem));
     if (err != cudaSuccess) return err;
-    return launch_pdl(breed_kernel<false>, dim3(grid), dim3(BreedShape<false>::kThreads), breed_smem_bytes<false>(),
-                      stream, r,
+    return launch_pdl(kernel, dim3(grid), dim3(32 * kWarps), kBreedSmem, stream, r, host_philox_keys(a.seed),
                       static_cast<const BreedRun*>(nullptr), 1, items, static_cast<const uint32_t*>(nullptr), status);
 }
 
-cudaError_t launch_breed_runs(const BreedRun* runs_dev, int32_t n_runs, int64_t n_items, const uint32_t* gen_dev,
-                              unsigned int* status, cudaStream_t stream)
+cudaError_t launch_breed_runs(const BreedArgs& common, const BreedRun* runs_dev, int32_t n_runs, int64_t n_items,
+                              const uint32_t* gen_dev, unsigned int* status, cudaStream_t stream)
 {
     int grid = 0;
     cudaError_t err = breed_grid(n_items, &grid);
     if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(breed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(breed_smem_bytes<true>()));
+    const BreedKernel kernel = breed_kernel_mut<true, true, true>(mut_mode(common.thr_mut));
+    err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBreedSmem));
     if (err != cudaSuccess) return err;
-    const BreedRun none{};
-    breed_kernel<true><<<grid, BreedShape<true>::kThreads, breed_smem_bytes<true>(), stream>>>(
-        none, runs_dev, n_runs, n_items, gen_dev, status);
+    BreedRun r{};
+    r.a = common;
+    kernel<<<grid, 32 * kWarps, kBreedSmem, stream>>>(r, PhiloxKeys{}, runs_dev, n_runs, n_items, gen_dev, status);
     return cudaGetLastError();
 }
 

@@ -1214,6 +1214,7 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
                 a.precision = prec;
                 a.n_w1 = static_cast<int64_t>(s->net.dims[0]) * s->net.dims[1];
                 a.sh_k = s->net.dims[0];
+                a.sh_row_mul = shadow_row_mul(a.sh_k);
                 a.sh_h = s->net.dims[1];
                 a.shadow = s->shadow[s->cur ^ 1];
                 a.sh_stride = s->sh_stride;

@@ -80,6 +80,7 @@ struct BreedArgs {
     int32_t precision;        // 1 BF16, 2 FP8-e4m3 scaled by 2^scale_exp[child]
     int64_t n_w1;             // multiple of 8
     int32_t sh_k, sh_h;       // d_0 and h: W1 is sh_h rows of sh_k
+    uint32_t sh_row_mul;      // shadow_row_mul(sh_k)
     uint8_t* shadow;          // child j's shadow at shadow + j * sh_stride (tiled, see shadow_offset)
     int64_t sh_stride;        // bytes, multiple of 128
     const int32_t* scale_exp;
@@ -153,10 +154,14 @@ struct BreedRun {
     int32_t chunks;      // work items per child
     int64_t item0;       // first of the run's pop * chunks items in the global list
 };
-cudaError_t launch_breed_runs(const BreedRun* runs_dev, int32_t n_runs, int64_t n_items, const uint32_t* gen_dev,
-                              unsigned int* status, cudaStream_t stream);
+// common: any run's arguments (the runs share the operators, the precision and
+// d_0).  Every run's populations are 32-byte aligned (cudaMalloc).
+cudaError_t launch_breed_runs(const BreedArgs& common, const BreedRun* runs_dev, int32_t n_runs, int64_t n_items,
+                              const uint32_t* gen_dev, unsigned int* status, cudaStream_t stream);
 // Items (chunks of genes) per child of a net with c_pad padded genes.
 int32_t breed_chunks(int64_t c_pad);
+// Multiplier whose high product with a unit of 8 genes of W1 is its row (d_0 = k, a multiple of 16).
+uint32_t shadow_row_mul(int32_t k);
 // Precision form: shadows of W1 for a whole population from its FP32 master
 // (exact max |W1| per individual, FP8 exponents from it).
 cudaError_t launch_make_shadow(int32_t pop, int32_t k, int32_t h, int64_t c_pad, const float* pop_dev,

@@ -48,6 +48,7 @@ struct leea_multi {
     cudaStream_t stream = nullptr;
     std::vector<RunBuf> runs;
     int64_t total_rows = 0, total_pop = 0, breed_items = 0;
+    BreedArgs breed_common{};  // what the runs' breeding has in common
     int32_t h_max = 0, cw_max = 0, pop_max = 0, eval_grid = 0;
     bool any_tiles = false;
     // The group evaluation (several individuals per MMA) when every run fits
@@ -185,6 +186,7 @@ cudaError_t build_step_tables(leea_multi* m, int c)
         b.a.n_w1 = static_cast<int64_t>(r.net.dims[0]) * r.net.dims[1];
         b.a.sh_k = r.net.dims[0];
         b.a.sh_h = r.net.dims[1];
+        b.a.sh_row_mul = shadow_row_mul(r.net.dims[0]);
         b.a.shadow = r.shadow[c ^ 1];
         b.a.sh_stride = r.sh_stride;
         b.a.scale_exp = r.scale_exp;
@@ -203,6 +205,7 @@ cudaError_t build_step_tables(leea_multi* m, int c)
         item += static_cast<int64_t>(br[i].a.pop) * br[i].chunks;
     }
     m->breed_items = item;
+    m->breed_common = br[0].a;
     cudaError_t err = upload(&m->sel_tab[c], sel);
     if (err == cudaSuccess) err = upload(&m->breed_tab[c], br);
     return err;
@@ -298,7 +301,7 @@ cudaError_t enqueue_step(leea_multi* m, int c, unsigned int* status, bool events
     if (err != cudaSuccess) return err;
     mark(0, 1);
     mark(1, 0);
-    err = launch_breed_runs(m->breed_tab[c], m->n_runs, m->breed_items, m->gen_dev, status, stream);
+    err = launch_breed_runs(m->breed_common, m->breed_tab[c], m->n_runs, m->breed_items, m->gen_dev, status, stream);
     if (err != cudaSuccess) return err;
     mark(1, 1);
     mark(2, 0);

@@ -353,6 +353,7 @@ BreedArgs surr_breed_args(leea_surr* s, int32_t n, const uint32_t* entity, uint8
         a.precision = 1;
         a.n_w1 = static_cast<int64_t>(s->net.dims[0]) * s->net.dims[1];
         a.sh_k = s->net.dims[0];
+        a.sh_row_mul = shadow_row_mul(a.sh_k);
         a.sh_h = s->net.dims[1];
         a.shadow = shadow;
         a.sh_stride = s->sh_stride;
