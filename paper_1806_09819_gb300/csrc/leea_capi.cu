@@ -259,7 +259,10 @@ leea_status dispatch_eval_u8(const NetLayout& net, int32_t pop, const float* pop
         }
         return LEEA_OK;
     }
-    const bool tc_ok = eval_u8_tc_supported(net, batch, pop_dev);
+    // AUTO also takes the tensor cores where TENSOR does not promise them
+    // (batches above 128, h up to 256 and not a multiple of 16).
+    const bool tc_ok = path == LEEA_EVAL_TENSOR ? eval_u8_tc_supported(net, pop, batch, pop_dev)
+                                                : eval_u8_wide_supported(net, pop, batch, pop_dev);
     if (path == LEEA_EVAL_TENSOR && !tc_ok)
         return fail(LEEA_EINVAL, "tensor-core evaluation of 8-bit inputs needs batch <= 128, d_0 %% 4 == 0, "
                                  "h %% 16 == 0, h <= 128, d_out <= 16 and a 16-byte aligned population");
@@ -267,9 +270,10 @@ leea_status dispatch_eval_u8(const NetLayout& net, int32_t pop, const float* pop
     if (tc_ok && path != LEEA_EVAL_SIMT) {
         unsigned int* status = device_status_ptr();
         if (!status) return fail(LEEA_ECUDA, "device status word unavailable");
-        void* own = nullptr;  // the call's own FP16 batch, freed in stream order after the evaluation
+        void* own = nullptr;  // the call's own scratch, freed in stream order after the evaluation
         if (!x16) {
-            LEEA_CUDA_TRY(cudaMallocAsync(&own, eval_u8_x16_bytes(net, batch), stream), "batch staging allocation");
+            LEEA_CUDA_TRY(cudaMallocAsync(&own, eval_u8_scratch_bytes(net, pop, batch), stream),
+                          "batch staging allocation");
             x16 = own;
             x16_staged = false;
         }
@@ -773,8 +777,9 @@ struct leea_state {
     void* mlp_scratch;
     size_t mlp_scratch_bytes;
     // tensor-core evaluation of d_0-h-d_out nets on 8-bit inputs: the batch as
-    // FP16 (at most 128 samples), staged once per generation
+    // FP16, staged once per generation, and several tiles' sums (grown with the batch)
     void* x16;
+    size_t x16_bytes;
     // precision form: the batch as the pair kernel's operand tiles (grown with the batch)
     void* xop;
     size_t xop_bytes;
@@ -953,8 +958,10 @@ leea_status leea_create(int32_t pop, const int32_t* dims, int32_t n_dims, const 
         err = cudaMalloc(&s->mlp_scratch, s->mlp_scratch_bytes);
     }
     if (s->net.n_layers == 2 && p->precision == 0 && err == cudaSuccess &&
-        eval_u8_tc_supported(s->net, 128, s->popbuf[0]))
-        err = cudaMalloc(&s->x16, eval_u8_x16_bytes(s->net, 128));
+        eval_u8_tc_supported(s->net, pop, 128, s->popbuf[0])) {
+        s->x16_bytes = eval_u8_scratch_bytes(s->net, pop, 128);  // grown with the batch
+        err = cudaMalloc(&s->x16, s->x16_bytes);
+    }
     if (p->sigma_ctl == LEEA_SIGMA_SELF) {
         for (int b = 0; b < 2 && err == cudaSuccess; ++b) err = cudaMalloc(&s->sigma[b], sizeof(float) * np);
         if (err == cudaSuccess) {  // every individual starts with the sigma gene p->sigma
@@ -1156,8 +1163,22 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
                                     u8 ? nullptr : static_cast<const float*>(x_dev), u8 ? x_div : 1.0f, y_dev, batch);
     // The tensor-core evaluation of 8-bit inputs reads the batch as FP16: a
     // breeding generation stages it beside the selection.
-    const bool stage_early = !first && !fused && u8 && prec == 0 && s->x16 && s->prm.eval_path != LEEA_EVAL_SIMT &&
-                             s->net.n_layers == 2 && eval_u8_tc_supported(s->net, batch, s->popbuf[0]);
+    const bool eval_u8_tc = !fused && u8 && prec == 0 && s->prm.eval_path != LEEA_EVAL_SIMT && s->net.n_layers == 2 &&
+                            (s->prm.eval_path == LEEA_EVAL_TENSOR
+                                 ? eval_u8_tc_supported(s->net, s->pop, batch, s->popbuf[0])
+                                 : eval_u8_wide_supported(s->net, s->pop, batch, s->popbuf[0]));
+    if (eval_u8_tc) {
+        const size_t need = eval_u8_scratch_bytes(s->net, s->pop, batch);
+        if (need > s->x16_bytes) {
+            LEEA_CUDA_TRY(cudaStreamSynchronize(s->stream), "staging sync");
+            cudaFree(s->x16);
+            s->x16 = nullptr;
+            s->x16_bytes = 0;
+            LEEA_CUDA_TRY(cudaMalloc(&s->x16, need), "batch staging allocation");
+            s->x16_bytes = need;
+        }
+    }
+    const bool stage_early = eval_u8_tc && !first;
     if (!first) {
         const uint32_t g = s->gen + 1;
         const float sigma_g = sigma_of_breed(s->prm, g);
@@ -1265,7 +1286,8 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
         else if (u8)
             st = dispatch_eval_u8(s->net, s->pop, s->popbuf[s->cur], static_cast<const uint8_t*>(x_dev), x_div, y_dev,
                                   batch, s->prm.alpha, first ? nullptr : s->f_inh, s->f_raw, s->f_adj, s->correct,
-                                  s->prm.eval_path, s->stream, s->mlp_scratch, s->x16, stage_early);
+                                  s->prm.eval_path, s->stream, s->mlp_scratch, eval_u8_tc ? s->x16 : nullptr,
+                                  stage_early);
         else
             st = dispatch_eval(s->net, s->pop, s->popbuf[s->cur], static_cast<const float*>(x_dev), y_dev, batch,
                                s->prm.alpha, first ? nullptr : s->f_inh, s->f_raw, s->f_adj, s->correct,

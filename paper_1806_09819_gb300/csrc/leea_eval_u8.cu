@@ -13,36 +13,49 @@
 // layer 1 with FP32 FFMA from global memory instead of the accumulator.
 //
 // Shape.  A tcgen05.mma of M = 128 and K = 16 costs about the same time for any
-// N up to 256, so two individuals share every MMA: the batch tile (<= 128
-// samples, the M side) is the A operand and the stacked W1 pieces of two
-// individuals (N = 2h) the B operand, and 2 x 49 MMAs evaluate a pair at
-// d_0 = 784.  The batch, staged once per evaluation as FP16 in global memory
-// (stage_x16_kernel; it stays in L2), arrives by TMA in K-stage tiles next to
-// the weights.  A K stage is 64 inputs (128-byte swizzled FP16 rows, 256-byte
-// FP32 rows) when three such stages fit in shared memory (h <= 112), else 32
-// (64-byte swizzle): the wider slices stream HBM faster (measured with no
-// compute: 4.8 against 4.0-4.4 TB/s for the same 351 MB).
+// N up to 256, so two individuals share every MMA where both fit (hp = h rounded
+// up to 16, 2 hp <= 256; rows past h arrive as zeros): a 128-sample tile of the
+// batch (the M side) is the A operand and the stacked W1 pieces of the
+// individuals (N = ni hp) the B operand.  The batch, staged once per evaluation
+// as FP16 in global memory (stage_x16_kernel; it stays in L2), arrives by TMA
+// in K-stage tiles next to the weights.  A batch of several tiles takes them
+// two per unit (TILES = 2), so that a weight slice is loaded and converted once
+// for both; the tiles' sums meet in scratch memory and are added in tile order.
+// A K stage is 64 inputs (128-byte swizzled FP16 rows, 256-byte FP32 rows) when
+// three such stages fit in shared memory, else 32 (64-byte swizzle): the wider
+// slices stream HBM faster (measured with no compute: 4.8 against 4.0-4.4 TB/s
+// for the same 351 MB).
+//
+// Measured, P = 1000, 784-112-10: batch 100 84 us (4.2 TB/s of weights; without
+// the epilogue's arithmetic 76), 256 124, 512 217, 1024 417, against 1.2 ms
+// (256) to 9.8 ms (1024) on the CUDA cores; 333 nets 784-100-10, batch 50: 37
+// (295).  Several tiles are bound by the weight stream (once per two tiles, the
+// repeats from L2) and by the epilogue, which cannot overlap the next unit when
+// the unit's accumulators take more than half of tensor memory (165 us at 512
+// without its arithmetic).
 //
 // Pipeline (persistent CTA, one per SM; each CTA takes a contiguous range of
-// individuals, as pairs, the last one alone when the range is odd):
+// individuals, as pairs, the last one alone when the range is odd, or of units,
+// see UnitWalk):
 //   warp 0      TMEM allocation and the single MMA-issuing thread
-//   warp 1      producer: per stage, one TMA of the batch tile (the batch's
-//               rows rounded up to 8, from L2) and one TMA per individual of
-//               its FP32 W1 slice.  A stage is [batch tile][slot 0][slot 1]:
-//               the MMA reads 128 rows of A, and rows past the tile fall on
-//               the slots' data, which only accumulator rows past the batch see
+//   warp 1      producer: per stage, one TMA per batch tile (a lone tile's rows
+//               rounded up to 8, from L2) and one TMA per individual of its
+//               FP32 W1 slice.  A stage is [batch tiles][slot 0][slot 1]: the
+//               MMA reads 128 rows of A, and rows past a lone tile fall on the
+//               slots' data, which only accumulator rows past the batch see
 //   warps 2-9   converters: each 8-row group of a raw FP32 slice is read by
 //               one warp and overwritten in place by its two FP16 pieces in
 //               the swizzled K-major layout (piece q in the group's q-th half,
 //               so the pieces of all 2h rows form two operands whose 8-row
 //               groups are one group apart); a warp reads the groups of a
 //               batch before it writes any of them
-//   warps 10-17 epilogue, 4 warps (one per TMEM lane quarter = 32 samples)
-//               per individual: while the unit's MMAs run, b1, W2 (transposed)
+//   warps 10-17 epilogue, two groups of 4 warps (one per TMEM lane quarter = 32
+//               samples), each with an individual or a tile of the unit: while the unit's MMAs run, b1, W2 (transposed)
 //               and b2 are loaded into shared memory; then bias, ReLU, layer
 //               2, softmax cross-entropy, fixed-order batch sum, inheritance
-//               blend; accumulators are double-buffered in TMEM (columns 0
-//               and 256), so a pair's epilogue overlaps the next pair's MMAs
+//               blend; accumulators of at most 256 columns are double-buffered
+//               in TMEM (columns 0 and 256), so a unit's epilogue overlaps the
+//               next unit's MMAs
 // Every mbarrier wait is bounded in time; on expiry the kernel sets
 // kStatusEvalTimeout, lets its copies and MMAs in flight finish and exits.
 #include <cuda.h>
@@ -65,6 +78,7 @@ constexpr int kU8Threads = 32 * (kFirstEpiWarp + kEpiWarps);
 constexpr int kMinStages = 3;
 constexpr int kMaxStages = 6;
 constexpr int kMaxOutU8 = 16;
+constexpr size_t kMaxScratchU8 = size_t{256} << 20;
 constexpr int kMaxGroups = 2 * 128 / 8;  // 8-row groups of the widest pair
 constexpr int kFlagSlots = 16;          // unit-tagged range flags; converters run at most a few units ahead
 constexpr uint32_t kTmemCols = 512;
@@ -88,10 +102,14 @@ struct StageShape {
 
 struct EvalU8Args {
     int32_t pop, k, h, d_out, dpad, batch, k16, k_stages, n_stages;
-    int32_t per_cta, extra;  // individuals per CTA: per_cta, one more for the first `extra` CTAs
-    uint32_t slot_bytes;     // one individual's slice of a stage: h raw rows
-    uint32_t a_bytes;        // the batch tile: round_up(batch, 8) rows of FP16 levels
-    uint32_t stage_bytes;    // the batch tile and two slots, rounded up to 1 KB
+    int32_t hp;              // hidden units rounded up to 16: the rows of a slot, the columns of an accumulator
+    int32_t ni;              // individuals per unit: 2, or 1 (hp > 128, or too few units for the SMs)
+    int32_t tiles, groups;   // 128-sample tiles of the batch; groups of TILES of them
+    int32_t n_bufs;          // accumulator buffers: 2 where a unit's columns fit twice
+    int32_t per_cta, extra;  // work per CTA: per_cta, one more for the first `extra` CTAs
+    uint32_t slot_bytes;     // one individual's slice of a stage: hp raw rows
+    uint32_t a_bytes;        // one batch tile: round_up(batch, 8) (or, with several tiles, 128) rows of FP16 levels
+    uint32_t stage_bytes;    // the batch tiles and the slots, rounded up to 1 KB
     int64_t c_pad;
     float inv_div, alpha;
     const float* popv;
@@ -101,25 +119,28 @@ struct EvalU8Args {
     float* f_raw;
     float* f_adj;
     int32_t* correct;
+    int32_t wide;            // sum the losses in FP64 (shapes beyond eval_u8_tc_supported)
+    double* part;            // several tiles: [tiles][pop] loss sums of the tiles,
+    int32_t* part_ok;        // and their correct counts
     unsigned int* status;
 };
 
 struct U8Smem {
     uint8_t* ring;       // n_stages x stage_bytes, 1024-aligned: the batch tile, then W1 slices (raw, then pieces)
-    float* w2t;          // [2 slots][h][dpad]
-    float* b1;           // [2 slots][h]
-    float* b2;           // [2 slots][16]
-    float* red_loss;     // [2 slots][4 quarters]
-    int32_t* red_ok;     // [2 slots][4 quarters]
+    float* w2t;          // [2 epilogue groups][hp][dpad]
+    float* b1;           // [2 groups][hp]
+    float* b2;           // [2 groups][16]
+    double* red_loss;    // [2 groups][2 tiles][4 quarters]
+    int32_t* red_ok;     // [2 groups][2 tiles][4 quarters]
     uint32_t* flag;      // [kFlagSlots][2]: u + 1 if unit u's individual in that slot has |w| >= 128
     uint32_t* accflag;   // [2]: the flags of the unit in that accumulator, for the epilogue
-    int* ep_go;          // [2 slots]: the epilogue groups' go words
+    int* ep_go;          // [2 groups]: their go words
     uint32_t* tmem_holder;
     volatile int* abort_flag;
     uint64_t *full, *a_full, *empty, *acc_full, *acc_empty, *drain;
 };
 
-constexpr size_t kTailFixed = sizeof(float) * 8 + sizeof(int32_t) * 8 + sizeof(uint32_t) * (2 * kFlagSlots + 2) +
+constexpr size_t kTailFixed = 8 + sizeof(double) * 16 + sizeof(int32_t) * 16 + sizeof(uint32_t) * (2 * kFlagSlots + 2) +
                               sizeof(int) * 2 + 16 + 16;
 
 size_t u8_tail_bytes(int32_t h, int32_t dpad, int32_t n_stages)
@@ -133,15 +154,16 @@ __device__ __forceinline__ U8Smem carve(uint8_t* raw, const EvalU8Args& a)
     s.ring = raw + ((1024u - (ptx::smem_u32(raw) & 1023u)) & 1023u);
     uint8_t* p = s.ring + static_cast<size_t>(a.n_stages) * a.stage_bytes;
     s.w2t = reinterpret_cast<float*>(p);
-    p += sizeof(float) * 2 * a.h * a.dpad;
+    p += sizeof(float) * 2 * a.hp * a.dpad;
     s.b1 = reinterpret_cast<float*>(p);
-    p += sizeof(float) * 2 * a.h;
+    p += sizeof(float) * 2 * a.hp;
     s.b2 = reinterpret_cast<float*>(p);
     p += sizeof(float) * 32;
-    s.red_loss = reinterpret_cast<float*>(p);
-    p += sizeof(float) * 8;
+    p += (8u - (ptx::smem_u32(p) & 7u)) & 7u;
+    s.red_loss = reinterpret_cast<double*>(p);
+    p += sizeof(double) * 16;
     s.red_ok = reinterpret_cast<int32_t*>(p);
-    p += sizeof(int32_t) * 8;
+    p += sizeof(int32_t) * 16;
     s.flag = reinterpret_cast<uint32_t*>(p);
     p += sizeof(uint32_t) * 2 * kFlagSlots;
     s.accflag = reinterpret_cast<uint32_t*>(p);
@@ -162,38 +184,43 @@ __device__ __forceinline__ U8Smem carve(uint8_t* raw, const EvalU8Args& a)
     return s;
 }
 
+// How a population and a batch are cut into units.
+struct U8Shape {
+    int32_t hp, ni, tiles_per_unit, ks, n_stages;
+};
+
 uint32_t u8_a_bytes(int32_t batch, int32_t ks)
 {
-    return static_cast<uint32_t>((batch + 7) / 8 * 8) * 2u * static_cast<uint32_t>(ks);
+    return static_cast<uint32_t>(batch > 128 ? 128 : (batch + 7) / 8 * 8) * 2u * static_cast<uint32_t>(ks);
 }
 
-// A stage holds the batch tile and two slots, and at least the 128 rows of A
+// A stage holds the batch tiles and the slots, and at least the 128 rows of A
 // the MMA reads from its start.
-uint32_t u8_stage_bytes(int32_t h, int32_t batch, int32_t ks)
+uint32_t u8_stage_bytes(const U8Shape& u, int32_t batch)
 {
-    const uint32_t b = u8_a_bytes(batch, ks) + 2u * static_cast<uint32_t>(h) * 4u * static_cast<uint32_t>(ks);
-    return std::max((b + 1023u) & ~1023u, 128u * 2u * static_cast<uint32_t>(ks));
+    const uint32_t ks = static_cast<uint32_t>(u.ks);
+    const uint32_t b = static_cast<uint32_t>(u.tiles_per_unit) * u8_a_bytes(batch, u.ks) +
+                       static_cast<uint32_t>(u.ni) * static_cast<uint32_t>(u.hp) * 4u * ks;
+    return std::max((b + 1023u) & ~1023u, 128u * 2u * ks);
 }
 
-size_t u8_smem_bytes(int32_t h, int32_t d_out, int32_t batch, int32_t ks, int32_t n_stages)
+size_t u8_smem_bytes(const U8Shape& u, int32_t d_out, int32_t batch)
 {
     const int32_t dpad = (d_out + 3) / 4 * 4;
-    return 1024 + static_cast<size_t>(n_stages) * u8_stage_bytes(h, batch, ks) + u8_tail_bytes(h, dpad, n_stages);
+    return 1024 + static_cast<size_t>(u.n_stages) * u8_stage_bytes(u, batch) + u8_tail_bytes(u.hp, dpad, u.n_stages);
 }
 
-// The deepest ring of K stage `ks` that fits in 227 KB of shared memory; 0 if
-// not even kMinStages do.
-int32_t u8_stages(int32_t h, int32_t d_out, int32_t batch, int32_t ks)
+// K stage and ring depth: 64 inputs when at least kMinStages such stages fit in
+// 227 KB of shared memory, else 32; false if neither fits.
+bool u8_ring(U8Shape* u, int32_t d_out, int32_t batch)
 {
-    for (int32_t ns = kMaxStages; ns >= kMinStages; --ns)
-        if (u8_smem_bytes(h, d_out, batch, ks, ns) <= 227u * 1024u) return ns;
-    return 0;
-}
-
-// K stage of a net: 64 inputs when kMinStages of them fit, else 32 (0: neither).
-int32_t u8_kstage(int32_t h, int32_t d_out, int32_t batch)
-{
-    return u8_stages(h, d_out, batch, 64) > 0 ? 64 : (u8_stages(h, d_out, batch, 32) > 0 ? 32 : 0);
+    for (int32_t ks : { 64, 32 })
+        for (int32_t ns = kMaxStages; ns >= kMinStages; --ns) {
+            u->ks = ks;
+            u->n_stages = ns;
+            if (u8_smem_bytes(*u, d_out, batch) <= 227u * 1024u) return true;
+        }
+    return false;
 }
 
 __device__ __forceinline__ void raise_abort(const U8Smem& s, const EvalU8Args& a)
@@ -242,15 +269,47 @@ __device__ __forceinline__ void put_pieces(uint8_t* group, int r, int c4, const 
     *reinterpret_cast<uint2*>(group + S::kPieceOff + off) = make_uint2(lo[1], hi[1]);
 }
 
-// This CTA's individuals: [first, first + count).
-__device__ __forceinline__ void cta_range(const EvalU8Args& a, int& first, int& count)
-{
-    const int b = static_cast<int>(blockIdx.x);
-    first = b * a.per_cta + min(b, a.extra);
-    count = a.per_cta + (b < a.extra ? 1 : 0);
-}
+// Unit u of this CTA: individuals [p0, p0 + n) on the tiles [t0, t0 + nt).
+// One group of tiles: every CTA takes a contiguous range of individuals, ni at
+// a time (the last unit may be smaller), so that the load stays even to one
+// individual.  Several groups: a contiguous range of (ni individuals, group)
+// units, the groups of the same individuals in a row, so that all but the
+// first find their weights in L2.
+struct Unit {
+    int p0, n, t0, nt;
+};
 
-template <int KS>
+template <int TILES>
+struct UnitWalk {
+    int first, count, u = 0;
+    __device__ __forceinline__ explicit UnitWalk(const EvalU8Args& a)
+    {
+        const int b = static_cast<int>(blockIdx.x);
+        first = b * a.per_cta + min(b, a.extra);
+        count = a.per_cta + (b < a.extra ? 1 : 0);
+    }
+    __device__ __forceinline__ bool next(const EvalU8Args& a, Unit& x)
+    {
+        if (a.groups == 1) {
+            if (a.ni * u >= count) return false;
+            x.p0 = first + a.ni * u;
+            x.n = min(a.ni, count - a.ni * u);
+            x.t0 = 0;
+            x.nt = a.tiles;
+        } else {
+            if (u >= count) return false;
+            const int id = first + u, blk = id / a.groups;
+            x.p0 = blk * a.ni;
+            x.n = min(a.ni, a.pop - x.p0);
+            x.t0 = (id - blk * a.groups) * TILES;
+            x.nt = min(TILES, a.tiles - x.t0);
+        }
+        ++u;
+        return true;
+    }
+};
+
+template <int KS, int TILES>
 __global__ void __launch_bounds__(kU8Threads, 1)
 eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                const EvalU8Args a)
@@ -259,8 +318,11 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     const U8Smem s = carve(smem_raw, a);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int first = 0, count = 0;
-    cta_range(a, first, count);
+    const uint32_t slots_off = TILES * a.a_bytes;          // the slots within a stage
+    const uint32_t tile_cols = static_cast<uint32_t>(a.ni * a.hp);  // a tile's accumulator columns
+    // Accumulator buffer and phase of unit u.
+    auto buf_of = [&](int u) { return a.n_bufs == 2 ? static_cast<uint32_t>(u) & 1u : 0u; };
+    auto phase_of = [&](int u) { return (a.n_bufs == 2 ? static_cast<uint32_t>(u) >> 1 : static_cast<uint32_t>(u)) & 1u; };
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < a.n_stages; ++i) {
@@ -290,23 +352,23 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     if (warp == 0) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            const uint32_t idesc1 = ptx::idesc_f16(128, static_cast<uint32_t>(a.h));
-            const uint32_t idesc2 = ptx::idesc_f16(128, 2u * static_cast<uint32_t>(a.h));
+            const uint32_t idesc1 = ptx::idesc_f16(128, static_cast<uint32_t>(a.hp));
+            const uint32_t idesc2 = ptx::idesc_f16(128, 2u * static_cast<uint32_t>(a.hp));
             const uint32_t ring = ptx::smem_u32(s.ring);
             uint32_t stage = 0, phase = 0;
             bool ok = true;
-            for (int u = 0; ok && 2 * u < count; ++u) {
-                const int n = min(2, count - 2 * u);
-                const uint32_t buf = static_cast<uint32_t>(u) & 1u;
-                if (!ptx::mbar_wait_bounded(&s.acc_empty[buf], ((static_cast<uint32_t>(u) >> 1) & 1u) ^ 1u,
-                                            s.abort_flag, kWaitLimitNs)) {
+            UnitWalk<TILES> walk(a);
+            Unit x;
+            for (int u = 0; ok && walk.next(a, x); ++u) {
+                const uint32_t buf = buf_of(u);
+                if (!ptx::mbar_wait_bounded(&s.acc_empty[buf], phase_of(u) ^ 1u, s.abort_flag, kWaitLimitNs)) {
                     raise_abort(s, a);
                     ok = false;
                     break;
                 }
                 ptx::tc_fence_after();
                 const uint32_t d = tmem_base + buf * kAccStride;
-                const uint32_t idesc = n == 2 ? idesc2 : idesc1;
+                const uint32_t idesc = x.n == 2 ? idesc2 : idesc1;
                 for (int kc = 0; kc < a.k_stages; ++kc) {
                     if (!ptx::mbar_wait_bounded(&s.full[stage], phase, s.abort_flag, kWaitLimitNs)) {
                         raise_abort(s, a);
@@ -318,12 +380,17 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
 #pragma unroll
                     for (int kk = 0; kk < KS / 16; ++kk) {
                         if (kc * KS + kk * 16 >= a.k16) break;
-                        const uint64_t ad = ptx::smem_desc(sb + 32u * kk, 8u * S::kPieceRow, S::kSwizzle);
 #pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const uint64_t bd =
-                                ptx::smem_desc(sb + a.a_bytes + S::kPieceOff * q + 32u * kk, S::kGroup, S::kSwizzle);
-                            ptx::mma_f16(d, ad, bd, idesc, (kc | kk | q) != 0 ? 1u : 0u);
+                        for (int t = 0; t < TILES; ++t) {
+                            if (t >= x.nt) break;
+                            const uint64_t ad =
+                                ptx::smem_desc(sb + t * a.a_bytes + 32u * kk, 8u * S::kPieceRow, S::kSwizzle);
+#pragma unroll
+                            for (int q = 0; q < 2; ++q) {
+                                const uint64_t bd =
+                                    ptx::smem_desc(sb + slots_off + S::kPieceOff * q + 32u * kk, S::kGroup, S::kSwizzle);
+                                ptx::mma_f16(d + t * tile_cols, ad, bd, idesc, (kc | kk | q) != 0 ? 1u : 0u);
+                            }
                         }
                     }
                     ptx::mma_commit(&s.empty[stage]);
@@ -349,8 +416,9 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
             ptx::grid_dep_wait();  // the population (breeding) and the staged batch come from earlier kernels
             uint32_t stage = 0, phase = 0, issued_mask = 0, parity_mask = 0;
             bool ok = true;
-            for (int u = 0; ok && 2 * u < count; ++u) {
-                const int n = min(2, count - 2 * u), p0 = first + 2 * u;
+            UnitWalk<TILES> walk(a);
+            Unit x;
+            while (ok && walk.next(a, x)) {
                 for (int kc = 0; kc < a.k_stages; ++kc) {
                     if (!ptx::mbar_wait_bounded(&s.empty[stage], phase ^ 1u, s.abort_flag, kWaitLimitNs)) {
                         raise_abort(s, a);
@@ -358,11 +426,13 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                         break;
                     }
                     uint8_t* sb = s.ring + stage * a.stage_bytes;
-                    ptx::mbar_arrive_expect_tx(&s.a_full[stage], a.a_bytes + static_cast<uint32_t>(n) * a.slot_bytes);
-                    ptx::tma_load_2d(sb, &tmap_x, &s.a_full[stage], kc * KS, 0);
-                    for (int j = 0; j < n; ++j)
-                        ptx::tma_load_3d(sb + a.a_bytes + j * a.slot_bytes, &tmap_w, &s.a_full[stage], kc * KS, 0,
-                                         p0 + j);
+                    ptx::mbar_arrive_expect_tx(&s.a_full[stage], static_cast<uint32_t>(x.nt) * a.a_bytes +
+                                                                     static_cast<uint32_t>(x.n) * a.slot_bytes);
+                    for (int t = 0; t < x.nt; ++t)
+                        ptx::tma_load_2d(sb + t * a.a_bytes, &tmap_x, &s.a_full[stage], kc * KS, (x.t0 + t) * 128);
+                    for (int j = 0; j < x.n; ++j)
+                        ptx::tma_load_3d(sb + slots_off + j * a.slot_bytes, &tmap_w, &s.a_full[stage], kc * KS, 0,
+                                         x.p0 + j);
                     issued_mask |= 1u << stage;
                     parity_mask = (parity_mask & ~(1u << stage)) | (phase << stage);
                     if (++stage == static_cast<uint32_t>(a.n_stages)) { stage = 0; phase ^= 1u; }
@@ -380,19 +450,20 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         // Lane l handles float4 f = l + 32 m (m < kF4) of each of its groups:
         // row f / (KS / 4), inputs 4 (f % (KS / 4)) .. + 3.
         const int cw = warp - kFirstConvWarp;
-        const int gps = a.h >> 3;  // 8-row groups per individual
+        const int gps = a.hp >> 3;  // 8-row groups per individual
         uint32_t stage = 0, phase = 0;
         bool ok = true;
-        for (int u = 0; ok && 2 * u < count; ++u) {
-            const int n = min(2, count - 2 * u);
-            const int groups = n * gps;
+        UnitWalk<TILES> walk(a);
+        Unit x;
+        for (int u = 0; ok && walk.next(a, x); ++u) {
+            const int groups = x.n * gps;
             for (int kc = 0; kc < a.k_stages; ++kc) {
                 if (!ptx::mbar_wait_bounded(&s.a_full[stage], phase, s.abort_flag, kWaitLimitNs)) {
                     raise_abort(s, a);
                     ok = false;
                     break;
                 }
-                uint8_t* sb = s.ring + stage * a.stage_bytes + a.a_bytes;  // the slots
+                uint8_t* sb = s.ring + stage * a.stage_bytes + slots_off;
                 bool bad0 = false, bad1 = false;
 #pragma unroll
                 for (int g0 = 0; g0 < kMaxGroups / kConvWarps; g0 += S::kBatch) {
@@ -438,73 +509,93 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         }
     } else {
         // ------------------------------------------------------------ epilogue
+        // Two groups of four warps.  Two individuals per unit: group g takes
+        // individual g on all tiles; one: group g takes the tiles of its parity.
         const int ew = warp - kFirstEpiWarp;
-        const int g = ew >> 2;        // slot: the pair's first or second individual
+        const int g = ew >> 2;
         const int q = warp & 3;       // TMEM lane quarter of this warp
         const int et = (ew & 3) * 32 + lane;
         const int row = q * 32 + lane;
         const uint32_t lane_addr = static_cast<uint32_t>(q * 32) << 16;
         const uint32_t bar_id = 1u + static_cast<uint32_t>(g);
-        const int32_t label = row < a.batch ? a.y[row] : 0;
-        float* b1s = s.b1 + g * a.h;
+        const int slot = a.ni == 2 ? g : 0;
+        const int t_first = a.ni == 2 ? 0 : g, t_step = a.ni == 2 ? 1 : 2;
+        float* b1s = s.b1 + g * a.hp;
         float* b2s = s.b2 + g * 16;
-        float* w2t = s.w2t + g * a.h * a.dpad;
+        float* w2t = s.w2t + g * a.hp * a.dpad;
         int* go = s.ep_go + g;
         ptx::grid_dep_wait();  // b1, W2, b2 come from the previous kernel (breeding)
-        for (int u = 0; 2 * u < count; ++u) {
-            const int n = min(2, count - 2 * u);
-            const int p = first + 2 * u + g;
-            const uint32_t buf = static_cast<uint32_t>(u) & 1u, bph = (static_cast<uint32_t>(u) >> 1) & 1u;
-            if (g < n) {
+        UnitWalk<TILES> walk(a);
+        Unit x;
+        for (int u = 0; walk.next(a, x); ++u) {
+            const int p = x.p0 + slot;
+            const uint32_t buf = buf_of(u);
+            const bool active = slot < x.n && t_first < x.nt;
+            if (active) {
                 // While this unit's MMAs run: b1, W2 transposed (rows padded to
-                // dpad with zeros) and b2 of this slot's individual, as stored
-                // after W1, into shared memory.  The group finished reading the
-                // previous ones at its barrier B.  Loads go through L2
-                // (ld.global.cg), not the read-only path: this grid starts while
-                // the breeding kernel that writes the masters still runs, and the
-                // read-only path assumes data no grid changes during the kernel.
+                // dpad with zeros, hidden units past h zero) and b2 of this
+                // group's individual, as stored after W1, into shared memory.
+                // The group finished reading the previous ones at its last
+                // barrier B.  Loads go through L2 (ld.global.cg), not the
+                // read-only path: this grid starts while the breeding kernel
+                // that writes the masters still runs, and the read-only path
+                // assumes data no grid changes during the kernel.
                 const float* src = a.popv + static_cast<int64_t>(p) * a.c_pad + static_cast<int64_t>(a.h) * a.k;
-                for (int i = et; i < a.h; i += 128) b1s[i] = __ldcg(src + i);
+                for (int i = et; i < a.hp; i += 128) b1s[i] = i < a.h ? __ldcg(src + i) : 0.0f;
                 for (int i = et; i < a.d_out * a.h; i += 128) {
                     const int o = i / a.h, col = i - o * a.h;
                     w2t[col * a.dpad + o] = __ldcg(src + a.h + i);
                 }
                 const int pad = a.dpad - a.d_out;
                 for (int i = et; i < a.h * pad; i += 128) w2t[(i / pad) * a.dpad + a.d_out + i % pad] = 0.0f;
+                for (int i = a.h * a.dpad + et; i < a.hp * a.dpad; i += 128) w2t[i] = 0.0f;
                 if (et < 16) b2s[et] = et < a.d_out ? __ldcg(src + a.h + a.d_out * a.h + et) : 0.0f;
             }
             if (et == 0) {
-                const bool got = ptx::mbar_wait_bounded(&s.acc_full[buf], bph, s.abort_flag, kWaitLimitNs);
+                const bool got = ptx::mbar_wait_bounded(&s.acc_full[buf], phase_of(u), s.abort_flag, kWaitLimitNs);
                 if (!got) raise_abort(s, a);
-                *go = !got ? 0 : (((s.accflag[buf] >> g) & 1u) ? 2 : 1);
+                *go = !got ? 0 : (((s.accflag[buf] >> slot) & 1u) ? 2 : 1);
             }
             ptx::named_barrier_sync(bar_id, 128);  // A: accumulator ready (or abort); parameters staged
             const int gov = *go;
             if (!gov) break;
             ptx::tc_fence_after();
+            if (!active) {
+                ptx::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(&s.acc_empty[buf]);
+                ptx::named_barrier_sync(bar_id, 128);  // everyone has read the go word
+                continue;
+            }
 
-            float loss = 0.0f;
-            int32_t good = 0;
-            if (g < n) {
+            for (int t = t_first; t < x.nt; t += t_step) {
+                const int smp = (x.t0 + t) * 128 + row;  // this thread's sample
+                const bool in = smp < a.batch;
+                float loss = 0.0f;
+                unsigned good = 0;
                 // Individuals with a weight outside the piece range: layer 1 by
                 // FP32 FFMA from global memory, k in order, in the accumulator's units.
                 const float* w1p = a.popv + static_cast<int64_t>(p) * a.c_pad;
-                const uint8_t* xrow = a.x + static_cast<int64_t>(row < a.batch ? row : 0) * a.k;
-                const uint32_t col0 = tmem_base + lane_addr + buf * kAccStride + static_cast<uint32_t>(g * a.h);
+                const uint8_t* xrow = a.x + static_cast<int64_t>(in ? smp : 0) * a.k;
+                const uint32_t col0 = tmem_base + lane_addr + buf * kAccStride + static_cast<uint32_t>(t) * tile_cols +
+                                      static_cast<uint32_t>(slot * a.hp);
                 float logit[kMaxOutU8];
 #pragma unroll
                 for (int o = 0; o < kMaxOutU8; ++o) logit[o] = 0.0f;
-                for (int c = 0; c < a.h; c += 16) {
+                for (int c = 0; c < a.hp; c += 16) {
                     float v[16];
                     ptx::tmem_ld16(col0 + static_cast<uint32_t>(c), v);
-                    if (row < a.batch) {
+                    if (in) {
                         if (gov == 2) {
 #pragma unroll
                             for (int j = 0; j < 16; ++j) {
-                                const float* wr = w1p + static_cast<int64_t>(c + j) * a.k;
-                                float acc = 0.0f;
-                                for (int kk = 0; kk < a.k; ++kk) acc = fmaf(wr[kk], static_cast<float>(xrow[kk]), acc);
-                                v[j] = acc * kPieceScale;
+                                if (c + j < a.h) {
+                                    const float* wr = w1p + static_cast<int64_t>(c + j) * a.k;
+                                    float acc = 0.0f;
+                                    for (int kk = 0; kk < a.k; ++kk)
+                                        acc = fmaf(wr[kk], static_cast<float>(xrow[kk]), acc);
+                                    v[j] = acc * kPieceScale;
+                                }
                             }
                         }
 #pragma unroll
@@ -525,7 +616,14 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                         }
                     }
                 }
-                if (row < a.batch) {
+                if (t + t_step >= x.nt) {
+                    // The accumulator is read: release it to the next unit's MMAs.
+                    ptx::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(&s.acc_empty[buf]);
+                }
+                if (in) {
+                    const int32_t label = a.y[smp];
                     float bo[kMaxOutU8];
 #pragma unroll
                     for (int o = 0; o < kMaxOutU8; ++o) bo[o] = b2s[o];
@@ -548,35 +646,53 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                         for (int o = 0; o < kMaxOutU8; ++o)
                             if (o == label) zl = logit[o] + bo[o];
                         loss = logf(se) + zmax - zl;
-                        good = (arg == label) ? 1 : 0;
+                        good = (arg == label) ? 1u : 0u;
                     } else {
                         loss = __int_as_float(0x7FC00000);
                     }
                 }
-            }
-            // The accumulator is read: release it to the next unit's MMAs.
-            ptx::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&s.acc_empty[buf]);
+                // Fixed-order sums: FP32 within TENSOR's shapes (the fused kernel
+                // gives the same bits), FP64 beyond them, where these roundings
+                // would be the larger part of the fitness's error.
+                double sum;
+                if (a.wide) {
+                    sum = static_cast<double>(loss);
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                loss += __shfl_xor_sync(0xFFFFFFFFu, loss, off);
-                good += __shfl_xor_sync(0xFFFFFFFFu, good, off);
-            }
-            if (lane == 0) {
-                s.red_loss[g * 4 + q] = loss;
-                s.red_ok[g * 4 + q] = good;
-            }
-            ptx::named_barrier_sync(bar_id, 128);  // B: quarter sums written; staged parameters no longer read
-            if (g < n && et == 0) {
-                const float* rl = s.red_loss + g * 4;
-                const int32_t* ro = s.red_ok + g * 4;
-                const float total = ((rl[0] + rl[1]) + rl[2]) + rl[3];
-                const int32_t n_ok = ro[0] + ro[1] + ro[2] + ro[3];
-                const float f = -(total / static_cast<float>(a.batch));
-                a.f_raw[p] = f;
-                if (a.f_adj) a.f_adj[p] = a.f_inh ? (1.0f - a.alpha) * a.f_inh[p] + a.alpha * f : f;
-                if (a.correct) a.correct[p] = n_ok;
+                    for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
+                } else {
+#pragma unroll
+                    for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xFFFFFFFFu, loss, off);
+                    sum = static_cast<double>(loss);
+                }
+                good = __reduce_add_sync(0xFFFFFFFFu, good);
+                double* rl = s.red_loss + (g * 2 + (t & 1)) * 4;
+                int32_t* ro = s.red_ok + (g * 2 + (t & 1)) * 4;
+                if (lane == 0) {
+                    rl[q] = sum;
+                    ro[q] = static_cast<int32_t>(good);
+                }
+                ptx::named_barrier_sync(bar_id, 128);  // B: quarter sums written; staged parameters no longer read
+                if (et == 0) {
+                    const int32_t n_ok = ro[0] + ro[1] + ro[2] + ro[3];
+                    const double total = ((rl[0] + rl[1]) + rl[2]) + rl[3];
+                    if (a.tiles == 1) {
+                        float f;
+                        if (a.wide) {
+                            f = static_cast<float>(-(total / static_cast<double>(a.batch)));
+                        } else {
+                            const float r0 = static_cast<float>(rl[0]), r1 = static_cast<float>(rl[1]),
+                                        r2 = static_cast<float>(rl[2]), r3 = static_cast<float>(rl[3]);
+                            f = -((((r0 + r1) + r2) + r3) / static_cast<float>(a.batch));
+                        }
+                        a.f_raw[p] = f;
+                        if (a.f_adj) a.f_adj[p] = a.f_inh ? (1.0f - a.alpha) * a.f_inh[p] + a.alpha * f : f;
+                        if (a.correct) a.correct[p] = n_ok;
+                    } else {
+                        const int64_t at = static_cast<int64_t>(x.t0 + t) * a.pop + p;
+                        a.part[at] = total;
+                        a.part_ok[at] = n_ok;
+                    }
+                }
             }
         }
     }
@@ -616,6 +732,25 @@ __global__ void __launch_bounds__(256) stage_x16_kernel(const uint8_t* __restric
     ptx::grid_dep_wait();
 }
 
+// A batch of several tiles: each individual's loss and correct count from its
+// tiles' sums, in tile order.
+__global__ void __launch_bounds__(256) combine_u8_tiles_kernel(const EvalU8Args a)
+{
+    ptx::grid_dep_wait();
+    const int p = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
+    if (p >= a.pop) return;
+    double total = 0.0;
+    int32_t n_ok = 0;
+    for (int t = 0; t < a.tiles; ++t) {
+        total += __ldcg(a.part + static_cast<int64_t>(t) * a.pop + p);
+        n_ok += __ldcg(a.part_ok + static_cast<int64_t>(t) * a.pop + p);
+    }
+    const float f = static_cast<float>(-(total / static_cast<double>(a.batch)));
+    a.f_raw[p] = f;
+    if (a.f_adj) a.f_adj[p] = a.f_inh ? (1.0f - a.alpha) * a.f_inh[p] + a.alpha * f : f;
+    if (a.correct) a.correct[p] = n_ok;
+}
+
 typedef CUresult (*U8EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                     const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                     CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -634,21 +769,56 @@ U8EncodeTiledFn u8_encode_fn()
     return fn;
 }
 
-}  // namespace
-
-bool eval_u8_tc_supported(const NetLayout& net, int32_t batch, const float* pop_dev)
+// The unit shape for a population and a batch: two individuals per MMA where
+// both fit its 256 columns, two tiles per unit where the batch has them (a
+// weight slice is converted once for both), less of either when that leaves
+// SMs without a unit.
+bool u8_shape(const NetLayout& net, int32_t pop, int32_t batch, int32_t sms, U8Shape* u)
 {
-    if (net.n_layers != 2) return false;
-    const int32_t k = net.dims[0], h = net.dims[1], d_out = net.dims[2];
-    if (k % 4 != 0 || h % 16 != 0 || h > 128 || d_out > kMaxOutU8 || batch < 1 || batch > 128) return false;
-    if (reinterpret_cast<uintptr_t>(pop_dev) & 15u) return false;
-    return u8_kstage(h, d_out, batch) > 0 && u8_encode_fn() != nullptr;
+    if (batch < 1 || eval_u8_scratch_bytes(net, pop, batch) > kMaxScratchU8) return false;
+    const int32_t tiles = (batch + 127) / 128;
+    u->hp = (net.dims[1] + 15) / 16 * 16;
+    u->ni = u->hp <= 128 ? 2 : 1;
+    u->tiles_per_unit = tiles > 1 ? 2 : 1;
+    if (tiles > 1) {
+        auto units = [&](int32_t ni, int32_t tp) {
+            return static_cast<int64_t>((pop + ni - 1) / ni) * ((tiles + tp - 1) / tp);
+        };
+        if (units(u->ni, 2) < sms) u->tiles_per_unit = 1;
+        if (u->ni == 2 && units(2, u->tiles_per_unit) < sms) u->ni = 1;
+    }
+    return u8_ring(u, net.dims[2], batch);
 }
 
-size_t eval_u8_x16_bytes(const NetLayout& net, int32_t batch)
+}  // namespace
+
+bool eval_u8_tc_supported(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev)
 {
-    const int64_t kp = (net.dims[0] + 7) / 8 * 8;
-    return static_cast<size_t>(batch) * static_cast<size_t>(kp) * 2u;
+    return net.dims[1] % 16 == 0 && net.dims[1] <= 128 && batch <= 128 &&
+           eval_u8_wide_supported(net, pop, batch, pop_dev);
+}
+
+bool eval_u8_wide_supported(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev)
+{
+    if (net.n_layers != 2) return false;
+    if (net.dims[0] % 4 != 0 || net.dims[1] > 256 || net.dims[2] > kMaxOutU8) return false;
+    if (reinterpret_cast<uintptr_t>(pop_dev) & 15u) return false;
+    U8Shape u;
+    return u8_shape(net, pop, batch, 1, &u) && u8_encode_fn() != nullptr;
+}
+
+// Scratch layout: the FP16 batch (rounded up to 256 bytes), then for several
+// tiles their loss sums and correct counts.
+static size_t x16_bytes(const NetLayout& net, int32_t batch)
+{
+    const size_t kp = static_cast<size_t>((net.dims[0] + 7) / 8 * 8);
+    return (static_cast<size_t>(batch) * kp * 2u + 255u) / 256u * 256u;
+}
+
+size_t eval_u8_scratch_bytes(const NetLayout& net, int32_t pop, int32_t batch)
+{
+    const size_t tiles = static_cast<size_t>((batch + 127) / 128);
+    return x16_bytes(net, batch) + (tiles > 1 ? 12u * tiles * static_cast<size_t>(pop) : 0u);
 }
 
 cudaError_t launch_stage_x16(const NetLayout& net, const uint8_t* x, int32_t batch, void* x16, cudaStream_t stream)
@@ -669,10 +839,18 @@ cudaError_t launch_stage_x16(const NetLayout& net, const uint8_t* x, int32_t bat
 }
 
 cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* pop_dev, const uint8_t* x,
-                              const void* x16, float x_div, const int32_t* y, int32_t batch, float alpha,
+                              void* scratch, float x_div, const int32_t* y, int32_t batch, float alpha,
                               const float* f_inh, float* f_raw, float* f_adj, int32_t* correct, unsigned int* status,
                               cudaStream_t stream)
 {
+    int dev = 0, sms = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (err != cudaSuccess) return err;
+    U8Shape u;
+    if (!u8_shape(net, pop, batch, sms, &u)) return cudaErrorInvalidValue;
+    const int32_t ks = u.ks;
     EvalU8Args a{};
     a.pop = pop;
     a.k = net.dims[0];
@@ -681,10 +859,13 @@ cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* po
     a.batch = batch;
     a.k16 = (a.k + 15) / 16 * 16;
     a.dpad = (a.d_out + 3) / 4 * 4;
-    const int32_t ks = u8_kstage(a.h, a.d_out, batch);
-    if (ks == 0) return cudaErrorInvalidValue;
     a.k_stages = (a.k + ks - 1) / ks;
-    a.n_stages = u8_stages(a.h, a.d_out, batch, ks);
+    a.n_stages = u.n_stages;
+    a.hp = u.hp;
+    a.ni = u.ni;
+    a.tiles = (batch + 127) / 128;
+    a.groups = (a.tiles + u.tiles_per_unit - 1) / u.tiles_per_unit;
+    a.n_bufs = u.tiles_per_unit * u.ni * u.hp <= static_cast<int32_t>(kAccStride) ? 2 : 1;
     a.c_pad = net.c_pad;
     a.inv_div = static_cast<float>(1.0 / (static_cast<double>(x_div) * kPieceScale));
     a.alpha = alpha;
@@ -695,20 +876,24 @@ cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* po
     a.f_raw = f_raw;
     a.f_adj = f_adj;
     a.correct = correct;
+    a.part = reinterpret_cast<double*>(static_cast<uint8_t*>(scratch) + x16_bytes(net, batch));
+    a.part_ok = reinterpret_cast<int32_t*>(a.part + static_cast<size_t>(a.tiles) * static_cast<size_t>(pop));
     a.status = status;
-    a.slot_bytes = static_cast<uint32_t>(a.h) * 4u * static_cast<uint32_t>(ks);
+    a.wide = a.tiles > 1 || a.h % 16 != 0 || a.h > 128;
+    a.slot_bytes = static_cast<uint32_t>(a.hp) * 4u * static_cast<uint32_t>(ks);
     a.a_bytes = u8_a_bytes(batch, ks);
-    a.stage_bytes = u8_stage_bytes(a.h, batch, ks);
-    const size_t smem = u8_smem_bytes(a.h, a.d_out, batch, ks, a.n_stages);
+    a.stage_bytes = u8_stage_bytes(u, batch);
+    const size_t smem = u8_smem_bytes(u, a.d_out, batch);
     U8EncodeTiledFn enc = u8_encode_fn();
     if (!enc) return cudaErrorNotSupported;
     CUtensorMap tw, tx;
     {
-        // W1 of every individual: [pop][h][k] FP32, rows k * 4 bytes apart.
+        // W1 of every individual: [pop][h][k] FP32, rows k * 4 bytes apart; rows
+        // h .. hp - 1 of a tile read as zero.
         const cuuint64_t dims[3] = { static_cast<cuuint64_t>(a.k), static_cast<cuuint64_t>(a.h),
                                      static_cast<cuuint64_t>(pop) };
         const cuuint64_t strides[2] = { static_cast<cuuint64_t>(a.k) * 4u, static_cast<cuuint64_t>(net.c_pad) * 4u };
-        const cuuint32_t box[3] = { static_cast<cuuint32_t>(ks), static_cast<cuuint32_t>(a.h), 1 };
+        const cuuint32_t box[3] = { static_cast<cuuint32_t>(ks), static_cast<cuuint32_t>(a.hp), 1 };
         const cuuint32_t es[3] = { 1, 1, 1 };
         if (enc(&tw, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(pop_dev), dims, strides, box, es,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -716,45 +901,36 @@ cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* po
             return cudaErrorInvalidValue;
     }
     {
-        // The staged batch: [batch][kp] FP16, tiles of round_up(batch, 8)
-        // rows; rows past the batch and levels past k read as zero.
+        // The staged batch: [batch][kp] FP16, tiles of round_up(batch, 8) rows
+        // (128 with several tiles); rows past the batch and levels past k read
+        // as zero.
         const int32_t kp = (a.k + 7) / 8 * 8;
         const cuuint64_t dims[2] = { static_cast<cuuint64_t>(a.k), static_cast<cuuint64_t>(batch) };
         const cuuint64_t strides[1] = { static_cast<cuuint64_t>(kp) * 2u };
-        const cuuint32_t box[2] = { static_cast<cuuint32_t>(ks), static_cast<cuuint32_t>((batch + 7) / 8 * 8) };
+        const cuuint32_t box[2] = { static_cast<cuuint32_t>(ks),
+                                    static_cast<cuuint32_t>(batch > 128 ? 128 : (batch + 7) / 8 * 8) };
         const cuuint32_t es[2] = { 1, 1 };
-        if (enc(&tx, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(x16), dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, ks == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
-                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        if (enc(&tx, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, scratch, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                ks == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    int dev = 0, sms = 0;
-    cudaError_t err = cudaGetDevice(&dev);
-    if (err != cudaSuccess) return err;
-    err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (err != cudaSuccess) return err;
-    const void* kern = ks == 64 ? reinterpret_cast<const void*>(eval_u8_kernel<64>)
-                                : reinterpret_cast<const void*>(eval_u8_kernel<32>);
+    typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const EvalU8Args);
+    const bool two = u.tiles_per_unit == 2;
+    const Kernel kern = ks == 64 ? (two ? eval_u8_kernel<64, 2> : eval_u8_kernel<64, 1>)
+                                 : (two ? eval_u8_kernel<32, 2> : eval_u8_kernel<32, 1>);
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (err != cudaSuccess) return err;
-    const int grid = pop < sms ? pop : sms;
-    a.per_cta = pop / grid;
-    a.extra = pop % grid;
+    const int64_t work = a.groups == 1 ? pop : static_cast<int64_t>((pop + a.ni - 1) / a.ni) * a.groups;
+    const int grid = static_cast<int>(work < sms ? work : sms);
+    a.per_cta = static_cast<int32_t>(work / grid);
+    a.extra = static_cast<int32_t>(work % grid);
     // Programmatic stream serialisation: CTAs may start (barriers, TMEM) while
     // the previous kernel finishes; the producer and the epilogue wait for it
     // before they read the population or the staged batch.
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kU8Threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return ks == 64 ? cudaLaunchKernelEx(&cfg, eval_u8_kernel<64>, tw, tx, a)
-                    : cudaLaunchKernelEx(&cfg, eval_u8_kernel<32>, tw, tx, a);
+    err = launch_pdl(kern, dim3(grid), dim3(kU8Threads), smem, stream, tw, tx, a);
+    if (err != cudaSuccess || a.tiles == 1) return err;
+    return launch_pdl(combine_u8_tiles_kernel, dim3((pop + 255) / 256), dim3(256), 0, stream, a);
 }
 
 }  // namespace leea
