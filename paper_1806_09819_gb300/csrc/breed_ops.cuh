@@ -240,4 +240,47 @@ __device__ __forceinline__ void mutate8_dense(float sigma, uint32_t gen, const K
     }
 }
 
+// ---- how mutation children draw their normals ------------------------------------
+// Rate from which a lane makes all its pairs itself: 16-bit threshold of
+// kDenseRate = 0.35.  Breeding mutation children alone at P = 1000, 784-112-10: the list
+// takes 129 us at q = 0.1 and 196 at 0.3, all pairs 190 at any q.
+constexpr uint32_t kDenseThr = 22937;
+enum MutMode { kMutNone, kMutSparse, kMutDense, kMutAll };
+inline MutMode mut_mode(uint32_t thr)
+{
+    return thr == 0u ? kMutNone : (thr >= 65536u ? kMutAll : (thr >= kDenseThr ? kMutDense : kMutSparse));
+}
+
+// ---- moving units -----------------------------------------------------------------
+// 8 consecutive floats; W32: the address is 32-byte aligned.  Parents are read
+// once per child, so they are kept out of L1.
+template <bool W32>
+__device__ __forceinline__ void load8(const float* p, float (&v)[8])
+{
+    if (W32) {
+        asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                     : "l"(p));
+    } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                         : "=f"(v[4 * h]), "=f"(v[4 * h + 1]), "=f"(v[4 * h + 2]), "=f"(v[4 * h + 3])
+                         : "l"(p + 4 * h));
+    }
+}
+
+template <bool W32>
+__device__ __forceinline__ void store8(float* p, const float (&v)[8])
+{
+    if (W32) {
+        asm volatile("st.global.v8.f32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"f"(v[0]), "f"(v[1]), "f"(v[2]),
+                     "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "l"(p)
+                     : "memory");
+    } else {
+        reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
+    }
+}
+
 }  // namespace leea

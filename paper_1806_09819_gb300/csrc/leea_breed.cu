@@ -56,20 +56,9 @@ constexpr int kUnitGenes = 8;
 constexpr int kUnits = 2;          // U: units per lane and item
 constexpr int kChunk = 32 * kUnits * kUnitGenes;  // genes per item
 constexpr int kJobSlots = 4 * 32 * kUnits;        // Box-Muller pairs of a warp's item
-// Rate from which a lane makes all its pairs itself: 16-bit threshold of
-// kDenseRate = 0.35.  Mutation children alone at P = 1000, 784-112-10: the list
-// takes 129 us at q = 0.1 and 196 at 0.3, all pairs 190 at any q.
-constexpr uint32_t kDenseThr = 22937;
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 constexpr uint64_t kDrainLimitNs = 200000000ull;
 constexpr int32_t kKindInvalid = -1;
-
-// How mutation children draw their normals.
-enum MutMode { kMutNone, kMutSparse, kMutDense, kMutAll };
-MutMode mut_mode(uint32_t thr)
-{
-    return thr == 0u ? kMutNone : (thr >= 65536u ? kMutAll : (thr >= kDenseThr ? kMutDense : kMutSparse));
-}
 
 // An item as its warp resolved it (one lane per item), so that the loop over
 // the items has no table look-ups or 64-bit products.
@@ -99,37 +88,6 @@ struct __align__(128) WarpSmem {
     int abort;                      // never set: the waits end by their limit
     uint8_t codes[kJobSlots];       // the listed pairs
 };
-
-// 8 consecutive floats; W32: the address is 32-byte aligned.  Parents are read
-// once per child, so they are kept out of L1.
-template <bool W32>
-__device__ __forceinline__ void load8(const float* p, float (&v)[8])
-{
-    if (W32) {
-        asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
-                     : "l"(p));
-    } else {
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-            asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
-                         : "=f"(v[4 * h]), "=f"(v[4 * h + 1]), "=f"(v[4 * h + 2]), "=f"(v[4 * h + 3])
-                         : "l"(p + 4 * h));
-    }
-}
-
-template <bool W32>
-__device__ __forceinline__ void store8(float* p, const float (&v)[8])
-{
-    if (W32) {
-        asm volatile("st.global.v8.f32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"f"(v[0]), "f"(v[1]), "f"(v[2]),
-                     "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "l"(p)
-                     : "memory");
-    } else {
-        reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
-        reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
-    }
-}
 
 // The shadow of unit u of W1 (8 genes of one row, as d_0 % 16 == 0): 8 BF16
 // (16 bytes) or 8 FP8-e4m3 of w 2^-e (saturating; 8 bytes), inside one 16-byte
@@ -443,19 +401,6 @@ BreedKernel breed_kernel_mut(MutMode mode)
     case kMutDense: return breed_kernel<MULTI, W32, kMutDense, SHADOW>;
     default: return breed_kernel<MULTI, W32, kMutAll, SHADOW>;
     }
-}
-
-PhiloxKeys host_philox_keys(uint64_t seed)
-{
-    PhiloxKeys k;
-    uint32_t a = static_cast<uint32_t>(seed), b = static_cast<uint32_t>(seed >> 32);
-    for (int r = 0; r < 10; ++r) {
-        k.k0[r] = a;
-        k.k1[r] = b;
-        a += kPhiloxW0;
-        b += kPhiloxW1;
-    }
-    return k;
 }
 
 constexpr size_t kBreedSmem = sizeof(WarpSmem) * kWarps;

@@ -119,4 +119,18 @@ __device__ __forceinline__ uint4 philox_keyed(uint4 ctr, const PhiloxKeys& k)
     return ctr;
 }
 
+// The same on the host, for kernels that take the keys as a parameter.
+inline PhiloxKeys host_philox_keys(uint64_t seed)
+{
+    PhiloxKeys k;
+    uint32_t a = static_cast<uint32_t>(seed), b = static_cast<uint32_t>(seed >> 32);
+    for (int r = 0; r < 10; ++r) {
+        k.k0[r] = a;
+        k.k1[r] = b;
+        a += kPhiloxW0;
+        b += kPhiloxW1;
+    }
+    return k;
+}
+
 }  // namespace leea
