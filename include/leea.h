@@ -318,10 +318,11 @@ leea_status leea_evaluate(int32_t pop, const int32_t* dims, int32_t n_dims,
  * |w| >= 128 gets its layer 1 in FP32 FFMA instead.  That path first writes the
  * batch as FP16 into a stream-ordered allocation of batch * round_up(d_0, 8) * 2
  * bytes, and above 128 samples 12 * ceil(batch / 128) * pop bytes for the
- * 128-sample tiles' sums (cudaMallocAsync on `stream`, freed after the
- * evaluation; beyond 256 MB AUTO takes the CUDA cores).  Otherwise, or with
- * LEEA_EVAL_SIMT, the CUDA-core kernel computes x = k / x_div in FP32.  x_div
- * must be finite and > 0. */
+ * 128-sample tiles' sums (freed in stream order after the evaluation; the
+ * library keeps at most 64 MB of such scratch per device between calls; beyond
+ * 256 MB AUTO takes the CUDA cores).  Otherwise, or with LEEA_EVAL_SIMT, the
+ * CUDA-core kernel computes x = k / x_div in FP32.  x_div must be finite and
+ * > 0. */
 leea_status leea_evaluate_u8(int32_t pop, const int32_t* dims, int32_t n_dims,
                              const float* pop_dev, const uint8_t* x_u8_dev, float x_div,
                              const int32_t* y_dev, int32_t batch, float alpha,

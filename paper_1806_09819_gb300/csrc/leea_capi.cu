@@ -12,6 +12,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <utility>
 #include <vector>
 
@@ -179,6 +180,44 @@ float* noalloc_scratch_ptr(cudaError_t* err)
     return hit;
 }
 
+// The step calls' scratch: stream-ordered allocations from a pool of the
+// library's own, one per device.  The device's default pool gives everything
+// back at each synchronisation, so that a caller who reads every result paid
+// for mapping the scratch again on every call (about 220 us); this one keeps
+// up to kScratchKeep bytes between calls and gives the rest back.  Allocation,
+// reuse across streams and threads are the pool's (ordered by the streams);
+// the table of pools is guarded here.
+constexpr uint64_t kScratchKeep = uint64_t{64} << 20;
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t stream)
+{
+    constexpr int kMaxDevices = 64;
+    static std::mutex mu;
+    static cudaMemPool_t pools[kMaxDevices] = {};
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    cudaMemPool_t pool = nullptr;
+    if (dev < kMaxDevices) {
+        std::lock_guard<std::mutex> lock(mu);
+        if (!pools[dev]) {
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t made = nullptr;
+            uint64_t keep = kScratchKeep;
+            if (cudaMemPoolCreate(&made, &props) == cudaSuccess) {
+                if (cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess) pools[dev] = made;
+                else cudaMemPoolDestroy(made);
+            }
+            if (!pools[dev]) cudaGetLastError();  // the default pool serves as well
+        }
+        pool = pools[dev];
+    }
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, stream) : cudaMallocAsync(p, bytes, stream);
+}
+
 // Synchronises `stream`, reads and clears the status word.
 leea_status check_device_status(cudaStream_t stream, uint32_t* flags_out)
 {
@@ -272,8 +311,7 @@ leea_status dispatch_eval_u8(const NetLayout& net, int32_t pop, const float* pop
         if (!status) return fail(LEEA_ECUDA, "device status word unavailable");
         void* own = nullptr;  // the call's own scratch, freed in stream order after the evaluation
         if (!x16) {
-            LEEA_CUDA_TRY(cudaMallocAsync(&own, eval_u8_scratch_bytes(net, pop, batch), stream),
-                          "batch staging allocation");
+            LEEA_CUDA_TRY(scratch_alloc(&own, eval_u8_scratch_bytes(net, pop, batch), stream), "batch staging allocation");
             x16 = own;
             x16_staged = false;
         }
