@@ -357,7 +357,11 @@ int64_t leea_shadow_scratch_bytes(int32_t pop, int32_t batch);
  * leaves it), x_u8_dev 16-byte aligned.  A batch above 128 samples is split into tiles of 128
  * whose partial sums go to scratch_dev (caller-owned, scratch_bytes >=
  * leea_shadow_scratch_bytes(pop, batch); NULL/0 allowed when that is 0) and
- * are combined in tile order.  Other arguments and outputs as in
+ * are combined in tile order.  With pop * ceil(batch / 128) of at least two per
+ * SM and h <= 128 the batch is first written as operand tiles into a
+ * stream-ordered allocation (16 KB per 128 samples and 64 BF16 or 128 FP8
+ * inputs, twice that for FP8), and two individuals share every tensor-core
+ * instruction; the results are the same bits.  Other arguments and outputs as in
  * leea_evaluate_u8. */
 leea_status leea_evaluate_shadow_u8(int32_t pop, const int32_t* dims, int32_t n_dims,
                                     const float* pop_dev, int32_t precision,

@@ -364,11 +364,37 @@ leea_status check_shadow_shape(const NetLayout& net, int32_t precision)
 leea_status dispatch_eval_shadow(const NetLayout& net, int32_t pop, const float* pop_dev, int32_t precision,
                                  const uint8_t* shadow, const int32_t* scale_exp, const uint8_t* x, float x_div,
                                  const int32_t* y, int32_t batch, float alpha, const float* f_inh, float* f_raw,
-                                 float* f_adj, int32_t* correct, float* scratch, cudaStream_t stream)
+                                 float* f_adj, int32_t* correct, float* scratch, cudaStream_t stream, bool may_allocate)
 {
     if (!(x_div > 0.0f) || std::isinf(x_div)) return fail(LEEA_EINVAL, "x_div must be finite and > 0");
     unsigned int* status = device_status_ptr();
     if (!status) return fail(LEEA_ECUDA, "device status word unavailable");
+    // Two individuals per MMA on the staged batch (the bits are the chunked
+    // kernel's), where the call may allocate the staging and there is a pair for
+    // every SM: below that the staging's launch costs more than the pairs save
+    // (BF16 784-112-10 on 24 samples: 200 nets 19 us chunked, 21 in pairs, 304
+    // 20 / 20, 400 24 / 21, 2,048 81 / 62; FP8 at 256 samples 139 / 92).
+    int dev = 0, sms = 0;
+    LEEA_CUDA_TRY(cudaGetDevice(&dev), "device query");
+    LEEA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device query");
+    if (may_allocate && static_cast<int64_t>(pop) * ((batch + 127) / 128) >= 2 * sms &&
+        eval_shadow_pair_supported(net, precision, batch)) {
+        void* xop = nullptr;
+        cudaError_t err = scratch_alloc(&xop, eval_shadow_pair_xop_bytes(net, precision, batch), stream);
+        if (err == cudaSuccess) {
+            err = launch_stage_xop(net, precision, x, batch, xop, stream);
+            if (err == cudaSuccess)
+                err = launch_eval_shadow_pair(net, pop, pop_dev, precision, shadow, shadow_stride_of(net, precision),
+                                              scale_exp, xop, x_div, y, batch, alpha, f_inh, f_raw, f_adj, correct,
+                                              scratch, status, stream);
+            const cudaError_t ferr = cudaFreeAsync(xop, stream);
+            if (err == cudaSuccess) err = ferr;
+            if (err != cudaSuccess) return cuda_fail(err, "shadow evaluate kernel");
+            return LEEA_OK;
+        }
+        if (err != cudaErrorMemoryAllocation) return cuda_fail(err, "batch staging allocation");
+        cudaGetLastError();  // no room for the staging: the chunked kernel needs none
+    }
     LEEA_CUDA_TRY(launch_eval_shadow(net, pop, pop_dev, precision, shadow, shadow_stride_of(net, precision),
                                      scale_exp, x, x_div, y, batch, alpha, f_inh, f_raw, f_adj, correct, scratch,
                                      status, stream),
@@ -689,7 +715,7 @@ leea_status leea_evaluate_shadow_u8(int32_t pop, const int32_t* dims, int32_t n_
         return fail(LEEA_EINVAL, "batch %d needs %lld scratch bytes", batch, static_cast<long long>(need));
     return dispatch_eval_shadow(net, pop, pop_dev, precision, shadow_dev, scale_exp_dev, x_u8_dev, x_div, y_dev,
                                 batch, alpha, f_inh_dev, f_raw_dev, f_adj_dev, correct_dev, scratch_dev,
-                                static_cast<cudaStream_t>(stream));
+                                static_cast<cudaStream_t>(stream), true);
 }
 
 leea_status leea_evaluate_shadow_u8_noalloc(int32_t pop, const int32_t* dims, int32_t n_dims, const float* pop_dev,

@@ -340,7 +340,7 @@ cudaError_t evaluate(leea_surr* s, const float* popv, const uint8_t* shadow, int
                                s->prm.eval_path, s->stream);
     else
         *st = dispatch_eval_shadow(s->net, n, popv, s->prm.precision, shadow, nullptr, x, x_div, y, batch,
-                                   s->prm.alpha, f_inh, f_raw, f_adj, correct, s->scratch, s->stream);
+                                   s->prm.alpha, f_inh, f_raw, f_adj, correct, s->scratch, s->stream, true);
     return cudaSuccess;
 }
 
