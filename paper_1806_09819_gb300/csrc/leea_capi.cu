@@ -248,7 +248,7 @@ leea_status check_device_status(cudaStream_t stream, uint32_t* flags_out)
 // Runs the evaluation kernel that `path` selects (LEEA_EVAL_*).
 leea_status dispatch_eval(const NetLayout& net, int32_t pop, const float* pop_dev, const float* x,
                           const int32_t* y, int32_t batch, float alpha, const float* f_inh, float* f_raw,
-                          float* f_adj, int32_t* correct, int32_t path, cudaStream_t stream)
+                          float* f_adj, int32_t* correct, int32_t path, cudaStream_t stream, void* scratch = nullptr)
 {
     if (net.n_layers > 2) {  // several hidden layers: CUDA-core FP32
         if (path == LEEA_EVAL_TENSOR) return fail(LEEA_EINVAL, "nets with several hidden layers evaluate on CUDA cores");
@@ -256,17 +256,48 @@ leea_status dispatch_eval(const NetLayout& net, int32_t pop, const float* pop_de
                       "evaluate kernel");
         return LEEA_OK;
     }
-    const bool tc_ok = eval_tc_supported(net, batch, pop_dev, x);
-    if (path == LEEA_EVAL_TENSOR && !tc_ok)
+    const bool tf32_ok = eval_tc_supported(net, batch, pop_dev, x);
+    if (path == LEEA_EVAL_TENSOR && !tf32_ok)
         return fail(LEEA_EINVAL, "tensor-core evaluation needs d_0 %% 4 == 0, h %% 16 == 0, h <= 256, "
                                  "d_out <= 16 and 16-byte aligned population and x");
-    cudaError_t err;
-    if (tc_ok && path != LEEA_EVAL_SIMT) {
-        unsigned int* status = device_status_ptr();
+    // AUTO: FP16 pieces of x and w, two individuals per MMA; where a weight is
+    // outside the pieces' range, that individual again with TF32 pieces (or, where
+    // the hidden width is off its 16, on the CUDA cores).
+    bool pieces = path == LEEA_EVAL_AUTO && (reinterpret_cast<uintptr_t>(x) & 15u) == 0 &&
+                        eval_u8_wide_supported(net, pop, batch, pop_dev, 2);
+    unsigned int* status = nullptr;
+    if (pieces || (tf32_ok && path != LEEA_EVAL_SIMT)) {
+        status = device_status_ptr();
         if (!status) return fail(LEEA_ECUDA, "device status word unavailable");
-        err = launch_eval_tc(net, pop, pop_dev, x, y, batch, alpha, f_inh, f_raw, f_adj, correct, status, stream);
-    } else {
-        err = launch_eval_simt(net, pop, pop_dev, x, y, batch, alpha, f_inh, f_raw, f_adj, correct, stream);
+    }
+    const int32_t* only = nullptr;
+    void* own = nullptr;  // the call's own scratch, freed in stream order after the evaluation
+    cudaError_t err = cudaSuccess;
+    if (pieces) {
+        if (!scratch) {
+            if (scratch_alloc(&own, eval_u8_scratch_bytes(net, pop, batch, 2), stream) != cudaSuccess) {
+                cudaGetLastError();
+                pieces = false;  // no memory for it: the kernels that need no scratch
+            }
+            scratch = own;
+        }
+    }
+    if (pieces) {
+        err = launch_stage_xf(net, pop, x, batch, scratch, stream);
+        if (err == cudaSuccess)
+            err = launch_eval_u8_tc(net, pop, pop_dev, 2, nullptr, scratch, 1.0f, y, batch, alpha, f_inh, f_raw, f_adj,
+                                    correct, status, stream);
+        only = eval_u8_flagged(net, pop, batch, 2, scratch);
+    }
+    if (err == cudaSuccess) {
+        if (tf32_ok && path != LEEA_EVAL_SIMT)
+            err = launch_eval_tc(net, pop, pop_dev, x, y, batch, alpha, f_inh, f_raw, f_adj, correct, status, stream, only);
+        else
+            err = launch_eval_simt(net, pop, pop_dev, x, y, batch, alpha, f_inh, f_raw, f_adj, correct, stream, only);
+    }
+    if (own) {
+        const cudaError_t ferr = cudaFreeAsync(own, stream);
+        if (err == cudaSuccess) err = ferr;
     }
     if (err != cudaSuccess) return cuda_fail(err, "evaluate kernel");
     return LEEA_OK;
@@ -300,25 +331,34 @@ leea_status dispatch_eval_u8(const NetLayout& net, int32_t pop, const float* pop
     }
     // AUTO also takes the tensor cores where TENSOR does not promise them
     // (batches above 128, h up to 256 and not a multiple of 16).
-    const bool tc_ok = path == LEEA_EVAL_TENSOR ? eval_u8_tc_supported(net, pop, batch, pop_dev)
-                                                : eval_u8_wide_supported(net, pop, batch, pop_dev);
+    const bool strict = eval_u8_tc_supported(net, pop, batch, pop_dev);
+    bool tc_ok = strict || (path != LEEA_EVAL_TENSOR && eval_u8_wide_supported(net, pop, batch, pop_dev));
     if (path == LEEA_EVAL_TENSOR && !tc_ok)
         return fail(LEEA_EINVAL, "tensor-core evaluation of 8-bit inputs needs batch <= 128, d_0 %% 4 == 0, "
                                  "h %% 16 == 0, h <= 128, d_out <= 16 and a 16-byte aligned population");
     cudaError_t err;
-    if (tc_ok && path != LEEA_EVAL_SIMT) {
-        unsigned int* status = device_status_ptr();
-        if (!status) return fail(LEEA_ECUDA, "device status word unavailable");
-        void* own = nullptr;  // the call's own scratch, freed in stream order after the evaluation
-        if (!x16) {
-            LEEA_CUDA_TRY(scratch_alloc(&own, eval_u8_scratch_bytes(net, pop, batch), stream), "batch staging allocation");
-            x16 = own;
-            x16_staged = false;
+    unsigned int* status = device_status_ptr();
+    if (tc_ok && path != LEEA_EVAL_SIMT && !status) return fail(LEEA_ECUDA, "device status word unavailable");
+    void* own = nullptr;  // the call's own scratch, freed in stream order after the evaluation
+    if (tc_ok && path != LEEA_EVAL_SIMT && !x16) {
+        err = scratch_alloc(&own, eval_u8_scratch_bytes(net, pop, batch, 1), stream);
+        if (err != cudaSuccess && strict) return cuda_fail(err, "batch staging allocation");
+        if (err != cudaSuccess) {  // no memory for it: the CUDA cores need none
+            cudaGetLastError();
+            tc_ok = false;
         }
-        err = x16_staged ? cudaSuccess : launch_stage_x16(net, x, batch, x16, stream);
+        x16 = own;
+        x16_staged = false;
+    }
+    if (tc_ok && path != LEEA_EVAL_SIMT) {
+        err = x16_staged ? cudaSuccess : launch_stage_x16(net, pop, x, batch, x16, stream);
         if (err == cudaSuccess)
-            err = launch_eval_u8_tc(net, pop, pop_dev, x, x16, x_div, y, batch, alpha, f_inh, f_raw, f_adj, correct,
+            err = launch_eval_u8_tc(net, pop, pop_dev, 1, x, x16, x_div, y, batch, alpha, f_inh, f_raw, f_adj, correct,
                                     status, stream);
+        const int32_t* only = eval_u8_flagged(net, pop, batch, 1, x16);  // a weight outside the pieces' range
+        if (err == cudaSuccess && only)
+            err = launch_eval_simt_u8(net, pop, pop_dev, x, x_div, y, batch, alpha, f_inh, f_raw, f_adj, correct, stream,
+                                      only);
         if (own) {
             const cudaError_t ferr = cudaFreeAsync(own, stream);
             if (err == cudaSuccess) err = ferr;
@@ -1023,7 +1063,7 @@ leea_status leea_create(int32_t pop, const int32_t* dims, int32_t n_dims, const 
     }
     if (s->net.n_layers == 2 && p->precision == 0 && err == cudaSuccess &&
         eval_u8_tc_supported(s->net, pop, 128, s->popbuf[0])) {
-        s->x16_bytes = eval_u8_scratch_bytes(s->net, pop, 128);  // grown with the batch
+        s->x16_bytes = eval_u8_scratch_bytes(s->net, pop, 128, 1);  // grown with the batch
         err = cudaMalloc(&s->x16, s->x16_bytes);
     }
     if (p->sigma_ctl == LEEA_SIGMA_SELF) {
@@ -1231,18 +1271,25 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
                             (s->prm.eval_path == LEEA_EVAL_TENSOR
                                  ? eval_u8_tc_supported(s->net, s->pop, batch, s->popbuf[0])
                                  : eval_u8_wide_supported(s->net, s->pop, batch, s->popbuf[0]));
-    if (eval_u8_tc) {
-        const size_t need = eval_u8_scratch_bytes(s->net, s->pop, batch);
+    const bool eval_f_tc = !fused && !u8 && prec == 0 && s->prm.eval_path == LEEA_EVAL_AUTO && s->net.n_layers == 2 &&
+                           eval_u8_wide_supported(s->net, s->pop, batch, s->popbuf[0], 2);
+    if (eval_u8_tc || eval_f_tc) {
+        const size_t need = eval_u8_scratch_bytes(s->net, s->pop, batch, u8 ? 1 : 2);
         if (need > s->x16_bytes) {
             LEEA_CUDA_TRY(cudaStreamSynchronize(s->stream), "staging sync");
             cudaFree(s->x16);
             s->x16 = nullptr;
             s->x16_bytes = 0;
-            LEEA_CUDA_TRY(cudaMalloc(&s->x16, need), "batch staging allocation");
-            s->x16_bytes = need;
+            const cudaError_t err = cudaMalloc(&s->x16, need);
+            if (err == cudaSuccess) {
+                s->x16_bytes = need;
+            } else {  // the evaluation then looks for itself, and does without where it may
+                s->x16 = nullptr;
+                cudaGetLastError();
+            }
         }
     }
-    const bool stage_early = eval_u8_tc && !first;
+    const bool stage_early = eval_u8_tc && s->x16 && !first;
     if (!first) {
         const uint32_t g = s->gen + 1;
         const float sigma_g = sigma_of_breed(s->prm, g);
@@ -1265,7 +1312,7 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
             LEEA_CUDA_TRY(launch_rank_select(a, s->f_adj, s->order, s->par1, s->par2, s->kind, s->f_inh, s->stream),
                           "rank/select kernel");
             if (stage_early)  // runs beside the selection; the breed that follows waits for both
-                LEEA_CUDA_TRY(launch_stage_x16(s->net, static_cast<const uint8_t*>(x_dev), batch, s->x16, s->stream),
+                LEEA_CUDA_TRY(launch_stage_x16(s->net, s->pop, static_cast<const uint8_t*>(x_dev), batch, s->x16, s->stream),
                               "batch staging kernel");
             if ((shadow_pair || shadow_group) && !fused)
                 LEEA_CUDA_TRY(launch_stage_xop(s->net, prec, static_cast<const uint8_t*>(x_dev), batch, s->xop,
@@ -1355,7 +1402,7 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
         else
             st = dispatch_eval(s->net, s->pop, s->popbuf[s->cur], static_cast<const float*>(x_dev), y_dev, batch,
                                s->prm.alpha, first ? nullptr : s->f_inh, s->f_raw, s->f_adj, s->correct,
-                               s->prm.eval_path, s->stream);
+                               s->prm.eval_path, s->stream, eval_f_tc ? s->x16 : nullptr);
         sc.done();
         if (st) return st;
     }

@@ -10,19 +10,25 @@
 // per-sample cross-entropy (maximum subtracted, FP32) and the sum over the
 // batch use fixed reduction orders: identical individuals give bitwise
 // identical fitness.
+#include <algorithm>
+
 #include "leea_internal.h"
+#include "tc_ptx.cuh"
 
 namespace leea {
 
 constexpr int kEvalThreads = 256;  // 16 x 16 thread grid
 constexpr int kBK = 16;
 constexpr int kMaxOut = 32;
+constexpr int kOnlyCtas = 304;  // CTAs of a launch for marked individuals: two per SM
 
 struct EvalSimtArgs {
     int32_t d_in, h, d_out, batch;
     int64_t c_pad;
     float alpha;
     float x_div;  // 8-bit inputs: x = k / x_div
+    int32_t pop;
+    const int32_t* only;  // NULL, or 1 for the individuals to evaluate
 };
 
 __device__ __forceinline__ float input_value(float v, float) { return v; }
@@ -63,7 +69,18 @@ eval_simt_kernel(EvalSimtArgs e, const float* __restrict__ popv, const XT* __res
 
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
-    const int p = blockIdx.x;
+    // One CTA per individual; for the marked ones only, a few CTAs share them all
+    // and most find no mark among theirs.
+    if (e.only) {
+        ptx::grid_dep_wait();
+        int any = 0;
+        for (int64_t p = blockIdx.x + static_cast<int64_t>(tid) * gridDim.x; p < e.pop;
+             p += static_cast<int64_t>(kEvalThreads) * gridDim.x)
+            any |= __ldcg(e.only + p);
+        if (!__syncthreads_or(any)) return;
+    }
+    for (int p = blockIdx.x; p < e.pop; p += gridDim.x) {
+    if (e.only && !__ldcg(e.only + p)) continue;
     const int K = e.d_in, H = e.h, D = e.d_out, Bt = e.batch;
     const float* W1 = popv + static_cast<int64_t>(p) * e.c_pad;
     const float* b1 = W1 + static_cast<int64_t>(H) * K;
@@ -226,6 +243,7 @@ eval_simt_kernel(EvalSimtArgs e, const float* __restrict__ popv, const XT* __res
         if (f_adj) f_adj[p] = f_inh ? (1.0f - e.alpha) * f_inh[p] + e.alpha * f : f;
         if (correct) correct[p] = n_correct;
     }
+    }
 }
 
 template <int TM, int TN, typename XT>
@@ -238,6 +256,9 @@ static cudaError_t launch_simt_t(const EvalSimtArgs& e, int32_t pop, const float
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            static_cast<int>(smem));
     if (err != cudaSuccess) return err;
+    if (e.only)
+        return launch_pdl(eval_simt_kernel<TM, TN, XT>, dim3(static_cast<unsigned>(std::min(pop, kOnlyCtas))),
+                          dim3(kEvalThreads), smem, stream, e, popv, x, y, f_inh, f_raw, f_adj, correct);
     eval_simt_kernel<TM, TN, XT><<<pop, kEvalThreads, smem, stream>>>(e, popv, x, y, f_inh, f_raw, f_adj,
                                                                        correct);
     return cudaGetLastError();
@@ -251,10 +272,11 @@ static int pick_micro(int extent)
 template <typename XT>
 static cudaError_t launch_simt_any(const NetLayout& net, int32_t pop, const float* pop_dev, const XT* x,
                                    float x_div, const int32_t* y, int32_t batch, float alpha, const float* f_inh,
-                                   float* f_raw, float* f_adj, int32_t* correct, cudaStream_t stream)
+                                   float* f_raw, float* f_adj, int32_t* correct, cudaStream_t stream,
+                                   const int32_t* only)
 {
     if (net.n_layers != 2 || net.dims[2] > kMaxOut) return cudaErrorInvalidValue;
-    EvalSimtArgs e{ net.dims[0], net.dims[1], net.dims[2], batch, net.c_pad, alpha, x_div };
+    EvalSimtArgs e{ net.dims[0], net.dims[1], net.dims[2], batch, net.c_pad, alpha, x_div, pop, only };
     const int tm = pick_micro(e.h), tn = pick_micro(batch);
 #define LEEA_SIMT_CASE(A, B)                                                                      \
     if (tm == A && tn == B)                                                                       \
@@ -269,18 +291,19 @@ static cudaError_t launch_simt_any(const NetLayout& net, int32_t pop, const floa
 cudaError_t launch_eval_simt(const NetLayout& net, int32_t pop, const float* pop_dev,
                              const float* x, const int32_t* y, int32_t batch, float alpha,
                              const float* f_inh, float* f_raw, float* f_adj, int32_t* correct,
-                             cudaStream_t stream)
+                             cudaStream_t stream, const int32_t* only)
 {
     return launch_simt_any<float>(net, pop, pop_dev, x, 1.0f, y, batch, alpha, f_inh, f_raw, f_adj, correct,
-                                  stream);
+                                  stream, only);
 }
 
 cudaError_t launch_eval_simt_u8(const NetLayout& net, int32_t pop, const float* pop_dev, const uint8_t* x,
                                 float x_div, const int32_t* y, int32_t batch, float alpha, const float* f_inh,
-                                float* f_raw, float* f_adj, int32_t* correct, cudaStream_t stream)
+                                float* f_raw, float* f_adj, int32_t* correct, cudaStream_t stream,
+                                const int32_t* only)
 {
     return launch_simt_any<uint8_t>(net, pop, pop_dev, x, x_div, y, batch, alpha, f_inh, f_raw, f_adj, correct,
-                                    stream);
+                                    stream, only);
 }
 
 }  // namespace leea

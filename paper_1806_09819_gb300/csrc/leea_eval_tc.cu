@@ -48,6 +48,7 @@ struct EvalTcArgs {
     float* f_raw;
     float* f_adj;
     int32_t* correct;
+    const int32_t* only;  // NULL, or 1 for the individuals to evaluate
     unsigned int* status;
 };
 
@@ -107,6 +108,14 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
     const TcSmem s = carve(smem_raw, a);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
+    if (a.only) {  // no marked individual among this CTA's: nothing to do
+        ptx::grid_dep_wait();
+        int any = 0;
+        for (int64_t p = blockIdx.x + static_cast<int64_t>(threadIdx.x) * gridDim.x; p < a.pop;
+             p += static_cast<int64_t>(kTcThreads) * gridDim.x)
+            any |= __ldcg(a.only + p);
+        if (!__syncthreads_or(any)) return;
+    }
     if (threadIdx.x == 0) {
         for (int i = 0; i < a.stages; ++i) {
             ptx::mbar_init(&s.full[i], 1);
@@ -137,6 +146,7 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             uint32_t issued_mask = 0, parity_mask = 0;  // per stage: issued at all / parity of the last issue
             bool ok = true;
             for (int p = blockIdx.x; ok && p < a.pop; p += gridDim.x) {
+                if (a.only && !__ldcg(a.only + p)) continue;
                 for (int mt = 0; ok && mt < a.m_tiles; ++mt) {
                     for (int kc = 0; kc < a.k_chunks; ++kc) {
                         if (!ptx::mbar_wait_bounded(&s.empty[stage], phase ^ 1u, s.abort_flag, kWaitLimitNs)) {
@@ -168,6 +178,7 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
             bool ok = true;
             for (int p = blockIdx.x; ok && p < a.pop; p += gridDim.x) {
+                if (a.only && !__ldcg(a.only + p)) continue;
                 for (int mt = 0; ok && mt < a.m_tiles; ++mt) {
                     if (!ptx::mbar_wait_bounded(&s.acc_empty[acc], acc_phase ^ 1u, s.abort_flag, kWaitLimitNs)) {
                         raise_abort(s, a);
@@ -218,6 +229,7 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
         uint32_t stage = 0, phase = 0;
         bool ok = true;
         for (int p = blockIdx.x; ok && p < a.pop; p += gridDim.x) {
+            if (a.only && !__ldcg(a.only + p)) continue;
             for (int mt = 0; ok && mt < a.m_tiles; ++mt) {
                 for (int kc = 0; kc < a.k_chunks; ++kc) {
                     if (!ptx::mbar_wait_bounded(&s.full[stage], phase, s.abort_flag, kWaitLimitNs)) {
@@ -261,6 +273,7 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
         int32_t n_ok = 0;
         bool ok = true;
         for (int p = blockIdx.x; ok && p < a.pop; p += gridDim.x) {
+            if (a.only && !__ldcg(a.only + p)) continue;
             for (int mt = 0; mt < a.m_tiles; ++mt) {
                 if (mt == 0) {
                     const float* src = a.popv + static_cast<int64_t>(p) * a.c_pad + static_cast<int64_t>(a.h) * a.k;
@@ -401,7 +414,8 @@ bool eval_tc_supported(const NetLayout& net, int32_t batch, const float* pop_dev
 
 cudaError_t launch_eval_tc(const NetLayout& net, int32_t pop, const float* pop_dev, const float* x,
                            const int32_t* y, int32_t batch, float alpha, const float* f_inh, float* f_raw,
-                           float* f_adj, int32_t* correct, unsigned int* status, cudaStream_t stream)
+                           float* f_adj, int32_t* correct, unsigned int* status, cudaStream_t stream,
+                           const int32_t* only)
 {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
@@ -452,6 +466,7 @@ cudaError_t launch_eval_tc(const NetLayout& net, int32_t pop, const float* pop_d
     a.f_raw = f_raw;
     a.f_adj = f_adj;
     a.correct = correct;
+    a.only = only;
     a.status = status;
 
     const uint32_t stage_bytes = 2u * kXTileBytes + 2u * static_cast<uint32_t>(npad) * 128u;
@@ -471,6 +486,8 @@ cudaError_t launch_eval_tc(const NetLayout& net, int32_t pop, const float* pop_d
     err = cudaFuncSetAttribute(eval_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (err != cudaSuccess) return err;
     const int grid = pop < sms ? pop : sms;
+    if (only)
+        return launch_pdl(eval_tc_kernel, dim3(static_cast<unsigned>(grid)), dim3(kTcThreads), smem, stream, tx, tw, a);
     eval_tc_kernel<<<grid, kTcThreads, smem, stream>>>(tx, tw, a);
     return cudaGetLastError();
 }

@@ -1,16 +1,20 @@
-// leea_eval_u8.cu -- fitness of every individual (Eq. 1; Section 3.3) for
-// minibatches of 8-bit image levels, x = k / x_div with k in [0, 255] (MNIST's
-// encoding), on the tcgen05 tensor cores with FP32-class accuracy.
+// leea_eval_u8.cu -- fitness of every individual (Eq. 1; Section 3.3) on the
+// tcgen05 tensor cores with FP32-class accuracy, for minibatches of 8-bit image
+// levels, x = k / x_div with k in [0, 255] (MNIST's encoding), and of floats.
 //
-// Numerics.  The integers k are exact in FP16, and every FP32 weight, scaled
+// Numerics.  The integers k are exact in FP16 (XP = 1), a float sample is two
+// FP16 pieces of 2^e x (XP = 2, see stage_xf_kernel), and every FP32 weight, scaled
 // by 2^8, is split into two FP16 pieces: w1 = fp16(2^8 w) and
 // w2 = fp16(2^8 w - w1), with the remainder exact in FP32.  So
 // |2^8 w - w1 - w2| <= max(2^-22 2^8 |w|, 2^-25): a 22-bit significand
-// against FP32's 24, and D = K (w1 + w2)^T is formed from exact products; only
-// the FP32 accumulation in the tensor core rounds.  The epilogue scales by
-// 2^-8 / x_div.  An individual with a weight |w| >= 128 (its scaled w1 could
-// overflow FP16) is flagged by the converters, and the epilogue forms its
-// layer 1 with FP32 FFMA from global memory instead of the accumulator.
+// against FP32's 24, and D = K (w1 + w2)^T (for floats x1 w1 + x1 w2 + x2 w1) is
+// formed from exact products; only the FP32 accumulation in the tensor core
+// rounds.  The epilogue scales by 2^-8 / x_div or by the sample's own factor.
+// The converters find the individuals that the pieces cannot carry
+// (outside_pieces).  On 8-bit levels within TENSOR's shapes the epilogue forms
+// their layer 1 with FP32 FFMA from global memory; elsewhere it marks them and
+// a launch of the TF32 or the CUDA-core kernel for the marked ones follows
+// (2 us when there are none).
 //
 // Shape.  A tcgen05.mma of M = 128 and K = 16 costs about the same time for any
 // N up to 256, so two individuals share every MMA where both fit (hp = h rounded
@@ -28,11 +32,15 @@
 //
 // Measured, P = 1000, 784-112-10: batch 100 84 us (4.2 TB/s of weights; without
 // the epilogue's arithmetic 76), 256 124, 512 217, 1024 417, against 1.2 ms
-// (256) to 9.8 ms (1024) on the CUDA cores; 333 nets 784-100-10, batch 50: 37
+// (256) to 9.8 ms (1024) on the CUDA cores; 333 nets 784-100-10, batch 50: 40
 // (295).  Several tiles are bound by the weight stream (once per two tiles, the
 // repeats from L2) and by the epilogue, which cannot overlap the next unit when
 // the unit's accumulators take more than half of tensor memory (165 us at 512
-// without its arithmetic).
+// without its arithmetic).  Floats: P = 1000, 784-112-10, batch 100: 85 us,
+// against 184 with TF32 pieces (12 MMAs of K = 8 per 32 inputs and individual
+// instead of 6 of K = 16 per pair); batch 512 268 (711); 784-100-10, batch 50,
+// 82 (341 on the CUDA cores).  Max error against 64 bits over 1000 nets 6.6e-8
+// (TF32 pieces 1.4e-7).
 //
 // Pipeline (persistent CTA, one per SM; each CTA takes a contiguous range of
 // individuals, as pairs, the last one alone when the range is odd, or of units,
@@ -61,6 +69,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cuda_fp16.h>
 
 #include "leea_internal.h"
@@ -108,12 +117,14 @@ struct EvalU8Args {
     int32_t n_bufs;          // accumulator buffers: 2 where a unit's columns fit twice
     int32_t per_cta, extra;  // work per CTA: per_cta, one more for the first `extra` CTAs
     uint32_t slot_bytes;     // one individual's slice of a stage: hp raw rows
-    uint32_t a_bytes;        // one batch tile: round_up(batch, 8) (or, with several tiles, 128) rows of FP16 levels
+    uint32_t a_bytes;        // one piece of a batch tile: round_up(batch, 8) (or, with several tiles, 128) FP16 rows
     uint32_t stage_bytes;    // the batch tiles and the slots, rounded up to 1 KB
     int64_t c_pad;
-    float inv_div, alpha;
+    float inv_div, alpha;    // 8-bit levels: accumulator units to x units
     const float* popv;
-    const uint8_t* x;        // the levels, for the FP32 fallback
+    const uint8_t* x;        // the levels, for the FP32 fallback inside TENSOR's shapes
+    const float* x_scale;    // float inputs: accumulator units to x units, per sample
+    int32_t* flagged;        // [pop]: 1 = a weight outside the pieces' range, to be evaluated again (or NULL: here)
     const int32_t* y;
     const float* f_inh;
     float* f_raw;
@@ -132,7 +143,7 @@ struct U8Smem {
     float* b2;           // [2 groups][16]
     double* red_loss;    // [2 groups][2 tiles][4 quarters]
     int32_t* red_ok;     // [2 groups][2 tiles][4 quarters]
-    uint32_t* flag;      // [kFlagSlots][2]: u + 1 if unit u's individual in that slot has |w| >= 128
+    uint32_t* flag;      // [kFlagSlots][2]: (u + 1) << 8 | the largest exponent field of unit u's individual
     uint32_t* accflag;   // [2]: the flags of the unit in that accumulator, for the epilogue
     int* ep_go;          // [2 groups]: their go words
     uint32_t* tmem_holder;
@@ -187,6 +198,7 @@ __device__ __forceinline__ U8Smem carve(uint8_t* raw, const EvalU8Args& a)
 // How a population and a batch are cut into units.
 struct U8Shape {
     int32_t hp, ni, tiles_per_unit, ks, n_stages;
+    int32_t xp;  // FP16 pieces of an input: 1 for 8-bit levels, 2 for floats
 };
 
 uint32_t u8_a_bytes(int32_t batch, int32_t ks)
@@ -194,14 +206,14 @@ uint32_t u8_a_bytes(int32_t batch, int32_t ks)
     return static_cast<uint32_t>(batch > 128 ? 128 : (batch + 7) / 8 * 8) * 2u * static_cast<uint32_t>(ks);
 }
 
-// A stage holds the batch tiles and the slots, and at least the 128 rows of A
-// the MMA reads from its start.
+// A stage holds the batch tiles (each of xp pieces) and the slots, and at least
+// the 128 rows of A the MMA reads from the start of each.
 uint32_t u8_stage_bytes(const U8Shape& u, int32_t batch)
 {
     const uint32_t ks = static_cast<uint32_t>(u.ks);
-    const uint32_t b = static_cast<uint32_t>(u.tiles_per_unit) * u8_a_bytes(batch, u.ks) +
-                       static_cast<uint32_t>(u.ni) * static_cast<uint32_t>(u.hp) * 4u * ks;
-    return std::max((b + 1023u) & ~1023u, 128u * 2u * ks);
+    const uint32_t n_a = static_cast<uint32_t>(u.tiles_per_unit * u.xp), a = u8_a_bytes(batch, u.ks);
+    const uint32_t b = n_a * a + static_cast<uint32_t>(u.ni) * static_cast<uint32_t>(u.hp) * 4u * ks;
+    return (std::max(b, (n_a - 1u) * a + 128u * 2u * ks) + 1023u) & ~1023u;
 }
 
 size_t u8_smem_bytes(const U8Shape& u, int32_t d_out, int32_t batch)
@@ -246,10 +258,14 @@ __device__ __forceinline__ void split2x2(float w0, float w1, uint32_t& p1, uint3
     p2 = half2_bits(__floats2half2_rn(s0 - f1.x, s1 - f1.y));
 }
 
-__device__ __forceinline__ bool out_of_piece_range(const float4& v)
+// Whether an individual whose largest |w| has this exponent field is outside
+// the pieces' range: |w| >= 128 overflows them; with float inputs also no
+// weight of 2^-10 or more (but not all zero), because a piece pair resolves
+// 2^-33 and so would carry less than the 22 bits the TF32 pieces carry.
+template <int XP>
+__device__ __forceinline__ bool outside_pieces(uint32_t exponent)
 {
-    return fabsf(v.x) >= kPieceRange || fabsf(v.y) >= kPieceRange || fabsf(v.z) >= kPieceRange ||
-           fabsf(v.w) >= kPieceRange;
+    return exponent >= 127u + 7u || (XP == 2 && exponent != 0u && exponent < 127u - 10u);
 }
 
 // Four weights of row r (0..7) of an 8-row group, inputs 4 c4 .. 4 c4 + 3 of
@@ -309,16 +325,17 @@ struct UnitWalk {
     }
 };
 
-template <int KS, int TILES>
+template <int KS, int TILES, int XP>
 __global__ void __launch_bounds__(kU8Threads, 1)
 eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                const EvalU8Args a)
 {
     using S = StageShape<KS>;
+    if (a.flagged) ptx::grid_dep_launch();  // the kernel for the marked individuals starts by waiting for this one
     extern __shared__ uint8_t smem_raw[];
     const U8Smem s = carve(smem_raw, a);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t slots_off = TILES * a.a_bytes;          // the slots within a stage
+    const uint32_t slots_off = TILES * XP * a.a_bytes;          // the slots within a stage
     const uint32_t tile_cols = static_cast<uint32_t>(a.ni * a.hp);  // a tile's accumulator columns
     // Accumulator buffer and phase of unit u.
     auto buf_of = [&](int u) { return a.n_bufs == 2 ? static_cast<uint32_t>(u) & 1u : 0u; };
@@ -383,13 +400,16 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
 #pragma unroll
                         for (int t = 0; t < TILES; ++t) {
                             if (t >= x.nt) break;
-                            const uint64_t ad =
-                                ptx::smem_desc(sb + t * a.a_bytes + 32u * kk, 8u * S::kPieceRow, S::kSwizzle);
+                            // x1 w1, x1 w2 and, for two-piece inputs, x2 w1 (x2 w2 is
+                            // below 2^-22 of the product).
 #pragma unroll
-                            for (int q = 0; q < 2; ++q) {
-                                const uint64_t bd =
-                                    ptx::smem_desc(sb + slots_off + S::kPieceOff * q + 32u * kk, S::kGroup, S::kSwizzle);
-                                ptx::mma_f16(d + t * tile_cols, ad, bd, idesc, (kc | kk | q) != 0 ? 1u : 0u);
+                            for (int e = 0; e < 1 + XP; ++e) {
+                                const int xq = e >> 1, wq = e & 1;
+                                const uint64_t ad = ptx::smem_desc(sb + (t * XP + xq) * a.a_bytes + 32u * kk,
+                                                                   8u * S::kPieceRow, S::kSwizzle);
+                                const uint64_t bd = ptx::smem_desc(sb + slots_off + S::kPieceOff * wq + 32u * kk,
+                                                                   S::kGroup, S::kSwizzle);
+                                ptx::mma_f16(d + t * tile_cols, ad, bd, idesc, (kc | kk | e) != 0 ? 1u : 0u);
                             }
                         }
                     }
@@ -399,11 +419,10 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 if (!ok) break;
                 ptx::mma_commit(&s.acc_full[buf]);
                 // Every converter arrival of this unit was acquired above, so
-                // its range flags are final; hand them to the epilogue with a
-                // releasing arrival on the same barrier.
+                // its exponents are final; hand the verdicts to the epilogue with
+                // a releasing arrival on the same barrier.
                 const volatile uint32_t* fl = s.flag + 2 * (u % kFlagSlots);
-                const uint32_t tag = static_cast<uint32_t>(u) + 1u;
-                s.accflag[buf] = (fl[0] == tag ? 1u : 0u) | (fl[1] == tag ? 2u : 0u);
+                s.accflag[buf] = (outside_pieces<XP>(fl[0] & 255u) ? 1u : 0u) | (outside_pieces<XP>(fl[1] & 255u) ? 2u : 0u);
                 ptx::mbar_arrive(&s.acc_full[buf]);
             }
             ptx::mma_commit(s.drain);
@@ -426,10 +445,13 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                         break;
                     }
                     uint8_t* sb = s.ring + stage * a.stage_bytes;
-                    ptx::mbar_arrive_expect_tx(&s.a_full[stage], static_cast<uint32_t>(x.nt) * a.a_bytes +
+                    ptx::mbar_arrive_expect_tx(&s.a_full[stage], static_cast<uint32_t>(x.nt * XP) * a.a_bytes +
                                                                      static_cast<uint32_t>(x.n) * a.slot_bytes);
                     for (int t = 0; t < x.nt; ++t)
-                        ptx::tma_load_2d(sb + t * a.a_bytes, &tmap_x, &s.a_full[stage], kc * KS, (x.t0 + t) * 128);
+#pragma unroll
+                        for (int e = 0; e < XP; ++e)
+                            ptx::tma_load_3d(sb + (t * XP + e) * a.a_bytes, &tmap_x, &s.a_full[stage], kc * KS,
+                                             (x.t0 + t) * 128, e);
                     for (int j = 0; j < x.n; ++j)
                         ptx::tma_load_3d(sb + slots_off + j * a.slot_bytes, &tmap_w, &s.a_full[stage], kc * KS, 0,
                                          x.p0 + j);
@@ -457,6 +479,7 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         Unit x;
         for (int u = 0; ok && walk.next(a, x); ++u) {
             const int groups = x.n * gps;
+            float top0 = 0.0f, top1 = 0.0f;  // this warp's largest |w| of each individual (NaN aside)
             for (int kc = 0; kc < a.k_stages; ++kc) {
                 if (!ptx::mbar_wait_bounded(&s.a_full[stage], phase, s.abort_flag, kWaitLimitNs)) {
                     raise_abort(s, a);
@@ -464,7 +487,6 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                     break;
                 }
                 uint8_t* sb = s.ring + stage * a.stage_bytes + slots_off;
-                bool bad0 = false, bad1 = false;
 #pragma unroll
                 for (int g0 = 0; g0 < kMaxGroups / kConvWarps; g0 += S::kBatch) {
                     // Read a batch of this warp's groups, then overwrite them.
@@ -483,23 +505,27 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                     for (int b = 0; b < S::kBatch; ++b) {
                         const int g = cw + kConvWarps * (g0 + b);
                         if (g < groups) {
-                            bool bad = false;
+                            float top = 0.0f;
 #pragma unroll
                             for (int m = 0; m < S::kF4; ++m) {
                                 const int fi = lane + 32 * m;
                                 put_pieces<KS>(sb + g * S::kGroup, fi / (KS / 4), fi % (KS / 4), f[b][m]);
-                                bad |= out_of_piece_range(f[b][m]);
+                                top = fmaxf(fmaxf(top, fmaxf(fabsf(f[b][m].x), fabsf(f[b][m].y))),
+                                            fmaxf(fabsf(f[b][m].z), fabsf(f[b][m].w)));
                             }
-                            if (g < gps) bad0 |= bad; else bad1 |= bad;
+                            if (g < gps) top0 = fmaxf(top0, top); else top1 = fmaxf(top1, top);
                         }
                     }
                     __syncwarp();
                 }
-                const bool any0 = __any_sync(0xFFFFFFFFu, bad0), any1 = __any_sync(0xFFFFFFFFu, bad1);
-                if (lane == 0) {
-                    const uint32_t tag = static_cast<uint32_t>(u) + 1u;
-                    if (any0) atomicExch(&s.flag[2 * (u % kFlagSlots)], tag);
-                    if (any1) atomicExch(&s.flag[2 * (u % kFlagSlots) + 1], tag);
+                if (kc == a.k_stages - 1) {
+                    const uint32_t e0 = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(top0)) >> 23;
+                    const uint32_t e1 = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(top1)) >> 23;
+                    const uint32_t tag = (static_cast<uint32_t>(u) + 1u) << 8;
+                    if (lane == 0) {
+                        atomicMax(&s.flag[2 * (u % kFlagSlots)], tag | e0);
+                        atomicMax(&s.flag[2 * (u % kFlagSlots) + 1], tag | e1);
+                    }
                 }
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
@@ -573,8 +599,13 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 const bool in = smp < a.batch;
                 float loss = 0.0f;
                 unsigned good = 0;
-                // Individuals with a weight outside the piece range: layer 1 by
-                // FP32 FFMA from global memory, k in order, in the accumulator's units.
+                // Individuals with a weight outside the piece range: marked for the
+                // evaluation that follows or, within TENSOR's shapes on 8-bit levels,
+                // layer 1 here by FP32 FFMA from global memory, k in order, in the
+                // accumulator's units.
+                const bool redo = XP == 1 && gov == 2 && !a.flagged;
+                const float scale = XP == 1 ? a.inv_div : (in ? __ldcg(a.x_scale + smp) : 0.0f);
+                if (a.flagged && (gov == 2 || scale != scale)) a.flagged[p] = 1;
                 const float* w1p = a.popv + static_cast<int64_t>(p) * a.c_pad;
                 const uint8_t* xrow = a.x + static_cast<int64_t>(in ? smp : 0) * a.k;
                 const uint32_t col0 = tmem_base + lane_addr + buf * kAccStride + static_cast<uint32_t>(t) * tile_cols +
@@ -586,7 +617,7 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                     float v[16];
                     ptx::tmem_ld16(col0 + static_cast<uint32_t>(c), v);
                     if (in) {
-                        if (gov == 2) {
+                        if (redo) {
 #pragma unroll
                             for (int j = 0; j < 16; ++j) {
                                 if (c + j < a.h) {
@@ -601,7 +632,7 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
                             const int col = c + j;
-                            const float hv = fmaxf(fmaf(v[j], a.inv_div, b1s[col]), 0.0f);
+                            const float hv = fmaxf(fmaf(v[j], scale, b1s[col]), 0.0f);
                             const float4* wr = reinterpret_cast<const float4*>(w2t + col * a.dpad);
 #pragma unroll
                             for (int o4 = 0; o4 < kMaxOutU8 / 4; ++o4) {
@@ -710,9 +741,11 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
 // 8) with zero padding: the A operand tiles of eval_u8_kernel.  It reads only
 // the caller's levels, so it lets the next kernel start at once; before it
 // ends it waits for its own predecessor, so that a successor that waits for it
-// also sees everything earlier on the stream complete.
+// also sees everything earlier on the stream complete.  Then it clears the
+// marks, which an earlier evaluation may have been reading until now.
 __global__ void __launch_bounds__(256) stage_x16_kernel(const uint8_t* __restrict__ x, int32_t batch, int32_t k,
-                                                        int32_t kp, __half* __restrict__ x16)
+                                                        int32_t kp, __half* __restrict__ x16,
+                                                        int32_t* __restrict__ flagged, int32_t pop)
 {
     ptx::grid_dep_launch();
     const int32_t per_row = kp >> 3;
@@ -730,6 +763,64 @@ __global__ void __launch_bounds__(256) stage_x16_kernel(const uint8_t* __restric
         *reinterpret_cast<uint4*>(x16 + static_cast<int64_t>(b) * kp + k0) = make_uint4(w[0], w[1], w[2], w[3]);
     }
     ptx::grid_dep_wait();
+    if (flagged)
+        for (int64_t p = i; p < pop; p += static_cast<int64_t>(gridDim.x) * blockDim.x) flagged[p] = 0;
+}
+
+// A float batch as two FP16 pieces of 2^e x, [2][batch][kp]: e per sample, so
+// that its largest |x| lands in [2^14, 2^15); x1 rounds 2^e x, x2 the remainder
+// (exact in FP32), so the pieces carry 22 bits of every value near the largest
+// and absolute errors of 2^-39 of it below.  x_scale[b] = 2^-(e + 8) turns the
+// accumulator's units (2^e x times 2^8 w) into x w; NaN for a sample with an
+// infinite or NaN input, whose individuals are all evaluated again by a kernel
+// that multiplies x itself.  A CTA per sample.
+__global__ void __launch_bounds__(256) stage_xf_kernel(const float* __restrict__ x, int32_t batch, int32_t k, int32_t kp,
+                                                       __half* __restrict__ x16, float* __restrict__ x_scale,
+                                                       int32_t* __restrict__ flagged, int32_t pop)
+{
+    __shared__ uint32_t top[8];
+    ptx::grid_dep_launch();
+    const int32_t b = blockIdx.x;
+    const float4* src = reinterpret_cast<const float4*>(x + static_cast<int64_t>(b) * k);  // k % 4 == 0
+    uint32_t mx = 0;
+    for (int32_t i = threadIdx.x; i < k / 4; i += blockDim.x) {
+        const float4 v = src[i];
+        mx = max(max(max(mx, __float_as_uint(v.x) & 0x7FFFFFFFu), __float_as_uint(v.y) & 0x7FFFFFFFu),
+                 max(__float_as_uint(v.z) & 0x7FFFFFFFu, __float_as_uint(v.w) & 0x7FFFFFFFu));
+    }
+    mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+    if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    mx = 0;
+    for (int w = 0; w < 8; ++w) mx = max(mx, top[w]);
+    // 2^e x of the largest in [2^14, 2^15), e within what FP32 scales exactly.
+    int e = 0;
+    if (mx != 0u && mx < 0x7F800000u) {
+        int ex = 0;
+        frexpf(__uint_as_float(mx), &ex);  // in [2^(ex-1), 2^ex)
+        e = min(15 - ex, 126);
+    }
+    const float up = ldexpf(1.0f, e);
+    for (int32_t i = threadIdx.x; i < kp / 4; i += blockDim.x) {
+        const float4 v = 4 * i < k ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float s[4] = { v.x * up, v.y * up, v.z * up, v.w * up };
+        uint32_t p1[2], p2[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const __half2 h1 = __floats2half2_rn(s[2 * h], s[2 * h + 1]);
+            const float2 f1 = __half22float2(h1);
+            p1[h] = half2_bits(h1);
+            p2[h] = half2_bits(__floats2half2_rn(s[2 * h] - f1.x, s[2 * h + 1] - f1.y));
+        }
+        uint2* dst = reinterpret_cast<uint2*>(x16 + static_cast<int64_t>(b) * kp) + i;
+        dst[0] = make_uint2(p1[0], p1[1]);
+        dst[static_cast<int64_t>(batch) * kp / 4] = make_uint2(p2[0], p2[1]);
+    }
+    if (threadIdx.x == 0) x_scale[b] = mx < 0x7F800000u ? ldexpf(1.0f, -e - 8) : __int_as_float(0x7FC00000);
+    ptx::grid_dep_wait();
+    for (int64_t p = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; p < pop;
+         p += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        flagged[p] = 0;
 }
 
 // A batch of several tiles: each individual's loss and correct count from its
@@ -773,9 +864,10 @@ U8EncodeTiledFn u8_encode_fn()
 // both fit its 256 columns, two tiles per unit where the batch has them (a
 // weight slice is converted once for both), less of either when that leaves
 // SMs without a unit.
-bool u8_shape(const NetLayout& net, int32_t pop, int32_t batch, int32_t sms, U8Shape* u)
+bool u8_shape(const NetLayout& net, int32_t pop, int32_t batch, int32_t xp, int32_t sms, U8Shape* u)
 {
-    if (batch < 1 || eval_u8_scratch_bytes(net, pop, batch) > kMaxScratchU8) return false;
+    if (batch < 1 || eval_u8_scratch_bytes(net, pop, batch, xp) > kMaxScratchU8) return false;
+    u->xp = xp;
     const int32_t tiles = (batch + 127) / 128;
     u->hp = (net.dims[1] + 15) / 16 * 16;
     u->ni = u->hp <= 128 ? 2 : 1;
@@ -792,53 +884,115 @@ bool u8_shape(const NetLayout& net, int32_t pop, int32_t batch, int32_t sms, U8S
 
 }  // namespace
 
-bool eval_u8_tc_supported(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev)
+// Shapes that eval_path TENSOR promises for 8-bit levels: their fitness is the
+// fused kernel's, bit for bit.
+static bool in_tensor_shapes(const NetLayout& net, int32_t batch)
 {
-    return net.dims[1] % 16 == 0 && net.dims[1] <= 128 && batch <= 128 &&
-           eval_u8_wide_supported(net, pop, batch, pop_dev);
+    return net.dims[1] % 16 == 0 && net.dims[1] <= 128 && batch <= 128;
 }
 
-bool eval_u8_wide_supported(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev)
+// Whether the pieces pay where another kernel could take the call: staging the
+// batch and looking for marked individuals are two more launches, and a call
+// takes 25 us with them however small it is (784-100-10 and 50 samples: 152
+// nets 23 us, 1000 nets 79), 14 without.  The other kernel's time is modelled
+// from its waves, fitted to k = 32 .. 784, h = 10 .. 256, batches 20 .. 512:
+// TF32 pieces, one CTA per SM, per wave and 128 samples 2.5 + 0.085 h + (0.011 +
+// 0.00013 h) k us; CUDA cores, two per SM, per wave, 128 hidden units and 64
+// samples 5 + 0.08 k us, half of it for h <= 32.  Measured around the line: 152
+// nets of k-112-10 on 100 float samples, k = 256 23 us without and 25 with, k =
+// 400 27 and 26; 333 nets of k-100-10 on 50 8-bit samples, k = 32 21 and 25, k =
+// 128 43 and 25.  A pair of nets costs an SM 4.8 us at least, which the CUDA
+// cores beat on the smallest nets at any population (4000 of 32-10-10 on 20
+// samples: 58 and 63 us).
+static bool pieces_pay(const NetLayout& net, int32_t pop, int32_t batch, int32_t xp)
+{
+    constexpr double kSms = 152.0, kPiecesUs = 25.0, kPairUs = 4.8;
+    const double k = net.dims[0], h = net.dims[1], b = batch;
+    if (xp == 2 && net.dims[1] % 16 == 0) {
+        const double wave = std::ceil(b / 128.0) * (2.5 + 0.085 * h + (0.011 + 0.00013 * h) * k);
+        return std::ceil(pop / kSms) * wave >= kPiecesUs;
+    }
+    const double wave = std::ceil(h / 128.0) * std::ceil(b / 64.0) * (5.0 + 0.08 * k) * (h <= 32.0 ? 0.5 : 1.0);
+    return wave >= kPairUs && std::ceil(pop / (2.0 * kSms)) * wave >= kPiecesUs;
+}
+
+static bool pieces_fit(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev, int32_t xp)
 {
     if (net.n_layers != 2) return false;
     if (net.dims[0] % 4 != 0 || net.dims[1] > 256 || net.dims[2] > kMaxOutU8) return false;
     if (reinterpret_cast<uintptr_t>(pop_dev) & 15u) return false;
     U8Shape u;
-    return u8_shape(net, pop, batch, 1, &u) && u8_encode_fn() != nullptr;
+    return u8_shape(net, pop, batch, xp, 1, &u) && u8_encode_fn() != nullptr;
 }
 
-// Scratch layout: the FP16 batch (rounded up to 256 bytes), then for several
-// tiles their loss sums and correct counts.
-static size_t x16_bytes(const NetLayout& net, int32_t batch)
+bool eval_u8_tc_supported(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev)
 {
-    const size_t kp = static_cast<size_t>((net.dims[0] + 7) / 8 * 8);
-    return (static_cast<size_t>(batch) * kp * 2u + 255u) / 256u * 256u;
+    return in_tensor_shapes(net, batch) && pieces_fit(net, pop, batch, pop_dev, 1);
 }
 
-size_t eval_u8_scratch_bytes(const NetLayout& net, int32_t pop, int32_t batch)
+bool eval_u8_wide_supported(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev, int32_t xp)
 {
-    const size_t tiles = static_cast<size_t>((batch + 127) / 128);
-    return x16_bytes(net, batch) + (tiles > 1 ? 12u * tiles * static_cast<size_t>(pop) : 0u);
+    if (!pieces_fit(net, pop, batch, pop_dev, xp)) return false;
+    return (xp == 1 && in_tensor_shapes(net, batch)) || pieces_pay(net, pop, batch, xp);
 }
 
-cudaError_t launch_stage_x16(const NetLayout& net, const uint8_t* x, int32_t batch, void* x16, cudaStream_t stream)
+bool eval_u8_marks(const NetLayout& net, int32_t batch, int32_t xp) { return xp == 2 || !in_tensor_shapes(net, batch); }
+
+// Scratch layout, each part rounded up to 256 bytes: the FP16 pieces of the
+// batch, the float samples' scales, the marks, several tiles' loss sums and
+// correct counts.
+namespace {
+struct U8Scratch {
+    size_t scale, flagged, part, part_ok, bytes;
+};
+
+U8Scratch u8_scratch(const NetLayout& net, int32_t pop, int32_t batch, int32_t xp)
+{
+    auto up = [](size_t n) { return (n + 255u) / 256u * 256u; };
+    const size_t kp = static_cast<size_t>((net.dims[0] + 7) / 8 * 8), nb = static_cast<size_t>(batch);
+    const size_t np = static_cast<size_t>(pop), tiles = (nb + 127u) / 128u;
+    U8Scratch s;
+    s.scale = up(static_cast<size_t>(xp) * nb * kp * 2u);
+    s.flagged = s.scale + (xp == 2 ? up(4u * nb) : 0u);
+    s.part = s.flagged + (eval_u8_marks(net, batch, xp) ? up(4u * np) : 0u);
+    s.part_ok = s.part + (tiles > 1 ? up(8u * tiles * np) : 0u);
+    s.bytes = s.part_ok + (tiles > 1 ? up(4u * tiles * np) : 0u);
+    return s;
+}
+}  // namespace
+
+size_t eval_u8_scratch_bytes(const NetLayout& net, int32_t pop, int32_t batch, int32_t xp)
+{
+    return u8_scratch(net, pop, batch, xp).bytes;
+}
+
+int32_t* eval_u8_flagged(const NetLayout& net, int32_t pop, int32_t batch, int32_t xp, void* scratch)
+{
+    if (!eval_u8_marks(net, batch, xp)) return nullptr;
+    return reinterpret_cast<int32_t*>(static_cast<uint8_t*>(scratch) + u8_scratch(net, pop, batch, xp).flagged);
+}
+
+cudaError_t launch_stage_x16(const NetLayout& net, int32_t pop, const uint8_t* x, int32_t batch, void* scratch,
+                             cudaStream_t stream)
 {
     const int32_t k = net.dims[0], kp = (k + 7) / 8 * 8;
     const int64_t items = static_cast<int64_t>(batch) * (kp / 8);
     if (items <= 0) return cudaSuccess;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>((items + 255) / 256));
-    cfg.blockDim = dim3(256);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, stage_x16_kernel, x, batch, k, kp, static_cast<__half*>(x16));
+    return launch_pdl(stage_x16_kernel, dim3(static_cast<unsigned>((items + 255) / 256)), dim3(256), 0, stream, x, batch,
+                      k, kp, static_cast<__half*>(scratch), eval_u8_flagged(net, pop, batch, 1, scratch), pop);
 }
 
-cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* pop_dev, const uint8_t* x,
+cudaError_t launch_stage_xf(const NetLayout& net, int32_t pop, const float* x, int32_t batch, void* scratch,
+                            cudaStream_t stream)
+{
+    const U8Scratch u = u8_scratch(net, pop, batch, 2);
+    return launch_pdl(stage_xf_kernel, dim3(static_cast<unsigned>(batch)), dim3(256), 0, stream, x, batch, net.dims[0],
+                      (net.dims[0] + 7) / 8 * 8, static_cast<__half*>(scratch),
+                      reinterpret_cast<float*>(static_cast<uint8_t*>(scratch) + u.scale),
+                      eval_u8_flagged(net, pop, batch, 2, scratch), pop);
+}
+
+cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* pop_dev, int32_t xp, const uint8_t* x,
                               void* scratch, float x_div, const int32_t* y, int32_t batch, float alpha,
                               const float* f_inh, float* f_raw, float* f_adj, int32_t* correct, unsigned int* status,
                               cudaStream_t stream)
@@ -849,7 +1003,7 @@ cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* po
     err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return err;
     U8Shape u;
-    if (!u8_shape(net, pop, batch, sms, &u)) return cudaErrorInvalidValue;
+    if (!u8_shape(net, pop, batch, xp, sms, &u)) return cudaErrorInvalidValue;
     const int32_t ks = u.ks;
     EvalU8Args a{};
     a.pop = pop;
@@ -876,10 +1030,14 @@ cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* po
     a.f_raw = f_raw;
     a.f_adj = f_adj;
     a.correct = correct;
-    a.part = reinterpret_cast<double*>(static_cast<uint8_t*>(scratch) + x16_bytes(net, batch));
-    a.part_ok = reinterpret_cast<int32_t*>(a.part + static_cast<size_t>(a.tiles) * static_cast<size_t>(pop));
+    const U8Scratch sc = u8_scratch(net, pop, batch, xp);
+    uint8_t* base = static_cast<uint8_t*>(scratch);
+    a.x_scale = reinterpret_cast<const float*>(base + sc.scale);
+    a.flagged = eval_u8_flagged(net, pop, batch, xp, scratch);
+    a.part = reinterpret_cast<double*>(base + sc.part);
+    a.part_ok = reinterpret_cast<int32_t*>(base + sc.part_ok);
     a.status = status;
-    a.wide = a.tiles > 1 || a.h % 16 != 0 || a.h > 128;
+    a.wide = xp == 2 || !in_tensor_shapes(net, batch);
     a.slot_bytes = static_cast<uint32_t>(a.hp) * 4u * static_cast<uint32_t>(ks);
     a.a_bytes = u8_a_bytes(batch, ks);
     a.stage_bytes = u8_stage_bytes(u, batch);
@@ -901,24 +1059,27 @@ cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* po
             return cudaErrorInvalidValue;
     }
     {
-        // The staged batch: [batch][kp] FP16, tiles of round_up(batch, 8) rows
-        // (128 with several tiles); rows past the batch and levels past k read
-        // as zero.
+        // The staged batch: [xp][batch][kp] FP16, tiles of round_up(batch, 8)
+        // rows (128 with several tiles); rows past the batch and inputs past k
+        // read as zero.
         const int32_t kp = (a.k + 7) / 8 * 8;
-        const cuuint64_t dims[2] = { static_cast<cuuint64_t>(a.k), static_cast<cuuint64_t>(batch) };
-        const cuuint64_t strides[1] = { static_cast<cuuint64_t>(kp) * 2u };
-        const cuuint32_t box[2] = { static_cast<cuuint32_t>(ks),
-                                    static_cast<cuuint32_t>(batch > 128 ? 128 : (batch + 7) / 8 * 8) };
-        const cuuint32_t es[2] = { 1, 1 };
-        if (enc(&tx, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, scratch, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        const cuuint64_t dims[3] = { static_cast<cuuint64_t>(a.k), static_cast<cuuint64_t>(batch),
+                                     static_cast<cuuint64_t>(xp) };
+        const cuuint64_t strides[2] = { static_cast<cuuint64_t>(kp) * 2u,
+                                        static_cast<cuuint64_t>(kp) * 2u * static_cast<cuuint64_t>(batch) };
+        const cuuint32_t box[3] = { static_cast<cuuint32_t>(ks),
+                                    static_cast<cuuint32_t>(batch > 128 ? 128 : (batch + 7) / 8 * 8), 1 };
+        const cuuint32_t es[3] = { 1, 1, 1 };
+        if (enc(&tx, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, scratch, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 ks == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
     typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const EvalU8Args);
-    const bool two = u.tiles_per_unit == 2;
-    const Kernel kern = ks == 64 ? (two ? eval_u8_kernel<64, 2> : eval_u8_kernel<64, 1>)
-                                 : (two ? eval_u8_kernel<32, 2> : eval_u8_kernel<32, 1>);
+    static const Kernel kernels[2][2][2] = {  // [K stage 64][two tiles][two pieces]
+        { { eval_u8_kernel<32, 1, 1>, eval_u8_kernel<32, 1, 2> }, { eval_u8_kernel<32, 2, 1>, eval_u8_kernel<32, 2, 2> } },
+        { { eval_u8_kernel<64, 1, 1>, eval_u8_kernel<64, 1, 2> }, { eval_u8_kernel<64, 2, 1>, eval_u8_kernel<64, 2, 2> } } };
+    const Kernel kern = kernels[ks == 64][u.tiles_per_unit == 2][xp == 2];
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (err != cudaSuccess) return err;
     const int64_t work = a.groups == 1 ? pop : static_cast<int64_t>((pop + a.ni - 1) / a.ni) * a.groups;

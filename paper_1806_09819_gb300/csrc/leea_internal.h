@@ -265,35 +265,44 @@ cudaError_t launch_eval_shadow_runs(int32_t k, int32_t d_out, int32_t precision,
                                     int32_t n_runs, int32_t pop_max, bool any_tiles, const ShadowRun* runs_dev,
                                     const ShadowSeg* segs_dev, const int32_t* seg_off_dev, int32_t grid,
                                     unsigned int* status, cudaStream_t stream);
-// Evaluation of d_0-h-d_out nets (one hidden layer), SIMT FP32.
+// Evaluation of d_0-h-d_out nets (one hidden layer), SIMT FP32.  only (here and
+// below): if not NULL, just the individuals p with only[p] != 0.
 cudaError_t launch_eval_simt(const NetLayout& net, int32_t pop, const float* pop_dev,
                              const float* x, const int32_t* y, int32_t batch, float alpha,
                              const float* f_inh, float* f_raw, float* f_adj, int32_t* correct,
-                             cudaStream_t stream);
+                             cudaStream_t stream, const int32_t* only = nullptr);
 // Evaluation on the tcgen05 tensor cores (3xTF32), d_0-h-d_out with d_0 % 4 == 0,
 // h % 16 == 0, h <= 256, d_out <= 16 and 16-byte aligned population and x.
 bool eval_tc_supported(const NetLayout& net, int32_t batch, const float* pop_dev, const float* x);
 cudaError_t launch_eval_tc(const NetLayout& net, int32_t pop, const float* pop_dev, const float* x,
                            const int32_t* y, int32_t batch, float alpha, const float* f_inh, float* f_raw,
-                           float* f_adj, int32_t* correct, unsigned int* status, cudaStream_t stream);
-// 8-bit inputs x = k / x_div: CUDA-core FP32 evaluation of any shape, and the
-// tensor-core evaluation (two individuals per MMA, exact FP16 pieces) for
-// d_0 % 4 == 0, h <= 256, d_out <= 16 and a scratch of at most 256 MB
-// (eval_u8_wide_supported);
-// LEEA_EVAL_TENSOR promises only batch <= 128, h % 16 == 0, h <= 128
-// (eval_u8_tc_supported).  It reads the batch as FP16 from scratch
-// (eval_u8_scratch_bytes(net, pop, batch) bytes, 256-byte aligned; several
-// 128-sample tiles put their sums behind it), which launch_stage_x16 fills from
-// the levels earlier on the same stream; the staging kernel lets its successor
-// start at once and waits for its own predecessor before it ends.
+                           float* f_adj, int32_t* correct, unsigned int* status, cudaStream_t stream,
+                           const int32_t* only = nullptr);
+// CUDA-core FP32 evaluation of 8-bit inputs x = k / x_div, any shape.
 cudaError_t launch_eval_simt_u8(const NetLayout& net, int32_t pop, const float* pop_dev, const uint8_t* x,
                                 float x_div, const int32_t* y, int32_t batch, float alpha, const float* f_inh,
-                                float* f_raw, float* f_adj, int32_t* correct, cudaStream_t stream);
+                                float* f_raw, float* f_adj, int32_t* correct, cudaStream_t stream,
+                                const int32_t* only = nullptr);
+// The tensor-core evaluation with FP16 operand pieces (two individuals per MMA)
+// for d_0 % 4 == 0, h <= 256, d_out <= 16 and a scratch of at most 256 MB
+// (eval_u8_wide_supported): 8-bit levels as one exact piece (xp = 1) or float
+// inputs as two (xp = 2, x 16-byte aligned), the weights as two.
+// LEEA_EVAL_TENSOR promises for 8-bit levels only batch <= 128, h % 16 == 0,
+// h <= 128 (eval_u8_tc_supported).  It reads the batch from scratch
+// (eval_u8_scratch_bytes, 256-byte aligned), which launch_stage_x16 or _xf fills
+// earlier on the same stream; the staging kernels let their successor start at
+// once and wait for their own predecessor before they end.  Where
+// eval_u8_flagged is not NULL, individuals with a weight |w| >= 128 are marked
+// there and their results are to be taken from another kernel ("only" below).
 bool eval_u8_tc_supported(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev);
-bool eval_u8_wide_supported(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev);
-size_t eval_u8_scratch_bytes(const NetLayout& net, int32_t pop, int32_t batch);
-cudaError_t launch_stage_x16(const NetLayout& net, const uint8_t* x, int32_t batch, void* x16, cudaStream_t stream);
-cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* pop_dev, const uint8_t* x,
+bool eval_u8_wide_supported(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev, int32_t xp = 1);
+size_t eval_u8_scratch_bytes(const NetLayout& net, int32_t pop, int32_t batch, int32_t xp);
+int32_t* eval_u8_flagged(const NetLayout& net, int32_t pop, int32_t batch, int32_t xp, void* scratch);
+cudaError_t launch_stage_x16(const NetLayout& net, int32_t pop, const uint8_t* x, int32_t batch, void* scratch,
+                             cudaStream_t stream);
+cudaError_t launch_stage_xf(const NetLayout& net, int32_t pop, const float* x, int32_t batch, void* scratch,
+                            cudaStream_t stream);
+cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* pop_dev, int32_t xp, const uint8_t* x,
                               void* scratch, float x_div, const int32_t* y, int32_t batch, float alpha,
                               const float* f_inh, float* f_raw, float* f_adj, int32_t* correct, unsigned int* status,
                               cudaStream_t stream);
