@@ -30,17 +30,20 @@
 // slices stream HBM faster (measured with no compute: 4.8 against 4.0-4.4 TB/s
 // for the same 351 MB).
 //
-// Measured, P = 1000, 784-112-10: batch 100 84 us (4.2 TB/s of weights; without
-// the epilogue's arithmetic 76), 256 124, 512 217, 1024 417, against 1.2 ms
-// (256) to 9.8 ms (1024) on the CUDA cores; 333 nets 784-100-10, batch 50: 40
-// (295).  Several tiles are bound by the weight stream (once per two tiles, the
-// repeats from L2) and by the epilogue, which cannot overlap the next unit when
-// the unit's accumulators take more than half of tensor memory (165 us at 512
-// without its arithmetic).  Floats: P = 1000, 784-112-10, batch 100: 85 us,
-// against 184 with TF32 pieces (12 MMAs of K = 8 per 32 inputs and individual
-// instead of 6 of K = 16 per pair); batch 512 268 (711); 784-100-10, batch 50,
-// 82 (341 on the CUDA cores).  Max error against 64 bits over 1000 nets 6.6e-8
-// (TF32 pieces 1.4e-7).
+// Measured, P = 1000, 784-112-10: batch 100 76 us (4.6 TB/s of weights), 256
+// 111, 512 195, 1000 356, against 1.2 ms (256) to 9.8 ms (1024) on the CUDA
+// cores; 333 nets 784-100-10, batch 50: 40 (295).  Floats: P = 1000, 784-112-10,
+// batch 100: 83, against 184 with TF32 pieces (12 MMAs of K = 8 per 32 inputs and
+// individual instead of 6 of K = 16 per pair); batch 512 246 (711); 784-100-10,
+// batch 50, 77 (341 on the CUDA cores).  Max error against 64 bits over 1000 nets
+// 6.6e-8 (TF32 pieces 1.4e-7).
+//
+// What bounds it: shared memory.  Per K stage of 64 inputs a unit of one net and
+// two tiles has 61 KB written by TMA, 57 KB read and written by the converters
+// and 123 KB of operands read by the MMAs (A again for each weight piece), 1.9k
+// cycles at 128 bytes a cycle of the 2.1k that a stage takes; the epilogue's
+// reads of W2 come on top (quad_logits).  One lone tile is also close to the
+// weight stream itself (52 us at 6.8 TB/s).
 //
 // Pipeline (persistent CTA, one per SM; each CTA takes a contiguous range of
 // individuals, as pairs, the last one alone when the range is odd, or of units,
@@ -93,7 +96,6 @@ constexpr int kFlagSlots = 16;          // unit-tagged range flags; converters r
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kAccStride = 256;    // the two accumulators: columns 0 and 256
 constexpr float kPieceScale = 256.0f;   // 2^8: weights enter the pieces as 2^8 w
-constexpr float kPieceRange = 128.0f;   // |w| below this: 2^8 |w| < 2^15, finite in FP16
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 constexpr uint64_t kDrainLimitNs = 200000000ull;
 
@@ -110,7 +112,8 @@ struct StageShape {
 };
 
 struct EvalU8Args {
-    int32_t pop, k, h, d_out, dpad, batch, k16, k_stages, n_stages;
+    int32_t pop, k, h, d_out, batch, k16, k_stages, n_stages;
+    int32_t no4, wst;        // output groups of four; floats between W2's rows in shared memory
     int32_t hp;              // hidden units rounded up to 16: the rows of a slot, the columns of an accumulator
     int32_t ni;              // individuals per unit: 2, or 1 (hp > 128, or too few units for the SMs)
     int32_t tiles, groups;   // 128-sample tiles of the batch; groups of TILES of them
@@ -138,7 +141,7 @@ struct EvalU8Args {
 
 struct U8Smem {
     uint8_t* ring;       // n_stages x stage_bytes, 1024-aligned: the batch tile, then W1 slices (raw, then pieces)
-    float* w2t;          // [2 epilogue groups][hp][dpad]
+    float* w2t;          // [2 epilogue groups][hp][wst]
     float* b1;           // [2 groups][hp]
     float* b2;           // [2 groups][16]
     double* red_loss;    // [2 groups][2 tiles][4 quarters]
@@ -154,9 +157,18 @@ struct U8Smem {
 constexpr size_t kTailFixed = 8 + sizeof(double) * 16 + sizeof(int32_t) * 16 + sizeof(uint32_t) * (2 * kFlagSlots + 2) +
                               sizeof(int) * 2 + 16 + 16;
 
-size_t u8_tail_bytes(int32_t h, int32_t dpad, int32_t n_stages)
+// Floats between the rows (a hidden unit's outputs) of W2 in shared memory: the
+// rows 0, 2, 4 and 6 that a quad reads together (quad_logits) fall on
+// different banks.
+int32_t w2_stride(int32_t d_out)
 {
-    return sizeof(float) * (2u * h * dpad + 2u * h + 32u) + kTailFixed + 8u * (3u * n_stages + 5u);
+    const int32_t no4 = (d_out + 3) / 4;
+    return no4 == 2 ? 12 : (no4 == 4 ? 20 : 4 * no4);
+}
+
+size_t u8_tail_bytes(int32_t h, int32_t wst, int32_t n_stages)
+{
+    return sizeof(float) * (2u * h * wst + 2u * h + 32u) + kTailFixed + 8u * (3u * n_stages + 5u);
 }
 
 __device__ __forceinline__ U8Smem carve(uint8_t* raw, const EvalU8Args& a)
@@ -165,7 +177,7 @@ __device__ __forceinline__ U8Smem carve(uint8_t* raw, const EvalU8Args& a)
     s.ring = raw + ((1024u - (ptx::smem_u32(raw) & 1023u)) & 1023u);
     uint8_t* p = s.ring + static_cast<size_t>(a.n_stages) * a.stage_bytes;
     s.w2t = reinterpret_cast<float*>(p);
-    p += sizeof(float) * 2 * a.hp * a.dpad;
+    p += sizeof(float) * 2 * a.hp * a.wst;
     s.b1 = reinterpret_cast<float*>(p);
     p += sizeof(float) * 2 * a.hp;
     s.b2 = reinterpret_cast<float*>(p);
@@ -218,8 +230,7 @@ uint32_t u8_stage_bytes(const U8Shape& u, int32_t batch)
 
 size_t u8_smem_bytes(const U8Shape& u, int32_t d_out, int32_t batch)
 {
-    const int32_t dpad = (d_out + 3) / 4 * 4;
-    return 1024 + static_cast<size_t>(u.n_stages) * u8_stage_bytes(u, batch) + u8_tail_bytes(u.hp, dpad, u.n_stages);
+    return 1024 + static_cast<size_t>(u.n_stages) * u8_stage_bytes(u, batch) + u8_tail_bytes(u.hp, w2_stride(d_out), u.n_stages);
 }
 
 // K stage and ring depth: 64 inputs when at least kMinStages such stages fit in
@@ -325,12 +336,84 @@ struct UnitWalk {
     }
 };
 
+// Layer 2 of the 32 samples of a warp (TMEM lanes of col0) for the shapes beyond
+// TENSOR's: logits [4 O4, 4 O4 + 4 NO4) of one sample per lane, sample 8 (lane %
+// 4) + lane / 4 of the 32.  W2 comes from shared memory, which gives a warp that
+// reads one address 4 bytes a cycle; with a sample per lane the reads alone
+// (h x 12 floats per warp) take 10.7k cycles per 256 samples of a 112-10 net,
+// longer than its MMAs.  So a lane takes four samples and a quarter of the hidden
+// units (the 16x256b shape of the accumulator): the four lanes of a quad read
+// different rows of W2 in one go, each for four samples, a quarter of the
+// cycles, and their partial logits are added across the quad.
+template <int NO4, int O4>
+__device__ __forceinline__ void quad_logits(uint32_t col0, int hp, const float (&scale)[4], const float* b1s,
+                                            const float* w2t, int wst, float* z)
+{
+    const int lane = threadIdx.x & 31, m = lane & 3;
+    float2 acc[4][2 * NO4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int o = 0; o < 2 * NO4; ++o) acc[j][o] = make_float2(0.0f, 0.0f);
+    for (int c = 0; c < hp; c += 16) {
+        uint32_t v[16];
+        ptx::tmem_ld_16x256_nowait(col0 + static_cast<uint32_t>(c), v);
+        ptx::tmem_ld_16x256_nowait(col0 + (16u << 16) + static_cast<uint32_t>(c), v + 8);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const int col = c + 8 * half + 2 * m;
+            const float2 b = *reinterpret_cast<const float2*>(b1s + col);
+            float2 h[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int at = 8 * (j >> 1) + 4 * half + 2 * (j & 1);
+                h[j] = __ffma2_rn(make_float2(__uint_as_float(v[at]), __uint_as_float(v[at + 1])),
+                                  make_float2(scale[j], scale[j]), b);
+                h[j].x = fmaxf(h[j].x, 0.0f);
+                h[j].y = fmaxf(h[j].y, 0.0f);
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float4* wr = reinterpret_cast<const float4*>(w2t + (col + e) * wst) + O4;
+#pragma unroll
+                for (int o = 0; o < NO4; ++o) {
+                    const float4 w = wr[o];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float hj = e ? h[j].y : h[j].x;
+                        acc[j][2 * o] = __ffma2_rn(make_float2(w.x, w.y), make_float2(hj, hj), acc[j][2 * o]);
+                        acc[j][2 * o + 1] = __ffma2_rn(make_float2(w.z, w.w), make_float2(hj, hj), acc[j][2 * o + 1]);
+                    }
+                }
+            }
+        }
+    }
+    // Lane m of a quad keeps row m: two of the four rows across lane ^ 2, one
+    // of those across lane ^ 1.
+    const bool up = m & 2, odd = m & 1;
+#pragma unroll
+    for (int o = 0; o < 2 * NO4; ++o) {
+        float2 keep[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float2 give = up ? acc[j][o] : acc[2 + j][o], mine = up ? acc[2 + j][o] : acc[j][o];
+            keep[j].x = mine.x + __shfl_xor_sync(0xFFFFFFFFu, give.x, 2);
+            keep[j].y = mine.y + __shfl_xor_sync(0xFFFFFFFFu, give.y, 2);
+        }
+        const float2 give = odd ? keep[0] : keep[1], mine = odd ? keep[1] : keep[0];
+        z[4 * O4 + 2 * o] = mine.x + __shfl_xor_sync(0xFFFFFFFFu, give.x, 1);
+        z[4 * O4 + 2 * o + 1] = mine.y + __shfl_xor_sync(0xFFFFFFFFu, give.y, 1);
+    }
+}
+
 template <int KS, int TILES, int XP>
 __global__ void __launch_bounds__(kU8Threads, 1)
 eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                const EvalU8Args a)
 {
     using S = StageShape<KS>;
+    constexpr bool kQuads = TILES == 2;
     if (a.flagged) ptx::grid_dep_launch();  // the kernel for the marked individuals starts by waiting for this one
     extern __shared__ uint8_t smem_raw[];
     const U8Smem s = carve(smem_raw, a);
@@ -368,17 +451,25 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
 
     if (warp == 0) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        // The whole warp runs the loops, one lane issues: see mma_f16_lo.
+        {
+            const uint32_t lead = ptx::elect_one();
+            const uint32_t a_hi = static_cast<uint32_t>(ptx::smem_desc(0u, 8u * S::kPieceRow, S::kSwizzle) >> 32);
+            const uint32_t b_hi = static_cast<uint32_t>(ptx::smem_desc(0u, S::kGroup, S::kSwizzle) >> 32);
+            const uint32_t a_units = a.a_bytes >> 4;
             const uint32_t idesc1 = ptx::idesc_f16(128, static_cast<uint32_t>(a.hp));
             const uint32_t idesc2 = ptx::idesc_f16(128, 2u * static_cast<uint32_t>(a.hp));
             const uint32_t ring = ptx::smem_u32(s.ring);
             uint32_t stage = 0, phase = 0;
             bool ok = true;
+            auto wait = [&](uint64_t* bar, uint32_t parity) {
+                return __all_sync(0xFFFFFFFFu, ptx::mbar_wait_bounded(bar, parity, s.abort_flag, kWaitLimitNs)) != 0;
+            };
             UnitWalk<TILES> walk(a);
             Unit x;
             for (int u = 0; ok && walk.next(a, x); ++u) {
                 const uint32_t buf = buf_of(u);
-                if (!ptx::mbar_wait_bounded(&s.acc_empty[buf], phase_of(u) ^ 1u, s.abort_flag, kWaitLimitNs)) {
+                if (!wait(&s.acc_empty[buf], phase_of(u) ^ 1u)) {
                     raise_abort(s, a);
                     ok = false;
                     break;
@@ -387,13 +478,15 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 const uint32_t d = tmem_base + buf * kAccStride;
                 const uint32_t idesc = x.n == 2 ? idesc2 : idesc1;
                 for (int kc = 0; kc < a.k_stages; ++kc) {
-                    if (!ptx::mbar_wait_bounded(&s.full[stage], phase, s.abort_flag, kWaitLimitNs)) {
+                    if (!wait(&s.full[stage], phase)) {
                         raise_abort(s, a);
                         ok = false;
                         break;
                     }
                     ptx::tc_fence_after();
-                    const uint32_t sb = ring + stage * a.stage_bytes;
+                    const uint32_t sa = ptx::desc_lo(ring + stage * a.stage_bytes);
+                    const uint32_t sw = sa + (slots_off >> 4);
+                    const uint32_t acc = kc == 0 ? 0u : 1u;
 #pragma unroll
                     for (int kk = 0; kk < KS / 16; ++kk) {
                         if (kc * KS + kk * 16 >= a.k16) break;
@@ -405,27 +498,28 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
 #pragma unroll
                             for (int e = 0; e < 1 + XP; ++e) {
                                 const int xq = e >> 1, wq = e & 1;
-                                const uint64_t ad = ptx::smem_desc(sb + (t * XP + xq) * a.a_bytes + 32u * kk,
-                                                                   8u * S::kPieceRow, S::kSwizzle);
-                                const uint64_t bd = ptx::smem_desc(sb + slots_off + S::kPieceOff * wq + 32u * kk,
-                                                                   S::kGroup, S::kSwizzle);
-                                ptx::mma_f16(d + t * tile_cols, ad, bd, idesc, (kc | kk | e) != 0 ? 1u : 0u);
+                                ptx::mma_f16_lo(d + t * tile_cols, sa + (t * XP + xq) * a_units + 2u * kk,
+                                                sw + (S::kPieceOff >> 4) * wq + 2u * kk, a_hi, b_hi, idesc,
+                                                (kk | e) != 0 ? 1u : acc, lead);
                             }
                         }
                     }
-                    ptx::mma_commit(&s.empty[stage]);
+                    if (lead) ptx::mma_commit(&s.empty[stage]);
                     if (++stage == static_cast<uint32_t>(a.n_stages)) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
-                ptx::mma_commit(&s.acc_full[buf]);
+                if (lead) ptx::mma_commit(&s.acc_full[buf]);
                 // Every converter arrival of this unit was acquired above, so
                 // its exponents are final; hand the verdicts to the epilogue with
                 // a releasing arrival on the same barrier.
-                const volatile uint32_t* fl = s.flag + 2 * (u % kFlagSlots);
-                s.accflag[buf] = (outside_pieces<XP>(fl[0] & 255u) ? 1u : 0u) | (outside_pieces<XP>(fl[1] & 255u) ? 2u : 0u);
-                ptx::mbar_arrive(&s.acc_full[buf]);
+                if (lead) {
+                    const volatile uint32_t* fl = s.flag + 2 * (u % kFlagSlots);
+                    s.accflag[buf] = (outside_pieces<XP>(fl[0] & 255u) ? 1u : 0u) | (outside_pieces<XP>(fl[1] & 255u) ? 2u : 0u);
+                    ptx::mbar_arrive(&s.acc_full[buf]);
+                }
             }
-            ptx::mma_commit(s.drain);
+            if (lead) ptx::mma_commit(s.drain);
+            __syncwarp();
             volatile int never = 0;
             ptx::mbar_wait_bounded(s.drain, 0u, &never, ok ? kWaitLimitNs : kDrainLimitNs);
         }
@@ -541,14 +635,13 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         const int g = ew >> 2;
         const int q = warp & 3;       // TMEM lane quarter of this warp
         const int et = (ew & 3) * 32 + lane;
-        const int row = q * 32 + lane;
         const uint32_t lane_addr = static_cast<uint32_t>(q * 32) << 16;
         const uint32_t bar_id = 1u + static_cast<uint32_t>(g);
         const int slot = a.ni == 2 ? g : 0;
         const int t_first = a.ni == 2 ? 0 : g, t_step = a.ni == 2 ? 1 : 2;
         float* b1s = s.b1 + g * a.hp;
         float* b2s = s.b2 + g * 16;
-        float* w2t = s.w2t + g * a.hp * a.dpad;
+        float* w2t = s.w2t + g * a.hp * a.wst;
         int* go = s.ep_go + g;
         ptx::grid_dep_wait();  // b1, W2, b2 come from the previous kernel (breeding)
         UnitWalk<TILES> walk(a);
@@ -559,7 +652,7 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
             const bool active = slot < x.n && t_first < x.nt;
             if (active) {
                 // While this unit's MMAs run: b1, W2 transposed (rows padded to
-                // dpad with zeros, hidden units past h zero) and b2 of this
+                // wst with zeros, hidden units past h zero) and b2 of this
                 // group's individual, as stored after W1, into shared memory.
                 // The group finished reading the previous ones at its last
                 // barrier B.  Loads go through L2 (ld.global.cg), not the
@@ -568,15 +661,20 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 // assumes data no grid changes during the kernel.
                 const float* src = a.popv + static_cast<int64_t>(p) * a.c_pad + static_cast<int64_t>(a.h) * a.k;
                 for (int i = et; i < a.hp; i += 128) b1s[i] = i < a.h ? __ldcg(src + i) : 0.0f;
-                for (int i = et; i < a.d_out * a.h; i += 128) {
-                    const int o = i / a.h, col = i - o * a.h;
-                    w2t[col * a.dpad + o] = __ldcg(src + a.h + i);
+                for (int col = et; col < a.hp; col += 128) {
+                    float w[kMaxOutU8];  // all in flight at once
+#pragma unroll
+                    for (int o = 0; o < kMaxOutU8; ++o)
+                        w[o] = o < a.d_out && col < a.h ? __ldcg(src + a.h + o * a.h + col) : 0.0f;
+#pragma unroll
+                    for (int o4 = 0; o4 < kMaxOutU8 / 4; ++o4)
+                        if (4 * o4 < a.wst)
+                            *reinterpret_cast<float4*>(w2t + col * a.wst + 4 * o4) =
+                                make_float4(w[4 * o4], w[4 * o4 + 1], w[4 * o4 + 2], w[4 * o4 + 3]);
                 }
-                const int pad = a.dpad - a.d_out;
-                for (int i = et; i < a.h * pad; i += 128) w2t[(i / pad) * a.dpad + a.d_out + i % pad] = 0.0f;
-                for (int i = a.h * a.dpad + et; i < a.hp * a.dpad; i += 128) w2t[i] = 0.0f;
                 if (et < 16) b2s[et] = et < a.d_out ? __ldcg(src + a.h + a.d_out * a.h + et) : 0.0f;
             }
+            const float inherited = active && et == 0 && a.f_inh && a.tiles == 1 ? a.f_inh[p] : 0.0f;
             if (et == 0) {
                 const bool got = ptx::mbar_wait_bounded(&s.acc_full[buf], phase_of(u), s.abort_flag, kWaitLimitNs);
                 if (!got) raise_abort(s, a);
@@ -595,24 +693,43 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
             }
 
             for (int t = t_first; t < x.nt; t += t_step) {
-                const int smp = (x.t0 + t) * 128 + row;  // this thread's sample
+                const int first = (x.t0 + t) * 128 + q * 32;  // the warp's samples
+                const int smp = first + (kQuads ? 8 * (lane & 3) + (lane >> 2) : lane);  // this thread's sample
                 const bool in = smp < a.batch;
+                const int32_t label = in ? a.y[smp] : 0;
                 float loss = 0.0f;
                 unsigned good = 0;
-                // Individuals with a weight outside the piece range: marked for the
-                // evaluation that follows or, within TENSOR's shapes on 8-bit levels,
-                // layer 1 here by FP32 FFMA from global memory, k in order, in the
-                // accumulator's units.
-                const bool redo = XP == 1 && gov == 2 && !a.flagged;
-                const float scale = XP == 1 ? a.inv_div : (in ? __ldcg(a.x_scale + smp) : 0.0f);
-                if (a.flagged && (gov == 2 || scale != scale)) a.flagged[p] = 1;
-                const float* w1p = a.popv + static_cast<int64_t>(p) * a.c_pad;
-                const uint8_t* xrow = a.x + static_cast<int64_t>(in ? smp : 0) * a.k;
                 const uint32_t col0 = tmem_base + lane_addr + buf * kAccStride + static_cast<uint32_t>(t) * tile_cols +
                                       static_cast<uint32_t>(slot * a.hp);
-                float logit[kMaxOutU8];
+                // Individuals with a weight outside the piece range, and samples that
+                // the pieces cannot carry: marked for the evaluation that follows or,
+                // within TENSOR's shapes on 8-bit levels, layer 1 here by FP32 FFMA
+                // from global memory, k in order.
+                float scale[4];  // accumulator units to x units, per sample
 #pragma unroll
-                for (int o = 0; o < kMaxOutU8; ++o) logit[o] = 0.0f;
+                for (int j = 0; j < 4; ++j) {
+                    const int sj = kQuads ? first + 8 * j + (lane >> 2) : smp;
+                    scale[j] = XP == 1 ? a.inv_div : (sj < a.batch ? __ldcg(a.x_scale + sj) : 0.0f);
+                    if (a.flagged && (gov == 2 || scale[j] != scale[j])) a.flagged[p] = 1;
+                    if (!kQuads) break;
+                }
+                float logit[kMaxOutU8];
+                if constexpr (kQuads) {
+                    switch (a.no4) {
+                    case 1: quad_logits<1, 0>(col0, a.hp, scale, b1s, w2t, a.wst, logit); break;
+                    case 2: quad_logits<2, 0>(col0, a.hp, scale, b1s, w2t, a.wst, logit); break;
+                    case 3: quad_logits<3, 0>(col0, a.hp, scale, b1s, w2t, a.wst, logit); break;
+                    default:
+                        quad_logits<2, 0>(col0, a.hp, scale, b1s, w2t, a.wst, logit);
+                        quad_logits<2, 2>(col0, a.hp, scale, b1s, w2t, a.wst, logit);
+                    }
+                } else {
+                const bool redo = XP == 1 && gov == 2 && !a.flagged;
+                const float* w1p = a.popv + static_cast<int64_t>(p) * a.c_pad;
+                const uint8_t* xrow = a.x + static_cast<int64_t>(in ? smp : 0) * a.k;
+                float2 logit2[kMaxOutU8 / 2];
+#pragma unroll
+                for (int o = 0; o < kMaxOutU8 / 2; ++o) logit2[o] = make_float2(0.0f, 0.0f);
                 for (int c = 0; c < a.hp; c += 16) {
                     float v[16];
                     ptx::tmem_ld16(col0 + static_cast<uint32_t>(c), v);
@@ -629,23 +746,33 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                                 }
                             }
                         }
+                        const float2 scale2 = make_float2(scale[0], scale[0]);
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const int col = c + j;
-                            const float hv = fmaxf(fmaf(v[j], scale, b1s[col]), 0.0f);
-                            const float4* wr = reinterpret_cast<const float4*>(w2t + col * a.dpad);
+                        for (int j2 = 0; j2 < 8; ++j2) {
+                            const float2 b = *reinterpret_cast<const float2*>(b1s + c + 2 * j2);
+                            const float2 z = __ffma2_rn(make_float2(v[2 * j2], v[2 * j2 + 1]), scale2, b);
+                            const float hv[2] = { fmaxf(z.x, 0.0f), fmaxf(z.y, 0.0f) };
 #pragma unroll
-                            for (int o4 = 0; o4 < kMaxOutU8 / 4; ++o4) {
-                                if (4 * o4 < a.d_out) {
-                                    const float4 w = wr[o4];
-                                    logit[4 * o4 + 0] = fmaf(w.x, hv, logit[4 * o4 + 0]);
-                                    logit[4 * o4 + 1] = fmaf(w.y, hv, logit[4 * o4 + 1]);
-                                    logit[4 * o4 + 2] = fmaf(w.z, hv, logit[4 * o4 + 2]);
-                                    logit[4 * o4 + 3] = fmaf(w.w, hv, logit[4 * o4 + 3]);
+                            for (int e = 0; e < 2; ++e) {
+                                const float4* wr = reinterpret_cast<const float4*>(w2t + (c + 2 * j2 + e) * a.wst);
+                                const float2 h2 = make_float2(hv[e], hv[e]);
+#pragma unroll
+                                for (int o4 = 0; o4 < kMaxOutU8 / 4; ++o4) {
+                                    if (4 * o4 < a.d_out) {
+                                        const float4 w = wr[o4];
+                                        logit2[2 * o4] = __ffma2_rn(make_float2(w.x, w.y), h2, logit2[2 * o4]);
+                                        logit2[2 * o4 + 1] = __ffma2_rn(make_float2(w.z, w.w), h2, logit2[2 * o4 + 1]);
+                                    }
                                 }
                             }
                         }
                     }
+                }
+#pragma unroll
+                for (int o = 0; o < kMaxOutU8 / 2; ++o) {
+                    logit[2 * o] = logit2[o].x;
+                    logit[2 * o + 1] = logit2[o].y;
+                }
                 }
                 if (t + t_step >= x.nt) {
                     // The accumulator is read: release it to the next unit's MMAs.
@@ -654,7 +781,6 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                     if (lane == 0) ptx::mbar_arrive(&s.acc_empty[buf]);
                 }
                 if (in) {
-                    const int32_t label = a.y[smp];
                     float bo[kMaxOutU8];
 #pragma unroll
                     for (int o = 0; o < kMaxOutU8; ++o) bo[o] = b2s[o];
@@ -716,7 +842,7 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                             f = -((((r0 + r1) + r2) + r3) / static_cast<float>(a.batch));
                         }
                         a.f_raw[p] = f;
-                        if (a.f_adj) a.f_adj[p] = a.f_inh ? (1.0f - a.alpha) * a.f_inh[p] + a.alpha * f : f;
+                        if (a.f_adj) a.f_adj[p] = a.f_inh ? (1.0f - a.alpha) * inherited + a.alpha * f : f;
                         if (a.correct) a.correct[p] = n_ok;
                     } else {
                         const int64_t at = static_cast<int64_t>(x.t0 + t) * a.pop + p;
@@ -876,6 +1002,12 @@ bool u8_shape(const NetLayout& net, int32_t pop, int32_t batch, int32_t xp, int3
         auto units = [&](int32_t ni, int32_t tp) {
             return static_cast<int64_t>((pop + ni - 1) / ni) * ((tiles + tp - 1) / tp);
         };
+        // Two tiles of two individuals fill tensor memory from h = 65 on, and the
+        // epilogue then waits for the MMAs and they for it; one individual leaves
+        // room for the next unit.  It pays where a unit's MMAs are long (1000 nets
+        // k-112-10, 512 samples: k = 784 200 against 207 us, k = 100 108 against 96;
+        // 784-64-10, two buffers either way: 150 against 130).
+        if (u->hp > 64 && net.dims[0] >= 256) u->ni = 1;
         if (units(u->ni, 2) < sms) u->tiles_per_unit = 1;
         if (u->ni == 2 && units(2, u->tiles_per_unit) < sms) u->ni = 1;
     }
@@ -1012,7 +1144,8 @@ cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* po
     a.d_out = net.dims[2];
     a.batch = batch;
     a.k16 = (a.k + 15) / 16 * 16;
-    a.dpad = (a.d_out + 3) / 4 * 4;
+    a.no4 = (a.d_out + 3) / 4;
+    a.wst = w2_stride(a.d_out);
     a.k_stages = (a.k + ks - 1) / ks;
     a.n_stages = u.n_stages;
     a.hp = u.hp;
