@@ -2,53 +2,59 @@
 // as the paper's 196-256-128-64-10 (Section 4.1), on the tcgen05 tensor cores
 // with FP32-class accuracy, for minibatches of 8-bit levels x = k / x_div.
 //
-// A unit is one individual on one 128-sample tile.  Layers 1-3 are MMAs with
-// the samples as M = 128 and FP32 accumulation in tensor memory (layer 1 in
-// columns [0, d1), layers 2 and 3 both from column d1: layer 3 starts after
-// the epilogue has read layer 2):
+// A unit is one individual on one 128-sample tile.  All four layers are MMAs
+// with the samples as M = 128 and FP32 accumulation in tensor memory:
 //   layer 1     A = the tile's levels k, exact in FP16; B = 2^8 W1 as two FP16
 //               pieces hi = fp16(2^8 w), lo = fp16(2^8 w - hi) (the remainder is
 //               exact in FP32): 2 MMAs per 16 inputs, only the accumulation rounds
-//   layers 2, 3 A = 2^8 h of the layer below and B = 2^8 W, both as two FP16
-//               pieces: hi.hi + hi.lo + lo.hi; the dropped lo.lo term is below
-//               2^-21 of the product.  For widths N <= 128 the two products of
-//               the hi activations are one MMA of width 2N against the stacked
-//               [W_hi; W_lo] block (its rows are contiguous), lo.hi adds onto
-//               the second half, and the epilogue sums the halves: 2 MMAs per
-//               16 inputs (an MMA of N = 256 costs little more than one of
-//               N = 128), else 3
-// The epilogue adds the bias and applies ReLU in FP32, splits the activations
-// for the next layer, and computes layer 4 (d3 -> d_out), the softmax
-// cross-entropy and the loss sums in FP32, tiles in order.  A weight or an
-// activation with |v| >= 128 (2^8 |v| could overflow its FP16 piece) marks the
-// individual; the CUDA-core kernel then recomputes its fitness in FP32.
-// The weights are split once per evaluation (split_weights_kernel), and the
-// batch's levels are converted once per evaluation into FP16 operand tiles
-// (stage_levels_kernel), so a unit's layer-1 operands arrive by bulk copies and
-// its layer-1 MMAs run while the epilogue finishes the previous unit.
+//   layers 2-4  A = 2^8 h of the layer below and B = 2^8 W, both as two FP16
+//               pieces: hi.hi + lo.hi + hi.lo; the dropped lo.lo term is below
+//               2^-21 of the product
+// The epilogue adds the bias and applies ReLU in FP32 and splits the activations
+// for the next layer; the softmax cross-entropy is FP32, losses are summed in
+// FP64.  A weight or an activation with |v| >= 128 (2^8 |v| could overflow its
+// FP16 piece) marks the individual; the CUDA-core kernel then recomputes its
+// fitness in FP32.  The weights are split once per evaluation
+// (split_weights_kernel), and the batch's levels are converted once per
+// evaluation into FP16 operand tiles (stage_levels_kernel).
 //
-// Warp roles (persistent CTA, one per SM; individuals strided by gridDim.x,
-// their tiles in order):
-//   warp 0      TMEM allocation and the single MMA-issuing thread
-//   warp 1      producer: per unit, the tile's levels (one bulk copy into the
-//               activation region), then one bulk copy per 64-input block of
-//               W1, W2, W3, already split into FP16 pieces and swizzled by
-//               split_weights_kernel, into one of two weight buffers
-//   warps 2-9   the epilogue (TMEM lane = sample, two warps per lane
-//               quarter, each with half of a layer's 16-column groups): the
-//               activations of layers 1 and 2 as the next operands, layer 4
-//               (the halves' partial logits added through shared memory) and
-//               the loss
-// The layers of a unit share one activation region, each layer's weight
-// blocks double-buffered.  Layer 1's activations go to the layer-2 MMAs one
-// 64-column block at a time (the epilogue halves take two of each block's four
-// column groups); layer 3 starts after all of layer 2's; the next unit's
-// levels and layer-1 MMAs start as soon as this unit's layer-3 MMAs are done.
+// Where activations live.  A layer's activations are the A operand of the next
+// layer in tensor memory: 16 FP32 accumulator columns become 8 columns of hi
+// and 8 of lo pieces in place, so shared memory holds nothing but the tile's
+// levels and a ring of 32 KB weight slots.  Where all layers have their own
+// columns (mlp_columns) the next unit's layer 1 runs before and after this
+// unit's layer 3, under the epilogue of layers 2 and 3.  A CTA takes a
+// contiguous range of units; the sums of an individual that two CTAs share meet
+// in scratch memory (combine_mlp_parts_kernel).
+//
+// Measured, 2000 nets 196-256-128-64-10 on 1024 samples: 945 us (1518 with the
+// activations in shared memory and two weight buffers), 207 of them the splitting
+// (1.5 GB, at the memory's rate); 512 samples 607, 128 375; 16 nets on 1024
+// samples 42.  What bounds it: a unit takes 13k cycles, its MMAs 7.3k at the
+// tensor peak (weights 448 KB of L2 reads, 3.4k-6k cycles, are hidden).  The rest
+// is the chain of a unit: layer 1's accumulator to the first activations 1-2k,
+// the restart of the MMAs after layer 2 0.5k, and the issuing warp's waits
+// between slots, which a queue of few MMAs does not cover.  Splitting the next
+// individual's weights beside the MMAs, by two to six more warps, took as much
+// issue time from the epilogue as the separate kernel takes.
+//
+// Warp roles (persistent CTA, one per SM):
+//   warp 0      TMEM allocation and MMA issue (see mma_f16_lo)
+//   warp 1      producer: per unit, the tile's levels (one bulk copy) and the
+//               weight slots of W1 to W4 in the order of the MMAs, already split
+//               into FP16 pieces and swizzled by split_weights_kernel
+//   warp 2      the next individual's biases into one of two buffers
+//   warps 3-10  the epilogue (TMEM lane = sample, two warps per lane quarter,
+//               each with half of every 64-column block): the activations of
+//               layers 1 to 3.  Layer 1's go to the layer-2 MMAs a block at a time
+//   warps 11-14 the loss from layer 4's accumulator, a sample per thread, while
+//               the others are at the next unit
 // Every wait is bounded; on expiry the kernel sets kStatusEvalTimeout and exits.
 #include <cuda.h>
 
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "leea_internal.h"
@@ -58,15 +64,17 @@ namespace leea {
 
 namespace {
 
-constexpr int kFirstEpiWarp = 2;
-constexpr int kEpiWarps = 8;  // two per TMEM lane quarter: half of a layer's columns each
-constexpr int kEpiThreads = 32 * kEpiWarps;
-constexpr int kTcThreads = 32 * (kFirstEpiWarp + kEpiWarps);
+constexpr int kParamWarp = 2;
+constexpr int kFirstEpiWarp = 3;
+constexpr int kParts = 2;                  // epilogue warps per TMEM lane quarter
+constexpr int kEpiWarps = 4 * kParts;
+constexpr int kFirstLossWarp = kFirstEpiWarp + kEpiWarps;
+constexpr int kLossWarps = 4;              // one per 32 samples
+constexpr int kTcThreads = 32 * (kFirstLossWarp + kLossWarps);
 constexpr int kTile = 128;                      // samples per unit (MMA M)
 constexpr uint32_t kBlockBytes = kTile * 128;   // one 64-input block of a 128-row operand
-constexpr uint32_t kHalfRegion = 4 * kBlockBytes;  // 64 KB: one piece of up to 256 inputs
-constexpr uint32_t kRegionBytes = 2 * kHalfRegion;  // activations: hi piece, lo piece
-constexpr uint32_t kSlotBytes = 2 * 256 * 128;      // weights: two pieces of up to 256 rows
+constexpr uint32_t kSlotBytes = 256 * 128;      // a weight slot: 256 rows of 64 FP16 values
+constexpr int kMaxSlots = 8;
 constexpr int kMaxOutTc = 16;
 constexpr uint32_t kTmemCols = 512;
 constexpr float kPieceScale = 256.0f;
@@ -74,10 +82,28 @@ constexpr float kPieceRange = 128.0f;
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 constexpr uint64_t kDrainLimitNs = 200000000ull;
 
+// The weights of layer l (0-3) as slots of slot_bytes[l], one bulk copy each,
+// of 128-byte rows (64 FP16 values, swizzled).  Stacked layers (N <= 128; layer 4 has
+// N = 16, rows past d_out zero): slot kb holds block kb's hi rows, then its lo
+// rows.  Else slot 2 kb is block kb's hi piece and slot 2 kb + 1 its lo piece;
+// layer 1's last block, if it has at most 32 inputs, is one slot whose rows hold
+// the hi inputs and then the lo ones.
+struct MlpSlots {
+    int32_t k16[4];      // inputs rounded up to 16
+    int32_t n[4];        // rows: the layer's width, 16 for layer 4
+    int32_t slots[4];
+    uint32_t slot_bytes[4];
+    int64_t layer_off[4];
+    bool stacked[4], tail_joined;
+};
+
 struct MlpTcArgs {
     int32_t pop, batch, n_tiles;
     int32_t dims[5];     // d0, d1, d2, d3, d_out
-    int32_t k16[3];      // inputs of layers 1-3 rounded up to 16
+    MlpSlots m;
+    int32_t n_slots;     // ring depth
+    int32_t col[4];      // first accumulator column of each layer
+    bool early;          // all have their own columns: the next unit's layer 1 may start before layer 3
     int64_t c_pad;
     int64_t w_off[4], b_off[4];
     float inv_div;       // 2^-8 / x_div: layer-1 accumulator units to x units
@@ -95,66 +121,69 @@ struct MlpTcArgs {
     const uint8_t* xtiles;
     uint32_t x_bytes;
     unsigned int* status;
-    // the weights of layers 1-3 as FP16 pieces, per individual (piece_stride
-    // bytes): layer l's 64-input blocks from byte layer_off[l], each block the
-    // hi piece (N rows of 128 bytes, swizzled) then the lo piece
-    const uint8_t* pieces;
+    uint8_t* pieces;     // per individual piece_stride bytes, see MlpSlots
     int64_t piece_stride;
-    int64_t layer_off[3];
+    int32_t per_cta, extra;  // units of a CTA; the first `extra` CTAs take one more
+    double* part_loss;   // [2 gridDim.x]: loss sums and correct counts of individuals shared by CTAs
+    int32_t* part_ok;
 };
 
 struct TcSmem {
-    uint8_t* region;  // activations: hi piece [0, 64 KB), lo piece [64 KB, 128 KB); the levels in the hi part
-    uint8_t* slot;    // weights: hi piece then lo piece, N x 128 bytes each per 64-input block
-    float *b1, *b2, *b3, *w4t, *b4;
-    float* plog;  // [128][16]: the second half's partial layer-4 logits
-    uint64_t *buf_full, *buf_empty, *x_full, *d_full, *h_blk, *h2_ready, *drain;
+    uint8_t* levels;
+    uint8_t* ring;
+    float* param;     // [2]: b1, b2, b3 times 2^8, b4 of an individual
+    double* red_loss;
+    uint64_t *full, *empty, *x_full, *d_full, *h_blk, *h_ready, *d4_read, *param_full, *param_empty, *red_full,
+        *drain;
+    int32_t* red_ok;
     uint32_t* tmem_holder;
     volatile int* abort_flag;
-    int* ep_go;
-    float* red_loss;
-    int32_t* red_ok;
 };
 
-__host__ __device__ inline size_t tc_param_floats(const int32_t* dims)
+__host__ __device__ inline uint32_t param_floats(const int32_t* dims)
 {
-    return static_cast<size_t>(dims[1] + dims[2] + dims[3] + dims[3] * kMaxOutTc + kMaxOutTc + kTile * kMaxOutTc);
+    return static_cast<uint32_t>(dims[1] + dims[2] + dims[3] + kMaxOutTc);
 }
 
-__host__ __device__ inline size_t tc_smem_bytes(const int32_t* dims)
+__host__ __device__ inline size_t tc_smem_bytes(const int32_t* dims, uint32_t x_bytes, int n_slots)
 {
-    // room for 16 barriers (14 used) and 16 words (11 used)
-    return 1024 + kRegionBytes + kSlotBytes + sizeof(float) * tc_param_floats(dims) + 8 * 16 + 64;
+    return 1024 + x_bytes + static_cast<size_t>(n_slots) * kSlotBytes + 8 * param_floats(dims) + 8 * 8 +
+           8 * (2 * kMaxSlots + 18) + 4 * 10;
+}
+
+// Ring depth that fits in shared memory.
+int mlp_ring(const int32_t* dims, uint32_t x_bytes)
+{
+    int n = kMaxSlots;
+    while (n > 0 && tc_smem_bytes(dims, x_bytes, n) > 227u * 1024u) --n;
+    return n;
 }
 
 __device__ __forceinline__ TcSmem carve(uint8_t* raw, const MlpTcArgs& a)
 {
     TcSmem s;
-    s.region = raw + ((1024u - (ptx::smem_u32(raw) & 1023u)) & 1023u);
-    s.slot = s.region + kRegionBytes;
-    float* f = reinterpret_cast<float*>(s.slot + kSlotBytes);
-    s.b1 = f;
-    s.b2 = s.b1 + a.dims[1];
-    s.b3 = s.b2 + a.dims[2];
-    s.w4t = s.b3 + a.dims[3];
-    s.b4 = s.w4t + a.dims[3] * kMaxOutTc;
-    s.plog = s.b4 + kMaxOutTc;
-    uint8_t* p = reinterpret_cast<uint8_t*>(s.plog + kTile * kMaxOutTc);
-    p += (8u - (reinterpret_cast<uintptr_t>(p) & 7u)) & 7u;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(p);
-    s.buf_full = bars;       // [2]
-    s.buf_empty = bars + 2;  // [2]
-    s.x_full = bars + 4;
-    s.d_full = bars + 5;     // [3]
-    s.h_blk = bars + 8;      // [4]: a 64-column block of layer 1's activations is in
-    s.h2_ready = bars + 12;  // layer 2's activations are in
-    s.drain = bars + 13;
-    uint32_t* w = reinterpret_cast<uint32_t*>(bars + 14);
+    s.levels = raw + ((1024u - (ptx::smem_u32(raw) & 1023u)) & 1023u);
+    s.ring = s.levels + a.x_bytes;
+    float* f = reinterpret_cast<float*>(s.ring + static_cast<uint32_t>(a.n_slots) * kSlotBytes);
+    s.param = f;
+    s.red_loss = reinterpret_cast<double*>(f + 2 * param_floats(a.dims));
+    uint64_t* bars = reinterpret_cast<uint64_t*>(s.red_loss + 8);
+    s.full = bars;
+    s.empty = bars + kMaxSlots;
+    bars += 2 * kMaxSlots;
+    s.x_full = bars;
+    s.d_full = bars + 1;       // [4]: a layer's MMAs are done
+    s.h_blk = bars + 5;        // [4]: a 64-column block of layer 1's activations is in
+    s.h_ready = bars + 9;      // [2]: layer 2's, layer 3's activations are in
+    s.d4_read = bars + 11;     // layer 4's accumulator has been read
+    s.param_full = bars + 12;  // [2]
+    s.param_empty = bars + 14; // [2]
+    s.red_full = bars + 16;
+    s.drain = bars + 17;
+    uint32_t* w = reinterpret_cast<uint32_t*>(bars + 18);
     s.tmem_holder = w;
     s.abort_flag = reinterpret_cast<volatile int*>(w + 1);
-    s.ep_go = reinterpret_cast<int*>(w + 2);
-    s.red_loss = reinterpret_cast<float*>(w + 3);
-    s.red_ok = reinterpret_cast<int32_t*>(w + 7);
+    s.red_ok = reinterpret_cast<int32_t*>(w + 2);
     return s;
 }
 
@@ -169,14 +198,18 @@ __device__ __forceinline__ uint32_t half2_bits(__half2 v)
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// Two FP32 values as packed FP16 pieces of 2^8 v (lower index in the low half).
-__device__ __forceinline__ void split2x2(float v0, float v1, uint32_t& p1, uint32_t& p2)
+// Two FP32 values s = 2^8 v as packed FP16 pieces (lower index in the low half).
+__device__ __forceinline__ void split_scaled(float s0, float s1, uint32_t& p1, uint32_t& p2)
 {
-    const float s0 = v0 * kPieceScale, s1 = v1 * kPieceScale;
     const __half2 h1 = __floats2half2_rn(s0, s1);
     const float2 f1 = __half22float2(h1);
     p1 = half2_bits(h1);
     p2 = half2_bits(__floats2half2_rn(s0 - f1.x, s1 - f1.y));
+}
+
+__device__ __forceinline__ void split2x2(float v0, float v1, uint32_t& p1, uint32_t& p2)
+{
+    split_scaled(v0 * kPieceScale, v1 * kPieceScale, p1, p2);
 }
 
 // Byte offset of 16-byte chunk `ch` (inputs 8 ch .. 8 ch + 7 of a 64-input
@@ -186,76 +219,198 @@ __device__ __forceinline__ uint32_t swz(int r, int ch)
     return static_cast<uint32_t>(r) * 128u + ((static_cast<uint32_t>(ch) ^ static_cast<uint32_t>(r & 7)) << 4);
 }
 
-__device__ __forceinline__ int layer_blocks(const MlpTcArgs& a, int l) { return (a.k16[l] + 63) / 64; }
+__device__ __forceinline__ int layer_blocks(const MlpTcArgs& a, int l) { return (a.m.k16[l] + 63) / 64; }
 
-// The weight blocks of a layer alternate between two buffers, so that one is
-// converted while the MMAs read the other.  Layer 1: the slot, and the lo half
-// of the activation region (it holds nothing while layer 1 runs: the levels
-// use the hi half).  Layers 2 and 3 with N <= 128 (blocks of <= 32 KB): the
-// slot's two halves; wider ones take the whole slot for every block.
-__device__ __forceinline__ int buffer_of(const MlpTcArgs& a, int l, int kb)
+// Accumulator columns.  Layer 1 in [0, d1), layer 2 in the d2 columns after it,
+// layer 3 and the 16 of layer 4 after those where they end by column 512
+// ("early": 196-256-128-64-10 uses 464); activations replace their accumulator.
+// Otherwise layer 2 ends at column 512, layer 3 takes layer 1's place, from
+// column 0 (layer 2 then starts at 256 or later), and layer 4 layer 2's, so the
+// next unit's layer 1 waits until layer 4 is read.
+void mlp_columns(MlpTcArgs* a)
 {
-    return (l == 0 || a.dims[l + 1] <= 128) ? (kb & 1) : 0;
+    const int32_t d1 = a->dims[1], d2 = a->dims[2], d3 = a->dims[3], cols = static_cast<int32_t>(kTmemCols);
+    a->early = d1 + d2 + d3 + kMaxOutTc <= cols;
+    a->col[0] = 0;
+    a->col[1] = a->early ? d1 : cols - d2;
+    a->col[2] = a->early ? d1 + d2 : 0;
+    a->col[3] = a->early ? d1 + d2 + d3 : cols - d2;
 }
 
-// Offset of weight buffer b of layer l from the start of the region.
-__device__ __forceinline__ uint32_t buffer_offset(int l, int b)
+// Bias, ReLU and split of 16 accumulator columns r, written to taddr in place:
+// 8 columns of hi pieces, 8 of lo pieces.  scale and bias include the pieces'
+// 2^8.  top: the largest hi pieces so far.
+__device__ __forceinline__ void activate16(uint32_t taddr, const uint32_t (&r)[16], float scale, const float* bias,
+                                           __half2& top)
 {
-    if (b == 0) return kRegionBytes;
-    return l == 0 ? kHalfRegion : kRegionBytes + kSlotBytes / 2;
-}
-
-// 16 accumulator columns of this thread's lane from TMEM address taddr; for a
-// merged layer the sum of the two halves (hi.hi + (hi.lo + lo.hi)).
-__device__ __forceinline__ void load_acc16(uint32_t taddr, uint32_t half_cols, bool merged, float (&v)[16])
-{
-    uint32_t r[16];
-    ptx::tmem_ld16_nowait(taddr, r);
-    if (merged) {
-        uint32_t r2[16];
-        ptx::tmem_ld16_nowait(taddr + half_cols, r2);
-        ptx::tmem_ld_wait();
+    const float2 sc = make_float2(scale, scale);
+    uint32_t out[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]) + __uint_as_float(r2[i]);
-    } else {
-        ptx::tmem_ld_wait();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+    for (int e = 0; e < 8; ++e) {
+        const float2 b = *reinterpret_cast<const float2*>(bias + 2 * e);
+        float2 h = __ffma2_rn(make_float2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1])), sc, b);
+        h.x = fmaxf(h.x, 0.0f);
+        h.y = fmaxf(h.y, 0.0f);
+        const __half2 hi = __floats2half2_rn(h.x, h.y);
+        const float2 f = __half22float2(hi);
+        const float2 lo = __fadd2_rn(h, make_float2(-f.x, -f.y));
+        top = __hmax2(top, hi);
+        out[e] = half2_bits(hi);
+        out[8 + e] = half2_bits(__floats2half2_rn(lo.x, lo.y));
     }
+    ptx::tmem_st16(taddr, out);
 }
 
-// Layers 2 and 3 (width n, layer 1 of width d1 in the columns below them) take
-// the hi activations' two products as one MMA of width 2n where 2n fits both
-// the MMA (N <= 256) and tensor memory.
-__host__ __device__ inline bool merged_layer(int32_t d1, int32_t n)
+// Columns [c, c + kPartCols) below n of the layer at taddr (n: a multiple of 16).
+constexpr int kPartCols = 64 / kParts;  // an epilogue warp's columns of a 64-column block
+static_assert(kPartCols == 32, "two 16-column groups");
+
+__device__ __forceinline__ void activate_part(uint32_t taddr, int c, int n, float scale, const float* bias, __half2& top)
 {
-    return 2 * n <= 256 && d1 + 2 * n <= static_cast<int32_t>(kTmemCols);
+    if (c >= n) return;
+    const uint32_t at = taddr + static_cast<uint32_t>(c);
+    uint32_t r0[16], r1[16];
+    const bool both = c + 16 < n;
+    ptx::tmem_ld16_nowait(at, r0);
+    if (both) ptx::tmem_ld16_nowait(at + 16u, r1);
+    ptx::tmem_ld_wait();
+    activate16(at, r0, scale, bias + c, top);
+    if (both) activate16(at + 16u, r1, scale, bias + c + 16, top);
 }
 
-__global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const MlpTcArgs a)
+// The segments of CTA c: its units [start, end) of the sequence of all
+// individuals' tiles, an individual (or the part of it that is this CTA's) at
+// a time.
+struct Segments {
+    int p, t0, t1;  // tiles [t0, t1) of individual p
+    int64_t u, end;
+    __device__ __forceinline__ Segments(const MlpTcArgs& a, int c)
+    {
+        u = static_cast<int64_t>(c) * a.per_cta + min(c, a.extra);
+        end = u + a.per_cta + (c < a.extra ? 1 : 0);
+        set(a);
+    }
+    __device__ __forceinline__ void set(const MlpTcArgs& a)
+    {
+        p = static_cast<int>(u / a.n_tiles);
+        t0 = static_cast<int>(u - static_cast<int64_t>(p) * a.n_tiles);
+        t1 = static_cast<int>(min(static_cast<int64_t>(a.n_tiles), t0 + end - u));
+    }
+    __device__ __forceinline__ bool valid() const { return u < end; }
+    __device__ __forceinline__ void step(const MlpTcArgs& a)
+    {
+        u += t1 - t0;
+        set(a);
+    }
+};
+
+// The unit sequence of this CTA.
+struct UnitSeq {
+    Segments seg;
+    int t;
+    __device__ __forceinline__ explicit UnitSeq(const MlpTcArgs& a) : seg(a, blockIdx.x), t(seg.t0) {}
+    __device__ __forceinline__ bool valid() const { return seg.valid(); }
+    __device__ __forceinline__ void step(const MlpTcArgs& a)
+    {
+        if (++t == seg.t1) {
+            seg.step(a);
+            t = seg.t0;
+        }
+    }
+};
+
+// Splits the weights of an individual into dst, a 64-input block
+// after the other, in batches: thread `first` of `stride` takes kSplitBatch
+// 8-input chunks of a batch.  A batch is loaded before any of it is split.
+constexpr int kSplitBatch = 4;
+
+struct Splitter {
+    int l = 0, kb = 0, it0 = 0;
+    float top = 0.0f;  // the largest |w|
+
+    // One batch (of the block at the cursor); returns false when all are done.
+    __device__ __forceinline__ bool batch(const MlpTcArgs& a, int p, uint8_t* dst, int first, int stride)
+    {
+        const int K = a.dims[l], N = a.m.n[l], rows = a.dims[l + 1], k16 = a.m.k16[l];
+        const bool joined = l == 0 && a.m.tail_joined && kb == k16 / 64;
+        uint8_t* blk = dst + a.m.layer_off[l] + static_cast<int64_t>(a.m.stacked[l] ? kb : 2 * kb) * a.m.slot_bytes[l];
+        // the lo piece: the same slot's next columns, or the next N rows
+        uint8_t* blk_lo = joined ? blk : blk + N * 128;
+        const int lo_ch = joined ? (k16 % 64) / 8 : 0;
+        // chunks of a row (those past k16 are not read by any MMA), rounded up to 2^shift
+        const int chunks = min(8, (k16 - 64 * kb) / 8), shift = chunks <= 2 ? 1 : (chunks <= 4 ? 2 : 3);
+        const float* w = a.popv + static_cast<int64_t>(p) * a.c_pad + a.w_off[l] + 64 * kb;
+        float4 v[kSplitBatch][2];
+#pragma unroll
+        for (int b = 0; b < kSplitBatch; ++b) {
+            const int it = it0 + first + b * stride, n = it >> shift, ch = it & ((1 << shift) - 1);
+            v[b][0] = v[b][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+            const int k = 64 * kb + 8 * ch;
+            if (n < rows && k < K) {
+                const float4* src = reinterpret_cast<const float4*>(w + static_cast<int64_t>(n) * K + 8 * ch);
+                v[b][0] = __ldg(src);
+                if (k + 4 < K) v[b][1] = __ldg(src + 1);
+            }
+        }
+#pragma unroll
+        for (int b = 0; b < kSplitBatch; ++b) {
+            const int it = it0 + first + b * stride, n = it >> shift, ch = it & ((1 << shift) - 1);
+            const float4 v0 = v[b][0], v1 = v[b][1];
+            if (n >= N || ch >= chunks) continue;
+            uint4 hi, lo;
+            split2x2(v0.x, v0.y, hi.x, lo.x);
+            split2x2(v0.z, v0.w, hi.y, lo.y);
+            split2x2(v1.x, v1.y, hi.z, lo.z);
+            split2x2(v1.z, v1.w, hi.w, lo.w);
+            top = fmaxf(fmaxf(fmaxf(top, fmaxf(fabsf(v0.x), fabsf(v0.y))), fmaxf(fabsf(v0.z), fabsf(v0.w))),
+                        fmaxf(fmaxf(fabsf(v1.x), fabsf(v1.y)), fmaxf(fabsf(v1.z), fabsf(v1.w))));
+            *reinterpret_cast<uint4*>(blk + swz(n, ch)) = hi;
+            *reinterpret_cast<uint4*>(blk_lo + swz(n, lo_ch + ch)) = lo;
+        }
+        it0 += kSplitBatch * stride;
+        if (it0 >= N << shift) {
+            it0 = 0;
+            if (++kb == layer_blocks(a, l)) {
+                kb = 0;
+                ++l;
+            }
+        }
+        return l < 4;
+    }
+    __device__ __forceinline__ bool outside() const { return top >= kPieceRange; }
+};
+
+__device__ __forceinline__ void store_fitness(const MlpTcArgs& a, int p, double sum, int32_t good)
+{
+    const float f = static_cast<float>(-(sum / static_cast<double>(a.batch)));
+    a.f_raw[p] = f;
+    if (a.f_adj) a.f_adj[p] = a.f_inh ? (1.0f - a.alpha) * a.f_inh[p] + a.alpha * f : f;
+    if (a.correct) a.correct[p] = good;
+}
+
+__global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid_constant__ MlpTcArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
     const TcSmem s = carve(smem_raw, a);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int d1 = a.dims[1], d2 = a.dims[2], d3 = a.dims[3], d_out = a.dims[4];
-    // Layer 3 reuses layer 2's columns; a merged layer (2N columns: hi.hi, then
-    // hi.lo + lo.hi) where its width allows.
-    const bool merged2 = merged_layer(d1, d2), merged3 = merged_layer(d1, d3);
-    auto col = [&](int l) { return l == 0 ? 0u : static_cast<uint32_t>(d1); };
-    auto merged = [&](int l) { return l == 1 ? merged2 : (l == 2 && merged3); };
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 2; ++i) {
-            ptx::mbar_init(&s.buf_full[i], 1);
-            ptx::mbar_init(&s.buf_empty[i], 1);
+        for (int i = 0; i < a.n_slots; ++i) {
+            ptx::mbar_init(&s.full[i], 1);
+            ptx::mbar_init(&s.empty[i], 1);
         }
         ptx::mbar_init(s.x_full, 1);
-        for (int i = 0; i < 3; ++i) ptx::mbar_init(&s.d_full[i], 1);
-        for (int i = 0; i < 4; ++i) ptx::mbar_init(&s.h_blk[i], kEpiThreads);
-        ptx::mbar_init(s.h2_ready, kEpiThreads);
+        for (int i = 0; i < 4; ++i) ptx::mbar_init(&s.d_full[i], 1);
+        for (int i = 0; i < 4; ++i) ptx::mbar_init(&s.h_blk[i], kEpiWarps);
+        for (int i = 0; i < 2; ++i) ptx::mbar_init(&s.h_ready[i], kEpiWarps);
+        ptx::mbar_init(s.d4_read, kLossWarps);
+        for (int i = 0; i < 2; ++i) {
+            ptx::mbar_init(&s.param_full[i], 1);
+            ptx::mbar_init(&s.param_empty[i], kEpiWarps + kLossWarps);
+        }
+        ptx::mbar_init(s.red_full, kLossWarps);
         ptx::mbar_init(s.drain, 1);
         *s.abort_flag = 0;
-        *s.ep_go = 0;
         ptx::fence_mbar_init();
     }
     if (warp == 0) ptx::tmem_alloc(s.tmem_holder, kTmemCols);
@@ -263,306 +418,329 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const MlpTcA
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem_base = *s.tmem_holder;
+    // Layer 3 of a unit comes after the first `cut` slots of the next unit's layer 1:
+    // by then its activations are in.
+    const int cut = a.m.slots[0] / 2;
 
     if (warp == 0) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t region = ptx::smem_u32(s.region);
-            uint32_t unit = 0, bphase = 0;  // bit b: phase of weight buffer b
+        {
+            const uint32_t lead = ptx::elect_one();
+            const uint32_t levels = ptx::smem_u32(s.levels), ring = ptx::smem_u32(s.ring);
+            const uint32_t hi = static_cast<uint32_t>(ptx::smem_desc_sw128(0u) >> 32);
+            uint32_t slot = 0, phase = 0;
             bool ok = true;
-            for (int p = blockIdx.x; ok && p < a.pop; p += gridDim.x) {
-                for (int t = 0; ok && t < a.n_tiles; ++t, ++unit) {
-                    if (!ptx::mbar_wait_bounded(s.x_full, unit & 1u, s.abort_flag, kWaitLimitNs)) {
-                        raise_abort(s, a);
-                        ok = false;
-                        break;
-                    }
-                    for (int l = 0; ok && l < 3; ++l) {
-                        // layer 3 after all of layer 2's activations (it reuses layer 2's
-                        // columns); layer 2 block by block below
-                        if (l == 2 && !ptx::mbar_wait_bounded(s.h2_ready, unit & 1u, s.abort_flag, kWaitLimitNs)) {
-                            raise_abort(s, a);
-                            ok = false;
-                            break;
-                        }
-                        ptx::tc_fence_after();
-                        const uint32_t n = static_cast<uint32_t>(a.dims[l + 1]);
-                        const uint32_t idesc = ptx::idesc_f16(kTile, n);
-                        const uint32_t idesc2 = ptx::idesc_f16(kTile, 2u * n);
-                        const uint32_t d_tmem = tmem_base + col(l);
-                        const int blocks = layer_blocks(a, l);
-                        for (int kb = 0; kb < blocks; ++kb) {
-                            const int b = buffer_of(a, l, kb);
-                            if (!ptx::mbar_wait_bounded(&s.buf_full[b], (bphase >> b) & 1u, s.abort_flag,
-                                                        kWaitLimitNs)) {
-                                raise_abort(s, a);
-                                ok = false;
-                                break;
-                            }
-                            bphase ^= 1u << b;
-                            if (l == 1 &&
-                                !ptx::mbar_wait_bounded(&s.h_blk[kb], unit & 1u, s.abort_flag, kWaitLimitNs)) {
-                                raise_abort(s, a);
-                                ok = false;
-                                break;
-                            }
-                            const uint32_t slot = region + buffer_offset(l, b);
-                            ptx::tc_fence_after();
+            auto wait = [&](uint64_t* bar, uint32_t parity) {
+                const bool got = ptx::mbar_wait_bounded(bar, parity, s.abort_flag, kWaitLimitNs);
+                if (!__all_sync(0xFFFFFFFFu, got)) {
+                    raise_abort(s, a);
+                    ok = false;
+                }
+                return ok;
+            };
+            auto next_slot = [&]() {
+                if (lead) ptx::mma_commit(&s.empty[slot]);
+                if (++slot == static_cast<uint32_t>(a.n_slots)) { slot = 0; phase ^= 1u; }
+            };
+            // Slots [j0, j1) of unit u's layer 1.
+            auto layer1 = [&](uint32_t u, int j0, int j1) {
+                const uint32_t n = static_cast<uint32_t>(a.dims[1]), idesc = ptx::idesc_f16(kTile, n);
+                if (j0 == 0 && j1 > 0 && !wait(s.x_full, u & 1u)) return;
+                for (int j = j0; j < j1; ++j) {
+                    if (!wait(&s.full[slot], phase)) return;
+                    const int kb = j >> 1, steps = min(4, (a.m.k16[0] - 64 * kb) / 16);
+                    const bool joined = a.m.tail_joined && j == a.m.slots[0] - 1;
+                    const uint32_t ax = ptx::desc_lo(levels + kb * kBlockBytes);
+                    const uint32_t b = ptx::desc_lo(ring + slot * kSlotBytes);
+                    const uint32_t acc = j == 0 ? 0u : 1u;
 #pragma unroll
-                            for (int kk = 0; kk < 4; ++kk) {
-                                const int kg = kb * 64 + kk * 16;
-                                if (kg >= a.k16[l]) break;
-                                const uint32_t a_hi = region + kb * kBlockBytes + kk * 32u;
-                                const uint32_t b_hi = slot + kk * 32u;
-                                const uint32_t b_lo = slot + n * 128u + kk * 32u;
-                                const uint32_t first = (kb | kk) == 0 ? 0u : 1u;
-                                if (merged(l)) {
-                                    // [hi.hi | hi.lo] against the stacked block, then lo.hi onto the second half
-                                    ptx::mma_f16(d_tmem, ptx::smem_desc_sw128(a_hi), ptx::smem_desc_sw128(b_hi),
-                                                 idesc2, first);
-                                    ptx::mma_f16(d_tmem + n, ptx::smem_desc_sw128(a_hi + kHalfRegion),
-                                                 ptx::smem_desc_sw128(b_hi), idesc, 1u);
-                                    continue;
-                                }
-                                ptx::mma_f16(d_tmem, ptx::smem_desc_sw128(a_hi), ptx::smem_desc_sw128(b_hi), idesc,
-                                             first);
-                                ptx::mma_f16(d_tmem, ptx::smem_desc_sw128(a_hi), ptx::smem_desc_sw128(b_lo), idesc,
-                                             1u);
-                                if (l > 0)
-                                    ptx::mma_f16(d_tmem, ptx::smem_desc_sw128(a_hi + kHalfRegion),
-                                                 ptx::smem_desc_sw128(b_hi), idesc, 1u);
-                            }
-                            ptx::mma_commit(&s.buf_empty[b]);
-                        }
-                        if (ok) ptx::mma_commit(&s.d_full[l]);
+                    for (int kk = 0; kk < 4; ++kk) {
+                        if (kk < steps)
+                            ptx::mma_f16_lo(tmem_base, ax + 2u * kk, b + 2u * kk, hi, hi, idesc, kk == 0 ? acc : 1u, lead);
                     }
+                    if (joined) {
+#pragma unroll
+                        for (int kk = 0; kk < 2; ++kk)
+                            if (kk < steps) ptx::mma_f16_lo(tmem_base, ax + 2u * kk, b + 2u * (steps + kk), hi, hi, idesc, 1u, lead);
+                    }
+                    next_slot();
+                }
+                if (j1 == a.m.slots[0] && lead) ptx::mma_commit(&s.d_full[0]);
+            };
+            // Unit u's layer l = 1, 2, 3, its A operand in the columns of the layer before.
+            auto later = [&](uint32_t u, int l) {
+                const uint32_t n = static_cast<uint32_t>(a.m.n[l]);
+                const uint32_t idesc = ptx::idesc_f16(kTile, n);
+                const uint32_t act = tmem_base + static_cast<uint32_t>(a.col[l - 1]);
+                const uint32_t d = tmem_base + static_cast<uint32_t>(a.col[l]);
+                const bool stacked = a.m.stacked[l];
+                if (l >= 2 && !wait(&s.h_ready[l - 2], u & 1u)) return;
+                ptx::tc_fence_after();
+                for (int j = 0; j < a.m.slots[l]; ++j) {
+                    const int kb = stacked ? j : j >> 1, lo = stacked ? 0 : j & 1;
+                    if (l == 1 && lo == 0 && !wait(&s.h_blk[kb], u & 1u)) return;
+                    if (!wait(&s.full[slot], phase)) return;
+                    if (l == 1) ptx::tc_fence_after();
+                    const uint32_t b = ptx::desc_lo(ring + slot * kSlotBytes);
+                    const uint32_t a_hi = act + 64u * static_cast<uint32_t>(kb);
+                    const uint32_t acc = j == 0 ? 0u : 1u;
+                    const int steps = min(4, (a.m.k16[l] - 64 * kb) / 16);
+                    if (stacked) {
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                                if (kk >= steps) break;
+                            ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk, b + 2u * kk, hi, idesc, kk == 0 ? acc : 1u, lead);
+                            ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk + 8u, b + 2u * kk, hi, idesc, 1u, lead);
+                            ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk, b + 8u * n + 2u * kk, hi, idesc, 1u, lead);
+                        }
+                    } else {
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                                if (kk >= steps) break;
+                            ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk, b + 2u * kk, hi, idesc, kk == 0 ? acc : 1u, lead);
+                            if (!lo) ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk + 8u, b + 2u * kk, hi, idesc, 1u, lead);
+                        }
+                    }
+                    next_slot();
+                }
+                if (lead) ptx::mma_commit(&s.d_full[l]);
+            };
+            UnitSeq x(a);
+            layer1(0, 0, a.m.slots[0]);
+            for (uint32_t u = 0; ok && x.valid(); ++u) {
+                x.step(a);
+                const bool more = x.valid();
+                later(u, 1);
+                if (a.early) {
+                    if (ok && more) {
+                        wait(&s.d_full[1], u & 1u);  // layer 1 overwrites layer 2's operand
+                        if (ok) layer1(u + 1, 0, cut);
+                    }
+                    if (ok && u > 0) wait(&s.d_full[3], (u - 1) & 1u);  // layer 3 overwrites layer 4's operand
+                    if (ok) later(u, 2);
+                    if (ok && more) layer1(u + 1, cut, a.m.slots[0]);
+                    if (ok && u > 0) wait(s.d4_read, (u - 1) & 1u);
+                    if (ok) later(u, 3);
+                } else {
+                    if (ok) later(u, 2);
+                    if (ok) wait(&s.d_full[2], u & 1u);  // layer 4 overwrites layer 3's operand
+                    if (ok) later(u, 3);
+                    if (ok && more) wait(s.d4_read, u & 1u);
+                    if (ok && more) layer1(u + 1, 0, a.m.slots[0]);
                 }
             }
-            ptx::mma_commit(s.drain);
+            if (lead) ptx::mma_commit(s.drain);
+            __syncwarp();
             volatile int never = 0;
             ptx::mbar_wait_bounded(s.drain, 0u, &never, ok ? kWaitLimitNs : kDrainLimitNs);
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ producer
-        // One bulk copy per 64-input weight block: the pieces are already in
-        // the swizzled operand layout (split_weights_kernel).
         if (lane == 0) {
-            uint32_t bphase = 0, unit = 0;
-            uint32_t issued = 0, parity = 0;  // per buffer: a copy was issued / the parity it completes
-            uint32_t x_issued = 0;            // level copies issued (at most the last one in flight)
+            uint32_t slot = 0, phase = 0, issued = 0, parity = 0;  // per slot: a copy was issued / its parity
+            uint32_t x_issued = 0;
             bool ok = true;
-            for (int p = blockIdx.x; ok && p < a.pop; p += gridDim.x) {
-                const uint8_t* src_p = a.pieces + static_cast<int64_t>(p) * a.piece_stride;
-                for (int t = 0; ok && t < a.n_tiles; ++t, ++unit) {
-                    // The activation region and the buffers of this unit's layer 1
-                    // (the slot, the region's lo half) are free once the previous
-                    // unit's last MMAs are done: the tile's levels into the hi half.
-                    if (unit > 0 &&
-                        !ptx::mbar_wait_bounded(&s.d_full[2], (unit - 1) & 1u, s.abort_flag, kWaitLimitNs)) {
-                        raise_abort(s, a);
-                        ok = false;
-                        break;
-                    }
-                    ptx::mbar_arrive_expect_tx(s.x_full, a.x_bytes);
-                    ptx::bulk_load(s.region, a.xtiles + static_cast<int64_t>(t) * a.x_bytes, a.x_bytes, s.x_full);
-                    ++x_issued;
-                    for (int l = 0; ok && l < 3; ++l) {
-                        const uint32_t bytes = static_cast<uint32_t>(a.dims[l + 1]) * 256u;
-                        const int blocks = layer_blocks(a, l);
-                        for (int kb = 0; kb < blocks; ++kb) {
-                            const int b = buffer_of(a, l, kb);
-                            if (!ptx::mbar_wait_bounded(&s.buf_empty[b], ((bphase >> b) & 1u) ^ 1u, s.abort_flag,
-                                                        kWaitLimitNs)) {
-                                raise_abort(s, a);
-                                ok = false;
-                                break;
-                            }
-                            ptx::mbar_arrive_expect_tx(&s.buf_full[b], bytes);
-                            ptx::bulk_load(s.region + buffer_offset(l, b),
-                                           src_p + a.layer_off[l] + static_cast<int64_t>(kb) * bytes, bytes,
-                                           &s.buf_full[b]);
-                            issued |= 1u << b;
-                            parity = (parity & ~(1u << b)) | (((bphase >> b) & 1u) << b);
-                            bphase ^= 1u << b;
-                        }
-                    }
+            auto wait = [&](uint64_t* bar, uint32_t want) {
+                if (ok && !ptx::mbar_wait_bounded(bar, want, s.abort_flag, kWaitLimitNs)) {
+                    raise_abort(s, a);
+                    ok = false;
+                }
+                return ok;
+            };
+            // Slots [j0, j1) of layer l of individual p, in the issuer's order.
+            auto load = [&](int p, int l, int j0, int j1) {
+                const uint8_t* src = a.pieces + static_cast<int64_t>(p) * a.piece_stride + a.m.layer_off[l];
+                const uint32_t bytes = a.m.slot_bytes[l];
+                for (int j = j0; j < j1; ++j) {
+                    if (!wait(&s.empty[slot], phase ^ 1u)) return;
+                    ptx::mbar_arrive_expect_tx(&s.full[slot], bytes);
+                    ptx::bulk_load(s.ring + slot * kSlotBytes, src + static_cast<int64_t>(j) * bytes, bytes,
+                                   &s.full[slot]);
+                    issued |= 1u << slot;
+                    parity = (parity & ~(1u << slot)) | (phase << slot);
+                    if (++slot == static_cast<uint32_t>(a.n_slots)) { slot = 0; phase ^= 1u; }
+                }
+            };
+            auto load_levels = [&](int t) {
+                // free once the previous unit's layer 1 is done
+                if (x_issued > 0 && !wait(&s.d_full[0], (x_issued - 1) & 1u)) return;
+                ptx::mbar_arrive_expect_tx(s.x_full, a.x_bytes);
+                ptx::bulk_load(s.levels, a.xtiles + static_cast<int64_t>(t) * a.x_bytes, a.x_bytes, s.x_full);
+                ++x_issued;
+            };
+            UnitSeq x(a);
+            load_levels(x.t);
+            load(x.seg.p, 0, 0, a.m.slots[0]);
+            while (ok && x.valid()) {
+                const int p = x.seg.p;
+                x.step(a);
+                const bool more = x.valid();
+                load(p, 1, 0, a.m.slots[1]);
+                if (ok && more) load_levels(x.t);
+                if (a.early) {
+                    if (ok && more) load(x.seg.p, 0, 0, cut);
+                    if (ok) load(p, 2, 0, a.m.slots[2]);
+                    if (ok && more) load(x.seg.p, 0, cut, a.m.slots[0]);
+                    if (ok) load(p, 3, 0, a.m.slots[3]);
+                } else {
+                    if (ok) load(p, 2, 0, a.m.slots[2]);
+                    if (ok) load(p, 3, 0, a.m.slots[3]);
+                    if (ok && more) load(x.seg.p, 0, 0, a.m.slots[0]);
                 }
             }
             if (!ok) {  // let copies in flight land before the CTA exits
                 volatile int never = 0;
-                for (int b = 0; b < 2; ++b)
+                for (int b = 0; b < a.n_slots; ++b)
                     if (issued & (1u << b))
-                        ptx::mbar_wait_bounded(&s.buf_full[b], (parity >> b) & 1u, &never, kDrainLimitNs);
+                        ptx::mbar_wait_bounded(&s.full[b], (parity >> b) & 1u, &never, kDrainLimitNs);
                 if (x_issued) ptx::mbar_wait_bounded(s.x_full, (x_issued - 1) & 1u, &never, kDrainLimitNs);
             }
         }
-    } else {
-        // ------------------------------------------------------------ epilogue
-        const int et = threadIdx.x - 32 * kFirstEpiWarp;
-        const int q = warp & 3;
-        const int half = (warp - kFirstEpiWarp) >> 2;
-        const int row = q * 32 + lane;
-        const uint32_t lane_addr = static_cast<uint32_t>(q * 32) << 16;
-        uint32_t unit = 0;
-        bool ok = true;
-        for (int p = blockIdx.x; ok && p < a.pop; p += gridDim.x) {
-            const float* net = a.popv + static_cast<int64_t>(p) * a.c_pad;
-            // Biases and layer 4 of individual p (row-major W4 -> [d3][16]).
-            ptx::named_barrier_sync(1, kEpiThreads);  // the previous individual's parameters are no longer read
-            for (int i = et; i < d1; i += kEpiThreads) s.b1[i] = net[a.b_off[0] + i];
-            for (int i = et; i < d2; i += kEpiThreads) s.b2[i] = net[a.b_off[1] + i];
-            for (int i = et; i < d3; i += kEpiThreads) s.b3[i] = net[a.b_off[2] + i];
-            for (int i = et; i < d3 * kMaxOutTc; i += kEpiThreads) {
-                const int c = i / kMaxOutTc, o = i % kMaxOutTc;
-                s.w4t[i] = o < d_out ? net[a.w_off[3] + static_cast<int64_t>(o) * d3 + c] : 0.0f;
+    } else if (warp < kFirstEpiWarp) {
+        // ------------------------------------------------------------ biases
+        const int d1 = a.dims[1], d2 = a.dims[2], d3 = a.dims[3], d_out = a.dims[4];
+        auto wait = [&](uint64_t* bar, uint32_t parity) {
+            const bool got = ptx::mbar_wait_sleeping(bar, parity, s.abort_flag, kWaitLimitNs, 200u);
+            if (__all_sync(0xFFFFFFFFu, got)) return true;
+            raise_abort(s, a);
+            return false;
+        };
+        uint32_t k = 0;
+        for (Segments seg(a, blockIdx.x); warp == kParamWarp && seg.valid(); ++k) {
+            {
+                if (!wait(&s.param_empty[k & 1u], ((k >> 1) & 1u) ^ 1u)) break;
+                const float* net = a.popv + static_cast<int64_t>(seg.p) * a.c_pad;
+                float* b = s.param + (k & 1u) * param_floats(a.dims);
+                for (int e = lane; e < d1; e += 32) b[e] = net[a.b_off[0] + e] * kPieceScale;
+                for (int e = lane; e < d2; e += 32) b[d1 + e] = net[a.b_off[1] + e] * kPieceScale;
+                for (int e = lane; e < d3; e += 32) b[d1 + d2 + e] = net[a.b_off[2] + e] * kPieceScale;
+                if (lane < kMaxOutTc) b[d1 + d2 + d3 + lane] = lane < d_out ? net[a.b_off[3] + lane] : 0.0f;
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(&s.param_full[k & 1u]);
             }
-            if (et < kMaxOutTc) s.b4[et] = et < d_out ? net[a.b_off[3] + et] : 0.0f;
-            ptx::named_barrier_sync(1, kEpiThreads);
-            float total = 0.0f;
-            int32_t n_ok = 0;
-            bool bad = false;
-            for (int t = 0; t < a.n_tiles; ++t, ++unit) {
-                const int smp = t * kTile + row;
-                const bool live = smp < a.batch;
-                // layers 1 and 2: bias, ReLU, split for the next layer; layer 3: ReLU, layer 4, loss
-                for (int l = 0; l < 3; ++l) {
-                    if (et == 0) {
-                        const bool got = ptx::mbar_wait_bounded(&s.d_full[l], unit & 1u, s.abort_flag, kWaitLimitNs);
-                        if (!got) raise_abort(s, a);
-                        *s.ep_go = got ? 1 : 0;
-                    }
-                    ptx::named_barrier_sync(1, kEpiThreads);
-                    if (!*s.ep_go) { ok = false; break; }
+            seg.step(a);
+        }
+    } else {
+        const int d1 = a.dims[1], d2 = a.dims[2], d3 = a.dims[3], d_out = a.dims[4];
+        const int q = warp & 3, row = q * 32 + lane;
+        auto wait = [&](uint64_t* bar, uint32_t parity) {
+            const bool got = ptx::mbar_wait_sleeping(bar, parity, s.abort_flag, kWaitLimitNs, 20u);
+            if (__all_sync(0xFFFFFFFFu, got)) return true;
+            raise_abort(s, a);
+            return false;
+        };
+        auto arrive = [&](uint64_t* bar) {
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(bar);
+        };
+        uint32_t u = 0, k = 0;  // units and individuals so far
+        bool ok = true;
+        if (warp < kFirstLossWarp) {
+            // -------------------------------------------------------- epilogue
+            const int part = (warp - kFirstEpiWarp) >> 2;
+            const uint32_t acc = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
+            const float scale1 = a.inv_div * kPieceScale;
+            for (Segments seg(a, blockIdx.x); ok && seg.valid(); seg.step(a), ++k) {
+                const float* b1 = s.param + (k & 1u) * param_floats(a.dims);
+                const float *b2 = b1 + d1, *b3 = b2 + d2;
+                if (!wait(&s.param_full[k & 1u], (k >> 1) & 1u)) break;
+                __half2 top = __float2half2_rn(0.0f);  // the largest hi pieces: activations times 2^8
+                for (int t = seg.t0; t < seg.t1; ++t, ++u) {
+                    // layer 1, a 64-column block at a time, one group per part
+                    if (!(ok = wait(&s.d_full[0], u & 1u))) break;
                     ptx::tc_fence_after();
-                    const int N = a.dims[l + 1];
-                    const float* bias = l == 0 ? s.b1 : (l == 1 ? s.b2 : s.b3);
-                    const float scale = l == 0 ? a.inv_div : 1.0f / (kPieceScale * kPieceScale);
-                    // this half's 16-column groups
-                    const int groups = N / 16, g0 = half ? groups / 2 : 0, g1 = half ? groups : groups / 2;
-                    if (l < 2) {
-                        // 64-column blocks in order, two of each block's four groups per
-                        // half; layer 1's blocks go to the layer-2 MMAs one by one
-                        for (int gi = 0; gi < 2 * ((N + 63) / 64); ++gi) {
-                            const int kb = gi >> 1, g = 4 * kb + 2 * half + (gi & 1);
-                            const int c = 16 * g;
-                            if (g < groups) {
-                                float v[16];
-                                load_acc16(tmem_base + lane_addr + col(l) + static_cast<uint32_t>(c),
-                                           static_cast<uint32_t>(N), merged(l), v);
-                                uint32_t hi[8], lo[8];
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) {
-                                    const float h0 = fmaxf(fmaf(v[2 * e], scale, bias[c + 2 * e]), 0.0f);
-                                    const float h1 = fmaxf(fmaf(v[2 * e + 1], scale, bias[c + 2 * e + 1]), 0.0f);
-                                    bad |= h0 >= kPieceRange || h1 >= kPieceRange;
-                                    split2x2(h0, h1, hi[e], lo[e]);
-                                }
-                                uint8_t* dst = s.region + (c >> 6) * kBlockBytes;
-                                const int ch = (c & 63) >> 3;
-                                *reinterpret_cast<uint4*>(dst + swz(row, ch)) =
-                                    make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                                *reinterpret_cast<uint4*>(dst + swz(row, ch + 1)) =
-                                    make_uint4(hi[4], hi[5], hi[6], hi[7]);
-                                *reinterpret_cast<uint4*>(dst + kHalfRegion + swz(row, ch)) =
-                                    make_uint4(lo[0], lo[1], lo[2], lo[3]);
-                                *reinterpret_cast<uint4*>(dst + kHalfRegion + swz(row, ch + 1)) =
-                                    make_uint4(lo[4], lo[5], lo[6], lo[7]);
-                            }
-                            if (l == 0 && (gi & 1)) {
-                                ptx::fence_proxy_async_smem();
-                                ptx::tc_fence_before();
-                                ptx::mbar_arrive(&s.h_blk[kb]);
-                            }
-                        }
-                        if (l == 1) {
-                            ptx::fence_proxy_async_smem();
-                            ptx::tc_fence_before();
-                            ptx::mbar_arrive(s.h2_ready);
-                        }
-                    } else {
-                        // layer 3's ReLU, then layer 4 and the loss in FP32
-                        float logit[kMaxOutTc];
-#pragma unroll
-                        for (int o = 0; o < kMaxOutTc; ++o) logit[o] = 0.0f;
-                        for (int c = 16 * g0; c < 16 * g1; c += 16) {
-                            float v[16];
-                            load_acc16(tmem_base + lane_addr + col(l) + static_cast<uint32_t>(c),
-                                       static_cast<uint32_t>(N), merged(l), v);
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) {
-                                const float h = fmaxf(fmaf(v[j], scale, bias[c + j]), 0.0f);
-                                const float4* wr = reinterpret_cast<const float4*>(s.w4t + (c + j) * kMaxOutTc);
-#pragma unroll
-                                for (int o4 = 0; o4 < kMaxOutTc / 4; ++o4) {
-                                    if (4 * o4 < d_out) {
-                                        const float4 w4 = wr[o4];
-                                        logit[4 * o4 + 0] = fmaf(w4.x, h, logit[4 * o4 + 0]);
-                                        logit[4 * o4 + 1] = fmaf(w4.y, h, logit[4 * o4 + 1]);
-                                        logit[4 * o4 + 2] = fmaf(w4.z, h, logit[4 * o4 + 2]);
-                                        logit[4 * o4 + 3] = fmaf(w4.w, h, logit[4 * o4 + 3]);
-                                    }
-                                }
-                            }
-                        }
+                    for (int kb = 0; kb < (d1 + 63) / 64; ++kb) {
+                        activate_part(acc, 64 * kb + kPartCols * part, d1, scale1, b1, top);
+                        ptx::tmem_st_wait();
                         ptx::tc_fence_before();
-                        if (half == 1) {
+                        arrive(&s.h_blk[kb]);
+                    }
+                    // layers 2 and 3
+                    for (int l = 1; ok && l < 3; ++l) {
+                        if (!(ok = wait(&s.d_full[l], u & 1u))) break;
+                        ptx::tc_fence_after();
+                        for (int c = kPartCols * part; c < a.dims[l + 1]; c += 64)
+                            activate_part(acc + static_cast<uint32_t>(a.col[l]), c, a.dims[l + 1], 1.0f / kPieceScale,
+                                          l == 1 ? b2 : b3, top);
+                        ptx::tmem_st_wait();
+                        ptx::tc_fence_before();
+                        arrive(&s.h_ready[l - 1]);
+                    }
+                    if (!ok) break;
+                }
+                if (!ok) break;
+                arrive(&s.param_empty[k & 1u]);
+                const float2 largest = __half22float2(top);
+                if (__any_sync(0xFFFFFFFFu, fmaxf(largest.x, largest.y) >= kPieceRange * kPieceScale) && lane == 0)
+                    a.flagged[seg.p] = 1;
+            }
+        } else {
+            // -------------------------------------------------------- loss, one sample per thread
+            for (Segments seg(a, blockIdx.x); ok && seg.valid(); seg.step(a), ++k) {
+                const float* b4 = s.param + (k & 1u) * param_floats(a.dims) + d1 + d2 + d3;
+                if (!wait(&s.param_full[k & 1u], (k >> 1) & 1u)) break;
+                double total = 0.0;
+                int32_t n_ok = 0;
+                for (int t = seg.t0; t < seg.t1; ++t, ++u) {
+                    const int smp = t * kTile + row;
+                    const int32_t lbl = smp < a.batch ? a.y[smp] : 0;
+                    if (!(ok = wait(&s.d_full[3], u & 1u))) break;
+                    ptx::tc_fence_after();
+                    float z[kMaxOutTc];
+                    ptx::tmem_ld16(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(a.col[3]), z);
+                    ptx::tc_fence_before();
+                    arrive(s.d4_read);
+                    float zmax = 0.0f, zl = 0.0f;
+                    int arg = 0;
 #pragma unroll
-                            for (int o = 0; o < kMaxOutTc; ++o) s.plog[row * kMaxOutTc + o] = logit[o];
+                    for (int o = 0; o < kMaxOutTc; ++o) {
+                        if (o < d_out) {
+                            z[o] = fmaf(z[o], 1.0f / (kPieceScale * kPieceScale), b4[o]);
+                            if (o == 0 || z[o] > zmax) { zmax = z[o]; arg = o; }
+                            if (o == lbl) zl = z[o];
                         }
-                        ptx::named_barrier_sync(1, kEpiThreads);  // the second half's partial logits are in
-                        float loss = 0.0f;
-                        int32_t good = 0;
-                        if (live && half == 0) {
-                            float z[kMaxOutTc];
+                    }
+                    if (smp < a.batch) {
+                        float se = 0.0f;
 #pragma unroll
-                            for (int o = 0; o < kMaxOutTc; ++o)
-                                z[o] = o < d_out ? (logit[o] + s.plog[row * kMaxOutTc + o]) + s.b4[o] : 0.0f;
-                            float zmax = z[0];
-                            int arg = 0;
-#pragma unroll
-                            for (int o = 1; o < kMaxOutTc; ++o)
-                                if (o < d_out && z[o] > zmax) { zmax = z[o]; arg = o; }
-                            float se = 0.0f;
-#pragma unroll
-                            for (int o = 0; o < kMaxOutTc; ++o)
-                                if (o < d_out) se += expf(z[o] - zmax);
-                            const int32_t lbl = a.y[smp];
-                            if (lbl >= 0 && lbl < d_out) {
-                                float zl = 0.0f;
-#pragma unroll
-                                for (int o = 0; o < kMaxOutTc; ++o)
-                                    if (o == lbl) zl = z[o];
-                                loss = logf(se) + zmax - zl;
-                                good = arg == lbl ? 1 : 0;
-                            } else {
-                                loss = __int_as_float(0x7FC00000);
-                            }
-                        }
-#pragma unroll
-                        for (int off = 16; off > 0; off >>= 1) {
-                            loss += __shfl_xor_sync(0xFFFFFFFFu, loss, off);
-                            good += __shfl_xor_sync(0xFFFFFFFFu, good, off);
-                        }
-                        if (lane == 0 && half == 0) {
-                            s.red_loss[q] = loss;
-                            s.red_ok[q] = good;
-                        }
-                        ptx::named_barrier_sync(1, kEpiThreads);
-                        if (et == 0) {
-                            total += ((s.red_loss[0] + s.red_loss[1]) + s.red_loss[2]) + s.red_loss[3];
-                            n_ok += s.red_ok[0] + s.red_ok[1] + s.red_ok[2] + s.red_ok[3];
-                        }
+                        for (int o = 0; o < kMaxOutTc; ++o)
+                            if (o < d_out) se += expf(z[o] - zmax);
+                        const bool valid = lbl >= 0 && lbl < d_out;
+                        total += static_cast<double>(valid ? logf(se) + zmax - zl : __int_as_float(0x7FC00000));
+                        n_ok += valid && arg == lbl ? 1 : 0;
                     }
                 }
                 if (!ok) break;
-            }
-            if (!ok) break;
-            if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) a.flagged[p] = 1;
-            if (et == 0) {
-                const float f = -(total / static_cast<float>(a.batch));
-                a.f_raw[p] = f;
-                if (a.f_adj) a.f_adj[p] = a.f_inh ? (1.0f - a.alpha) * a.f_inh[p] + a.alpha * f : f;
-                if (a.correct) a.correct[p] = n_ok;
+                arrive(&s.param_empty[k & 1u]);
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) {
+                    total += __shfl_xor_sync(0xFFFFFFFFu, total, off);
+                    n_ok += __shfl_xor_sync(0xFFFFFFFFu, n_ok, off);
+                }
+                // Two buffers: the sums of individual k + 2 come after layer 4 of its
+                // units, which waits for d4_read of a unit of k + 1, for which warp q = 0
+                // arrives when it has read these.
+                double* red_loss = s.red_loss + 4 * (k & 1u);
+                int32_t* red_ok = s.red_ok + 4 * (k & 1u);
+                if (lane == 0) {
+                    red_loss[q] = total;
+                    red_ok[q] = n_ok;
+                    ptx::mbar_arrive(s.red_full);
+                }
+                if (q == 0) {
+                    if (!(ok = wait(s.red_full, k & 1u))) break;
+                    if (lane == 0) {
+                        const double sum = ((red_loss[0] + red_loss[1]) + red_loss[2]) + red_loss[3];
+                        const int32_t good = red_ok[0] + red_ok[1] + red_ok[2] + red_ok[3];
+                        if (seg.t0 == 0 && seg.t1 == a.n_tiles) {
+                            store_fitness(a, seg.p, sum, good);
+                        } else {  // at most one segment of a CTA starts, and one ends, inside an individual
+                            const int e = 2 * static_cast<int>(blockIdx.x) + (seg.t0 == 0 ? 1 : 0);
+                            a.part_loss[e] = sum;
+                            a.part_ok[e] = good;
+                        }
+                    }
+                }
             }
         }
     }
@@ -576,44 +754,44 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const MlpTcA
     }
 }
 
+// The fitness of the individuals that several CTAs share: the sums of their
+// segments in order of the tiles.
+__global__ void __launch_bounds__(256) combine_mlp_parts_kernel(const MlpTcArgs a)
+{
+    const int p = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
+    if (p >= a.pop) return;
+    const int64_t big = static_cast<int64_t>(a.extra) * (a.per_cta + 1);  // units of the CTAs with one more
+    auto owner = [&](int64_t u) {
+        return static_cast<int>(u < big ? u / (a.per_cta + 1) : a.extra + (u - big) / a.per_cta);
+    };
+    const int64_t first = static_cast<int64_t>(p) * a.n_tiles;
+    const int c0 = owner(first), c1 = owner(first + a.n_tiles - 1);
+    if (c0 == c1) return;
+    double sum = 0.0;
+    int32_t good = 0;
+    for (int c = c0; c <= c1; ++c) {
+        const int e = 2 * c + (c == c0 ? 1 : 0);
+        sum += a.part_loss[e];
+        good += a.part_ok[e];
+    }
+    store_fitness(a, p, sum, good);
+}
+
 // Each individual's weights of layers 1-3 as FP16 pieces of 2^8 w in the
-// swizzled operand layout (individuals strided over blockIdx.y); a weight
-// |w| >= 128 marks the individual for the FP32 recomputation.
+// swizzled operand layout (blockIdx.x: the 64-input block); a weight |w| >= 128
+// marks the individual for the FP32 recomputation.
 __global__ void __launch_bounds__(256) split_weights_kernel(const MlpTcArgs a)
 {
+    // block blockIdx.x of the individual
+    int l = 0, kb = static_cast<int>(blockIdx.x);
+    while (kb >= layer_blocks(a, l)) kb -= layer_blocks(a, l++);
     for (int p = blockIdx.y; p < a.pop; p += gridDim.y) {
-        const float* net = a.popv + static_cast<int64_t>(p) * a.c_pad;
-        uint8_t* dst_p = const_cast<uint8_t*>(a.pieces) + static_cast<int64_t>(p) * a.piece_stride;
-        int n_items[3];
-        for (int l = 0; l < 3; ++l) n_items[l] = layer_blocks(a, l) * a.dims[l + 1] * 8;
-        const int total = n_items[0] + n_items[1] + n_items[2];
-        bool bad = false;
-        for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < total; it += gridDim.x * blockDim.x) {
-            int l = 0, r = it;
-            while (r >= n_items[l]) r -= n_items[l++];
-            const int K = a.dims[l], N = a.dims[l + 1];
-            const int kb = r / (N * 8), rem = r - kb * N * 8;
-            const int n = rem >> 3, ch = rem & 7;
-            const int k = kb * 64 + 8 * ch;
-            float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
-            if (k < K) {
-                const float4* src = reinterpret_cast<const float4*>(net + a.w_off[l] + static_cast<int64_t>(n) * K + k);
-                v0 = __ldg(src);
-                if (k + 4 < K) v1 = __ldg(src + 1);
-            }
-            const float w[8] = { v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w };
-            uint32_t hi[4], lo[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                split2x2(w[2 * e], w[2 * e + 1], hi[e], lo[e]);
-                bad |= fabsf(w[2 * e]) >= kPieceRange || fabsf(w[2 * e + 1]) >= kPieceRange;
-            }
-            uint8_t* blk = dst_p + a.layer_off[l] + static_cast<int64_t>(kb) * N * 256;
-            const uint32_t off = swz(n, ch);
-            *reinterpret_cast<uint4*>(blk + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-            *reinterpret_cast<uint4*>(blk + N * 128 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-        }
-        if (bad) a.flagged[p] = 1;
+        Splitter split;
+        split.l = l;
+        split.kb = kb;
+        while (split.batch(a, p, a.pieces + static_cast<int64_t>(p) * a.piece_stride, static_cast<int>(threadIdx.x), 256) &&
+               split.l == l && split.kb == kb) {}
+        if (split.outside()) a.flagged[p] = 1;
     }
 }
 
@@ -669,16 +847,23 @@ uint8_t* shared_scratch(size_t bytes)
     return buf[dev];
 }
 
-// Bytes of one individual's weight pieces; byte offset of each layer's blocks.
-int64_t piece_layout(const NetLayout& net, int64_t* layer_off)
+// The slots of an individual's weights; its bytes of pieces.
+int64_t piece_layout(const NetLayout& net, MlpSlots* m)
 {
     int64_t off = 0;
-    for (int l = 0; l < 3; ++l) {
-        layer_off[l] = off;
-        const int64_t k16 = (net.dims[l] + 15) / 16 * 16;
-        off += (k16 + 63) / 64 * net.dims[l + 1] * 256;
+    for (int l = 0; l < 4; ++l) {
+        const int32_t k16 = (net.dims[l] + 15) / 16 * 16, n = l < 3 ? net.dims[l + 1] : kMaxOutTc, tail = k16 % 64;
+        m->k16[l] = k16;
+        m->n[l] = n;
+        m->stacked[l] = l > 0 && 2 * n <= 256;
+        m->tail_joined = l == 0 ? (tail > 0 && tail <= 32) : m->tail_joined;
+        const int32_t blocks = (k16 + 63) / 64;
+        m->slots[l] = m->stacked[l] ? blocks : 2 * blocks - (l == 0 && m->tail_joined ? 1 : 0);
+        m->slot_bytes[l] = static_cast<uint32_t>(n) * (m->stacked[l] ? 256u : 128u);
+        m->layer_off[l] = off;
+        off += static_cast<int64_t>(m->slots[l]) * m->slot_bytes[l];
     }
-    return off;
+    return (off + 255) / 256 * 256;
 }
 
 // Bytes of one tile's levels (64-input blocks of 128 rows of 128 bytes).
@@ -687,21 +872,41 @@ uint32_t level_tile_bytes(const NetLayout& net)
     return static_cast<uint32_t>((net.dims[0] + 63) / 64) * kBlockBytes;
 }
 
-// Scratch layout: the pieces (a multiple of 256 bytes), the marks (rounded up
-// to 256 bytes), the level tiles.
-size_t marks_bytes(int32_t pop)
+int sm_count()
 {
-    return (sizeof(int32_t) * static_cast<size_t>(pop) + 255) / 256 * 256;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    return cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? sms : 0;
+}
+
+// Scratch layout, each part a multiple of 256 bytes: the pieces, the marks, the
+// level tiles, the sums of shared individuals.
+struct MlpScratch {
+    int32_t grid;
+    size_t marks, tiles, part_loss, part_ok, bytes;
+};
+
+MlpScratch mlp_scratch_layout(const NetLayout& net, int32_t pop, int32_t batch)
+{
+    auto up = [](size_t n) { return (n + 255) / 256 * 256; };
+    MlpSlots m{};
+    const size_t stride = static_cast<size_t>(piece_layout(net, &m)), np = static_cast<size_t>(pop);
+    const int32_t tiles = (batch + kTile - 1) / kTile, sms = sm_count();
+    MlpScratch s{};
+    s.grid = static_cast<int32_t>(std::min<int64_t>(sms, static_cast<int64_t>(pop) * tiles));
+    s.marks = stride * np;
+    s.tiles = s.marks + up(sizeof(int32_t) * np);
+    s.part_loss = s.tiles + static_cast<size_t>(tiles) * level_tile_bytes(net);
+    s.part_ok = s.part_loss + up(16 * static_cast<size_t>(sms));
+    s.bytes = s.part_ok + up(8 * static_cast<size_t>(sms));
+    return s;
 }
 
 }  // namespace
 
 size_t eval_mlp_tc_scratch_bytes(const NetLayout& net, int32_t pop, int32_t batch)
 {
-    int64_t layer_off[3];
-    const size_t pieces = static_cast<size_t>(piece_layout(net, layer_off)) * static_cast<size_t>(pop);
-    const size_t tiles = static_cast<size_t>((batch + kTile - 1) / kTile);
-    return pieces + marks_bytes(pop) + tiles * level_tile_bytes(net);
+    return mlp_scratch_layout(net, pop, batch).bytes;
 }
 
 bool eval_mlp_tc_supported(const NetLayout& net, const float* pop_dev)
@@ -711,13 +916,10 @@ bool eval_mlp_tc_supported(const NetLayout& net, const float* pop_dev)
     if (d0 % 4 != 0 || d0 > 256 || d_out > kMaxOutTc) return false;
     for (int32_t n : { d1, d2, d3 })
         if (n % 16 != 0 || n < 16 || n > 256) return false;
-    // layer 1 in [0, d1), layers 2 and 3 from column d1 (2n columns if merged)
-    for (int32_t n : { d2, d3 })
-        if (d1 + (merged_layer(d1, n) ? 2 * n : n) > static_cast<int32_t>(kTmemCols)) return false;
-    for (int l = 0; l < 3; ++l)
+    for (int l = 0; l < 4; ++l)
         if (net.w_off[l] % 4 != 0) return false;
     if (reinterpret_cast<uintptr_t>(pop_dev) & 15u) return false;
-    return tc_smem_bytes(net.dims) <= 227u * 1024u;
+    return mlp_ring(net.dims, (d0 + 63) / 64 * kBlockBytes) >= 2;
 }
 
 cudaError_t launch_eval_mlp_tc(const NetLayout& net, int32_t pop, const float* pop_dev, const uint8_t* x, float x_div,
@@ -730,7 +932,6 @@ cudaError_t launch_eval_mlp_tc(const NetLayout& net, int32_t pop, const float* p
     a.batch = batch;
     a.n_tiles = (batch + kTile - 1) / kTile;
     for (int l = 0; l <= 4; ++l) a.dims[l] = net.dims[l];
-    for (int l = 0; l < 3; ++l) a.k16[l] = (net.dims[l] + 15) / 16 * 16;
     a.c_pad = net.c_pad;
     for (int l = 0; l < 4; ++l) {
         a.w_off[l] = net.w_off[l];
@@ -746,35 +947,42 @@ cudaError_t launch_eval_mlp_tc(const NetLayout& net, int32_t pop, const float* p
     a.f_adj = f_adj;
     a.correct = correct;
     a.status = status;
-    a.piece_stride = piece_layout(net, a.layer_off);
-    const size_t pieces = static_cast<size_t>(a.piece_stride) * static_cast<size_t>(pop);
-    uint8_t* base =
-        scratch ? static_cast<uint8_t*>(scratch) : shared_scratch(eval_mlp_tc_scratch_bytes(net, pop, batch));
+    a.piece_stride = piece_layout(net, &a.m);
+    mlp_columns(&a);
+    const MlpScratch sc = mlp_scratch_layout(net, pop, batch);
+    uint8_t* base = static_cast<uint8_t*>(scratch ? scratch : shared_scratch(sc.bytes));
     if (!base) return cudaErrorMemoryAllocation;
+    if (sc.grid <= 0) return cudaErrorInvalidValue;
     a.pieces = base;
-    a.flagged = reinterpret_cast<int32_t*>(base + pieces);  // pieces: a multiple of 256 bytes
+    a.flagged = reinterpret_cast<int32_t*>(base + sc.marks);
     a.x_bytes = level_tile_bytes(net);
-    a.xtiles = base + pieces + marks_bytes(pop);
+    a.xtiles = base + sc.tiles;
+    a.part_loss = reinterpret_cast<double*>(base + sc.part_loss);
+    a.part_ok = reinterpret_cast<int32_t*>(base + sc.part_ok);
+    const int64_t units = static_cast<int64_t>(pop) * a.n_tiles;
+    a.per_cta = static_cast<int32_t>(units / sc.grid);
+    a.extra = static_cast<int32_t>(units % sc.grid);
     cudaError_t err = cudaMemsetAsync(a.flagged, 0, sizeof(int32_t) * static_cast<size_t>(pop), stream);
     if (err != cudaSuccess) return err;
     {
-        int items = 0;
-        for (int l = 0; l < 3; ++l) items += ((a.k16[l] + 63) / 64) * net.dims[l + 1] * 8;
-        split_weights_kernel<<<dim3((items + 255) / 256, pop < 65535 ? pop : 65535), 256, 0, stream>>>(a);
+        int blocks = 0;
+        for (int l = 0; l < 4; ++l) blocks += (a.m.k16[l] + 63) / 64;
+        split_weights_kernel<<<dim3(blocks, pop < 65535 ? pop : 65535), 256, 0, stream>>>(a);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         const int level_items = a.n_tiles * ((a.dims[0] + 63) / 64) * kTile * 8;
         stage_levels_kernel<<<(level_items + 255) / 256, 256, 0, stream>>>(a, x);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
     }
-    const size_t smem = tc_smem_bytes(net.dims);
+    a.n_slots = mlp_ring(net.dims, a.x_bytes);
+    const size_t smem = tc_smem_bytes(net.dims, a.x_bytes, a.n_slots);
     err = cudaFuncSetAttribute(eval_mlp_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (err != cudaSuccess) return err;
-    int dev = 0, sms = 0;
-    if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
-    if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return err;
-    const int grid = pop < sms ? pop : sms;
-    eval_mlp_tc_kernel<<<grid, kTcThreads, smem, stream>>>(a);
+    eval_mlp_tc_kernel<<<sc.grid, kTcThreads, smem, stream>>>(a);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    if (a.extra != 0 || a.per_cta % a.n_tiles != 0) {
+        combine_mlp_parts_kernel<<<(pop + 255) / 256, 256, 0, stream>>>(a);
+        if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    }
     // Individuals with a weight or activation outside the FP16 pieces' range:
     // their fitness again, in FP32 on the CUDA cores.
     return launch_eval_mlp_u8_only(net, pop, pop_dev, x, x_div, y, batch, alpha, f_inh, f_raw, f_adj, correct,
