@@ -174,6 +174,12 @@ __device__ __forceinline__ void cta_work(const PairArgs& a, int& mt, int& first,
     count = a.per_grp + (g < a.extra ? 1 : 0);
 }
 
+// i / d for 0 <= i with i d < 2^32, from reciprocal(d): the epilogue divides nine
+// indices per unit to stage the parameters, between a pair's results and the
+// next pair's layer 2.
+__device__ __forceinline__ uint32_t reciprocal(int d) { return 0xFFFFFFFFu / static_cast<uint32_t>(d) + 1u; }
+__device__ __forceinline__ int divide(int i, uint32_t per_d) { return static_cast<int>(__umulhi(static_cast<uint32_t>(i), per_d)); }
+
 template <int PREC, int DOUT>  // DOUT: d_out when fixed at compile time (10), else 0
 __global__ void __launch_bounds__(kPairThreads, 1) eval_shadow_pair_kernel(const PairArgs a)
 {
@@ -418,6 +424,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) eval_shadow_pair_kernel(const
                 }
             }
         };
+        const uint32_t per_h = reciprocal(a.h);
         load_prm(0);
         for (int u = 0; 2 * u < count; ++u) {
             const int n = min(2, count - 2 * u);
@@ -431,7 +438,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) eval_shadow_pair_kernel(const
                     if (i < a.h) {
                         b1[i] = prm[j];
                     } else if (i < a.h + d_out * a.h) {
-                        const int o = (i - a.h) / a.h, col = (i - a.h) - o * a.h;
+                        const int o = divide(i - a.h, per_h), col = (i - a.h) - o * a.h;
                         w2t[col * dpad + o] = prm[j];
                     } else if (i < a.n_prm) {
                         b2[i - a.h - d_out * a.h] = prm[j];
