@@ -15,6 +15,8 @@
 // per sample (maximum subtracted, FP32), and the argmax.  Each tile's two warp
 // sums are added in order, the tiles in order: identical individuals give
 // bitwise identical fitness.
+#include <algorithm>
+
 #include "leea_internal.h"
 
 namespace leea {
@@ -31,13 +33,14 @@ constexpr int kWStride = kMaxWidth + 4;      // WT[kk][o] row stride (floats)
 constexpr int kLogitStride = kMaxOutMlp + 1;
 
 struct MlpArgs {
-    int32_t n_layers, batch;
+    int32_t n_layers, batch, pop;
     int32_t dims[kMaxLayers + 1];
     int64_t w_off[kMaxLayers], b_off[kMaxLayers];
     int64_t c_pad;
     float alpha, x_div;
 };
 
+constexpr int kOnlyCtas = 152;  // CTAs of a launch for marked individuals: one per SM
 constexpr size_t kMlpSmemBytes =
     sizeof(float) * (2 * kMaxWidth * kActStride + 2 * kKC * kWStride + kTS * kLogitStride) + 64;
 
@@ -146,7 +149,6 @@ eval_mlp_kernel(const MlpArgs e, const float* __restrict__ popv, const XT* __res
                 const int32_t* __restrict__ y, const float* __restrict__ f_inh, float* __restrict__ f_raw,
                 float* __restrict__ f_adj, int32_t* __restrict__ correct, const int32_t* __restrict__ only)
 {
-    if (only && only[blockIdx.x] == 0) return;  // only the marked individuals
     extern __shared__ float4 smem4[];
     float* smem = reinterpret_cast<float*>(smem4);
     float* act[2] = { smem, smem + kMaxWidth * kActStride };
@@ -155,7 +157,17 @@ eval_mlp_kernel(const MlpArgs e, const float* __restrict__ popv, const XT* __res
     float* red = logits + kTS * kLogitStride;        // [2]: per-warp loss sums of a tile
     int32_t* red_ok = reinterpret_cast<int32_t*>(red + 2);
     const int tid = threadIdx.x;
-    const int p = blockIdx.x;
+    // One CTA per individual; for the marked ones only, a few CTAs share them all
+    // and most find no mark among theirs (2000 nets: 10 us with a CTA each).
+    if (only) {
+        int any = 0;
+        for (int64_t p = blockIdx.x + static_cast<int64_t>(tid) * gridDim.x; p < e.pop;
+             p += static_cast<int64_t>(kMlpThreads) * gridDim.x)
+            any |= only[p];
+        if (!__syncthreads_or(any)) return;
+    }
+    for (int p = blockIdx.x; p < e.pop; p += gridDim.x) {
+    if (only && only[p] == 0) continue;
     const float* net = popv + static_cast<int64_t>(p) * e.c_pad;
     const int d0 = e.dims[0], d_out = e.dims[e.n_layers];
     float total = 0.0f;
@@ -226,6 +238,7 @@ eval_mlp_kernel(const MlpArgs e, const float* __restrict__ popv, const XT* __res
         if (f_adj) f_adj[p] = f_inh ? (1.0f - e.alpha) * f_inh[p] + e.alpha * f : f;
         if (correct) correct[p] = n_ok;
     }
+    }
 }
 
 template <typename XT>
@@ -271,7 +284,9 @@ cudaError_t launch_mlp(const NetLayout& net, int32_t pop, const float* pop_dev, 
     cudaError_t err = cudaFuncSetAttribute(eval_mlp_kernel<XT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            static_cast<int>(kMlpSmemBytes));
     if (err != cudaSuccess) return err;
-    eval_mlp_kernel<XT><<<pop, kMlpThreads, kMlpSmemBytes, stream>>>(mlp_args(net, batch, alpha, x_div), pop_dev, x, y,
+    MlpArgs e = mlp_args(net, batch, alpha, x_div);
+    e.pop = pop;
+    eval_mlp_kernel<XT><<<only ? std::min(pop, kOnlyCtas) : pop, kMlpThreads, kMlpSmemBytes, stream>>>(e, pop_dev, x, y,
                                                                     f_inh, f_raw, f_adj, correct, only);
     return cudaGetLastError();
 }
