@@ -109,12 +109,12 @@ STAGES = ("select", "breed", "evaluate")
 # DRAM traffic per launch from one ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum), valid only while the kernel source is unchanged.
 TRAFFIC = {
-    "breed": {"bytes_per_launch": 472.53e6, "src_sha": "3ba6876d0f989830", "capture": "P=1000 plain workload"},
-    "evaluate": {"bytes_per_launch": 368.68e6, "src_sha": "921b0e7934e40403", "capture": "P=1000 plain workload"},
+    "breed": {"bytes_per_launch": 467.92e6, "src_sha": "7ef2dd3ff5ab01c5", "capture": "P=1000 plain workload"},
+    "evaluate": {"bytes_per_launch": 369.01e6, "src_sha": "29de9ecff4f9f1bf", "capture": "P=1000 plain workload"},
     "breed_evaluate": {"bytes_per_launch": 738.19e6, "src_sha": "23e25d83744d9797", "capture": "P=1000 plain workload"},
     # eval_mlp_tc_kernel alone (each individual's weight pieces read once from
     # DRAM, the other tiles from L2); the stage also splits the weights
-    "evaluate_paper_net": {"bytes_per_launch": 869.79e6, "src_sha": "407558790a9f32f1",
+    "evaluate_paper_net": {"bytes_per_launch": 1059.44e6, "src_sha": "bcad002c4ce3d228",
                            "capture": "paper-net workload, eval_mlp_tc_kernel"},
 }
 
@@ -692,15 +692,16 @@ def run_paper_net(args, rank: int, world: int, local_rank: int):
                        "kernel_timing": f"CUDA events around each kernel of every {PROFILE_EVERY}th generation "
                                         "inside the timed region",
                        "input": "uint8 levels k of 28x28 images, x = k/255, pooled on the GPU each step",
-                       "eval_kernel": ("tcgen05, FP16 operand pieces (FP32-class), FP32 accumulation in TMEM; layer 4 "
-                                       "and the loss in FP32" if tensor else
+                       "eval_kernel": ("tcgen05, FP16 operand pieces (FP32-class) in all four layers, FP32 accumulation "
+                                       "in TMEM; the loss in FP32" if tensor else
                                        "CUDA-core FP32, layers chained in shared memory (64-sample tiles)"),
                        "l2": f"inputs larger than L2 (2 population buffers of "
                              f"{pop * leea.leea_padded_params(dims) * 4 / 1e6:.0f} MB), no flush"},
             "network_samples_per_sec": gen_per_s * pop * batch, "e2e": e2e,
-            # + the max-pool; the tensor-core evaluation is four launches: the weight split, the level
-            # tiles, the kernel and the FP32 recomputation of marked individuals
-            "gpu_launches": int(steps * (1 + (3 if tensor else 0) + sum(kernels_per_generation(pop, batch, 0).values()))),
+            # + the max-pool; the tensor-core evaluation is five launches: the weight split, the level
+            # tiles, the kernel, the sums of individuals shared by CTAs and the FP32
+            # recomputation of marked individuals
+            "gpu_launches": int(steps * (1 + (4 if tensor else 0) + sum(kernels_per_generation(pop, batch, 0).values()))),
             "roofline": roofline, "kernels": kernels, "clocks": clk}
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         x_last = xtr[idx[warmup + steps]].astype(np.float64)

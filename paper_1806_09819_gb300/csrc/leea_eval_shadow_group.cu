@@ -4,7 +4,7 @@
 // individuals of a run per tcgen05 MMA; b1, W2, b2 and the softmax
 // cross-entropy in FP32 from the masters.
 //
-// A tcgen05.mma of M = 128 costs about the same for any N up to 256, so a
+// An MMA's issue and the batch tile it reads cost the same for any N, so a
 // run of hidden width h puts group = min(16, 256 / h) individuals side by
 // side in N (their pre-tiled shadow blocks stacked as the B operand); the
 // 128-sample batch tile is the A operand, staged once per evaluation as

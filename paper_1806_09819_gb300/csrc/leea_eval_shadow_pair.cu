@@ -3,10 +3,10 @@
 // of W1 with FP32 accumulation, two individuals per tcgen05 MMA; b1, W2, b2
 // and the softmax cross-entropy in FP32 from the master.
 //
-// A tcgen05.mma of M = 128 costs about the same time for any N up to 256,
-// and the shadows carry half (BF16) or a quarter (FP8) of the master's bytes,
-// so the MMA rate bounds this evaluation unless two individuals share every
-// MMA: the batch tile is the A operand (128 samples, the M side) and the
+// The shadows carry half (BF16) or a quarter (FP8) of the master's bytes, so
+// what an MMA costs besides them bounds this evaluation: its issue (about 100
+// to 130 cycles each here) and the batch tile it reads.  Two individuals
+// therefore share every MMA: the batch tile is the A operand (128 samples, the M side) and the
 // pair's shadow blocks, side by side, the B operand (N = 2h).  The batch is
 // staged once per evaluation as operand tiles in global memory, in the
 // 128-byte-swizzled K-major image the tensor core reads (stage_xop_kernel:

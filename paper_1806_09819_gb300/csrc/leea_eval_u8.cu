@@ -16,8 +16,8 @@
 // a launch of the TF32 or the CUDA-core kernel for the marked ones follows
 // (2 us when there are none).
 //
-// Shape.  A tcgen05.mma of M = 128 and K = 16 costs about the same time for any
-// N up to 256, so two individuals share every MMA where both fit (hp = h rounded
+// Shape.  Two individuals share every MMA where both fit, so that the batch tile
+// is streamed and read from shared memory once for both (hp = h rounded
 // up to 16, 2 hp <= 256; rows past h arrive as zeros): a 128-sample tile of the
 // batch (the M side) is the A operand and the stacked W1 pieces of the
 // individuals (N = ni hp) the B operand.  The batch, staged once per evaluation
