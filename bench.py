@@ -110,7 +110,7 @@ STAGES = ("select", "breed", "evaluate")
 # dram__bytes_write.sum), valid only while the kernel source is unchanged.
 TRAFFIC = {
     "breed": {"bytes_per_launch": 467.92e6, "src_sha": "7ef2dd3ff5ab01c5", "capture": "P=1000 plain workload"},
-    "evaluate": {"bytes_per_launch": 369.01e6, "src_sha": "29de9ecff4f9f1bf", "capture": "P=1000 plain workload"},
+    "evaluate": {"bytes_per_launch": 369.01e6, "src_sha": "12869056f17ba4e8", "capture": "P=1000 plain workload"},
     "breed_evaluate": {"bytes_per_launch": 738.19e6, "src_sha": "23e25d83744d9797", "capture": "P=1000 plain workload"},
     # eval_mlp_tc_kernel alone (each individual's weight pieces read once from
     # DRAM, the other tiles from L2); the stage also splits the weights

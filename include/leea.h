@@ -124,9 +124,10 @@ enum { LEEA_SIGMA_CONST = 0, LEEA_SIGMA_DECAY = 1, LEEA_SIGMA_SELF = 2 };
  * h <= 256, d_out <= 16 and 16-byte aligned buffers the tensor cores with FP16
  * operand pieces (an 8-bit level exactly, a float input and a weight as two, 22
  * bits; FP32 accumulation; individuals and samples that the pieces cannot hold
- * again with TF32 pieces or on the CUDA cores), else, or where so small a call
- * does not pay for the staging, TENSOR's kernel or SIMT's.  SIMT: exact FP32 FFMA on the
- * CUDA cores.  TENSOR: tcgen05 tensor cores with a three-term TF32 split
+ * again with TF32 pieces or on the CUDA cores) -- floats with h % 16 == 0,
+ * 8-bit levels in TENSOR's shapes or from 48 samples on -- else, or where so
+ * small a call does not pay for the staging, TENSOR's kernel or SIMT's.  SIMT:
+ * exact FP32 FFMA on the CUDA cores.  TENSOR: tcgen05 tensor cores with a three-term TF32 split
  * (X_hi W_hi + X_hi W_lo + X_lo W_hi, FP32 accumulation), which is within
  * ~1e-6 relative of FP32; LEEA_EINVAL if the shape does not allow it.
  * FUSED (state object, 8-bit generation calls, precision 0): every breeding

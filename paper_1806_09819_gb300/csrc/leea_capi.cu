@@ -260,13 +260,12 @@ leea_status dispatch_eval(const NetLayout& net, int32_t pop, const float* pop_de
     if (path == LEEA_EVAL_TENSOR && !tf32_ok)
         return fail(LEEA_EINVAL, "tensor-core evaluation needs d_0 %% 4 == 0, h %% 16 == 0, h <= 256, "
                                  "d_out <= 16 and 16-byte aligned population and x");
-    // AUTO: FP16 pieces of x and w, two individuals per MMA; where a weight is
-    // outside the pieces' range, that individual again with TF32 pieces (or, where
-    // the hidden width is off its 16, on the CUDA cores).
-    bool pieces = path == LEEA_EVAL_AUTO && (reinterpret_cast<uintptr_t>(x) & 15u) == 0 &&
-                        eval_u8_wide_supported(net, pop, batch, pop_dev, 2);
+    // AUTO, where TENSOR's kernel applies: FP16 pieces of x and w, two individuals
+    // per MMA; where a weight is outside the pieces' range, that individual again
+    // with TF32 pieces.
+    bool pieces = path == LEEA_EVAL_AUTO && tf32_ok && eval_u8_wide_supported(net, pop, batch, pop_dev, 2);
     unsigned int* status = nullptr;
-    if (pieces || (tf32_ok && path != LEEA_EVAL_SIMT)) {
+    if (tf32_ok && path != LEEA_EVAL_SIMT) {
         status = device_status_ptr();
         if (!status) return fail(LEEA_ECUDA, "device status word unavailable");
     }
@@ -277,7 +276,7 @@ leea_status dispatch_eval(const NetLayout& net, int32_t pop, const float* pop_de
         if (!scratch) {
             if (scratch_alloc(&own, eval_u8_scratch_bytes(net, pop, batch, 2), stream) != cudaSuccess) {
                 cudaGetLastError();
-                pieces = false;  // no memory for it: the kernels that need no scratch
+                pieces = false;  // no memory for it: TF32 pieces need no scratch
             }
             scratch = own;
         }
@@ -293,7 +292,7 @@ leea_status dispatch_eval(const NetLayout& net, int32_t pop, const float* pop_de
         if (tf32_ok && path != LEEA_EVAL_SIMT)
             err = launch_eval_tc(net, pop, pop_dev, x, y, batch, alpha, f_inh, f_raw, f_adj, correct, status, stream, only);
         else
-            err = launch_eval_simt(net, pop, pop_dev, x, y, batch, alpha, f_inh, f_raw, f_adj, correct, stream, only);
+            err = launch_eval_simt(net, pop, pop_dev, x, y, batch, alpha, f_inh, f_raw, f_adj, correct, stream);
     }
     if (own) {
         const cudaError_t ferr = cudaFreeAsync(own, stream);

@@ -291,10 +291,10 @@ static cudaError_t launch_simt_any(const NetLayout& net, int32_t pop, const floa
 cudaError_t launch_eval_simt(const NetLayout& net, int32_t pop, const float* pop_dev,
                              const float* x, const int32_t* y, int32_t batch, float alpha,
                              const float* f_inh, float* f_raw, float* f_adj, int32_t* correct,
-                             cudaStream_t stream, const int32_t* only)
+                             cudaStream_t stream)
 {
     return launch_simt_any<float>(net, pop, pop_dev, x, 1.0f, y, batch, alpha, f_inh, f_raw, f_adj, correct,
-                                  stream, only);
+                                  stream, nullptr);
 }
 
 cudaError_t launch_eval_simt_u8(const NetLayout& net, int32_t pop, const float* pop_dev, const uint8_t* x,

@@ -13,8 +13,9 @@
 // The converters find the individuals that the pieces cannot carry
 // (outside_pieces).  On 8-bit levels within TENSOR's shapes the epilogue forms
 // their layer 1 with FP32 FFMA from global memory; elsewhere it marks them and
-// a launch of the TF32 or the CUDA-core kernel for the marked ones follows
-// (2 us when there are none).
+// a launch of the kernel that has the call otherwise follows for the marked
+// ones (floats: TF32 pieces, 8-bit levels: the CUDA cores; 2 us when there are
+// none).
 //
 // Shape.  Two individuals share every MMA where both fit, so that the batch tile
 // is streamed and read from shared memory once for both (hp = h rounded
@@ -34,9 +35,8 @@
 // 111, 512 195, 1000 356, against 1.2 ms (256) to 9.8 ms (1024) on the CUDA
 // cores; 333 nets 784-100-10, batch 50: 40 (295).  Floats: P = 1000, 784-112-10,
 // batch 100: 83, against 184 with TF32 pieces (12 MMAs of K = 8 per 32 inputs and
-// individual instead of 6 of K = 16 per pair); batch 512 246 (711); 784-100-10,
-// batch 50, 77 (341 on the CUDA cores).  Max error against 64 bits over 1000 nets
-// 6.6e-8 (TF32 pieces 1.4e-7).
+// individual instead of 6 of K = 16 per pair); batch 512 246 (711).  Error against
+// 64 bits over 1000 nets 6.6e-8 (TF32 pieces 1.4e-7); see pieces_exact.
 //
 // What bounds it: shared memory.  Per K stage of 64 inputs a unit of one net and
 // two tiles has 61 KB written by TMA, 57 KB read and written by the converters
@@ -1023,10 +1023,11 @@ static bool in_tensor_shapes(const NetLayout& net, int32_t batch)
     return net.dims[1] % 16 == 0 && net.dims[1] <= 128 && batch <= 128;
 }
 
-// Whether the pieces pay where another kernel could take the call: staging the
-// batch and looking for marked individuals are two more launches, and a call
-// takes 25 us with them however small it is (784-100-10 and 50 samples: 152
-// nets 23 us, 1000 nets 79), 14 without.  The other kernel's time is modelled
+// Whether the pieces pay where another kernel could take the call (floats: TF32
+// pieces; 8-bit levels: the CUDA cores): staging the batch and looking for marked
+// individuals are two more launches, and a call takes 25 us with them however
+// small it is (784-100-10 and 50 samples: 152 nets 23 us, 1000 nets 79), 14
+// without.  The other kernel's time is modelled
 // from its waves, fitted to k = 32 .. 784, h = 10 .. 256, batches 20 .. 512:
 // TF32 pieces, one CTA per SM, per wave and 128 samples 2.5 + 0.085 h + (0.011 +
 // 0.00013 h) k us; CUDA cores, two per SM, per wave, 128 hidden units and 64
@@ -1040,7 +1041,7 @@ static bool pieces_pay(const NetLayout& net, int32_t pop, int32_t batch, int32_t
 {
     constexpr double kSms = 152.0, kPiecesUs = 25.0, kPairUs = 4.8;
     const double k = net.dims[0], h = net.dims[1], b = batch;
-    if (xp == 2 && net.dims[1] % 16 == 0) {
+    if (xp == 2) {
         const double wave = std::ceil(b / 128.0) * (2.5 + 0.085 * h + (0.011 + 0.00013 * h) * k);
         return std::ceil(pop / kSms) * wave >= kPiecesUs;
     }
@@ -1062,10 +1063,24 @@ bool eval_u8_tc_supported(const NetLayout& net, int32_t pop, int32_t batch, cons
     return in_tensor_shapes(net, batch) && pieces_fit(net, pop, batch, pop_dev, 1);
 }
 
+// Whether the pieces are at least as exact as the kernel they replace, by the
+// RMS error of the fitness against 64 bits (1200 initial nets each, k = 784, h = 17
+// .. 250).  The tensor core's accumulation truncates, 98 times for 784 8-bit
+// inputs and 147 times for floats.  8-bit levels against the CUDA cores: 1.05 to
+// 1.2 times at 8 to 24 samples, 0.96 to 1.05 at 32, 0.91 to 0.98 at 50, 0.92 to
+// 1.01 at 64, 0.75 to 0.93 from 100 on, where the loss sums in FP64 make up for
+// it.  Floats: 0.5 times the TF32 kernel's, but 1.2 to 1.4 times the CUDA cores',
+// so hidden widths off 16 stay there.
+static bool pieces_exact(const NetLayout& net, int32_t batch, int32_t xp)
+{
+    return xp == 2 ? net.dims[1] % 16 == 0 : batch >= 48;
+}
+
 bool eval_u8_wide_supported(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev, int32_t xp)
 {
     if (!pieces_fit(net, pop, batch, pop_dev, xp)) return false;
-    return (xp == 1 && in_tensor_shapes(net, batch)) || pieces_pay(net, pop, batch, xp);
+    if (xp == 1 && in_tensor_shapes(net, batch)) return true;
+    return pieces_exact(net, batch, xp) && pieces_pay(net, pop, batch, xp);
 }
 
 bool eval_u8_marks(const NetLayout& net, int32_t batch, int32_t xp) { return xp == 2 || !in_tensor_shapes(net, batch); }

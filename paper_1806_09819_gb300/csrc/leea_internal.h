@@ -265,14 +265,14 @@ cudaError_t launch_eval_shadow_runs(int32_t k, int32_t d_out, int32_t precision,
                                     int32_t n_runs, int32_t pop_max, bool any_tiles, const ShadowRun* runs_dev,
                                     const ShadowSeg* segs_dev, const int32_t* seg_off_dev, int32_t grid,
                                     unsigned int* status, cudaStream_t stream);
-// Evaluation of d_0-h-d_out nets (one hidden layer), SIMT FP32.  only (here and
-// below): if not NULL, just the individuals p with only[p] != 0.
+// Evaluation of d_0-h-d_out nets (one hidden layer), SIMT FP32.
 cudaError_t launch_eval_simt(const NetLayout& net, int32_t pop, const float* pop_dev,
                              const float* x, const int32_t* y, int32_t batch, float alpha,
                              const float* f_inh, float* f_raw, float* f_adj, int32_t* correct,
-                             cudaStream_t stream, const int32_t* only = nullptr);
+                             cudaStream_t stream);
 // Evaluation on the tcgen05 tensor cores (3xTF32), d_0-h-d_out with d_0 % 4 == 0,
-// h % 16 == 0, h <= 256, d_out <= 16 and 16-byte aligned population and x.
+// h % 16 == 0, h <= 256, d_out <= 16 and 16-byte aligned population and x.  only
+// (here and below): if not NULL, just the individuals p with only[p] != 0.
 bool eval_tc_supported(const NetLayout& net, int32_t batch, const float* pop_dev, const float* x);
 cudaError_t launch_eval_tc(const NetLayout& net, int32_t pop, const float* pop_dev, const float* x,
                            const int32_t* y, int32_t batch, float alpha, const float* f_inh, float* f_raw,

@@ -1,6 +1,6 @@
 """Evaluation of float inputs through FP16 pieces: edges of tiles, units and K stages, samples of very different
 magnitudes, and the individuals and samples that the pieces cannot carry.  Against the FP64 oracle with the fitness
-tolerance; for infinite and NaN inputs against the CUDA-core path."""
+tolerance; for infinite and NaN inputs against the TF32 path."""
 import numpy as np
 import pytest
 
@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 CASES = [  # dims, pop, batch
     ([784, 112, 10], 155, 100), ([784, 100, 10], 333, 50), ([784, 1, 10], 5, 3), ([4, 17, 2], 3, 1),
     ([20, 129, 16], 7, 130), ([784, 256, 16], 4, 256), ([784, 112, 10], 1, 1000), ([52, 112, 10], 305, 128),
-    ([36, 127, 5], 307, 257), ([68, 16, 10], 400, 127), ([784, 33, 10], 3, 1025), ([100, 128, 10], 153, 129),
+    ([36, 127, 5], 307, 257), ([68, 16, 10], 2400, 127), ([784, 33, 10], 3, 1025), ([100, 128, 10], 153, 129),
+    ([20, 128, 16], 700, 130), ([36, 112, 5], 400, 257), ([784, 32, 10], 300, 1025), ([784, 16, 10], 170, 3),
 ]
 
 
@@ -59,14 +60,14 @@ def test_float_pieces_match_oracle(gpu, oracle_mod, dims, pop, batch):
         assert f[0] == f[2]
 
 
-@pytest.mark.parametrize("dims", [[784, 100, 10], [36, 17, 5]])
-def test_float_pieces_non_finite_inputs(gpu, dims):
-    """Off the TF32 path's hidden widths: bit for bit what the CUDA cores give."""
+@pytest.mark.parametrize("dims,pop", [([784, 112, 10], 40), ([36, 64, 5], 400)])
+def test_float_pieces_non_finite_inputs(gpu, dims, pop):
+    """Bit for bit what the TF32 kernel gives."""
     rng = np.random.default_rng(3)
-    popd = to_device_pop(_population(gpu, dims, 40, rng), gpu.leea_padded_params(dims))
+    popd = to_device_pop(_population(gpu, dims, pop, rng), gpu.leea_padded_params(dims))
     y = rng.integers(0, dims[2], size=70).astype(np.int32)
     for v in (np.inf, -np.inf, np.nan):
         x = rng.random((70, dims[0])).astype(np.float32)
         x[33, 5] = v
-        for a, b in zip(_run(gpu, dims, popd, x, y, 0), _run(gpu, dims, popd, x, y, gpu.EVAL_SIMT)):
+        for a, b in zip(_run(gpu, dims, popd, x, y, 0), _run(gpu, dims, popd, x, y, gpu.EVAL_TENSOR)):
             np.testing.assert_array_equal(a, b)

@@ -12,6 +12,7 @@ CASES = [  # dims, pop, batch
     ([784, 100, 10], 333, 50), ([784, 1, 10], 5, 3), ([4, 17, 2], 3, 1), ([20, 129, 16], 7, 130), ([784, 255, 3], 3, 7),
     ([784, 256, 16], 2, 256), ([784, 112, 10], 1, 1000), ([784, 112, 10], 155, 384), ([52, 112, 10], 153, 129),
     ([36, 127, 5], 307, 257), ([68, 16, 10], 400, 512), ([784, 33, 10], 2, 1025),
+    ([784, 100, 10], 333, 47), ([784, 100, 10], 333, 48),
 ]
 
 
