@@ -9,7 +9,7 @@
 //               exact in FP32): 2 MMAs per 16 inputs, only the accumulation rounds
 //   layers 2-4  A = 2^8 h of the layer below and B = 2^8 W, both as two FP16
 //               pieces: hi.hi + lo.hi + hi.lo; the dropped lo.lo term is below
-//               2^-21 of the product
+//               2^-21 of the product (their order: kFewSamples)
 // The epilogue adds the bias and applies ReLU in FP32 and splits the activations
 // for the next layer; the softmax cross-entropy is FP32, losses are summed in
 // FP64.  A weight or an activation with |v| >= 128 (2^8 |v| could overflow its
@@ -75,6 +75,13 @@ constexpr int kTile = 128;                      // samples per unit (MMA M)
 constexpr uint32_t kBlockBytes = kTile * 128;   // one 64-input block of a 128-row operand
 constexpr uint32_t kSlotBytes = 256 * 128;      // a weight slot: 256 rows of 64 FP16 values
 constexpr int kMaxSlots = 8;
+// Up to here (FEW) the small products of a layer come first.  RMS error of the fitness
+// against 64 bits, 600 initial nets 196-256-128-64-10, in order of K / small
+// products first / with layer 4 in FFMA on the CUDA cores and the small products
+// in accumulators of their own: 8 samples 6.9e-8 / 5.3e-8 / 5.3e-8, 16 4.8 / 4.1 /
+// 4.9, 32 4.4 / 3.8 / 4.8, 128 4.0 / 3.5 / 4.7, 1024 3.7 / 3.3 / 5.2.
+// On so few samples that costs 2000 nets 370 us (368), 152 nets 53 (51).
+constexpr int kFewSamples = 32;
 constexpr int kMaxOutTc = 16;
 constexpr uint32_t kTmemCols = 512;
 constexpr float kPieceScale = 256.0f;
@@ -388,6 +395,7 @@ __device__ __forceinline__ void store_fitness(const MlpTcArgs& a, int p, double 
     if (a.correct) a.correct[p] = good;
 }
 
+template <bool FEW>
 __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid_constant__ MlpTcArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -476,6 +484,47 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                 const bool stacked = a.m.stacked[l];
                 if (l >= 2 && !wait(&s.h_ready[l - 2], u & 1u)) return;
                 ptx::tc_fence_after();
+                // The tensor core truncates every sum, to the size of what the accumulator
+                // holds by then.  With few samples, whose errors the fitness averages
+                // least, the small products lo.hi and hi.lo therefore come before hi.hi:
+                // per slot, and in layers 3 and 4, whose A operand is complete, over all
+                // slots, which the ring then holds at once (for the paper net on 1024
+                // samples 7 % of the time, and 2 % just by the longer code).
+                if (FEW && stacked) {
+                    const bool all = l >= 2 && a.m.slots[l] <= a.n_slots;
+                    const int slots = a.m.slots[l], group = all ? slots : 1;
+                    for (int j0 = 0; j0 < slots; j0 += group) {
+                        if (l == 1 && !wait(&s.h_blk[j0], u & 1u)) return;
+                        uint32_t at = slot, ph = phase;
+                        for (int j = j0; j < j0 + group; ++j) {
+                            if (!wait(&s.full[at], ph)) return;
+                            if (l == 1) ptx::tc_fence_after();
+                            const uint32_t b = ptx::desc_lo(ring + at * kSlotBytes);
+                            const uint32_t a_hi = act + 64u * static_cast<uint32_t>(j);
+                            const int steps = min(4, (a.m.k16[l] - 64 * j) / 16);
+#pragma unroll
+                            for (int kk = 0; kk < 4; ++kk) {
+                                if (kk >= steps) break;
+                                ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk + 8u, b + 2u * kk, hi, idesc, j + kk == 0 ? 0u : 1u, lead);
+                                ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk, b + 8u * n + 2u * kk, hi, idesc, 1u, lead);
+                            }
+                            if (++at == static_cast<uint32_t>(a.n_slots)) { at = 0; ph ^= 1u; }
+                        }
+                        for (int j = j0; j < j0 + group; ++j) {
+                            const uint32_t b = ptx::desc_lo(ring + slot * kSlotBytes);
+                            const uint32_t a_hi = act + 64u * static_cast<uint32_t>(j);
+                            const int steps = min(4, (a.m.k16[l] - 64 * j) / 16);
+#pragma unroll
+                            for (int kk = 0; kk < 4; ++kk) {
+                                if (kk >= steps) break;
+                                ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk, b + 2u * kk, hi, idesc, 1u, lead);
+                            }
+                            next_slot();
+                        }
+                    }
+                    if (lead) ptx::mma_commit(&s.d_full[l]);
+                    return;
+                }
                 for (int j = 0; j < a.m.slots[l]; ++j) {
                     const int kb = stacked ? j : j >> 1, lo = stacked ? 0 : j & 1;
                     if (l == 1 && lo == 0 && !wait(&s.h_blk[kb], u & 1u)) return;
@@ -975,9 +1024,10 @@ cudaError_t launch_eval_mlp_tc(const NetLayout& net, int32_t pop, const float* p
     }
     a.n_slots = mlp_ring(net.dims, a.x_bytes);
     const size_t smem = tc_smem_bytes(net.dims, a.x_bytes, a.n_slots);
-    err = cudaFuncSetAttribute(eval_mlp_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const auto kernel = batch <= kFewSamples ? eval_mlp_tc_kernel<true> : eval_mlp_tc_kernel<false>;
+    err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (err != cudaSuccess) return err;
-    eval_mlp_tc_kernel<<<sc.grid, kTcThreads, smem, stream>>>(a);
+    kernel<<<sc.grid, kTcThreads, smem, stream>>>(a);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     if (a.extra != 0 || a.per_cta % a.n_tiles != 0) {
         combine_mlp_parts_kernel<<<(pop + 255) / 256, 256, 0, stream>>>(a);

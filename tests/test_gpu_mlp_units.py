@@ -1,6 +1,6 @@
 """The tensor-core evaluation of nets with three hidden layers at the edges of its plan: individuals shared by several
-CTAs, last input blocks of 16, 32 and 48 inputs, widths on both sides of the stacked weight slots, and nets whose layers
-share accumulator columns.  Against the FP64 oracle with the fitness tolerance."""
+CTAs, last input blocks of 16, 32 and 48 inputs, widths on both sides of the stacked weight slots, nets whose layers share
+accumulator columns, and both orders of the products.  Against the FP64 oracle with the fitness tolerance."""
 import numpy as np
 import pytest
 
@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 CASES = [  # dims, pop, batch
     ([196, 256, 128, 64, 10], 160, 300), ([196, 256, 128, 64, 10], 3, 1024), ([256, 256, 256, 256, 16], 5, 260),
     ([48, 16, 16, 16, 2], 200, 129), ([80, 128, 144, 48, 7], 33, 400), ([32, 240, 256, 16, 3], 20, 200),
-    ([64, 64, 64, 64, 10], 1, 2000), ([200, 256, 192, 32, 10], 155, 128), ([4, 16, 256, 240, 5], 7, 1),
+    ([196, 256, 128, 64, 10], 160, 32), ([196, 256, 128, 64, 10], 160, 33), ([64, 256, 256, 112, 10], 33, 17),
+    ([36, 80, 128, 128, 16], 310, 8), ([64, 64, 64, 64, 10], 1, 2000), ([200, 256, 192, 32, 10], 155, 128), ([4, 16, 256, 240, 5], 7, 1),
 ]
 
 
