@@ -114,7 +114,7 @@ TRAFFIC = {
     "breed_evaluate": {"bytes_per_launch": 738.19e6, "src_sha": "23e25d83744d9797", "capture": "P=1000 plain workload"},
     # eval_mlp_tc_kernel alone (each individual's weight pieces read once from
     # DRAM, the other tiles from L2); the stage also splits the weights
-    "evaluate_paper_net": {"bytes_per_launch": 1059.44e6, "src_sha": "2e037631158b3b9a",
+    "evaluate_paper_net": {"bytes_per_launch": 1059.44e6, "src_sha": "98b4baf63d0ccc97",
                            "capture": "paper-net workload, eval_mlp_tc_kernel"},
 }
 

@@ -18,6 +18,7 @@
 #include <algorithm>
 
 #include "leea_internal.h"
+#include "tc_ptx.cuh"
 
 namespace leea {
 
@@ -160,14 +161,15 @@ eval_mlp_kernel(const MlpArgs e, const float* __restrict__ popv, const XT* __res
     // One CTA per individual; for the marked ones only, a few CTAs share them all
     // and most find no mark among theirs (2000 nets: 10 us with a CTA each).
     if (only) {
+        ptx::grid_dep_wait();
         int any = 0;
         for (int64_t p = blockIdx.x + static_cast<int64_t>(tid) * gridDim.x; p < e.pop;
              p += static_cast<int64_t>(kMlpThreads) * gridDim.x)
-            any |= only[p];
+            any |= __ldcg(only + p);
         if (!__syncthreads_or(any)) return;
     }
     for (int p = blockIdx.x; p < e.pop; p += gridDim.x) {
-    if (only && only[p] == 0) continue;
+    if (only && __ldcg(only + p) == 0) continue;
     const float* net = popv + static_cast<int64_t>(p) * e.c_pad;
     const int d0 = e.dims[0], d_out = e.dims[e.n_layers];
     float total = 0.0f;
@@ -286,8 +288,11 @@ cudaError_t launch_mlp(const NetLayout& net, int32_t pop, const float* pop_dev, 
     if (err != cudaSuccess) return err;
     MlpArgs e = mlp_args(net, batch, alpha, x_div);
     e.pop = pop;
-    eval_mlp_kernel<XT><<<only ? std::min(pop, kOnlyCtas) : pop, kMlpThreads, kMlpSmemBytes, stream>>>(e, pop_dev, x, y,
-                                                                    f_inh, f_raw, f_adj, correct, only);
+    if (only)
+        return launch_pdl(eval_mlp_kernel<XT>, dim3(static_cast<unsigned>(std::min(pop, kOnlyCtas))), dim3(kMlpThreads),
+                          kMlpSmemBytes, stream, e, pop_dev, x, y, f_inh, f_raw, f_adj, correct, only);
+    eval_mlp_kernel<XT><<<pop, kMlpThreads, kMlpSmemBytes, stream>>>(e, pop_dev, x, y, f_inh, f_raw, f_adj, correct,
+                                                                    nullptr);
     return cudaGetLastError();
 }
 

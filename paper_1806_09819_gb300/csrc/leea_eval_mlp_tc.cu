@@ -30,7 +30,10 @@
 // Measured, 2000 nets 196-256-128-64-10 on 1024 samples: 945 us (1518 with the
 // activations in shared memory and two weight buffers), 207 of them the splitting
 // (1.5 GB, at the memory's rate); 512 samples 607, 128 375; 16 nets on 1024
-// samples 42.  What bounds it: a unit takes 13k cycles, its MMAs 7.3k at the
+// samples 42.  The staging, this kernel and the one for the marked individuals are
+// each launched before their predecessor has ended and wait for it on the device:
+// 152 nets on 30 samples 42 us (51 without, 49 before), 2000 on 8 364 (368).
+// What bounds it: a unit takes 13k cycles, its MMAs 7.3k at the
 // tensor peak (weights 448 KB of L2 reads, 3.4k-6k cycles, are hidden).  The rest
 // is the chain of a unit: layer 1's accumulator to the first activations 1-2k,
 // the restart of the MMAs after layer 2 0.5k, and the issuing warp's waits
@@ -80,8 +83,9 @@ constexpr int kMaxSlots = 8;
 // products first / with layer 4 in FFMA on the CUDA cores and the small products
 // in accumulators of their own: 8 samples 6.9e-8 / 5.3e-8 / 5.3e-8, 16 4.8 / 4.1 /
 // 4.9, 32 4.4 / 3.8 / 4.8, 128 4.0 / 3.5 / 4.7, 1024 3.7 / 3.3 / 5.2.
-// On so few samples that costs 2000 nets 370 us (368), 152 nets 53 (51).
-constexpr int kFewSamples = 32;
+// On so few samples that costs 152 nets 44.5 us (42.4), 2000 nets 0.5 %.  The line
+// lies below 16, from where on the order of K is no worse than the third.
+constexpr int kFewSamples = 15;
 constexpr int kMaxOutTc = 16;
 constexpr uint32_t kTmemCols = 512;
 constexpr float kPieceScale = 256.0f;
@@ -426,6 +430,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem_base = *s.tmem_holder;
+    ptx::grid_dep_wait();  // the pieces and the levels are in
     // Layer 3 of a unit comes after the first `cut` slots of the next unit's layer 1:
     // by then its activations are in.
     const int cut = a.m.slots[0] / 2;
@@ -869,6 +874,7 @@ __global__ void __launch_bounds__(256) stage_levels_kernel(const MlpTcArgs a, co
         *reinterpret_cast<uint4*>(out + static_cast<int64_t>(t) * a.x_bytes + kb * kBlockBytes + swz(r, ch)) =
             make_uint4(h[0], h[1], h[2], h[3]);
     }
+    ptx::grid_dep_wait();  // the evaluation waits for this grid, so for the split as well
 }
 
 // Library-owned scratch (weight pieces, marks), grown on demand, for callers
@@ -1019,16 +1025,16 @@ cudaError_t launch_eval_mlp_tc(const NetLayout& net, int32_t pop, const float* p
         split_weights_kernel<<<dim3(blocks, pop < 65535 ? pop : 65535), 256, 0, stream>>>(a);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         const int level_items = a.n_tiles * ((a.dims[0] + 63) / 64) * kTile * 8;
-        stage_levels_kernel<<<(level_items + 255) / 256, 256, 0, stream>>>(a, x);
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
+        err = launch_pdl(stage_levels_kernel, dim3((level_items + 255) / 256), dim3(256), 0, stream, a, x);
+        if (err != cudaSuccess) return err;
     }
     a.n_slots = mlp_ring(net.dims, a.x_bytes);
     const size_t smem = tc_smem_bytes(net.dims, a.x_bytes, a.n_slots);
     const auto kernel = batch <= kFewSamples ? eval_mlp_tc_kernel<true> : eval_mlp_tc_kernel<false>;
     err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (err != cudaSuccess) return err;
-    kernel<<<sc.grid, kTcThreads, smem, stream>>>(a);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    err = launch_pdl(kernel, dim3(sc.grid), dim3(kTcThreads), smem, stream, a);
+    if (err != cudaSuccess) return err;
     if (a.extra != 0 || a.per_cta % a.n_tiles != 0) {
         combine_mlp_parts_kernel<<<(pop + 255) / 256, 256, 0, stream>>>(a);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
