@@ -709,7 +709,8 @@ leea_status leea_breed_entities(int32_t n_parents, const int32_t* dims, int32_t 
  * p->precision 0: the logits of the FP32 child (CUDA cores); >= 1: of the
  * child with W1 rounded to BF16 (nearest even) as the precision form holds
  * it, on the tensor cores, the probe inputs carried as two BF16 pieces
- * (needs h <= 128; probe_dev 4-byte aligned). */
+ * (needs h <= 128, and with 10 outputs d_0 <= 1024 for h = 16, 832 for h = 128:
+ * probe pieces and parameters live in shared memory; probe_dev 4-byte aligned). */
 leea_status leea_descriptors(int32_t n_parents, const int32_t* dims, int32_t n_dims, const leea_params* p,
                              uint64_t seed, uint32_t gen, const float* parents_dev, const float* f_adj_dev,
                              const int32_t* par1_dev, const int32_t* par2_dev, const int32_t* kind_dev,

@@ -41,6 +41,8 @@
 // and took 1,920 us: too few warps to hide the parents' loads.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "breed_ops.cuh"
 #include "leea_internal.h"
 #include "philox.cuh"
@@ -101,6 +103,19 @@ __host__ __device__ inline size_t tc_smem_bytes(int32_t k, int32_t h, int32_t d_
            2 * kProducerWarps * (sizeof(uint32_t) + sizeof(float)) + 8 * (2 * kMaxStages + 8 + 2) + 64;
 }
 
+// The shapes the call takes: probe pieces, both tail buffers and the activations
+// within kShapeBytes (with 10 outputs 1024 inputs for 16 hidden units, 832 for 128).
+// A limit of its own, so that the call's shapes do not move with the layout of the
+// rest.
+constexpr size_t kShapeBytes = 137008;
+
+inline bool tc_shape_fits(int32_t k, int32_t h, int32_t d_out)
+{
+    const size_t tail = static_cast<size_t>(h + d_out * h + d_out + 3) / 4 * 4;
+    return static_cast<size_t>(tc_n_kb(k)) * kXBlockBytes + sizeof(float) * (2 * tail + kMaxProbeTc * (h + 1)) <=
+           kShapeBytes;
+}
+
 // The deepest ring that fits in 227 KB; 0 if not even two stages do.  The
 // 128-row operand that an MMA reads from the last stage ends inside the probe
 // pieces and the task buffers behind the ring.
@@ -109,6 +124,30 @@ inline int32_t tc_stages(int32_t k, int32_t h, int32_t d_out)
     for (int32_t ns = kMaxStages; ns >= 2; --ns)
         if (tc_smem_bytes(k, h, d_out, ns) <= 227u * 1024u) return ns;
     return 0;
+}
+
+// Whether the ring is deep enough for its waits.  A producer warp waits for a stage
+// only where it has a task, by parity, which tells a stage's uses apart only in
+// turn: for use G of the ring the use before the previous one of that stage, G - 2
+// n_stages, must be known to be over.  It is, if the warp has waited for use G -
+// n_stages or a later one, so no two of its tasks in a row may be further apart
+// than the ring; or if it belongs to a recipe that the warp's last wait for a
+// tail buffer has seen finished (three before the current one).  (A wait on the
+// way, where the warp has no task, would not do: the stage can move on by two uses
+// before it looks.)
+inline bool tc_ring_holds(int32_t k, int32_t h, int32_t d_out, int32_t n_stages)
+{
+    const int32_t n_kb = tc_n_kb(k), whole = h / 4, last = h * ((k - (n_kb - 1) * kKB) / 8) / 32;
+    if (2 * n_stages >= 3 * n_kb) return true;
+    const int32_t n_w1 = (n_kb - 1) * whole + last;
+    const int32_t n = n_w1 + ((h + d_out * h + d_out + 7) / 8 + 31) / 32;  // tasks of a recipe, its tail's last
+    auto block = [&](int32_t t) { return t / n * n_kb + std::min(t % n / whole, n_kb - 1); };
+    for (int32_t t = 0; t < n_w1; ++t) {
+        int32_t next = t + kProducerWarps;
+        while (next % n >= n_w1) next += kProducerWarps;
+        if (block(next) - block(t) > n_stages) return false;
+    }
+    return true;
 }
 
 __device__ __forceinline__ TcSmem carve(uint8_t* raw, const ProbeArgs& a, int32_t n_stages)
@@ -565,8 +604,11 @@ probe_tc_kernel(const __grid_constant__ ProbeArgs a, const __grid_constant__ Phi
 
 bool probe_tc_supported(int32_t k, int32_t h, int32_t d_out, int32_t n_probe)
 {
-    return k % 16 == 0 && h % 16 == 0 && h >= 16 && h <= kMaxHiddenTc && d_out >= 1 && d_out <= 16 &&
-           n_probe >= 1 && n_probe <= kMaxProbeTc && tc_stages(k, h, d_out) > 0;
+    if (k % 16 != 0 || h % 16 != 0 || h < 16 || h > kMaxHiddenTc || d_out < 1 || d_out > 16 || n_probe < 1 ||
+        n_probe > kMaxProbeTc || !tc_shape_fits(k, h, d_out))
+        return false;
+    const int32_t n_stages = tc_stages(k, h, d_out);
+    return n_stages > 0 && tc_ring_holds(k, h, d_out, n_stages);
 }
 
 cudaError_t launch_descriptors_tc(const ProbeArgs& a, int32_t n_recipes, cudaStream_t stream)
