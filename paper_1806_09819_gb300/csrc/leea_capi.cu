@@ -248,7 +248,8 @@ leea_status check_device_status(cudaStream_t stream, uint32_t* flags_out)
 // Runs the evaluation kernel that `path` selects (LEEA_EVAL_*).
 leea_status dispatch_eval(const NetLayout& net, int32_t pop, const float* pop_dev, const float* x,
                           const int32_t* y, int32_t batch, float alpha, const float* f_inh, float* f_raw,
-                          float* f_adj, int32_t* correct, int32_t path, cudaStream_t stream, void* scratch = nullptr)
+                          float* f_adj, int32_t* correct, int32_t path, cudaStream_t stream, void* scratch = nullptr,
+                          bool x_ready = false)
 {
     if (net.n_layers > 2) {  // several hidden layers: CUDA-core FP32
         if (path == LEEA_EVAL_TENSOR) return fail(LEEA_EINVAL, "nets with several hidden layers evaluate on CUDA cores");
@@ -282,7 +283,7 @@ leea_status dispatch_eval(const NetLayout& net, int32_t pop, const float* pop_de
         }
     }
     if (pieces) {
-        err = launch_stage_xf(net, pop, x, batch, scratch, stream);
+        err = launch_stage_xf(net, pop, x, batch, scratch, x_ready && !own, stream);
         if (err == cudaSuccess)
             err = launch_eval_u8_tc(net, pop, pop_dev, 2, nullptr, scratch, 1.0f, y, batch, alpha, f_inh, f_raw, f_adj,
                                     correct, status, stream);
@@ -350,7 +351,7 @@ leea_status dispatch_eval_u8(const NetLayout& net, int32_t pop, const float* pop
         x16_staged = false;
     }
     if (tc_ok && path != LEEA_EVAL_SIMT) {
-        err = x16_staged ? cudaSuccess : launch_stage_x16(net, pop, x, batch, x16, stream);
+        err = x16_staged ? cudaSuccess : launch_stage_x16(net, pop, x, batch, x16, false, stream);
         if (err == cudaSuccess)
             err = launch_eval_u8_tc(net, pop, pop_dev, 1, x, x16, x_div, y, batch, alpha, f_inh, f_raw, f_adj, correct,
                                     status, stream);
@@ -421,7 +422,7 @@ leea_status dispatch_eval_shadow(const NetLayout& net, int32_t pop, const float*
         void* xop = nullptr;
         cudaError_t err = scratch_alloc(&xop, eval_shadow_pair_xop_bytes(net, precision, batch), stream);
         if (err == cudaSuccess) {
-            err = launch_stage_xop(net, precision, x, batch, xop, stream);
+            err = launch_stage_xop(net, precision, x, batch, xop, false, stream);
             if (err == cudaSuccess)
                 err = launch_eval_shadow_pair(net, pop, pop_dev, precision, shadow, shadow_stride_of(net, precision),
                                               scale_exp, xop, x_div, y, batch, alpha, f_inh, f_raw, f_adj, correct,
@@ -1311,10 +1312,11 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
             LEEA_CUDA_TRY(launch_rank_select(a, s->f_adj, s->order, s->par1, s->par2, s->kind, s->f_inh, s->stream),
                           "rank/select kernel");
             if (stage_early)  // runs beside the selection; the breed that follows waits for both
-                LEEA_CUDA_TRY(launch_stage_x16(s->net, s->pop, static_cast<const uint8_t*>(x_dev), batch, s->x16, s->stream),
+                LEEA_CUDA_TRY(launch_stage_x16(s->net, s->pop, static_cast<const uint8_t*>(x_dev), batch, s->x16, true,
+                                               s->stream),
                               "batch staging kernel");
             if ((shadow_pair || shadow_group) && !fused)
-                LEEA_CUDA_TRY(launch_stage_xop(s->net, prec, static_cast<const uint8_t*>(x_dev), batch, s->xop,
+                LEEA_CUDA_TRY(launch_stage_xop(s->net, prec, static_cast<const uint8_t*>(x_dev), batch, s->xop, true,
                                                s->stream),
                               "batch staging kernel");
             sc.done();
@@ -1368,7 +1370,7 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
             unsigned int* status = device_status_ptr();
             if (!status) return fail(LEEA_ECUDA, "device status word unavailable");
             if (first)
-                LEEA_CUDA_TRY(launch_stage_xop(s->net, prec, static_cast<const uint8_t*>(x_dev), batch, s->xop,
+                LEEA_CUDA_TRY(launch_stage_xop(s->net, prec, static_cast<const uint8_t*>(x_dev), batch, s->xop, false,
                                                s->stream),
                               "batch staging kernel");
             LEEA_CUDA_TRY(launch_eval_shadow_pair(s->net, s->pop, s->popbuf[s->cur], prec, s->shadow[s->cur],
@@ -1380,7 +1382,7 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
             unsigned int* status = device_status_ptr();
             if (!status) return fail(LEEA_ECUDA, "device status word unavailable");
             if (first)
-                LEEA_CUDA_TRY(launch_stage_xop(s->net, prec, static_cast<const uint8_t*>(x_dev), batch, s->xop,
+                LEEA_CUDA_TRY(launch_stage_xop(s->net, prec, static_cast<const uint8_t*>(x_dev), batch, s->xop, false,
                                                s->stream),
                               "batch staging kernel");
             LEEA_CUDA_TRY(launch_eval_shadow_group_run(s->net, s->pop, s->popbuf[s->cur], prec, s->shadow[s->cur],
@@ -1401,7 +1403,7 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
         else
             st = dispatch_eval(s->net, s->pop, s->popbuf[s->cur], static_cast<const float*>(x_dev), y_dev, batch,
                                s->prm.alpha, first ? nullptr : s->f_inh, s->f_raw, s->f_adj, s->correct,
-                               s->prm.eval_path, s->stream, eval_f_tc ? s->x16 : nullptr);
+                               s->prm.eval_path, s->stream, eval_f_tc ? s->x16 : nullptr, !first);
         sc.done();
         if (st) return st;
     }

@@ -582,13 +582,17 @@ __global__ void combine_pair_tiles_kernel(const PairArgs a)
 // zero past the batch) at 128 r, its 16-byte chunk c at chunk position
 // c ^ (r & 7).  BF16: 64 levels per row of a block; FP8: 128 levels, piece 0
 // holding 16 floor(k / 16), piece 1 k mod 16, both exact in e4m3.  One thread
-// per 16-byte chunk.  It reads only the caller's levels, so it lets the next
-// kernel start at once; it waits for its own predecessor before it ends.
+// per 16-byte chunk.  It lets the next kernel start at once, and waits for its own
+// predecessor before it ends; x_ready: the levels are complete and xop is free
+// before this kernel can start (a generation, behind its ranking), otherwise it
+// waits before it reads them.
 template <int PREC>
 __global__ void __launch_bounds__(256) stage_xop_kernel(const uint8_t* __restrict__ x, int32_t batch, int32_t k,
-                                                        int32_t m_tiles, int32_t k_blocks, uint8_t* __restrict__ xop)
+                                                        int32_t m_tiles, int32_t k_blocks, uint8_t* __restrict__ xop,
+                                                        bool x_ready)
 {
     ptx::grid_dep_launch();
+    if (!x_ready) ptx::grid_dep_wait();
     constexpr int kPieces = PREC == 1 ? 1 : 2;
     const int64_t chunks = static_cast<int64_t>(m_tiles) * k_blocks * kPieces * 128 * 8;
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -654,7 +658,7 @@ size_t eval_shadow_pair_xop_bytes(const NetLayout& net, int32_t precision, int32
 }
 
 cudaError_t launch_stage_xop(const NetLayout& net, int32_t precision, const uint8_t* x, int32_t batch, void* xop,
-                             cudaStream_t stream)
+                             bool x_ready, cudaStream_t stream)
 {
     const int32_t m_tiles = (batch + 127) / 128;
     const int32_t k_blocks = (net.dims[0] + (precision == 1 ? 63 : 127)) / (precision == 1 ? 64 : 128);
@@ -669,8 +673,8 @@ cudaError_t launch_stage_xop(const NetLayout& net, int32_t precision, const uint
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     uint8_t* dst = static_cast<uint8_t*>(xop);
-    return precision == 1 ? cudaLaunchKernelEx(&cfg, stage_xop_kernel<1>, x, batch, net.dims[0], m_tiles, k_blocks, dst)
-                          : cudaLaunchKernelEx(&cfg, stage_xop_kernel<2>, x, batch, net.dims[0], m_tiles, k_blocks, dst);
+    const auto kernel = precision == 1 ? stage_xop_kernel<1> : stage_xop_kernel<2>;
+    return cudaLaunchKernelEx(&cfg, kernel, x, batch, net.dims[0], m_tiles, k_blocks, dst, x_ready);
 }
 
 cudaError_t launch_eval_shadow_pair(const NetLayout& net, int32_t pop, const float* pop_dev, int32_t precision,

@@ -864,16 +864,20 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
 }
 
 // The batch's levels as FP16 (exact), row-major [batch][kp], kp = round_up(k,
-// 8) with zero padding: the A operand tiles of eval_u8_kernel.  It reads only
-// the caller's levels, so it lets the next kernel start at once; before it
+// 8) with zero padding: the A operand tiles of eval_u8_kernel.  x_ready: the
+// levels are complete and the buffer is free before this kernel can start (a
+// generation, behind its ranking); otherwise the kernel on the stream before it
+// may still be writing them, whoever launched that, and it waits.  It lets the
+// next kernel start at once; before it
 // ends it waits for its own predecessor, so that a successor that waits for it
 // also sees everything earlier on the stream complete.  Then it clears the
 // marks, which an earlier evaluation may have been reading until now.
 __global__ void __launch_bounds__(256) stage_x16_kernel(const uint8_t* __restrict__ x, int32_t batch, int32_t k,
                                                         int32_t kp, __half* __restrict__ x16,
-                                                        int32_t* __restrict__ flagged, int32_t pop)
+                                                        int32_t* __restrict__ flagged, int32_t pop, bool x_ready)
 {
     ptx::grid_dep_launch();
+    if (!x_ready) ptx::grid_dep_wait();
     const int32_t per_row = kp >> 3;
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i < static_cast<int64_t>(batch) * per_row) {
@@ -899,13 +903,14 @@ __global__ void __launch_bounds__(256) stage_x16_kernel(const uint8_t* __restric
 // and absolute errors of 2^-39 of it below.  x_scale[b] = 2^-(e + 8) turns the
 // accumulator's units (2^e x times 2^8 w) into x w; NaN for a sample with an
 // infinite or NaN input, whose individuals are all evaluated again by a kernel
-// that multiplies x itself.  A CTA per sample.
+// that multiplies x itself.  A CTA per sample.  x_ready as in stage_x16_kernel.
 __global__ void __launch_bounds__(256) stage_xf_kernel(const float* __restrict__ x, int32_t batch, int32_t k, int32_t kp,
                                                        __half* __restrict__ x16, float* __restrict__ x_scale,
-                                                       int32_t* __restrict__ flagged, int32_t pop)
+                                                       int32_t* __restrict__ flagged, int32_t pop, bool x_ready)
 {
     __shared__ uint32_t top[8];
     ptx::grid_dep_launch();
+    if (!x_ready) ptx::grid_dep_wait();
     const int32_t b = blockIdx.x;
     const float4* src = reinterpret_cast<const float4*>(x + static_cast<int64_t>(b) * k);  // k % 4 == 0
     uint32_t mx = 0;
@@ -1120,23 +1125,23 @@ int32_t* eval_u8_flagged(const NetLayout& net, int32_t pop, int32_t batch, int32
 }
 
 cudaError_t launch_stage_x16(const NetLayout& net, int32_t pop, const uint8_t* x, int32_t batch, void* scratch,
-                             cudaStream_t stream)
+                             bool x_ready, cudaStream_t stream)
 {
     const int32_t k = net.dims[0], kp = (k + 7) / 8 * 8;
     const int64_t items = static_cast<int64_t>(batch) * (kp / 8);
     if (items <= 0) return cudaSuccess;
     return launch_pdl(stage_x16_kernel, dim3(static_cast<unsigned>((items + 255) / 256)), dim3(256), 0, stream, x, batch,
-                      k, kp, static_cast<__half*>(scratch), eval_u8_flagged(net, pop, batch, 1, scratch), pop);
+                      k, kp, static_cast<__half*>(scratch), eval_u8_flagged(net, pop, batch, 1, scratch), pop, x_ready);
 }
 
 cudaError_t launch_stage_xf(const NetLayout& net, int32_t pop, const float* x, int32_t batch, void* scratch,
-                            cudaStream_t stream)
+                            bool x_ready, cudaStream_t stream)
 {
     const U8Scratch u = u8_scratch(net, pop, batch, 2);
     return launch_pdl(stage_xf_kernel, dim3(static_cast<unsigned>(batch)), dim3(256), 0, stream, x, batch, net.dims[0],
                       (net.dims[0] + 7) / 8 * 8, static_cast<__half*>(scratch),
                       reinterpret_cast<float*>(static_cast<uint8_t*>(scratch) + u.scale),
-                      eval_u8_flagged(net, pop, batch, 2, scratch), pop);
+                      eval_u8_flagged(net, pop, batch, 2, scratch), pop, x_ready);
 }
 
 cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* pop_dev, int32_t xp, const uint8_t* x,

@@ -198,11 +198,11 @@ bool eval_shadow_supported(const NetLayout& net, int32_t precision, int32_t batc
 // d_0 % 16 == 0, d_out <= 16): the batch staged by launch_stage_xop into
 // xop (eval_shadow_pair_xop_bytes, 16-byte aligned) earlier on the stream;
 // scratch as eval_shadow_scratch_bytes when the batch spans several
-// 128-sample tiles.
+// 128-sample tiles.  x_ready: see launch_stage_x16.
 bool eval_shadow_pair_supported(const NetLayout& net, int32_t precision, int32_t batch);
 size_t eval_shadow_pair_xop_bytes(const NetLayout& net, int32_t precision, int32_t batch);
 cudaError_t launch_stage_xop(const NetLayout& net, int32_t precision, const uint8_t* x, int32_t batch, void* xop,
-                             cudaStream_t stream);
+                             bool x_ready, cudaStream_t stream);
 cudaError_t launch_eval_shadow_pair(const NetLayout& net, int32_t pop, const float* pop_dev, int32_t precision,
                                     const uint8_t* shadow, int64_t sh_stride, const int32_t* scale_exp,
                                     const void* xop, float x_div, const int32_t* y, int32_t batch, float alpha,
@@ -291,7 +291,9 @@ cudaError_t launch_eval_simt_u8(const NetLayout& net, int32_t pop, const float* 
 // h <= 128 (eval_u8_tc_supported).  It reads the batch from scratch
 // (eval_u8_scratch_bytes, 256-byte aligned), which launch_stage_x16 or _xf fills
 // earlier on the same stream; the staging kernels let their successor start at
-// once and wait for their own predecessor before they end.  Where
+// once and wait for their own predecessor before they end, and before they read
+// the batch unless x_ready says that a kernel which the library has launched
+// since the caller's last starts only once the batch is complete.  Where
 // eval_u8_flagged is not NULL, individuals with a weight |w| >= 128 are marked
 // there and their results are to be taken from another kernel ("only" below).
 bool eval_u8_tc_supported(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev);
@@ -299,9 +301,9 @@ bool eval_u8_wide_supported(const NetLayout& net, int32_t pop, int32_t batch, co
 size_t eval_u8_scratch_bytes(const NetLayout& net, int32_t pop, int32_t batch, int32_t xp);
 int32_t* eval_u8_flagged(const NetLayout& net, int32_t pop, int32_t batch, int32_t xp, void* scratch);
 cudaError_t launch_stage_x16(const NetLayout& net, int32_t pop, const uint8_t* x, int32_t batch, void* scratch,
-                             cudaStream_t stream);
+                             bool x_ready, cudaStream_t stream);
 cudaError_t launch_stage_xf(const NetLayout& net, int32_t pop, const float* x, int32_t batch, void* scratch,
-                            cudaStream_t stream);
+                            bool x_ready, cudaStream_t stream);
 cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* pop_dev, int32_t xp, const uint8_t* x,
                               void* scratch, float x_div, const int32_t* y, int32_t batch, float alpha,
                               const float* f_inh, float* f_raw, float* f_adj, int32_t* correct, unsigned int* status,

@@ -20,8 +20,11 @@ __global__ void __launch_bounds__(32 * kRankWarps) rank_kernel(int32_t pop, cons
                                                               int32_t* __restrict__ order)
 {
     __shared__ uint64_t tile[kRankTile];
-    ptx::grid_dep_launch();
     ptx::grid_dep_wait();  // f_adj comes from the previous kernel
+    // Only now: what starts from here on (the selection, and a generation's staging
+    // of its batch beside it) finds everything earlier on the stream complete, the
+    // caller's minibatch too.
+    ptx::grid_dep_launch();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int32_t i = blockIdx.x * kRankWarps + warp;
     const uint64_t mine = i < pop ? rank_key(f_adj[i], i) : 0ull;
