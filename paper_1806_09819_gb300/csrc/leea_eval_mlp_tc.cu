@@ -771,9 +771,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                     total += __shfl_xor_sync(0xFFFFFFFFu, total, off);
                     n_ok += __shfl_xor_sync(0xFFFFFFFFu, n_ok, off);
                 }
-                // Two buffers: the sums of individual k + 2 come after layer 4 of its
-                // units, which waits for d4_read of a unit of k + 1, for which warp q = 0
-                // arrives when it has read these.
+                // red_full counts these four warps once per individual: an arrival for k
+                // before the last one for k - 1 would end that phase without the slowest
+                // warp's sum, so each waits for it first (by now it has long passed).  It
+                // also orders the two buffers: warp q = 0 has read the sums of k - 2 when
+                // it arrives for k - 1.
+                if (k > 0 && !(ok = wait(s.red_full, (k - 1) & 1u))) break;
                 double* red_loss = s.red_loss + 4 * (k & 1u);
                 int32_t* red_ok = s.red_ok + 4 * (k & 1u);
                 if (lane == 0) {

@@ -1,0 +1,37 @@
+"""How the tensor-core evaluation of deeper nets adds up an individual's loss: identical individuals get identical bits."""
+import numpy as np
+import pytest
+
+from helpers import to_device_pop
+
+pytestmark = pytest.mark.gpu
+
+
+def _evaluate(gpu, dims, pd, levels, y):
+    import torch
+    pop = pd.shape[0]
+    f = torch.full((pop,), float("nan"), device="cuda")
+    cor = torch.full((pop,), -1, dtype=torch.int32, device="cuda")
+    gpu.leea_evaluate_u8(pop, dims, pd, torch.from_numpy(levels).cuda(), 255.0, torch.from_numpy(y).cuda(), len(y), 1.0,
+                         None, f, None, cor, gpu.EVAL_TENSOR)
+    assert gpu.leea_device_status() == 0
+    return f.cpu().numpy(), cor.cpu().numpy()
+
+
+@pytest.mark.parametrize("dims,batch", [([16, 16, 16, 16, 2], 128), ([32, 16, 16, 16, 10], 1), ([64, 32, 16, 32, 5], 77)])
+def test_many_small_nets_of_one_tile(gpu, dims, batch):
+    """Net after net on every CTA with little between them: each one's sum holds all of its samples and no other's, so
+    that it has the bits of the net alone on a CTA (which the oracle checks elsewhere)."""
+    pop, kinds = 12000, 7
+    rng = np.random.default_rng(batch)
+    nets = rng.normal(0.0, 0.5, size=(kinds, gpu.leea_layout_num_params(dims))).astype(np.float32)
+    which = rng.integers(0, kinds, size=pop)
+    levels = rng.integers(0, 256, size=(batch, dims[0])).astype(np.uint8)
+    y = rng.integers(0, dims[-1], size=batch).astype(np.int32)
+    cp = gpu.leea_padded_params(dims)
+    alone, cor_alone = _evaluate(gpu, dims, to_device_pop(nets, cp), levels, y)
+    pd = to_device_pop(nets[which], cp)
+    for _ in range(3):
+        f, cor = _evaluate(gpu, dims, pd, levels, y)
+        np.testing.assert_array_equal(f, alone[which])
+        np.testing.assert_array_equal(cor, cor_alone[which])
