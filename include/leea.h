@@ -299,7 +299,7 @@ leea_status leea_breed_evaluate_u8(int32_t pop, const int32_t* dims, int32_t n_d
  * bias, ReLU, last layer and loss; an individual with a weight or activation
  * |v| >= 128 is recomputed in FP32 on the CUDA cores.  That path splits the
  * weights and converts the batch into a library-owned scratch buffer (388 KB
- * per individual for 196-256-128-64-10, plus 64 KB per 128 samples), one per
+ * per individual for 196-256-128-64-10, plus 68 KB per 128 samples), one per
  * device, shared by these step calls on that device, so such calls must not
  * overlap on one device; growing it frees the old buffer (which synchronises
  * the device).  The state object owns its own.  f_adj_dev and

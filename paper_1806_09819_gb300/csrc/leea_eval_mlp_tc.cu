@@ -24,8 +24,8 @@
 // levels and a ring of 32 KB weight slots.  Where all layers have their own
 // columns (mlp_columns) the next unit's layer 1 runs before and after this
 // unit's layer 3, under the epilogue of layers 2 and 3.  A CTA takes a
-// contiguous range of units; the sums of an individual that two CTAs share meet
-// in scratch memory (combine_mlp_parts_kernel).
+// contiguous range of units; the tiles' sums of an individual that several CTAs
+// share meet in scratch memory (combine_mlp_parts_kernel).
 //
 // Measured, 2000 nets 196-256-128-64-10 on 1024 samples: 945 us (1518 with the
 // activations in shared memory and two weight buffers), 207 of them the splitting
@@ -135,7 +135,7 @@ struct MlpTcArgs {
     uint8_t* pieces;     // per individual piece_stride bytes, see MlpSlots
     int64_t piece_stride;
     int32_t per_cta, extra;  // units of a CTA; the first `extra` CTAs take one more
-    double* part_loss;   // [2 gridDim.x]: loss sums and correct counts of individuals shared by CTAs
+    double* part_loss;   // [2 gridDim.x][n_tiles]: tiles' loss sums and correct counts of individuals shared by CTAs
     int32_t* part_ok;
 };
 
@@ -733,8 +733,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
             for (Segments seg(a, blockIdx.x); ok && seg.valid(); seg.step(a), ++k) {
                 const float* b4 = s.param + (k & 1u) * param_floats(a.dims) + d1 + d2 + d3;
                 if (!wait(&s.param_full[k & 1u], (k >> 1) & 1u)) break;
-                double total = 0.0;
-                int32_t n_ok = 0;
+                const bool whole = seg.t0 == 0 && seg.t1 == a.n_tiles;
+                double total = 0.0;  // warp q = 0, lane 0: the tiles so far, in their order
+                int32_t total_ok = 0;
                 for (int t = seg.t0; t < seg.t1; ++t, ++u) {
                     const int smp = t * kTile + row;
                     const int32_t lbl = smp < a.batch ? a.y[smp] : 0;
@@ -744,6 +745,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                     ptx::tmem_ld16(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(a.col[3]), z);
                     ptx::tc_fence_before();
                     arrive(s.d4_read);
+                    double loss = 0.0;
+                    int32_t n_ok = 0;
                     float zmax = 0.0f, zl = 0.0f;
                     int arg = 0;
 #pragma unroll
@@ -760,44 +763,44 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                         for (int o = 0; o < kMaxOutTc; ++o)
                             if (o < d_out) se += expf(z[o] - zmax);
                         const bool valid = lbl >= 0 && lbl < d_out;
-                        total += static_cast<double>(valid ? logf(se) + zmax - zl : __int_as_float(0x7FC00000));
-                        n_ok += valid && arg == lbl ? 1 : 0;
+                        loss = static_cast<double>(valid ? logf(se) + zmax - zl : __int_as_float(0x7FC00000));
+                        n_ok = valid && arg == lbl ? 1 : 0;
+                    }
+#pragma unroll
+                    for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xFFFFFFFFu, loss, off);
+                    n_ok = __reduce_add_sync(0xFFFFFFFFu, n_ok);
+                    // red_full counts these four warps once per unit: an arrival for u before
+                    // the last one for u - 1 would end that phase without the slowest warp's
+                    // sum, so each waits for it first (by now it has long passed).  It also
+                    // orders the two buffers: warp q = 0 has read the sums of u - 2 when it
+                    // arrives for u - 1.
+                    if (u > 0 && !(ok = wait(s.red_full, (u - 1) & 1u))) break;
+                    double* red_loss = s.red_loss + 4 * (u & 1u);
+                    int32_t* red_ok = s.red_ok + 4 * (u & 1u);
+                    if (lane == 0) {
+                        red_loss[q] = loss;
+                        red_ok[q] = n_ok;
+                        ptx::mbar_arrive(s.red_full);
+                    }
+                    if (q == 0) {
+                        if (!(ok = wait(s.red_full, u & 1u))) break;
+                        const double sum = ((red_loss[0] + red_loss[1]) + red_loss[2]) + red_loss[3];
+                        const int32_t good = red_ok[0] + red_ok[1] + red_ok[2] + red_ok[3];
+                        total += sum;
+                        total_ok += good;
+                        // An individual that this CTA shares: its tiles one by one, so that the sum
+                        // of all has the same order wherever they were cut.  At most one segment of
+                        // a CTA starts, and one ends, inside an individual.
+                        if (!whole && lane == 0) {
+                            const int64_t e = 2 * static_cast<int64_t>(blockIdx.x) + (seg.t0 == 0 ? 1 : 0);
+                            a.part_loss[e * a.n_tiles + t] = sum;
+                            a.part_ok[e * a.n_tiles + t] = good;
+                        }
                     }
                 }
                 if (!ok) break;
                 arrive(&s.param_empty[k & 1u]);
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) {
-                    total += __shfl_xor_sync(0xFFFFFFFFu, total, off);
-                    n_ok += __shfl_xor_sync(0xFFFFFFFFu, n_ok, off);
-                }
-                // red_full counts these four warps once per individual: an arrival for k
-                // before the last one for k - 1 would end that phase without the slowest
-                // warp's sum, so each waits for it first (by now it has long passed).  It
-                // also orders the two buffers: warp q = 0 has read the sums of k - 2 when
-                // it arrives for k - 1.
-                if (k > 0 && !(ok = wait(s.red_full, (k - 1) & 1u))) break;
-                double* red_loss = s.red_loss + 4 * (k & 1u);
-                int32_t* red_ok = s.red_ok + 4 * (k & 1u);
-                if (lane == 0) {
-                    red_loss[q] = total;
-                    red_ok[q] = n_ok;
-                    ptx::mbar_arrive(s.red_full);
-                }
-                if (q == 0) {
-                    if (!(ok = wait(s.red_full, k & 1u))) break;
-                    if (lane == 0) {
-                        const double sum = ((red_loss[0] + red_loss[1]) + red_loss[2]) + red_loss[3];
-                        const int32_t good = red_ok[0] + red_ok[1] + red_ok[2] + red_ok[3];
-                        if (seg.t0 == 0 && seg.t1 == a.n_tiles) {
-                            store_fitness(a, seg.p, sum, good);
-                        } else {  // at most one segment of a CTA starts, and one ends, inside an individual
-                            const int e = 2 * static_cast<int>(blockIdx.x) + (seg.t0 == 0 ? 1 : 0);
-                            a.part_loss[e] = sum;
-                            a.part_ok[e] = good;
-                        }
-                    }
-                }
+                if (whole && q == 0 && lane == 0) store_fitness(a, seg.p, total, total_ok);
             }
         }
     }
@@ -811,8 +814,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
     }
 }
 
-// The fitness of the individuals that several CTAs share: the sums of their
-// segments in order of the tiles.
+// The fitness of the individuals that several CTAs share: the sums of their tiles
+// in order, as for an individual inside one CTA.
 __global__ void __launch_bounds__(256) combine_mlp_parts_kernel(const MlpTcArgs a)
 {
     const int p = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
@@ -826,10 +829,14 @@ __global__ void __launch_bounds__(256) combine_mlp_parts_kernel(const MlpTcArgs 
     if (c0 == c1) return;
     double sum = 0.0;
     int32_t good = 0;
+    int t = 0;
     for (int c = c0; c <= c1; ++c) {
-        const int e = 2 * c + (c == c0 ? 1 : 0);
-        sum += a.part_loss[e];
-        good += a.part_ok[e];
+        const int64_t end = static_cast<int64_t>(c + 1) * a.per_cta + min(c + 1, a.extra) - first;  // the CTA's last tile + 1
+        const int64_t e = (2 * static_cast<int64_t>(c) + (c == c0 ? 1 : 0)) * a.n_tiles;
+        for (; t < a.n_tiles && t < end; ++t) {
+            sum += a.part_loss[e + t];
+            good += a.part_ok[e + t];
+        }
     }
     store_fitness(a, p, sum, good);
 }
@@ -955,8 +962,8 @@ MlpScratch mlp_scratch_layout(const NetLayout& net, int32_t pop, int32_t batch)
     s.marks = stride * np;
     s.tiles = s.marks + up(sizeof(int32_t) * np);
     s.part_loss = s.tiles + static_cast<size_t>(tiles) * level_tile_bytes(net);
-    s.part_ok = s.part_loss + up(16 * static_cast<size_t>(sms));
-    s.bytes = s.part_ok + up(8 * static_cast<size_t>(sms));
+    s.part_ok = s.part_loss + up(16 * static_cast<size_t>(sms) * static_cast<size_t>(tiles));
+    s.bytes = s.part_ok + up(8 * static_cast<size_t>(sms) * static_cast<size_t>(tiles));
     return s;
 }
 

@@ -35,3 +35,19 @@ def test_many_small_nets_of_one_tile(gpu, dims, batch):
         f, cor = _evaluate(gpu, dims, pd, levels, y)
         np.testing.assert_array_equal(f, alone[which])
         np.testing.assert_array_equal(cor, cor_alone[which])
+
+
+def test_twins_split_differently_among_ctas(gpu):
+    """Twins on three tiles, of which some lie within a CTA and others in two or three.  The losses make the order of the
+    sum visible in the result: 3 2^58 and 3 2^34 in the first tile, whose quotient by the 384 samples is a tie between two
+    floats, and 64, half an ulp of their FP64 sum, in each of the others."""
+    dims, pop, batch = [64, 16, 16, 16, 10], 228, 384
+    net = np.zeros(gpu.leea_layout_num_params(dims), dtype=np.float32)
+    net[-10:] = [0.0, -3.0 * 2.0 ** 58, -3.0 * 2.0 ** 34, -64.0] + [-200.0] * 6  # the output layer's biases
+    y = np.zeros(batch, dtype=np.int32)  # class 0: loss 0; class o: minus its bias
+    y[0], y[1], y[128 + 5], y[256 + 5] = 1, 2, 3, 3
+    levels = np.zeros((batch, dims[0]), dtype=np.uint8)
+    f, cor = _evaluate(gpu, dims, to_device_pop(np.tile(net, (pop, 1)), gpu.leea_padded_params(dims)), levels, y)
+    total = ((3.0 * 2.0 ** 58 + 3.0 * 2.0 ** 34) + 64.0) + 64.0
+    np.testing.assert_array_equal(f, np.full(pop, -np.float32(total / batch)))
+    assert (cor == batch - 4).all()
