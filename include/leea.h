@@ -303,7 +303,8 @@ leea_status leea_breed_evaluate_u8(int32_t pop, const int32_t* dims, int32_t n_d
  * device, shared by these step calls on that device, so such calls must not
  * overlap on one device; growing it frees the old buffer (which synchronises
  * the device).  The state object owns its own.  f_adj_dev and
- * correct_dev may be NULL; f_raw_dev may not.  eval_path: LEEA_EVAL_*. */
+ * correct_dev may be NULL; f_raw_dev may not.  f_adj_dev may be f_inh_dev, except
+ * for deeper nets on the tensor cores.  eval_path: LEEA_EVAL_*. */
 leea_status leea_evaluate(int32_t pop, const int32_t* dims, int32_t n_dims,
                           const float* pop_dev, const float* x_dev, const int32_t* y_dev,
                           int32_t batch, float alpha, const float* f_inh_dev,

@@ -706,11 +706,12 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 // within TENSOR's shapes on 8-bit levels, layer 1 here by FP32 FFMA
                 // from global memory, k in order.
                 float scale[4];  // accumulator units to x units, per sample
+                bool marked = gov == 2;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int sj = kQuads ? first + 8 * j + (lane >> 2) : smp;
                     scale[j] = XP == 1 ? a.inv_div : (sj < a.batch ? __ldcg(a.x_scale + sj) : 0.0f);
-                    if (a.flagged && (gov == 2 || scale[j] != scale[j])) a.flagged[p] = 1;
+                    marked = marked || scale[j] != scale[j];
                     if (!kQuads) break;
                 }
                 float logit[kMaxOutU8];
@@ -821,7 +822,7 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                     for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xFFFFFFFFu, loss, off);
                     sum = static_cast<double>(loss);
                 }
-                good = __reduce_add_sync(0xFFFFFFFFu, good);
+                good = __reduce_add_sync(0xFFFFFFFFu, good | (marked ? 1u << 16 : 0u));  // and the marks above
                 double* rl = s.red_loss + (g * 2 + (t & 1)) * 4;
                 int32_t* ro = s.red_ok + (g * 2 + (t & 1)) * 4;
                 if (lane == 0) {
@@ -830,9 +831,13 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 }
                 ptx::named_barrier_sync(bar_id, 128);  // B: quarter sums written; staged parameters no longer read
                 if (et == 0) {
-                    const int32_t n_ok = ro[0] + ro[1] + ro[2] + ro[3];
+                    const int32_t sum_ok = ro[0] + ro[1] + ro[2] + ro[3], n_ok = sum_ok & 0xFFFF;
                     const double total = ((rl[0] + rl[1]) + rl[2]) + rl[3];
-                    if (a.tiles == 1) {
+                    // A marked individual's results all come from the evaluation that follows,
+                    // which reads f_inh: f_adj may be the same array.
+                    const bool again = a.flagged && sum_ok > 0xFFFF;
+                    if (again) a.flagged[p] = 1;
+                    if (a.tiles == 1 && !again) {
                         float f;
                         if (a.wide) {
                             f = static_cast<float>(-(total / static_cast<double>(a.batch)));
@@ -844,7 +849,7 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                         a.f_raw[p] = f;
                         if (a.f_adj) a.f_adj[p] = a.f_inh ? (1.0f - a.alpha) * inherited + a.alpha * f : f;
                         if (a.correct) a.correct[p] = n_ok;
-                    } else {
+                    } else if (a.tiles > 1) {
                         const int64_t at = static_cast<int64_t>(x.t0 + t) * a.pop + p;
                         a.part[at] = total;
                         a.part_ok[at] = n_ok;
@@ -955,12 +960,12 @@ __global__ void __launch_bounds__(256) stage_xf_kernel(const float* __restrict__
 }
 
 // A batch of several tiles: each individual's loss and correct count from its
-// tiles' sums, in tile order.
+// tiles' sums, in tile order, except for the marked ones.
 __global__ void __launch_bounds__(256) combine_u8_tiles_kernel(const EvalU8Args a)
 {
     ptx::grid_dep_wait();
     const int p = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
-    if (p >= a.pop) return;
+    if (p >= a.pop || (a.flagged && __ldcg(a.flagged + p))) return;
     double total = 0.0;
     int32_t n_ok = 0;
     for (int t = 0; t < a.tiles; ++t) {
