@@ -122,9 +122,11 @@ enum { LEEA_SIGMA_CONST = 0, LEEA_SIGMA_DECAY = 1, LEEA_SIGMA_SELF = 2 };
 
 /* Evaluation kernels.  AUTO takes the fastest for the shape: with d_0 % 4 == 0,
  * h <= 256, d_out <= 16 and 16-byte aligned buffers the tensor cores with FP16
- * operand pieces (an 8-bit level exactly, a float input and a weight as two, 22
- * bits; FP32 accumulation; individuals and samples that the pieces cannot hold
- * again with TF32 pieces or on the CUDA cores) -- floats with h % 16 == 0,
+ * operand pieces (an 8-bit level exactly; a float input and a weight as two, 22
+ * bits, but errors up to 2^-39 of the sample's largest input and 2^-33; FP32
+ * accumulation; individuals outside the pieces' range, or where those errors could
+ * move a logit by about one FP32 rounding of the loss, as with features of very
+ * different scale, again with TF32 pieces or on the CUDA cores) -- floats with h % 16 == 0,
  * 8-bit levels in TENSOR's shapes or from 48 samples on -- else, or where so
  * small a call does not pay for the staging, TENSOR's kernel or SIMT's.  SIMT:
  * exact FP32 FFMA on the CUDA cores.  TENSOR: tcgen05 tensor cores with a three-term TF32 split
@@ -320,7 +322,9 @@ leea_status leea_evaluate(int32_t pop, const int32_t* dims, int32_t n_dims,
  * scaled by 2^8, is split into two FP16 pieces (|2^8 w - w1 - w2| <=
  * max(2^-22 2^8 |w|, 2^-25), a 22-bit significand), so besides that split only
  * the tensor core's FP32 accumulation rounds; an individual with a weight
- * |w| >= 128 gets its layer 1 in FP32 FFMA instead.  That path first writes the
+ * |w| >= 128 gets its layer 1 in FP32 FFMA instead, and outside TENSOR's shapes
+ * so does one for which 2^-33 is too coarse (W1 small beside W2, a small x_div).
+ * That path first writes the
  * batch as FP16 into a stream-ordered allocation of batch * round_up(d_0, 8) * 2
  * bytes, and above 128 samples 12 * ceil(batch / 128) * pop bytes for the
  * 128-sample tiles' sums (freed in stream order after the evaluation; the

@@ -11,7 +11,8 @@
 // formed from exact products; only the FP32 accumulation in the tensor core
 // rounds.  The epilogue scales by 2^-8 / x_div or by the sample's own factor.
 // The converters find the individuals that the pieces cannot carry
-// (outside_pieces).  On 8-bit levels within TENSOR's shapes the epilogue forms
+// (outside_pieces), the epilogue those for which they are too coarse (kMarkTol).
+// On 8-bit levels within TENSOR's shapes the epilogue forms
 // their layer 1 with FP32 FFMA from global memory; elsewhere it marks them and
 // a launch of the kernel that has the call otherwise follows for the marked
 // ones (floats: TF32 pieces, 8-bit levels: the CUDA cores; 2 us when there are
@@ -127,6 +128,9 @@ struct EvalU8Args {
     const float* popv;
     const uint8_t* x;        // the levels, for the FP32 fallback inside TENSOR's shapes
     const float* x_scale;    // float inputs: accumulator units to x units, per sample
+    const float2* x_err;     // float inputs: what the pieces may err by, per sample (see kMarkTol)
+    float err;               // the same for 8-bit levels, times sqrt(h)
+    float sqrt_h;
     int32_t* flagged;        // [pop]: 1 = a weight outside the pieces' range, to be evaluated again (or NULL: here)
     const int32_t* y;
     const float* f_inh;
@@ -146,15 +150,17 @@ struct U8Smem {
     float* b2;           // [2 groups][16]
     double* red_loss;    // [2 groups][2 tiles][4 quarters]
     int32_t* red_ok;     // [2 groups][2 tiles][4 quarters]
+    uint32_t* w2_top;    // [2 groups][4 warps]: largest |w| of W2, as bits
     uint32_t* flag;      // [kFlagSlots][2]: (u + 1) << 8 | the largest exponent field of unit u's individual
-    uint32_t* accflag;   // [2]: the flags of the unit in that accumulator, for the epilogue
-    int* ep_go;          // [2 groups]: their go words
+    uint32_t* accflag;   // [2]: of the unit in that accumulator, for the epilogue: bit s: individual s is outside the
+                         // pieces; byte 1 + s: the exponent field of its largest weight
+    int* ep_go;          // [2 groups]: their go words, 1 or 2 (outside the pieces), and that exponent in byte 1
     uint32_t* tmem_holder;
     volatile int* abort_flag;
     uint64_t *full, *a_full, *empty, *acc_full, *acc_empty, *drain;
 };
 
-constexpr size_t kTailFixed = 8 + sizeof(double) * 16 + sizeof(int32_t) * 16 + sizeof(uint32_t) * (2 * kFlagSlots + 2) +
+constexpr size_t kTailFixed = 8 + sizeof(double) * 16 + sizeof(int32_t) * 16 + sizeof(uint32_t) * (8 + 2 * kFlagSlots + 2) +
                               sizeof(int) * 2 + 16 + 16;
 
 // Floats between the rows (a hidden unit's outputs) of W2 in shared memory: the
@@ -187,6 +193,8 @@ __device__ __forceinline__ U8Smem carve(uint8_t* raw, const EvalU8Args& a)
     p += sizeof(double) * 16;
     s.red_ok = reinterpret_cast<int32_t*>(p);
     p += sizeof(int32_t) * 16;
+    s.w2_top = reinterpret_cast<uint32_t*>(p);
+    p += sizeof(uint32_t) * 8;
     s.flag = reinterpret_cast<uint32_t*>(p);
     p += sizeof(uint32_t) * 2 * kFlagSlots;
     s.accflag = reinterpret_cast<uint32_t*>(p);
@@ -205,6 +213,13 @@ __device__ __forceinline__ U8Smem carve(uint8_t* raw, const EvalU8Args& a)
     s.acc_empty = s.acc_full + 2;
     s.drain = s.acc_empty + 2;
     return s;
+}
+
+// Largest |w| of the W2 that epilogue group g has staged.
+__device__ __forceinline__ float w2_top(const U8Smem& s, int g)
+{
+    const uint32_t* t = s.w2_top + 4 * g;
+    return __uint_as_float(max(max(t[0], t[1]), max(t[2], t[3])));
 }
 
 // How a population and a batch are cut into units.
@@ -278,6 +293,24 @@ __device__ __forceinline__ bool outside_pieces(uint32_t exponent)
 {
     return exponent >= 127u + 7u || (XP == 2 && exponent != 0u && exponent < 127u - 10u);
 }
+
+// The largest weight is not all there is to it.  A weight's pieces resolve 2^-32
+// and a float sample's 2^-38 of its largest input, so where large inputs meet small
+// weights (features of very different scale), or small inputs stand beside a large
+// one, products keep fewer than 22 bits.  The rounding errors, uniform in half a
+// step each way, reach a hidden unit as err = 2^-33 / sqrt(3) ||x|| + 2^-39 / sqrt(3)
+// max |x| max |w| sqrt(d_0) (root mean square; the second term for floats) and a
+// logit as at most err sqrt(h) max |W2|.  An individual with a sample where that
+// exceeds 2^-24 max(1, |largest logit|, loss), one rounding of the FP32 softmax
+// cross-entropy, is evaluated again (8-bit levels, whose ||x|| is at most 255
+// sqrt(d_0) / x_div: with the mean loss of a tile).  On images and initial weights
+// the two are 10 to 25 apart; 8 of 784 inputs of scale 1e3 and more, their weights
+// smaller in proportion, go beyond it (without this their loss erred by 1.1e-5
+// relative at 1e6, 2e-4 at the test's scales).  It costs 333 nets 784-100-10 on 50
+// samples 0.4 of 40 us, 1000 nets on 512 samples 1.4 of 196.
+constexpr float kMarkTol = 5.9604645e-8f;           // 2^-24
+constexpr float kWeightErr = 6.7212e-11f;           // 2^-33 / sqrt(3)
+constexpr float kInputErr = kWeightErr / 64.0f;     // 2^-39 / sqrt(3)
 
 // Four weights of row r (0..7) of an 8-row group, inputs 4 c4 .. 4 c4 + 3 of
 // the stage, as FP16 pieces at their swizzled positions (the 16-byte chunk
@@ -514,7 +547,9 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 // a releasing arrival on the same barrier.
                 if (lead) {
                     const volatile uint32_t* fl = s.flag + 2 * (u % kFlagSlots);
-                    s.accflag[buf] = (outside_pieces<XP>(fl[0] & 255u) ? 1u : 0u) | (outside_pieces<XP>(fl[1] & 255u) ? 2u : 0u);
+                    const uint32_t e0 = fl[0] & 255u, e1 = fl[1] & 255u;
+                    s.accflag[buf] = (outside_pieces<XP>(e0) ? 1u : 0u) | (outside_pieces<XP>(e1) ? 2u : 0u) |
+                                     (e0 << 8) | (e1 << 16);
                     ptx::mbar_arrive(&s.acc_full[buf]);
                 }
             }
@@ -661,11 +696,14 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 // assumes data no grid changes during the kernel.
                 const float* src = a.popv + static_cast<int64_t>(p) * a.c_pad + static_cast<int64_t>(a.h) * a.k;
                 for (int i = et; i < a.hp; i += 128) b1s[i] = i < a.h ? __ldcg(src + i) : 0.0f;
+                float top = 0.0f;
                 for (int col = et; col < a.hp; col += 128) {
                     float w[kMaxOutU8];  // all in flight at once
 #pragma unroll
                     for (int o = 0; o < kMaxOutU8; ++o)
                         w[o] = o < a.d_out && col < a.h ? __ldcg(src + a.h + o * a.h + col) : 0.0f;
+#pragma unroll
+                    for (int o = 0; o < kMaxOutU8; ++o) top = fmaxf(top, fabsf(w[o]));
 #pragma unroll
                     for (int o4 = 0; o4 < kMaxOutU8 / 4; ++o4)
                         if (4 * o4 < a.wst)
@@ -673,15 +711,20 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                                 make_float4(w[4 * o4], w[4 * o4 + 1], w[4 * o4 + 2], w[4 * o4 + 3]);
                 }
                 if (et < 16) b2s[et] = et < a.d_out ? __ldcg(src + a.h + a.d_out * a.h + et) : 0.0f;
+                if (a.flagged) {
+                    const uint32_t t = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(top));
+                    if (lane == 0) s.w2_top[ew] = t;
+                }
             }
             const float inherited = active && et == 0 && a.f_inh && a.tiles == 1 ? a.f_inh[p] : 0.0f;
             if (et == 0) {
                 const bool got = ptx::mbar_wait_bounded(&s.acc_full[buf], phase_of(u), s.abort_flag, kWaitLimitNs);
                 if (!got) raise_abort(s, a);
-                *go = !got ? 0 : (((s.accflag[buf] >> slot) & 1u) ? 2 : 1);
+                const uint32_t fl = s.accflag[buf];
+                *go = !got ? 0 : static_cast<int>(1u + ((fl >> slot) & 1u) + (((fl >> (8 + 8 * slot)) & 255u) << 8));
             }
             ptx::named_barrier_sync(bar_id, 128);  // A: accumulator ready (or abort); parameters staged
-            const int gov = *go;
+            const int gov = *go & 255;
             if (!gov) break;
             ptx::tc_fence_after();
             if (!active) {
@@ -701,17 +744,15 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 unsigned good = 0;
                 const uint32_t col0 = tmem_base + lane_addr + buf * kAccStride + static_cast<uint32_t>(t) * tile_cols +
                                       static_cast<uint32_t>(slot * a.hp);
-                // Individuals with a weight outside the piece range, and samples that
-                // the pieces cannot carry: marked for the evaluation that follows or,
-                // within TENSOR's shapes on 8-bit levels, layer 1 here by FP32 FFMA
-                // from global memory, k in order.
+                // Individuals with a weight outside the piece range are marked for the
+                // evaluation that follows or, within TENSOR's shapes on 8-bit levels, have
+                // layer 1 here by FP32 FFMA from global memory, k in order.
                 float scale[4];  // accumulator units to x units, per sample
                 bool marked = gov == 2;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int sj = kQuads ? first + 8 * j + (lane >> 2) : smp;
                     scale[j] = XP == 1 ? a.inv_div : (sj < a.batch ? __ldcg(a.x_scale + sj) : 0.0f);
-                    marked = marked || scale[j] != scale[j];
                     if (!kQuads) break;
                 }
                 float logit[kMaxOutU8];
@@ -808,6 +849,14 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                     } else {
                         loss = __int_as_float(0x7FC00000);
                     }
+                    // Marks a float sample that the pieces cannot carry (kMarkTol), one that is
+                    // not finite too (its x_err is NaN).
+                    if (XP == 2) {
+                        const float2 err = __ldcg(a.x_err + smp);
+                        const float w_top = __uint_as_float(min(static_cast<uint32_t>(*go >> 8) + 1u, 254u) << 23);
+                        const float reach = fmaf(err.y, w_top, err.x) * a.sqrt_h * w2_top(s, g);
+                        marked = marked || !(reach <= kMarkTol * fmaxf(fmaxf(fabsf(zmax), loss), 1.0f));
+                    }
                 }
                 // Fixed-order sums: FP32 within TENSOR's shapes (the fused kernel
                 // gives the same bits), FP64 beyond them, where these roundings
@@ -829,13 +878,16 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                     rl[q] = sum;
                     ro[q] = static_cast<int32_t>(good);
                 }
+                const float reach = XP == 1 && a.flagged && et == 0 ? a.err * w2_top(s, g) : 0.0f;
                 ptx::named_barrier_sync(bar_id, 128);  // B: quarter sums written; staged parameters no longer read
                 if (et == 0) {
                     const int32_t sum_ok = ro[0] + ro[1] + ro[2] + ro[3], n_ok = sum_ok & 0xFFFF;
                     const double total = ((rl[0] + rl[1]) + rl[2]) + rl[3];
                     // A marked individual's results all come from the evaluation that follows,
                     // which reads f_inh: f_adj may be the same array.
-                    const bool again = a.flagged && sum_ok > 0xFFFF;
+                    bool again = a.flagged && sum_ok > 0xFFFF;
+                    if (XP == 1 && a.flagged)
+                        again = again || !(reach <= kMarkTol * fmaxf(static_cast<float>(total) * (1.0f / 128.0f), 1.0f));
                     if (again) a.flagged[p] = 1;
                     if (a.tiles == 1 && !again) {
                         float f;
@@ -906,14 +958,17 @@ __global__ void __launch_bounds__(256) stage_x16_kernel(const uint8_t* __restric
 // that its largest |x| lands in [2^14, 2^15); x1 rounds 2^e x, x2 the remainder
 // (exact in FP32), so the pieces carry 22 bits of every value near the largest
 // and absolute errors of 2^-39 of it below.  x_scale[b] = 2^-(e + 8) turns the
-// accumulator's units (2^e x times 2^8 w) into x w; NaN for a sample with an
-// infinite or NaN input, whose individuals are all evaluated again by a kernel
-// that multiplies x itself.  A CTA per sample.  x_ready as in stage_x16_kernel.
+// accumulator's units (2^e x times 2^8 w) into x w.  x_err[b]: kWeightErr ||x|| and
+// kInputErr max |x| sqrt(k), what the pieces may err by (kMarkTol); NaN for a sample
+// with an infinite or NaN input, whose individuals are all evaluated again by a
+// kernel that multiplies x itself.  A CTA per sample.  x_ready as in
+// stage_x16_kernel.
 __global__ void __launch_bounds__(256) stage_xf_kernel(const float* __restrict__ x, int32_t batch, int32_t k, int32_t kp,
                                                        __half* __restrict__ x16, float* __restrict__ x_scale,
-                                                       int32_t* __restrict__ flagged, int32_t pop, bool x_ready)
+                                                       float2* __restrict__ x_err, int32_t* __restrict__ flagged, int32_t pop, bool x_ready)
 {
     __shared__ uint32_t top[8];
+    __shared__ float part_sq[8];
     ptx::grid_dep_launch();
     if (!x_ready) ptx::grid_dep_wait();
     const int32_t b = blockIdx.x;
@@ -937,10 +992,16 @@ __global__ void __launch_bounds__(256) stage_xf_kernel(const float* __restrict__
         e = min(15 - ex, 126);
     }
     const float up = ldexpf(1.0f, e);
+    float sq = 0.0f;  // of 2^(e - 15) x
     for (int32_t i = threadIdx.x; i < kp / 4; i += blockDim.x) {
         const float4 v = 4 * i < k ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
         const float s[4] = { v.x * up, v.y * up, v.z * up, v.w * up };
         uint32_t p1[2], p2[2];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float n = s[j] * 3.0517578e-5f;  // 2^-15
+            sq = fmaf(n, n, sq);
+        }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const __half2 h1 = __floats2half2_rn(s[2 * h], s[2 * h + 1]);
@@ -952,7 +1013,20 @@ __global__ void __launch_bounds__(256) stage_xf_kernel(const float* __restrict__
         dst[0] = make_uint2(p1[0], p1[1]);
         dst[static_cast<int64_t>(batch) * kp / 4] = make_uint2(p2[0], p2[1]);
     }
-    if (threadIdx.x == 0) x_scale[b] = mx < 0x7F800000u ? ldexpf(1.0f, -e - 8) : __int_as_float(0x7FC00000);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, off);
+    if ((threadIdx.x & 31) == 0) part_sq[threadIdx.x >> 5] = sq;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sq = 0.0f;
+        for (int w = 0; w < 8; ++w) sq += part_sq[w];
+        const bool finite = mx < 0x7F800000u;
+        const float nan = __int_as_float(0x7FC00000);
+        x_scale[b] = finite ? ldexpf(1.0f, -e - 8) : nan;
+        x_err[b] = finite ? make_float2(kWeightErr * ldexpf(sqrtf(sq), 15 - e),
+                                        kInputErr * __uint_as_float(mx) * sqrtf(static_cast<float>(k)))
+                          : make_float2(nan, nan);
+    }
     ptx::grid_dep_wait();
     for (int64_t p = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; p < pop;
          p += static_cast<int64_t>(gridDim.x) * blockDim.x)
@@ -1096,11 +1170,11 @@ bool eval_u8_wide_supported(const NetLayout& net, int32_t pop, int32_t batch, co
 bool eval_u8_marks(const NetLayout& net, int32_t batch, int32_t xp) { return xp == 2 || !in_tensor_shapes(net, batch); }
 
 // Scratch layout, each part rounded up to 256 bytes: the FP16 pieces of the
-// batch, the float samples' scales, the marks, several tiles' loss sums and
+// batch, the float samples' scales and errors, the marks, several tiles' loss sums and
 // correct counts.
 namespace {
 struct U8Scratch {
-    size_t scale, flagged, part, part_ok, bytes;
+    size_t scale, err, flagged, part, part_ok, bytes;
 };
 
 U8Scratch u8_scratch(const NetLayout& net, int32_t pop, int32_t batch, int32_t xp)
@@ -1110,7 +1184,8 @@ U8Scratch u8_scratch(const NetLayout& net, int32_t pop, int32_t batch, int32_t x
     const size_t np = static_cast<size_t>(pop), tiles = (nb + 127u) / 128u;
     U8Scratch s;
     s.scale = up(static_cast<size_t>(xp) * nb * kp * 2u);
-    s.flagged = s.scale + (xp == 2 ? up(4u * nb) : 0u);
+    s.err = s.scale + (xp == 2 ? up(4u * nb) : 0u);
+    s.flagged = s.err + (xp == 2 ? up(8u * nb) : 0u);
     s.part = s.flagged + (eval_u8_marks(net, batch, xp) ? up(4u * np) : 0u);
     s.part_ok = s.part + (tiles > 1 ? up(8u * tiles * np) : 0u);
     s.bytes = s.part_ok + (tiles > 1 ? up(4u * tiles * np) : 0u);
@@ -1146,6 +1221,7 @@ cudaError_t launch_stage_xf(const NetLayout& net, int32_t pop, const float* x, i
     return launch_pdl(stage_xf_kernel, dim3(static_cast<unsigned>(batch)), dim3(256), 0, stream, x, batch, net.dims[0],
                       (net.dims[0] + 7) / 8 * 8, static_cast<__half*>(scratch),
                       reinterpret_cast<float*>(static_cast<uint8_t*>(scratch) + u.scale),
+                      reinterpret_cast<float2*>(static_cast<uint8_t*>(scratch) + u.err),
                       eval_u8_flagged(net, pop, batch, 2, scratch), pop, x_ready);
 }
 
@@ -1191,6 +1267,9 @@ cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* po
     const U8Scratch sc = u8_scratch(net, pop, batch, xp);
     uint8_t* base = static_cast<uint8_t*>(scratch);
     a.x_scale = reinterpret_cast<const float*>(base + sc.scale);
+    a.x_err = reinterpret_cast<const float2*>(base + sc.err);
+    a.sqrt_h = std::sqrt(static_cast<float>(a.h));
+    a.err = static_cast<float>(static_cast<double>(kWeightErr) * 255.0 * std::sqrt(static_cast<double>(a.k) * a.h) / x_div);
     a.flagged = eval_u8_flagged(net, pop, batch, xp, scratch);
     a.part = reinterpret_cast<double*>(base + sc.part);
     a.part_ok = reinterpret_cast<int32_t*>(base + sc.part_ok);
