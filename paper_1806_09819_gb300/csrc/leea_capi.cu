@@ -207,10 +207,15 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t stream)
             props.location.id = dev;
             cudaMemPool_t made = nullptr;
             uint64_t keep = kScratchKeep;
+            // A first call may be one under stream capture (this thread's or another's),
+            // where creating a pool counts as unsafe and would end the capture.
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
             if (cudaMemPoolCreate(&made, &props) == cudaSuccess) {
                 if (cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess) pools[dev] = made;
                 else cudaMemPoolDestroy(made);
             }
+            cudaThreadExchangeStreamCaptureMode(&mode);
             if (!pools[dev]) cudaGetLastError();  // the default pool serves as well
         }
         pool = pools[dev];
