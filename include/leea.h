@@ -289,7 +289,9 @@ leea_status leea_breed_evaluate_u8(int32_t pop, const int32_t* dims, int32_t n_d
  * with the maximum subtracted; correct = #{b : argmax z_b = y_b} (ties to the
  * lowest class); f_adj = (1 - alpha) f_inh + alpha f, or f_adj = f when
  * f_inh_dev is NULL (the first evaluation).  Reductions have a fixed order,
- * so identical individuals get bitwise identical results.
+ * so identical individuals of a call get bitwise identical results.  Between
+ * calls under AUTO the last bits may differ with pop and batch, which select the
+ * kernel; name one with eval_path where they must not.
  * n_dims == 3 (d_0-h-d_out with d_out <= 32), or n_dims > 3 with every layer
  * input and hidden width <= 256 and d_out <= 32 (the paper's 196-256-128-64-10,
  * Section 4.1), layer by layer with ReLU between layers.  Deeper nets take
@@ -304,7 +306,13 @@ leea_status leea_breed_evaluate_u8(int32_t pop, const int32_t* dims, int32_t n_d
  * per individual for 196-256-128-64-10, plus 68 KB per 128 samples), one per
  * device, shared by these step calls on that device, so such calls must not
  * overlap on one device; growing it frees the old buffer (which synchronises
- * the device).  The state object owns its own.  f_adj_dev and
+ * the device).  The state object owns its own.  Float inputs of nets with one
+ * hidden layer may take the tensor cores with FP16 pieces under AUTO; the call
+ * then makes a stream-ordered allocation of 4 batch round_up(d_0, 8) + 12 batch +
+ * 4 pop bytes, and above 128 samples 12 ceil(batch / 128) pop more (see
+ * leea_evaluate_u8; a state object keeps its own, grown with the batch).  Without
+ * the memory, and while `stream` is being captured, TENSOR's kernel takes the
+ * call.  f_adj_dev and
  * correct_dev may be NULL; f_raw_dev may not.  f_adj_dev may be f_inh_dev, except
  * for deeper nets on the tensor cores.  eval_path: LEEA_EVAL_*. */
 leea_status leea_evaluate(int32_t pop, const int32_t* dims, int32_t n_dims,
@@ -329,7 +337,8 @@ leea_status leea_evaluate(int32_t pop, const int32_t* dims, int32_t n_dims,
  * bytes, and above 128 samples 12 * ceil(batch / 128) * pop bytes for the
  * 128-sample tiles' sums (freed in stream order after the evaluation; the
  * library keeps at most 64 MB of such scratch per device between calls; beyond
- * 256 MB AUTO takes the CUDA cores).  Otherwise, or with LEEA_EVAL_SIMT, the
+ * 256 MB, and outside TENSOR's shapes while `stream` is being captured, AUTO takes
+ * the CUDA cores).  Otherwise, or with LEEA_EVAL_SIMT, the
  * CUDA-core kernel computes x = k / x_div in FP32.  x_div must be finite and
  * > 0. */
 leea_status leea_evaluate_u8(int32_t pop, const int32_t* dims, int32_t n_dims,
@@ -370,7 +379,7 @@ int64_t leea_shadow_scratch_bytes(int32_t pop, int32_t batch);
  * SM and h <= 128 the batch is first written as operand tiles into a
  * stream-ordered allocation (16 KB per 128 samples and 64 BF16 or 128 FP8
  * inputs, twice that for FP8), and two individuals share every tensor-core
- * instruction; the results are the same bits.  Other arguments and outputs as in
+ * instruction (not while `stream` is being captured); the results are the same bits.  Other arguments and outputs as in
  * leea_evaluate_u8. */
 leea_status leea_evaluate_shadow_u8(int32_t pop, const int32_t* dims, int32_t n_dims,
                                     const float* pop_dev, int32_t precision,

@@ -223,6 +223,19 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t stream)
     return pool ? cudaMallocFromPoolAsync(p, bytes, pool, stream) : cudaMallocAsync(p, bytes, stream);
 }
 
+// Whether work on `stream` is being recorded into a graph.  Scratch would become
+// memory nodes there, and such a graph can be instantiated once at a time and not
+// be a child of another; calls that have a way without scratch take it.
+bool capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus state = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &state) != cudaSuccess) {
+        cudaGetLastError();  // the legacy stream beside a capture: the launches will say so
+        return false;
+    }
+    return state != cudaStreamCaptureStatusNone;
+}
+
 // Synchronises `stream`, reads and clears the status word.
 leea_status check_device_status(cudaStream_t stream, uint32_t* flags_out)
 {
@@ -278,14 +291,14 @@ leea_status dispatch_eval(const NetLayout& net, int32_t pop, const float* pop_de
     const int32_t* only = nullptr;
     void* own = nullptr;  // the call's own scratch, freed in stream order after the evaluation
     cudaError_t err = cudaSuccess;
-    if (pieces) {
-        if (!scratch) {
-            if (scratch_alloc(&own, eval_u8_scratch_bytes(net, pop, batch, 2), stream) != cudaSuccess) {
-                cudaGetLastError();
-                pieces = false;  // no memory for it: TF32 pieces need no scratch
-            }
-            scratch = own;
+    if (pieces && !scratch) {  // TF32 pieces need no scratch
+        if (capturing(stream)) {
+            pieces = false;
+        } else if (scratch_alloc(&own, eval_u8_scratch_bytes(net, pop, batch, 2), stream) != cudaSuccess) {
+            cudaGetLastError();
+            pieces = false;
         }
+        scratch = own;
     }
     if (pieces) {
         err = launch_stage_xf(net, pop, x, batch, scratch, x_ready && !own, stream);
@@ -345,6 +358,7 @@ leea_status dispatch_eval_u8(const NetLayout& net, int32_t pop, const float* pop
     unsigned int* status = device_status_ptr();
     if (tc_ok && path != LEEA_EVAL_SIMT && !status) return fail(LEEA_ECUDA, "device status word unavailable");
     void* own = nullptr;  // the call's own scratch, freed in stream order after the evaluation
+    if (tc_ok && !strict && !x16 && capturing(stream)) tc_ok = false;  // the CUDA cores need no scratch
     if (tc_ok && path != LEEA_EVAL_SIMT && !x16) {
         err = scratch_alloc(&own, eval_u8_scratch_bytes(net, pop, batch, 1), stream);
         if (err != cudaSuccess && strict) return cuda_fail(err, "batch staging allocation");
@@ -423,7 +437,7 @@ leea_status dispatch_eval_shadow(const NetLayout& net, int32_t pop, const float*
     LEEA_CUDA_TRY(cudaGetDevice(&dev), "device query");
     LEEA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device query");
     if (may_allocate && static_cast<int64_t>(pop) * ((batch + 127) / 128) >= 2 * sms &&
-        eval_shadow_pair_supported(net, precision, batch)) {
+        eval_shadow_pair_supported(net, precision, batch) && !capturing(stream)) {
         void* xop = nullptr;
         cudaError_t err = scratch_alloc(&xop, eval_shadow_pair_xop_bytes(net, precision, batch), stream);
         if (err == cudaSuccess) {
@@ -1278,9 +1292,10 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
                                  : eval_u8_wide_supported(s->net, s->pop, batch, s->popbuf[0]));
     const bool eval_f_tc = !fused && !u8 && prec == 0 && s->prm.eval_path == LEEA_EVAL_AUTO && s->net.n_layers == 2 &&
                            eval_u8_wide_supported(s->net, s->pop, batch, s->popbuf[0], 2);
+    void* x16 = nullptr;
     if (eval_u8_tc || eval_f_tc) {
         const size_t need = eval_u8_scratch_bytes(s->net, s->pop, batch, u8 ? 1 : 2);
-        if (need > s->x16_bytes) {
+        if (need > s->x16_bytes && !capturing(s->stream)) {
             LEEA_CUDA_TRY(cudaStreamSynchronize(s->stream), "staging sync");
             cudaFree(s->x16);
             s->x16 = nullptr;
@@ -1293,8 +1308,9 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
                 cudaGetLastError();
             }
         }
+        if (need <= s->x16_bytes) x16 = s->x16;
     }
-    const bool stage_early = eval_u8_tc && s->x16 && !first;
+    const bool stage_early = eval_u8_tc && x16 && !first;
     if (!first) {
         const uint32_t g = s->gen + 1;
         const float sigma_g = sigma_of_breed(s->prm, g);
@@ -1317,7 +1333,7 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
             LEEA_CUDA_TRY(launch_rank_select(a, s->f_adj, s->order, s->par1, s->par2, s->kind, s->f_inh, s->stream),
                           "rank/select kernel");
             if (stage_early)  // runs beside the selection; the breed that follows waits for both
-                LEEA_CUDA_TRY(launch_stage_x16(s->net, s->pop, static_cast<const uint8_t*>(x_dev), batch, s->x16, true,
+                LEEA_CUDA_TRY(launch_stage_x16(s->net, s->pop, static_cast<const uint8_t*>(x_dev), batch, x16, true,
                                                s->stream),
                               "batch staging kernel");
             if ((shadow_pair || shadow_group) && !fused)
@@ -1403,12 +1419,12 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
         else if (u8)
             st = dispatch_eval_u8(s->net, s->pop, s->popbuf[s->cur], static_cast<const uint8_t*>(x_dev), x_div, y_dev,
                                   batch, s->prm.alpha, first ? nullptr : s->f_inh, s->f_raw, s->f_adj, s->correct,
-                                  s->prm.eval_path, s->stream, s->mlp_scratch, eval_u8_tc ? s->x16 : nullptr,
+                                  s->prm.eval_path, s->stream, s->mlp_scratch, x16,
                                   stage_early);
         else
             st = dispatch_eval(s->net, s->pop, s->popbuf[s->cur], static_cast<const float*>(x_dev), y_dev, batch,
                                s->prm.alpha, first ? nullptr : s->f_inh, s->f_raw, s->f_adj, s->correct,
-                               s->prm.eval_path, s->stream, eval_f_tc ? s->x16 : nullptr, !first);
+                               s->prm.eval_path, s->stream, x16, !first);
         sc.done();
         if (st) return st;
     }

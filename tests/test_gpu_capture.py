@@ -83,3 +83,40 @@ def test_first_call_of_a_process(gpu, name):
     code = FIRST_CALL.format(root=ROOT, tests=os.path.join(ROOT, "tests"), name=name)
     res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=ROOT, timeout=120)
     assert res.returncode == 0, res.stderr[-2000:]
+
+
+@pytest.mark.parametrize("name", list(CALLS))
+def test_captured_call(gpu, name):
+    """The same results to a rounding as outside, launched again and again; and where the call has a way without scratch
+    memory no memory nodes, so that the graph can be instantiated more than once."""
+    import torch
+    rt = _runtime()
+    call, pop = _setup(gpu, name)
+    s = torch.cuda.Stream()
+    direct, f = torch.zeros(pop, device="cuda"), torch.zeros(pop, device="cuda")
+    torch.cuda.synchronize()
+    call(s, direct)
+    s.synchronize()
+    graph = _capture(rt, call, s, f)
+    n = ctypes.c_size_t(0)
+    assert rt.cudaGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    nodes, kinds = (ctypes.c_void_p * n.value)(), []
+    assert rt.cudaGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+    for node in nodes:
+        t = ctypes.c_int()
+        assert rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(t)) == 0
+        kinds.append(t.value)
+    memory = bool(MEMORY_NODES & set(kinds))
+    assert memory == (name == "u8")
+    for _ in range(1 if memory else 2):
+        f.zero_()
+        torch.cuda.synchronize()
+        ex = _launch(rt, graph, s)
+        # FP32 evaluations of the same fitness: each within 1e-6 relative of it
+        assert torch.allclose(f, direct, rtol=2e-6, atol=0)
+        f.zero_()
+        torch.cuda.synchronize()
+        assert rt.cudaGraphLaunch(ex, ctypes.c_void_p(s.cuda_stream)) == 0
+        s.synchronize()
+        assert torch.allclose(f, direct, rtol=2e-6, atol=0)
+    assert gpu.leea_device_status() == 0
