@@ -41,7 +41,6 @@ struct MlpArgs {
     float alpha, x_div;
 };
 
-constexpr int kOnlyCtas = 152;  // CTAs of a launch for marked individuals: one per SM
 constexpr size_t kMlpSmemBytes =
     sizeof(float) * (2 * kMaxWidth * kActStride + 2 * kKC * kWStride + kTS * kLogitStride) + 64;
 
@@ -288,9 +287,11 @@ cudaError_t launch_mlp(const NetLayout& net, int32_t pop, const float* pop_dev, 
     if (err != cudaSuccess) return err;
     MlpArgs e = mlp_args(net, batch, alpha, x_div);
     e.pop = pop;
-    if (only)
-        return launch_pdl(eval_mlp_kernel<XT>, dim3(static_cast<unsigned>(std::min(pop, kOnlyCtas))), dim3(kMlpThreads),
-                          kMlpSmemBytes, stream, e, pop_dev, x, y, f_inh, f_raw, f_adj, correct, only);
+    if (only) {  // one CTA per SM
+        const unsigned grid = static_cast<unsigned>(std::max(1, std::min(pop, sm_count())));
+        return launch_pdl(eval_mlp_kernel<XT>, dim3(grid), dim3(kMlpThreads), kMlpSmemBytes, stream, e, pop_dev, x, y,
+                          f_inh, f_raw, f_adj, correct, only);
+    }
     eval_mlp_kernel<XT><<<pop, kMlpThreads, kMlpSmemBytes, stream>>>(e, pop_dev, x, y, f_inh, f_raw, f_adj, correct,
                                                                     nullptr);
     return cudaGetLastError();

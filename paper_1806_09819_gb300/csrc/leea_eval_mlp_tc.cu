@@ -937,13 +937,6 @@ uint32_t level_tile_bytes(const NetLayout& net)
     return static_cast<uint32_t>((net.dims[0] + 63) / 64) * kBlockBytes;
 }
 
-int sm_count()
-{
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    return cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? sms : 0;
-}
-
 // Scratch layout, each part a multiple of 256 bytes: the pieces, the marks, the
 // level tiles, the sums of shared individuals.
 struct MlpScratch {

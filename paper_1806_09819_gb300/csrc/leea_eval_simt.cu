@@ -21,7 +21,6 @@ namespace leea {
 constexpr int kEvalThreads = 256;  // 16 x 16 thread grid
 constexpr int kBK = 16;
 constexpr int kMaxOut = 32;
-constexpr int kOnlyCtas = 304;  // CTAs of a launch for marked individuals: two per SM
 
 struct EvalSimtArgs {
     int32_t d_in, h, d_out, batch;
@@ -263,8 +262,9 @@ static cudaError_t launch_simt_t(const EvalSimtArgs& e, int32_t pop, const float
             const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                          static_cast<int>(smem));
             if (err != cudaSuccess) return err;
-            return launch_pdl(kernel, dim3(static_cast<unsigned>(std::min(pop, kOnlyCtas))), dim3(kEvalThreads), smem,
-                              stream, e, popv, x, y, f_inh, f_raw, f_adj, correct);
+            const unsigned grid = static_cast<unsigned>(std::max(1, std::min(pop, 2 * sm_count())));  // two per SM
+            return launch_pdl(kernel, dim3(grid), dim3(kEvalThreads), smem, stream, e, popv, x, y, f_inh, f_raw, f_adj,
+                              correct);
         }
     }
     const auto kernel = eval_simt_kernel<TM, TN, XT, false>;

@@ -1123,14 +1123,16 @@ static bool in_tensor_shapes(const NetLayout& net, int32_t batch)
 // samples: 58 and 63 us).
 static bool pieces_pay(const NetLayout& net, int32_t pop, int32_t batch, int32_t xp)
 {
-    constexpr double kSms = 152.0, kPiecesUs = 25.0, kPairUs = 4.8;
+    constexpr double kPiecesUs = 25.0, kPairUs = 4.8;
+    const double sms = sm_count();
+    if (sms < 1.0) return false;
     const double k = net.dims[0], h = net.dims[1], b = batch;
     if (xp == 2) {
         const double wave = std::ceil(b / 128.0) * (2.5 + 0.085 * h + (0.011 + 0.00013 * h) * k);
-        return std::ceil(pop / kSms) * wave >= kPiecesUs;
+        return std::ceil(pop / sms) * wave >= kPiecesUs;
     }
     const double wave = std::ceil(h / 128.0) * std::ceil(b / 64.0) * (5.0 + 0.08 * k) * (h <= 32.0 ? 0.5 : 1.0);
-    return wave >= kPairUs && std::ceil(pop / (2.0 * kSms)) * wave >= kPiecesUs;
+    return wave >= kPairUs && std::ceil(pop / (2.0 * sms)) * wave >= kPiecesUs;
 }
 
 static bool pieces_fit(const NetLayout& net, int32_t pop, int32_t batch, const float* pop_dev, int32_t xp)

@@ -9,6 +9,14 @@ namespace leea {
 
 constexpr int kMaxLayers = 15;
 
+// SMs of the current device, 0 if there is none.
+inline int sm_count()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    return cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? sms : 0;
+}
+
 // Launches `kernel` with programmatic stream serialisation: its CTAs may be
 // scheduled while the previous kernel on the stream finishes, so the kernel
 // must wait (griddepcontrol.wait) before it reads that kernel's results.
