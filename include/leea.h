@@ -299,10 +299,11 @@ leea_status leea_breed_evaluate_u8(int32_t pop, const int32_t* dims, int32_t n_d
  * inputs and three hidden layers (widths multiples of 16 in [16, 256],
  * d_0 % 4 == 0, d_0 <= 256, d_out <= 16, 4-byte aligned x), the
  * tensor cores (AUTO or TENSOR): FP16 operand pieces of 2^8 w and 2^8 h
- * (hi.hi + hi.lo + lo.hi; the levels are exact), FP32 accumulation, FP32
- * bias, ReLU, last layer and loss; an individual with a weight or activation
- * |v| >= 128 is recomputed in FP32 on the CUDA cores.  That path splits the
- * weights and converts the batch into a library-owned scratch buffer (388 KB
+ * (hi.hi + hi.lo + lo.hi; the levels are exact) for the hidden layers, FP32
+ * accumulation, FP32 bias, ReLU, last layer and loss; an individual with a weight
+ * of the hidden layers, or an activation of the first two, of |v| >= 128 is
+ * recomputed in FP32 on the CUDA cores.  That path splits the
+ * weights and converts the batch into a library-owned scratch buffer (384 KB
  * per individual for 196-256-128-64-10, plus 68 KB per 128 samples), one per
  * device, shared by these step calls on that device, so such calls must not
  * overlap on one device; growing it frees the old buffer (which synchronises

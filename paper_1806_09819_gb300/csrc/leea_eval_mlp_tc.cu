@@ -2,38 +2,48 @@
 // as the paper's 196-256-128-64-10 (Section 4.1), on the tcgen05 tensor cores
 // with FP32-class accuracy, for minibatches of 8-bit levels x = k / x_div.
 //
-// A unit is one individual on one 128-sample tile.  All four layers are MMAs
-// with the samples as M = 128 and FP32 accumulation in tensor memory:
+// A unit is one individual on one 128-sample tile.  The three hidden layers are
+// MMAs with the samples as M = 128 and FP32 accumulation in tensor memory:
 //   layer 1     A = the tile's levels k, exact in FP16; B = 2^8 W1 as two FP16
 //               pieces hi = fp16(2^8 w), lo = fp16(2^8 w - hi) (the remainder is
 //               exact in FP32): 2 MMAs per 16 inputs, only the accumulation rounds
-//   layers 2-4  A = 2^8 h of the layer below and B = 2^8 W, both as two FP16
-//               pieces: hi.hi + lo.hi + hi.lo; the dropped lo.lo term is below
-//               2^-21 of the product (their order: kFewSamples)
+//   layers 2, 3 A = 2^8 h of the layer below and B = 2^8 W, both as two FP16
+//               pieces: lo.hi + hi.lo + hi.hi, in this order; the dropped lo.lo
+//               term is below 2^-21 of the product
+//   layer 4     FP32 FFMA on the CUDA cores, from FP32 weights and activations
 // The epilogue adds the bias and applies ReLU in FP32 and splits the activations
 // for the next layer; the softmax cross-entropy is FP32, losses are summed in
-// FP64.  A weight or an activation with |v| >= 128 (2^8 |v| could overflow its
-// FP16 piece) marks the individual; the CUDA-core kernel then recomputes its
-// fitness in FP32.  The weights are split once per evaluation
+// FP64.  A weight of layers 1 to 3 or an activation of layers 1 and 2 with |v| >=
+// 128 (2^8 |v| could overflow its FP16 piece) marks the individual; the CUDA-core
+// kernel then recomputes its fitness in FP32.  The weights are split once per evaluation
 // (split_weights_kernel), and the batch's levels are converted once per
 // evaluation into FP16 operand tiles (stage_levels_kernel).
+//
+// Error against 64 bits, RMS of the fitness of 600 nets, relative to the kernel that
+// kept the small products of layers 2 and 3 in accumulators of their own and summed
+// losses in FP32: initial nets 0.95 at 8 samples, 0.68 at 128, 0.61 at 1024; with
+// steps of 0.03 on every weight 0.98, 0.84 and 0.70; weights twice as large 1.58.
+// (In order of K, and with layer 4 as pieces too: 0.93, 0.83, 0.68; 1.08, 1.13,
+// 0.89; 2.5.)
 //
 // Where activations live.  A layer's activations are the A operand of the next
 // layer in tensor memory: 16 FP32 accumulator columns become 8 columns of hi
 // and 8 of lo pieces in place, so shared memory holds nothing but the tile's
-// levels and a ring of 32 KB weight slots.  Where all layers have their own
-// columns (mlp_columns) the next unit's layer 1 runs before and after this
-// unit's layer 3, under the epilogue of layers 2 and 3.  A CTA takes a
+// levels, a ring of 32 KB weight slots and W4.  Where the layers have columns of
+// their own (mlp_columns) the next unit's layer 1 runs before and after this
+// unit's layer 3, under the epilogue of layer 2 and layer 4.  A CTA takes a
 // contiguous range of units; the tiles' sums of an individual that several CTAs
 // share meet in scratch memory (combine_mlp_parts_kernel).
 //
-// Measured, 2000 nets 196-256-128-64-10 on 1024 samples: 945 us (1518 with the
-// activations in shared memory and two weight buffers), 207 of them the splitting
-// (1.5 GB, at the memory's rate); 512 samples 607, 128 375; 16 nets on 1024
-// samples 42.  The staging, this kernel and the one for the marked individuals are
-// each launched before their predecessor has ended and wait for it on the device:
-// 152 nets on 30 samples 42 us (51 without, 49 before), 2000 on 8 364 (368).
-// What bounds it: a unit takes 13k cycles, its MMAs 7.3k at the
+// Measured, 2000 nets 196-256-128-64-10 on 1024 samples: 922 us (930 with layer 4 on
+// the tensor cores, 1518 with the activations in shared memory and two weight
+// buffers), 207 of them the splitting (1.5 GB, at the memory's rate); 512 samples
+// 584, 128 362; 16 nets on 1024 samples 32.  The staging, this kernel and the one
+// for the marked individuals are each launched before their predecessor has ended
+// and wait for it on the device: 152 nets on 30 samples 44 us (52 without),
+// 2000 on 8 361.  A last layer of 256 x 16 is dearer on the CUDA cores: 300 nets
+// 256-256-256-256-16 on 512 samples 252 us (234).
+// What bounds it: a unit takes 12.8k cycles, its MMAs 7.2k at the
 // tensor peak (weights 448 KB of L2 reads, 3.4k-6k cycles, are hidden).  The rest
 // is the chain of a unit: layer 1's accumulator to the first activations 1-2k,
 // the restart of the MMAs after layer 2 0.5k, and the issuing warp's waits
@@ -44,13 +54,13 @@
 // Warp roles (persistent CTA, one per SM):
 //   warp 0      TMEM allocation and MMA issue (see mma_f16_lo)
 //   warp 1      producer: per unit, the tile's levels (one bulk copy) and the
-//               weight slots of W1 to W4 in the order of the MMAs, already split
+//               weight slots of W1 to W3 in the order of the MMAs, already split
 //               into FP16 pieces and swizzled by split_weights_kernel
-//   warp 2      the next individual's biases into one of two buffers
+//   warp 2      the next individual's biases and W4 into one of two buffers
 //   warps 3-10  the epilogue (TMEM lane = sample, two warps per lane quarter,
 //               each with half of every 64-column block): the activations of
-//               layers 1 to 3.  Layer 1's go to the layer-2 MMAs a block at a time
-//   warps 11-14 the loss from layer 4's accumulator, a sample per thread, while
+//               layers 1 and 2.  Layer 1's go to the layer-2 MMAs a block at a time
+//   warps 11-14 layer 4 and the loss from layer 3's accumulator (quad_logits), while
 //               the others are at the next unit
 // Every wait is bounded; on expiry the kernel sets kStatusEvalTimeout and exits.
 #include <cuda.h>
@@ -61,6 +71,7 @@
 #include <mutex>
 
 #include "leea_internal.h"
+#include "quad_logits.cuh"
 #include "tc_ptx.cuh"
 
 namespace leea {
@@ -78,14 +89,6 @@ constexpr int kTile = 128;                      // samples per unit (MMA M)
 constexpr uint32_t kBlockBytes = kTile * 128;   // one 64-input block of a 128-row operand
 constexpr uint32_t kSlotBytes = 256 * 128;      // a weight slot: 256 rows of 64 FP16 values
 constexpr int kMaxSlots = 8;
-// Up to here (FEW) the small products of a layer come first.  RMS error of the fitness
-// against 64 bits, 600 initial nets 196-256-128-64-10, in order of K / small
-// products first / with layer 4 in FFMA on the CUDA cores and the small products
-// in accumulators of their own: 8 samples 6.9e-8 / 5.3e-8 / 5.3e-8, 16 4.8 / 4.1 /
-// 4.9, 32 4.4 / 3.8 / 4.8, 128 4.0 / 3.5 / 4.7, 1024 3.7 / 3.3 / 5.2.
-// On so few samples that costs 152 nets 44.5 us (42.4), 2000 nets 0.5 %.  The line
-// lies below 16, from where on the order of K is no worse than the third.
-constexpr int kFewSamples = 15;
 constexpr int kMaxOutTc = 16;
 constexpr uint32_t kTmemCols = 512;
 constexpr float kPieceScale = 256.0f;
@@ -93,19 +96,19 @@ constexpr float kPieceRange = 128.0f;
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 constexpr uint64_t kDrainLimitNs = 200000000ull;
 
-// The weights of layer l (0-3) as slots of slot_bytes[l], one bulk copy each,
-// of 128-byte rows (64 FP16 values, swizzled).  Stacked layers (N <= 128; layer 4 has
-// N = 16, rows past d_out zero): slot kb holds block kb's hi rows, then its lo
+// The weights of layer l (0-2) as slots of slot_bytes[l], one bulk copy each,
+// of 128-byte rows (64 FP16 values, swizzled).  Stacked layers (N <= 128): slot kb
+// holds block kb's hi rows, then its lo
 // rows.  Else slot 2 kb is block kb's hi piece and slot 2 kb + 1 its lo piece;
 // layer 1's last block, if it has at most 32 inputs, is one slot whose rows hold
 // the hi inputs and then the lo ones.
 struct MlpSlots {
-    int32_t k16[4];      // inputs rounded up to 16
-    int32_t n[4];        // rows: the layer's width, 16 for layer 4
-    int32_t slots[4];
-    uint32_t slot_bytes[4];
-    int64_t layer_off[4];
-    bool stacked[4], tail_joined;
+    int32_t k16[3];      // inputs rounded up to 16
+    int32_t n[3];        // rows: the layer's width
+    int32_t slots[3];
+    uint32_t slot_bytes[3];
+    int64_t layer_off[3];
+    bool stacked[3], tail_joined;
 };
 
 struct MlpTcArgs {
@@ -113,14 +116,14 @@ struct MlpTcArgs {
     int32_t dims[5];     // d0, d1, d2, d3, d_out
     MlpSlots m;
     int32_t n_slots;     // ring depth
-    int32_t col[4];      // first accumulator column of each layer
+    int32_t col[3];      // first accumulator column of each layer
+    int32_t no4, wst;    // output groups of four; floats between W4's rows in shared memory
     bool early;          // all have their own columns: the next unit's layer 1 may start before layer 3
     int64_t c_pad;
     int64_t w_off[4], b_off[4];
     float inv_div;       // 2^-8 / x_div: layer-1 accumulator units to x units
     float alpha;
     const float* popv;
-    const uint8_t* x;
     const int32_t* y;
     const float* f_inh;
     float* f_raw;
@@ -142,24 +145,24 @@ struct MlpTcArgs {
 struct TcSmem {
     uint8_t* levels;
     uint8_t* ring;
-    float* param;     // [2]: b1, b2, b3 times 2^8, b4 of an individual
+    float* param;     // [2]: b1, b2, b3 times 2^8, b4, W4 (a row per hidden unit) of an individual
     double* red_loss;
-    uint64_t *full, *empty, *x_full, *d_full, *h_blk, *h_ready, *d4_read, *param_full, *param_empty, *red_full,
+    uint64_t *full, *empty, *x_full, *d_full, *h_blk, *h_ready, *d3_read, *param_full, *w4_full, *param_empty, *red_full,
         *drain;
     int32_t* red_ok;
     uint32_t* tmem_holder;
     volatile int* abort_flag;
 };
 
-__host__ __device__ inline uint32_t param_floats(const int32_t* dims)
+__host__ __device__ inline uint32_t param_floats(const int32_t* dims, int32_t wst)
 {
-    return static_cast<uint32_t>(dims[1] + dims[2] + dims[3] + kMaxOutTc);
+    return static_cast<uint32_t>(dims[1] + dims[2] + dims[3] + kMaxOutTc + dims[3] * wst);
 }
 
-__host__ __device__ inline size_t tc_smem_bytes(const int32_t* dims, uint32_t x_bytes, int n_slots)
+inline size_t tc_smem_bytes(const int32_t* dims, uint32_t x_bytes, int n_slots)
 {
-    return 1024 + x_bytes + static_cast<size_t>(n_slots) * kSlotBytes + 8 * param_floats(dims) + 8 * 8 +
-           8 * (2 * kMaxSlots + 18) + 4 * 10;
+    return 1024 + x_bytes + static_cast<size_t>(n_slots) * kSlotBytes + 8 * param_floats(dims, quad_row_floats(dims[4])) +
+           8 * 8 + 8 * (2 * kMaxSlots + 18) + 4 * 10;
 }
 
 // Ring depth that fits in shared memory.
@@ -177,17 +180,18 @@ __device__ __forceinline__ TcSmem carve(uint8_t* raw, const MlpTcArgs& a)
     s.ring = s.levels + a.x_bytes;
     float* f = reinterpret_cast<float*>(s.ring + static_cast<uint32_t>(a.n_slots) * kSlotBytes);
     s.param = f;
-    s.red_loss = reinterpret_cast<double*>(f + 2 * param_floats(a.dims));
+    s.red_loss = reinterpret_cast<double*>(f + 2 * param_floats(a.dims, a.wst));
     uint64_t* bars = reinterpret_cast<uint64_t*>(s.red_loss + 8);
     s.full = bars;
     s.empty = bars + kMaxSlots;
     bars += 2 * kMaxSlots;
     s.x_full = bars;
-    s.d_full = bars + 1;       // [4]: a layer's MMAs are done
-    s.h_blk = bars + 5;        // [4]: a 64-column block of layer 1's activations is in
-    s.h_ready = bars + 9;      // [2]: layer 2's, layer 3's activations are in
-    s.d4_read = bars + 11;     // layer 4's accumulator has been read
-    s.param_full = bars + 12;  // [2]
+    s.d_full = bars + 1;       // [3]: a layer's MMAs are done
+    s.h_blk = bars + 4;        // [4]: a 64-column block of layer 1's activations is in
+    s.h_ready = bars + 8;      // layer 2's activations are in
+    s.d3_read = bars + 9;      // layer 3's accumulator has been read
+    s.param_full = bars + 10;  // [2]: b1 and b2 are in
+    s.w4_full = bars + 12;     // [2]: b3, b4 and W4 are in
     s.param_empty = bars + 14; // [2]
     s.red_full = bars + 16;
     s.drain = bars + 17;
@@ -232,20 +236,19 @@ __device__ __forceinline__ uint32_t swz(int r, int ch)
 
 __device__ __forceinline__ int layer_blocks(const MlpTcArgs& a, int l) { return (a.m.k16[l] + 63) / 64; }
 
-// Accumulator columns.  Layer 1 in [0, d1), layer 2 in the d2 columns after it,
-// layer 3 and the 16 of layer 4 after those where they end by column 512
-// ("early": 196-256-128-64-10 uses 464); activations replace their accumulator.
-// Otherwise layer 2 ends at column 512, layer 3 takes layer 1's place, from
-// column 0 (layer 2 then starts at 256 or later), and layer 4 layer 2's, so the
-// next unit's layer 1 waits until layer 4 is read.
+// Accumulator columns.  Layer 1 in [0, d1), layer 2 in the d2 columns after it and
+// layer 3 after those where it ends by column 512 ("early": 196-256-128-64-10 uses
+// 448); the activations of layers 1 and 2 replace their accumulator.  Otherwise
+// layer 2 ends at column 512 and layer 3 takes layer 1's place, from column 0
+// (layer 2 then starts at 256 or later), so the next unit's layer 1 waits until
+// layer 3 is read.
 void mlp_columns(MlpTcArgs* a)
 {
     const int32_t d1 = a->dims[1], d2 = a->dims[2], d3 = a->dims[3], cols = static_cast<int32_t>(kTmemCols);
-    a->early = d1 + d2 + d3 + kMaxOutTc <= cols;
+    a->early = d1 + d2 + d3 <= cols;
     a->col[0] = 0;
     a->col[1] = a->early ? d1 : cols - d2;
     a->col[2] = a->early ? d1 + d2 : 0;
-    a->col[3] = a->early ? d1 + d2 + d3 : cols - d2;
 }
 
 // Bias, ReLU and split of 16 accumulator columns r, written to taddr in place:
@@ -386,7 +389,7 @@ struct Splitter {
                 ++l;
             }
         }
-        return l < 4;
+        return l < 3;
     }
     __device__ __forceinline__ bool outside() const { return top >= kPieceRange; }
 };
@@ -399,7 +402,6 @@ __device__ __forceinline__ void store_fitness(const MlpTcArgs& a, int p, double 
     if (a.correct) a.correct[p] = good;
 }
 
-template <bool FEW>
 __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid_constant__ MlpTcArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -412,12 +414,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
             ptx::mbar_init(&s.empty[i], 1);
         }
         ptx::mbar_init(s.x_full, 1);
-        for (int i = 0; i < 4; ++i) ptx::mbar_init(&s.d_full[i], 1);
+        for (int i = 0; i < 3; ++i) ptx::mbar_init(&s.d_full[i], 1);
         for (int i = 0; i < 4; ++i) ptx::mbar_init(&s.h_blk[i], kEpiWarps);
-        for (int i = 0; i < 2; ++i) ptx::mbar_init(&s.h_ready[i], kEpiWarps);
-        ptx::mbar_init(s.d4_read, kLossWarps);
+        ptx::mbar_init(s.h_ready, kEpiWarps);
+        ptx::mbar_init(s.d3_read, kLossWarps);
         for (int i = 0; i < 2; ++i) {
             ptx::mbar_init(&s.param_full[i], 1);
+            ptx::mbar_init(&s.w4_full[i], 1);
             ptx::mbar_init(&s.param_empty[i], kEpiWarps + kLossWarps);
         }
         ptx::mbar_init(s.red_full, kLossWarps);
@@ -480,23 +483,21 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                 }
                 if (j1 == a.m.slots[0] && lead) ptx::mma_commit(&s.d_full[0]);
             };
-            // Unit u's layer l = 1, 2, 3, its A operand in the columns of the layer before.
+            // Unit u's layer l = 1, 2, its A operand in the columns of the layer before.
             auto later = [&](uint32_t u, int l) {
                 const uint32_t n = static_cast<uint32_t>(a.m.n[l]);
                 const uint32_t idesc = ptx::idesc_f16(kTile, n);
                 const uint32_t act = tmem_base + static_cast<uint32_t>(a.col[l - 1]);
                 const uint32_t d = tmem_base + static_cast<uint32_t>(a.col[l]);
                 const bool stacked = a.m.stacked[l];
-                if (l >= 2 && !wait(&s.h_ready[l - 2], u & 1u)) return;
+                if (l == 2 && !wait(s.h_ready, u & 1u)) return;
                 ptx::tc_fence_after();
                 // The tensor core truncates every sum, to the size of what the accumulator
-                // holds by then.  With few samples, whose errors the fitness averages
-                // least, the small products lo.hi and hi.lo therefore come before hi.hi:
-                // per slot, and in layers 3 and 4, whose A operand is complete, over all
-                // slots, which the ring then holds at once (for the paper net on 1024
-                // samples 7 % of the time, and 2 % just by the longer code).
-                if (FEW && stacked) {
-                    const bool all = l >= 2 && a.m.slots[l] <= a.n_slots;
+                // holds by then, so the small products lo.hi and hi.lo come before hi.hi:
+                // per slot, and in layer 3, whose A operand is complete, over all slots,
+                // which the ring then holds at once.
+                if (stacked) {
+                    const bool all = l == 2 && a.m.slots[l] <= a.n_slots;
                     const int slots = a.m.slots[l], group = all ? slots : 1;
                     for (int j0 = 0; j0 < slots; j0 += group) {
                         if (l == 1 && !wait(&s.h_blk[j0], u & 1u)) return;
@@ -531,7 +532,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                     return;
                 }
                 for (int j = 0; j < a.m.slots[l]; ++j) {
-                    const int kb = stacked ? j : j >> 1, lo = stacked ? 0 : j & 1;
+                    const int kb = j >> 1, lo = j & 1;
                     if (l == 1 && lo == 0 && !wait(&s.h_blk[kb], u & 1u)) return;
                     if (!wait(&s.full[slot], phase)) return;
                     if (l == 1) ptx::tc_fence_after();
@@ -539,21 +540,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                     const uint32_t a_hi = act + 64u * static_cast<uint32_t>(kb);
                     const uint32_t acc = j == 0 ? 0u : 1u;
                     const int steps = min(4, (a.m.k16[l] - 64 * kb) / 16);
-                    if (stacked) {
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                                if (kk >= steps) break;
-                            ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk, b + 2u * kk, hi, idesc, kk == 0 ? acc : 1u, lead);
-                            ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk + 8u, b + 2u * kk, hi, idesc, 1u, lead);
-                            ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk, b + 8u * n + 2u * kk, hi, idesc, 1u, lead);
-                        }
-                    } else {
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                                if (kk >= steps) break;
-                            ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk, b + 2u * kk, hi, idesc, kk == 0 ? acc : 1u, lead);
-                            if (!lo) ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk + 8u, b + 2u * kk, hi, idesc, 1u, lead);
-                        }
+                    for (int kk = 0; kk < 4; ++kk) {
+                        if (kk >= steps) break;
+                        ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk, b + 2u * kk, hi, idesc, kk == 0 ? acc : 1u, lead);
+                        if (!lo) ptx::mma_f16_tmem_a_lo(d, a_hi + 16u * kk + 8u, b + 2u * kk, hi, idesc, 1u, lead);
                     }
                     next_slot();
                 }
@@ -570,16 +561,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                         wait(&s.d_full[1], u & 1u);  // layer 1 overwrites layer 2's operand
                         if (ok) layer1(u + 1, 0, cut);
                     }
-                    if (ok && u > 0) wait(&s.d_full[3], (u - 1) & 1u);  // layer 3 overwrites layer 4's operand
+                    if (ok && u > 0) wait(s.d3_read, (u - 1) & 1u);
                     if (ok) later(u, 2);
                     if (ok && more) layer1(u + 1, cut, a.m.slots[0]);
-                    if (ok && u > 0) wait(s.d4_read, (u - 1) & 1u);
-                    if (ok) later(u, 3);
                 } else {
                     if (ok) later(u, 2);
-                    if (ok) wait(&s.d_full[2], u & 1u);  // layer 4 overwrites layer 3's operand
-                    if (ok) later(u, 3);
-                    if (ok && more) wait(s.d4_read, u & 1u);
+                    if (ok && more) wait(s.d3_read, u & 1u);
                     if (ok && more) layer1(u + 1, 0, a.m.slots[0]);
                 }
             }
@@ -635,10 +622,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                     if (ok && more) load(x.seg.p, 0, 0, cut);
                     if (ok) load(p, 2, 0, a.m.slots[2]);
                     if (ok && more) load(x.seg.p, 0, cut, a.m.slots[0]);
-                    if (ok) load(p, 3, 0, a.m.slots[3]);
                 } else {
                     if (ok) load(p, 2, 0, a.m.slots[2]);
-                    if (ok) load(p, 3, 0, a.m.slots[3]);
                     if (ok && more) load(x.seg.p, 0, 0, a.m.slots[0]);
                 }
             }
@@ -651,7 +636,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
             }
         }
     } else if (warp < kFirstEpiWarp) {
-        // ------------------------------------------------------------ biases
+        // ------------------------------------------------------------ biases and W4
         const int d1 = a.dims[1], d2 = a.dims[2], d3 = a.dims[3], d_out = a.dims[4];
         auto wait = [&](uint64_t* bar, uint32_t parity) {
             const bool got = ptx::mbar_wait_sleeping(bar, parity, s.abort_flag, kWaitLimitNs, 200u);
@@ -664,19 +649,32 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
             {
                 if (!wait(&s.param_empty[k & 1u], ((k >> 1) & 1u) ^ 1u)) break;
                 const float* net = a.popv + static_cast<int64_t>(seg.p) * a.c_pad;
-                float* b = s.param + (k & 1u) * param_floats(a.dims);
+                float* b = s.param + (k & 1u) * param_floats(a.dims, a.wst);
                 for (int e = lane; e < d1; e += 32) b[e] = net[a.b_off[0] + e] * kPieceScale;
                 for (int e = lane; e < d2; e += 32) b[d1 + e] = net[a.b_off[1] + e] * kPieceScale;
-                for (int e = lane; e < d3; e += 32) b[d1 + d2 + e] = net[a.b_off[2] + e] * kPieceScale;
-                if (lane < kMaxOutTc) b[d1 + d2 + d3 + lane] = lane < d_out ? net[a.b_off[3] + lane] : 0.0f;
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(&s.param_full[k & 1u]);
+                for (int e = lane; e < d3; e += 32) b[d1 + d2 + e] = net[a.b_off[2] + e] * kPieceScale;
+                if (lane < kMaxOutTc) b[d1 + d2 + d3 + lane] = lane < d_out ? net[a.b_off[3] + lane] : 0.0f;
+                float* w4t = b + d1 + d2 + d3 + kMaxOutTc;
+                for (int col = lane; col < d3; col += 32) {
+                    float w[kMaxOutTc];  // all in flight at once
+#pragma unroll
+                    for (int o = 0; o < kMaxOutTc; ++o) w[o] = o < d_out ? net[a.w_off[3] + o * d3 + col] : 0.0f;
+#pragma unroll
+                    for (int o4 = 0; o4 < kMaxOutTc / 4; ++o4)
+                        if (o4 < a.no4)
+                            *reinterpret_cast<float4*>(w4t + col * a.wst + 4 * o4) =
+                                make_float4(w[4 * o4], w[4 * o4 + 1], w[4 * o4 + 2], w[4 * o4 + 3]);
+                }
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(&s.w4_full[k & 1u]);
             }
             seg.step(a);
         }
     } else {
         const int d1 = a.dims[1], d2 = a.dims[2], d3 = a.dims[3], d_out = a.dims[4];
-        const int q = warp & 3, row = q * 32 + lane;
+        const int q = warp & 3;
         auto wait = [&](uint64_t* bar, uint32_t parity) {
             const bool got = ptx::mbar_wait_sleeping(bar, parity, s.abort_flag, kWaitLimitNs, 20u);
             if (__all_sync(0xFFFFFFFFu, got)) return true;
@@ -695,8 +693,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
             const uint32_t acc = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
             const float scale1 = a.inv_div * kPieceScale;
             for (Segments seg(a, blockIdx.x); ok && seg.valid(); seg.step(a), ++k) {
-                const float* b1 = s.param + (k & 1u) * param_floats(a.dims);
-                const float *b2 = b1 + d1, *b3 = b2 + d2;
+                const float* b1 = s.param + (k & 1u) * param_floats(a.dims, a.wst);
+                const float* b2 = b1 + d1;
                 if (!wait(&s.param_full[k & 1u], (k >> 1) & 1u)) break;
                 __half2 top = __float2half2_rn(0.0f);  // the largest hi pieces: activations times 2^8
                 for (int t = seg.t0; t < seg.t1; ++t, ++u) {
@@ -709,18 +707,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                         ptx::tc_fence_before();
                         arrive(&s.h_blk[kb]);
                     }
-                    // layers 2 and 3
-                    for (int l = 1; ok && l < 3; ++l) {
-                        if (!(ok = wait(&s.d_full[l], u & 1u))) break;
-                        ptx::tc_fence_after();
-                        for (int c = kPartCols * part; c < a.dims[l + 1]; c += 64)
-                            activate_part(acc + static_cast<uint32_t>(a.col[l]), c, a.dims[l + 1], 1.0f / kPieceScale,
-                                          l == 1 ? b2 : b3, top);
-                        ptx::tmem_st_wait();
-                        ptx::tc_fence_before();
-                        arrive(&s.h_ready[l - 1]);
-                    }
-                    if (!ok) break;
+                    // layer 2
+                    if (!(ok = wait(&s.d_full[1], u & 1u))) break;
+                    ptx::tc_fence_after();
+                    for (int c = kPartCols * part; c < d2; c += 64)
+                        activate_part(acc + static_cast<uint32_t>(a.col[1]), c, d2, 1.0f / kPieceScale, b2, top);
+                    ptx::tmem_st_wait();
+                    ptx::tc_fence_before();
+                    arrive(s.h_ready);
                 }
                 if (!ok) break;
                 arrive(&s.param_empty[k & 1u]);
@@ -729,22 +723,27 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                     a.flagged[seg.p] = 1;
             }
         } else {
-            // -------------------------------------------------------- loss, one sample per thread
+            // -------------------------------------------------------- layer 4 and the loss, one sample per thread
             for (Segments seg(a, blockIdx.x); ok && seg.valid(); seg.step(a), ++k) {
-                const float* b4 = s.param + (k & 1u) * param_floats(a.dims) + d1 + d2 + d3;
-                if (!wait(&s.param_full[k & 1u], (k >> 1) & 1u)) break;
+                const float* b3 = s.param + (k & 1u) * param_floats(a.dims, a.wst) + d1 + d2;
+                const float *b4 = b3 + d3, *w4t = b4 + kMaxOutTc;
+                if (!wait(&s.w4_full[k & 1u], (k >> 1) & 1u)) break;
                 const bool whole = seg.t0 == 0 && seg.t1 == a.n_tiles;
                 double total = 0.0;  // warp q = 0, lane 0: the tiles so far, in their order
                 int32_t total_ok = 0;
                 for (int t = seg.t0; t < seg.t1; ++t, ++u) {
-                    const int smp = t * kTile + row;
+                    const int smp = t * kTile + q * 32 + 8 * (lane & 3) + (lane >> 2);
                     const int32_t lbl = smp < a.batch ? a.y[smp] : 0;
-                    if (!(ok = wait(&s.d_full[3], u & 1u))) break;
+                    if (!(ok = wait(&s.d_full[2], u & 1u))) break;
                     ptx::tc_fence_after();
+                    // 2^8 h of layer 3 in FP32, W4 in FP32: logits times 2^8.
+                    constexpr float kInv = 1.0f / kPieceScale;
+                    const float scale[4] = { kInv, kInv, kInv, kInv };
                     float z[kMaxOutTc];
-                    ptx::tmem_ld16(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(a.col[3]), z);
+                    quad_logits(a.no4, tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(a.col[2]), d3,
+                                scale, b3, w4t, a.wst, z);
                     ptx::tc_fence_before();
-                    arrive(s.d4_read);
+                    arrive(s.d3_read);
                     double loss = 0.0;
                     int32_t n_ok = 0;
                     float zmax = 0.0f, zl = 0.0f;
@@ -752,7 +751,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
 #pragma unroll
                     for (int o = 0; o < kMaxOutTc; ++o) {
                         if (o < d_out) {
-                            z[o] = fmaf(z[o], 1.0f / (kPieceScale * kPieceScale), b4[o]);
+                            z[o] = fmaf(z[o], kInv, b4[o]);
                             if (o == 0 || z[o] > zmax) { zmax = z[o]; arg = o; }
                             if (o == lbl) zl = z[o];
                         }
@@ -841,7 +840,7 @@ __global__ void __launch_bounds__(256) combine_mlp_parts_kernel(const MlpTcArgs 
     store_fitness(a, p, sum, good);
 }
 
-// Each individual's weights of layers 1-3 as FP16 pieces of 2^8 w in the
+// Each individual's weights of layers 1 to 3 as FP16 pieces of 2^8 w in the
 // swizzled operand layout (blockIdx.x: the 64-input block); a weight |w| >= 128
 // marks the individual for the FP32 recomputation.
 __global__ void __launch_bounds__(256) split_weights_kernel(const MlpTcArgs a)
@@ -916,8 +915,8 @@ uint8_t* shared_scratch(size_t bytes)
 int64_t piece_layout(const NetLayout& net, MlpSlots* m)
 {
     int64_t off = 0;
-    for (int l = 0; l < 4; ++l) {
-        const int32_t k16 = (net.dims[l] + 15) / 16 * 16, n = l < 3 ? net.dims[l + 1] : kMaxOutTc, tail = k16 % 64;
+    for (int l = 0; l < 3; ++l) {
+        const int32_t k16 = (net.dims[l] + 15) / 16 * 16, n = net.dims[l + 1], tail = k16 % 64;
         m->k16[l] = k16;
         m->n[l] = n;
         m->stacked[l] = l > 0 && 2 * n <= 256;
@@ -974,7 +973,7 @@ bool eval_mlp_tc_supported(const NetLayout& net, const float* pop_dev)
     if (d0 % 4 != 0 || d0 > 256 || d_out > kMaxOutTc) return false;
     for (int32_t n : { d1, d2, d3 })
         if (n % 16 != 0 || n < 16 || n > 256) return false;
-    for (int l = 0; l < 4; ++l)
+    for (int l = 0; l < 3; ++l)
         if (net.w_off[l] % 4 != 0) return false;
     if (reinterpret_cast<uintptr_t>(pop_dev) & 15u) return false;
     return mlp_ring(net.dims, (d0 + 63) / 64 * kBlockBytes) >= 2;
@@ -998,7 +997,6 @@ cudaError_t launch_eval_mlp_tc(const NetLayout& net, int32_t pop, const float* p
     a.inv_div = static_cast<float>(1.0 / (static_cast<double>(x_div) * kPieceScale));
     a.alpha = alpha;
     a.popv = pop_dev;
-    a.x = x;
     a.y = y;
     a.f_inh = f_inh;
     a.f_raw = f_raw;
@@ -1007,6 +1005,8 @@ cudaError_t launch_eval_mlp_tc(const NetLayout& net, int32_t pop, const float* p
     a.status = status;
     a.piece_stride = piece_layout(net, &a.m);
     mlp_columns(&a);
+    a.no4 = (a.dims[4] + 3) / 4;
+    a.wst = quad_row_floats(a.dims[4]);
     const MlpScratch sc = mlp_scratch_layout(net, pop, batch);
     uint8_t* base = static_cast<uint8_t*>(scratch ? scratch : shared_scratch(sc.bytes));
     if (!base) return cudaErrorMemoryAllocation;
@@ -1024,7 +1024,7 @@ cudaError_t launch_eval_mlp_tc(const NetLayout& net, int32_t pop, const float* p
     if (err != cudaSuccess) return err;
     {
         int blocks = 0;
-        for (int l = 0; l < 4; ++l) blocks += (a.m.k16[l] + 63) / 64;
+        for (int l = 0; l < 3; ++l) blocks += (a.m.k16[l] + 63) / 64;
         split_weights_kernel<<<dim3(blocks, pop < 65535 ? pop : 65535), 256, 0, stream>>>(a);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         const int level_items = a.n_tiles * ((a.dims[0] + 63) / 64) * kTile * 8;
@@ -1033,10 +1033,9 @@ cudaError_t launch_eval_mlp_tc(const NetLayout& net, int32_t pop, const float* p
     }
     a.n_slots = mlp_ring(net.dims, a.x_bytes);
     const size_t smem = tc_smem_bytes(net.dims, a.x_bytes, a.n_slots);
-    const auto kernel = batch <= kFewSamples ? eval_mlp_tc_kernel<true> : eval_mlp_tc_kernel<false>;
-    err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    err = cudaFuncSetAttribute(eval_mlp_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (err != cudaSuccess) return err;
-    err = launch_pdl(kernel, dim3(sc.grid), dim3(kTcThreads), smem, stream, a);
+    err = launch_pdl(eval_mlp_tc_kernel, dim3(sc.grid), dim3(kTcThreads), smem, stream, a);
     if (err != cudaSuccess) return err;
     if (a.extra != 0 || a.per_cta % a.n_tiles != 0) {
         combine_mlp_parts_kernel<<<(pop + 255) / 256, 256, 0, stream>>>(a);

@@ -77,6 +77,7 @@
 #include <cuda_fp16.h>
 
 #include "leea_internal.h"
+#include "quad_logits.cuh"
 #include "tc_ptx.cuh"
 
 namespace leea {
@@ -163,15 +164,6 @@ struct U8Smem {
 constexpr size_t kTailFixed = 8 + sizeof(double) * 16 + sizeof(int32_t) * 16 + sizeof(uint32_t) * (8 + 2 * kFlagSlots + 2) +
                               sizeof(int) * 2 + 16 + 16;
 
-// Floats between the rows (a hidden unit's outputs) of W2 in shared memory: the
-// rows 0, 2, 4 and 6 that a quad reads together (quad_logits) fall on
-// different banks.
-int32_t w2_stride(int32_t d_out)
-{
-    const int32_t no4 = (d_out + 3) / 4;
-    return no4 == 2 ? 12 : (no4 == 4 ? 20 : 4 * no4);
-}
-
 size_t u8_tail_bytes(int32_t h, int32_t wst, int32_t n_stages)
 {
     return sizeof(float) * (2u * h * wst + 2u * h + 32u) + kTailFixed + 8u * (3u * n_stages + 5u);
@@ -245,7 +237,7 @@ uint32_t u8_stage_bytes(const U8Shape& u, int32_t batch)
 
 size_t u8_smem_bytes(const U8Shape& u, int32_t d_out, int32_t batch)
 {
-    return 1024 + static_cast<size_t>(u.n_stages) * u8_stage_bytes(u, batch) + u8_tail_bytes(u.hp, w2_stride(d_out), u.n_stages);
+    return 1024 + static_cast<size_t>(u.n_stages) * u8_stage_bytes(u, batch) + u8_tail_bytes(u.hp, quad_row_floats(d_out), u.n_stages);
 }
 
 // K stage and ring depth: 64 inputs when at least kMinStages such stages fit in
@@ -368,77 +360,6 @@ struct UnitWalk {
         return true;
     }
 };
-
-// Layer 2 of the 32 samples of a warp (TMEM lanes of col0) for the shapes beyond
-// TENSOR's: logits [4 O4, 4 O4 + 4 NO4) of one sample per lane, sample 8 (lane %
-// 4) + lane / 4 of the 32.  W2 comes from shared memory, which gives a warp that
-// reads one address 4 bytes a cycle; with a sample per lane the reads alone
-// (h x 12 floats per warp) take 10.7k cycles per 256 samples of a 112-10 net,
-// longer than its MMAs.  So a lane takes four samples and a quarter of the hidden
-// units (the 16x256b shape of the accumulator): the four lanes of a quad read
-// different rows of W2 in one go, each for four samples, a quarter of the
-// cycles, and their partial logits are added across the quad.
-template <int NO4, int O4>
-__device__ __forceinline__ void quad_logits(uint32_t col0, int hp, const float (&scale)[4], const float* b1s,
-                                            const float* w2t, int wst, float* z)
-{
-    const int lane = threadIdx.x & 31, m = lane & 3;
-    float2 acc[4][2 * NO4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int o = 0; o < 2 * NO4; ++o) acc[j][o] = make_float2(0.0f, 0.0f);
-    for (int c = 0; c < hp; c += 16) {
-        uint32_t v[16];
-        ptx::tmem_ld_16x256_nowait(col0 + static_cast<uint32_t>(c), v);
-        ptx::tmem_ld_16x256_nowait(col0 + (16u << 16) + static_cast<uint32_t>(c), v + 8);
-        ptx::tmem_ld_wait();
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const int col = c + 8 * half + 2 * m;
-            const float2 b = *reinterpret_cast<const float2*>(b1s + col);
-            float2 h[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int at = 8 * (j >> 1) + 4 * half + 2 * (j & 1);
-                h[j] = __ffma2_rn(make_float2(__uint_as_float(v[at]), __uint_as_float(v[at + 1])),
-                                  make_float2(scale[j], scale[j]), b);
-                h[j].x = fmaxf(h[j].x, 0.0f);
-                h[j].y = fmaxf(h[j].y, 0.0f);
-            }
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const float4* wr = reinterpret_cast<const float4*>(w2t + (col + e) * wst) + O4;
-#pragma unroll
-                for (int o = 0; o < NO4; ++o) {
-                    const float4 w = wr[o];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float hj = e ? h[j].y : h[j].x;
-                        acc[j][2 * o] = __ffma2_rn(make_float2(w.x, w.y), make_float2(hj, hj), acc[j][2 * o]);
-                        acc[j][2 * o + 1] = __ffma2_rn(make_float2(w.z, w.w), make_float2(hj, hj), acc[j][2 * o + 1]);
-                    }
-                }
-            }
-        }
-    }
-    // Lane m of a quad keeps row m: two of the four rows across lane ^ 2, one
-    // of those across lane ^ 1.
-    const bool up = m & 2, odd = m & 1;
-#pragma unroll
-    for (int o = 0; o < 2 * NO4; ++o) {
-        float2 keep[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const float2 give = up ? acc[j][o] : acc[2 + j][o], mine = up ? acc[2 + j][o] : acc[j][o];
-            keep[j].x = mine.x + __shfl_xor_sync(0xFFFFFFFFu, give.x, 2);
-            keep[j].y = mine.y + __shfl_xor_sync(0xFFFFFFFFu, give.y, 2);
-        }
-        const float2 give = odd ? keep[0] : keep[1], mine = odd ? keep[1] : keep[0];
-        z[4 * O4 + 2 * o] = mine.x + __shfl_xor_sync(0xFFFFFFFFu, give.x, 1);
-        z[4 * O4 + 2 * o + 1] = mine.y + __shfl_xor_sync(0xFFFFFFFFu, give.y, 1);
-    }
-}
 
 template <int KS, int TILES, int XP>
 __global__ void __launch_bounds__(kU8Threads, 1)
@@ -757,14 +678,7 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 }
                 float logit[kMaxOutU8];
                 if constexpr (kQuads) {
-                    switch (a.no4) {
-                    case 1: quad_logits<1, 0>(col0, a.hp, scale, b1s, w2t, a.wst, logit); break;
-                    case 2: quad_logits<2, 0>(col0, a.hp, scale, b1s, w2t, a.wst, logit); break;
-                    case 3: quad_logits<3, 0>(col0, a.hp, scale, b1s, w2t, a.wst, logit); break;
-                    default:
-                        quad_logits<2, 0>(col0, a.hp, scale, b1s, w2t, a.wst, logit);
-                        quad_logits<2, 2>(col0, a.hp, scale, b1s, w2t, a.wst, logit);
-                    }
+                    quad_logits(a.no4, col0, a.hp, scale, b1s, w2t, a.wst, logit);
                 } else {
                 const bool redo = XP == 1 && gov == 2 && !a.flagged;
                 const float* w1p = a.popv + static_cast<int64_t>(p) * a.c_pad;
@@ -1248,7 +1162,7 @@ cudaError_t launch_eval_u8_tc(const NetLayout& net, int32_t pop, const float* po
     a.batch = batch;
     a.k16 = (a.k + 15) / 16 * 16;
     a.no4 = (a.d_out + 3) / 4;
-    a.wst = w2_stride(a.d_out);
+    a.wst = quad_row_floats(a.d_out);
     a.k_stages = (a.k + ks - 1) / ks;
     a.n_stages = u.n_stages;
     a.hp = u.hp;

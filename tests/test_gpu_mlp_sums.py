@@ -2,7 +2,7 @@
 import numpy as np
 import pytest
 
-from helpers import to_device_pop
+from helpers import assert_fitness_close, to_device_pop
 
 pytestmark = pytest.mark.gpu
 
@@ -51,3 +51,21 @@ def test_twins_split_differently_among_ctas(gpu):
     total = ((3.0 * 2.0 ** 58 + 3.0 * 2.0 ** 34) + 64.0) + 64.0
     np.testing.assert_array_equal(f, np.full(pop, -np.float32(total / batch)))
     assert (cor == batch - 4).all()
+
+
+@pytest.mark.parametrize("batch", [5, 40, 200])
+def test_last_layer_is_fp32(gpu, oracle_mod, batch):
+    """Last-layer weights of 24 bits that nearly cancel in pairs: 64 (1 + 2^-12 + 2^-23) - 64 (1 + 2^-12), eight times, a
+    logit of 2^-14 that weights of 22 bits lose."""
+    dims = [16, 16, 16, 16, 2]
+    net = np.zeros(gpu.leea_layout_num_params(dims), dtype=np.float32)
+    b3 = 3 * (16 * 16 + 16) - 16
+    net[b3:b3 + 16] = 64.0  # layer 3's activations
+    w4 = net[b3 + 16:b3 + 16 + 32].reshape(2, 16)
+    w4[0, 0::2] = 1.0 + 2.0 ** -12 + 2.0 ** -23
+    w4[0, 1::2] = -(1.0 + 2.0 ** -12)
+    levels, y = np.full((batch, 16), 7, dtype=np.uint8), np.zeros(batch, dtype=np.int32)
+    f, _ = _evaluate(gpu, dims, to_device_pop(np.tile(net, (3, 1)), gpu.leea_padded_params(dims)), levels, y)
+    ref, _ = oracle_mod.evaluate(np.tile(net, (3, 1)).astype(np.float64), dims, levels.astype(np.float64) / 255.0, y)
+    assert abs(ref[0] + np.log1p(np.exp(-2.0 ** -14))) < 1e-12  # the oracle's sum of `batch` equal losses
+    assert_fitness_close(f, ref)
