@@ -660,16 +660,15 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 const int first = (x.t0 + t) * 128 + q * 32;  // the warp's samples
                 const int smp = first + (kQuads ? 8 * (lane & 3) + (lane >> 2) : lane);  // this thread's sample
                 const bool in = smp < a.batch;
-                const int32_t label = in ? a.y[smp] : 0;
+                const int32_t label = in ? ptx::ld_here(a.y + smp) : 0;  // in flight during layer 2
                 float loss = 0.0f;
-                unsigned good = 0;
+                unsigned good = 0;  // and marked samples from bit 16 on
                 const uint32_t col0 = tmem_base + lane_addr + buf * kAccStride + static_cast<uint32_t>(t) * tile_cols +
                                       static_cast<uint32_t>(slot * a.hp);
                 // Individuals with a weight outside the piece range are marked for the
                 // evaluation that follows or, within TENSOR's shapes on 8-bit levels, have
                 // layer 1 here by FP32 FFMA from global memory, k in order.
                 float scale[4];  // accumulator units to x units, per sample
-                bool marked = gov == 2;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int sj = kQuads ? first + 8 * j + (lane >> 2) : smp;
@@ -769,7 +768,7 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                         const float2 err = __ldcg(a.x_err + smp);
                         const float w_top = __uint_as_float(min(static_cast<uint32_t>(*go >> 8) + 1u, 254u) << 23);
                         const float reach = fmaf(err.y, w_top, err.x) * a.sqrt_h * w2_top(s, g);
-                        marked = marked || !(reach <= kMarkTol * fmaxf(fmaxf(fabsf(zmax), loss), 1.0f));
+                        if (!(reach <= kMarkTol * fmaxf(fmaxf(fabsf(zmax), loss), 1.0f))) good |= 1u << 16;
                     }
                 }
                 // Fixed-order sums: FP32 within TENSOR's shapes (the fused kernel
@@ -785,7 +784,7 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                     for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xFFFFFFFFu, loss, off);
                     sum = static_cast<double>(loss);
                 }
-                good = __reduce_add_sync(0xFFFFFFFFu, good | (marked ? 1u << 16 : 0u));  // and the marks above
+                good = __reduce_add_sync(0xFFFFFFFFu, good);
                 double* rl = s.red_loss + (g * 2 + (t & 1)) * 4;
                 int32_t* ro = s.red_ok + (g * 2 + (t & 1)) * 4;
                 if (lane == 0) {
@@ -799,7 +798,7 @@ eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                     const double total = ((rl[0] + rl[1]) + rl[2]) + rl[3];
                     // A marked individual's results all come from the evaluation that follows,
                     // which reads f_inh: f_adj may be the same array.
-                    bool again = a.flagged && sum_ok > 0xFFFF;
+                    bool again = a.flagged && (sum_ok > 0xFFFF || (*go & 255) == 2);
                     if (XP == 1 && a.flagged)
                         again = again || !(reach <= kMarkTol * fmaxf(static_cast<float>(total) * (1.0f / 128.0f), 1.0f));
                     if (again) a.flagged[p] = 1;

@@ -94,6 +94,16 @@ __device__ __forceinline__ bool mbar_wait_sleeping(uint64_t* bar, uint32_t parit
 }
 
 // ---- programmatic dependent launch ---------------------------------------------------
+// A global load that stays where it is written: the compiler moves an ordinary one
+// down to its first use, where its latency is paid in full, when registers are
+// short in between.
+__device__ __forceinline__ int32_t ld_here(const int32_t* p)
+{
+    int32_t v;
+    asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // Lets the next kernel on the stream (launched with programmatic stream
 // serialisation) start its independent prologue before this grid ends.
 __device__ __forceinline__ void grid_dep_launch()
