@@ -43,12 +43,13 @@ leea_status dispatch_eval_u8(const NetLayout& net, int32_t pop, const float* pop
                              float* f_adj, int32_t* correct, int32_t path, cudaStream_t stream,
                              void* mlp_scratch = nullptr, void* x16 = nullptr, bool x16_staged = false);
 // The precision form's evaluation on W1 shadows (scratch: batch > 128);
-// may_allocate: a stream-ordered allocation for the staged batch is allowed.
+// may_allocate: a stream-ordered allocation for the staged batch is allowed;
+// x_ready: see launch_stage_x16.
 leea_status dispatch_eval_shadow(const NetLayout& net, int32_t pop, const float* pop_dev, int32_t precision,
                                  const uint8_t* shadow, const int32_t* scale_exp, const uint8_t* x, float x_div,
                                  const int32_t* y, int32_t batch, float alpha, const float* f_inh, float* f_raw,
                                  float* f_adj, int32_t* correct, float* scratch, cudaStream_t stream,
-                                 bool may_allocate = false);
+                                 bool may_allocate = false, bool x_ready = false);
 
 SelectArgs select_args(int32_t pop, const leea_params* p, uint64_t seed, uint32_t gen);
 BreedArgs breed_args(int32_t pop, const NetLayout& net, const leea_params* p, uint64_t seed, uint32_t gen);

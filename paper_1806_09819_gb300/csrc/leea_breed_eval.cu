@@ -72,6 +72,7 @@ struct FusedArgs {
     uint64_t seed;
     uint32_t gen;
     float inv_div, alpha;
+    bool x_ready;    // the batch is complete before this kernel can start (a generation, behind its ranking)
     uint32_t a_col;  // first TMEM column of the batch operand (the accumulator uses 0 .. h-1)
     // batch staging in the tail of the rings (as in the 8-bit evaluation)
     int32_t x_staged, x_kc, x_stride, x_off, n_early;
@@ -480,6 +481,7 @@ breed_eval_u8_kernel(const __grid_constant__ CUtensorMap tmap_par, const FusedAr
                 }
                 ptx::tmem_st16(tmem_base + lane_addr + a.a_col + static_cast<uint32_t>(16 * g), cols);
             };
+            if (!a.x_ready) ptx::grid_dep_wait();
             const uint8_t* xr = a.x + static_cast<int64_t>(row) * a.k;
             const bool live = row < a.batch;
             const int n_groups = (a.k16 + 31) / 32;
@@ -747,10 +749,11 @@ bool breed_eval_u8_supported(const NetLayout& net, int32_t batch, const float* p
 cudaError_t launch_breed_eval_u8(const BreedArgs& b, const NetLayout& net, const float* parents, const int32_t* par1,
                                  const int32_t* par2, const int32_t* kind, float* children, const uint8_t* x,
                                  float x_div, const int32_t* y, int32_t batch, float alpha, const float* f_inh,
-                                 float* f_raw, float* f_adj, int32_t* correct, unsigned int* status,
+                                 float* f_raw, float* f_adj, int32_t* correct, bool x_ready, unsigned int* status,
                                  cudaStream_t stream)
 {
     FusedArgs a{};
+    a.x_ready = x_ready;
     a.pop = b.pop;
     a.k = net.dims[0];
     a.h = net.dims[1];
@@ -821,8 +824,8 @@ cudaError_t launch_breed_eval_u8(const BreedArgs& b, const NetLayout& net, const
                                static_cast<int>(smem));
     if (err != cudaSuccess) return err;
     const int grid = a.pop < sms ? a.pop : sms;
-    // Programmatic stream serialisation: barriers, TMEM and the batch may be
-    // set up while the selection kernel finishes; every role waits for it
+    // Programmatic stream serialisation: barriers, TMEM and, with x_ready, the batch
+    // may be set up while the selection kernel finishes; every role waits for it
     // before it reads kinds, parents, sigma genes or f_inh.
     return launch_pdl(breed_eval_u8_kernel, dim3(grid), dim3(kFusedThreads), smem, stream, tp, a);
 }

@@ -423,7 +423,8 @@ leea_status check_shadow_shape(const NetLayout& net, int32_t precision)
 leea_status dispatch_eval_shadow(const NetLayout& net, int32_t pop, const float* pop_dev, int32_t precision,
                                  const uint8_t* shadow, const int32_t* scale_exp, const uint8_t* x, float x_div,
                                  const int32_t* y, int32_t batch, float alpha, const float* f_inh, float* f_raw,
-                                 float* f_adj, int32_t* correct, float* scratch, cudaStream_t stream, bool may_allocate)
+                                 float* f_adj, int32_t* correct, float* scratch, cudaStream_t stream, bool may_allocate,
+                                 bool x_ready)
 {
     if (!(x_div > 0.0f) || std::isinf(x_div)) return fail(LEEA_EINVAL, "x_div must be finite and > 0");
     unsigned int* status = device_status_ptr();
@@ -456,7 +457,7 @@ leea_status dispatch_eval_shadow(const NetLayout& net, int32_t pop, const float*
     }
     LEEA_CUDA_TRY(launch_eval_shadow(net, pop, pop_dev, precision, shadow, shadow_stride_of(net, precision),
                                      scale_exp, x, x_div, y, batch, alpha, f_inh, f_raw, f_adj, correct, scratch,
-                                     status, stream),
+                                     status, stream, 0, x_ready),
                   "shadow evaluate kernel");
     return LEEA_OK;
 }
@@ -658,7 +659,7 @@ leea_status leea_breed_evaluate_u8(int32_t pop, const int32_t* dims, int32_t n_d
     unsigned int* status = device_status_ptr();
     if (!status) return fail(LEEA_ECUDA, "device status word unavailable");
     LEEA_CUDA_TRY(launch_breed_eval_u8(a, net, parents_dev, par1_dev, par2_dev, kind_dev, children_dev, x_u8_dev,
-                                       x_div, y_dev, batch, alpha, f_inh_dev, f_raw_dev, f_adj_dev, correct_dev, status,
+                                       x_div, y_dev, batch, alpha, f_inh_dev, f_raw_dev, f_adj_dev, correct_dev, false, status,
                                        static_cast<cudaStream_t>(stream)),
                   "breed + evaluate kernel");
     return LEEA_OK;
@@ -1352,7 +1353,7 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
             LEEA_CUDA_TRY(launch_breed_eval_u8(a, s->net, s->popbuf[s->cur], s->par1, s->par2, s->kind,
                                                s->popbuf[s->cur ^ 1], static_cast<const uint8_t*>(x_dev), x_div,
                                                y_dev, batch, s->prm.alpha, s->f_inh, s->f_raw, s->f_adj, s->correct,
-                                               status, s->stream),
+                                               true, status, s->stream),
                           "breed + evaluate kernel");
             sc.done();
             s->cur ^= 1;
@@ -1415,7 +1416,7 @@ static leea_status run_generation(leea_state* s, const void* x_dev, bool u8, flo
             st = dispatch_eval_shadow(s->net, s->pop, s->popbuf[s->cur], prec, s->shadow[s->cur], s->scale_exp,
                                       static_cast<const uint8_t*>(x_dev), x_div, y_dev, batch, s->prm.alpha,
                                       first ? nullptr : s->f_inh, s->f_raw, s->f_adj, s->correct, s->scratch,
-                                      s->stream);
+                                      s->stream, false, !first);
         else if (u8)
             st = dispatch_eval_u8(s->net, s->pop, s->popbuf[s->cur], static_cast<const uint8_t*>(x_dev), x_div, y_dev,
                                   batch, s->prm.alpha, first ? nullptr : s->f_inh, s->f_raw, s->f_adj, s->correct,

@@ -67,6 +67,7 @@ struct EvalShArgs {
     const ShadowSeg* segs;   // many runs: CTA b walks segs[seg_off[b] .. seg_off[b+1])
     const int32_t* seg_off;
     ShadowRun run0;
+    bool x_ready;  // the batches are complete before this kernel can start
     unsigned int* status;
 };
 
@@ -247,6 +248,7 @@ eval_shadow_kernel(const __grid_constant__ EvalShArgs a, int32_t h_max)
     const ShSmem s = carve(smem_raw, a, h_max);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int32_t nseg = seg_count(a);
+    if (!a.x_ready) ptx::grid_dep_wait();
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < a.stages; ++i) {
@@ -646,9 +648,9 @@ cudaError_t launch(const EvalShArgs& a, int32_t precision, int32_t h_max, int32_
     auto kernel = precision == 1 ? eval_shadow_kernel<1> : eval_shadow_kernel<2>;
     cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (err != cudaSuccess) return err;
-    // Programmatic stream serialisation: CTAs may start (barriers, TMEM, the
-    // batch tile) while the previous kernel finishes; the copy producer waits
-    // for it before it reads shadows and masters.
+    // Programmatic stream serialisation: CTAs may start (barriers, TMEM and, with
+    // x_ready, the batch tile) while the previous kernel finishes; the copy
+    // producer waits for it before it reads shadows and masters.
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kShThreads);
@@ -731,13 +733,14 @@ cudaError_t launch_eval_shadow(const NetLayout& net, int32_t pop, const float* p
                                const uint8_t* shadow, int64_t sh_stride, const int32_t* scale_exp,
                                const uint8_t* x, float x_div, const int32_t* y, int32_t batch, float alpha,
                                const float* f_inh, float* f_raw, float* f_adj, int32_t* correct, float* scratch,
-                               unsigned int* status, cudaStream_t stream, int32_t chunk)
+                               unsigned int* status, cudaStream_t stream, int32_t chunk, bool x_ready)
 {
     const ShadowRun r = shadow_run(net, pop, pop_dev, precision, shadow, sh_stride, scale_exp, x, x_div, y, batch,
                                    alpha, f_inh, f_raw, f_adj, correct, scratch, chunk);
     if (r.m_tiles > 1 && !scratch) return cudaErrorInvalidValue;
     EvalShArgs a = common_args(net.dims[0], net.dims[2], precision, r.h, r.cw);
     a.run0 = r;
+    a.x_ready = x_ready;
     a.status = status;
     int dev = 0, sms = 0;
     cudaError_t err = cudaGetDevice(&dev);
@@ -771,12 +774,13 @@ cudaError_t launch_combine_shadow_run_tiles(const ShadowRun& run, cudaStream_t s
 cudaError_t launch_eval_shadow_runs(int32_t k, int32_t d_out, int32_t precision, int32_t h_max, int32_t cw_max,
                                     int32_t n_runs, int32_t pop_max, bool any_tiles, const ShadowRun* runs_dev,
                                     const ShadowSeg* segs_dev, const int32_t* seg_off_dev, int32_t grid,
-                                    unsigned int* status, cudaStream_t stream)
+                                    bool x_ready, unsigned int* status, cudaStream_t stream)
 {
     EvalShArgs a = common_args(k, d_out, precision, h_max, cw_max);
     a.runs = runs_dev;
     a.segs = segs_dev;
     a.seg_off = seg_off_dev;
+    a.x_ready = x_ready;
     a.status = status;
     return launch(a, precision, h_max, cw_max, grid, n_runs, pop_max, any_tiles, stream);
 }

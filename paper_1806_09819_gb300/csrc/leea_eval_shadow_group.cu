@@ -728,12 +728,14 @@ __global__ void __launch_bounds__(kGroupThreads, 1) eval_shadow_group_kernel(con
 // (zero past the tile's rows) at 128 r, its 16-byte chunk c at chunk position
 // c ^ (r & 7).  BF16: 64 levels per row of a block; FP8: 128 levels, piece 0
 // holding 16 floor(k / 16), piece 1 k mod 16, both exact in e4m3.  One thread
-// per 16-byte chunk.
+// per 16-byte chunk.  x_ready: the batches are complete before this kernel can
+// start (a step, behind its first kernel).
 template <int PREC>
 __global__ void __launch_bounds__(256) stage_xop_tiles_kernel(const XopTile* __restrict__ tiles, int32_t n_tiles,
-                                                              int32_t k, int32_t k_blocks)
+                                                              int32_t k, int32_t k_blocks, bool x_ready)
 {
     ptx::grid_dep_launch();
+    if (!x_ready) ptx::grid_dep_wait();
     constexpr int kPieces = PREC == 1 ? 1 : 2;
     const int64_t per_tile = static_cast<int64_t>(k_blocks) * kPieces * 128 * 8;
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -805,7 +807,7 @@ size_t eval_shadow_group_xop_bytes(int32_t k, int32_t precision, int32_t batch)
 }
 
 cudaError_t launch_stage_xop_tiles(const XopTile* tiles_dev, int32_t n_tiles, int32_t k, int32_t precision,
-                                   cudaStream_t stream)
+                                   bool x_ready, cudaStream_t stream)
 {
     if (n_tiles < 1) return cudaSuccess;
     const int32_t k_blocks = (k + (precision == 1 ? 63 : 127)) / (precision == 1 ? 64 : 128);
@@ -819,8 +821,8 @@ cudaError_t launch_stage_xop_tiles(const XopTile* tiles_dev, int32_t n_tiles, in
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return precision == 1 ? cudaLaunchKernelEx(&cfg, stage_xop_tiles_kernel<1>, tiles_dev, n_tiles, k, k_blocks)
-                          : cudaLaunchKernelEx(&cfg, stage_xop_tiles_kernel<2>, tiles_dev, n_tiles, k, k_blocks);
+    const auto kernel = precision == 1 ? stage_xop_tiles_kernel<1> : stage_xop_tiles_kernel<2>;
+    return cudaLaunchKernelEx(&cfg, kernel, tiles_dev, n_tiles, k, k_blocks, x_ready);
 }
 
 namespace {

@@ -250,14 +250,15 @@ cudaError_t launch_eval_shadow_group_run(const NetLayout& net, int32_t pop, cons
 bool eval_shadow_group_supported(int32_t k, int32_t d_out, int32_t precision, int32_t h, int32_t n_max);
 size_t eval_shadow_group_xop_bytes(int32_t k, int32_t precision, int32_t batch);
 cudaError_t launch_stage_xop_tiles(const XopTile* tiles_dev, int32_t n_tiles, int32_t k, int32_t precision,
-                                   cudaStream_t stream);
+                                   bool x_ready, cudaStream_t stream);
 cudaError_t launch_eval_shadow_group(int32_t k, int32_t d_out, int32_t precision, int32_t n_max,
                                      const ShadowRun* runs_dev, int32_t n_runs, int32_t pop_max, bool any_tiles,
                                      const GroupUnit* units_dev, int32_t n_units, int32_t* sched_dev, int32_t grid,
                                      unsigned int* status, cudaStream_t stream);
 // Widest hidden chunk the tensor memory leaves room for next to the batch tile.
 int32_t eval_shadow_max_chunk(int32_t precision, int32_t k);
-// chunk: hidden units per chunk (multiple of 16), 0 for the widest.
+// chunk: hidden units per chunk (multiple of 16), 0 for the widest.  x_ready (here and
+// below): see launch_stage_x16.
 ShadowRun shadow_run(const NetLayout& net, int32_t pop, const float* pop_dev, int32_t precision,
                      const uint8_t* shadow, int64_t sh_stride, const int32_t* scale_exp, const uint8_t* x,
                      float x_div, const int32_t* y, int32_t batch, float alpha, const float* f_inh, float* f_raw,
@@ -266,13 +267,13 @@ cudaError_t launch_eval_shadow(const NetLayout& net, int32_t pop, const float* p
                                const uint8_t* shadow, int64_t sh_stride, const int32_t* scale_exp,
                                const uint8_t* x, float x_div, const int32_t* y, int32_t batch, float alpha,
                                const float* f_inh, float* f_raw, float* f_adj, int32_t* correct, float* scratch,
-                               unsigned int* status, cudaStream_t stream, int32_t chunk = 0);
+                               unsigned int* status, cudaStream_t stream, int32_t chunk = 0, bool x_ready = false);
 // Many runs of d_0-h_r-d_out nets in one launch: runs_dev[n_runs], CTA b walks
 // segs_dev[seg_off_dev[b] .. seg_off_dev[b+1]); h_max and cw_max bound every run's.
 cudaError_t launch_eval_shadow_runs(int32_t k, int32_t d_out, int32_t precision, int32_t h_max, int32_t cw_max,
                                     int32_t n_runs, int32_t pop_max, bool any_tiles, const ShadowRun* runs_dev,
                                     const ShadowSeg* segs_dev, const int32_t* seg_off_dev, int32_t grid,
-                                    unsigned int* status, cudaStream_t stream);
+                                    bool x_ready, unsigned int* status, cudaStream_t stream);
 // Evaluation of d_0-h-d_out nets (one hidden layer), SIMT FP32.
 cudaError_t launch_eval_simt(const NetLayout& net, int32_t pop, const float* pop_dev,
                              const float* x, const int32_t* y, int32_t batch, float alpha,
@@ -358,7 +359,7 @@ bool breed_eval_u8_supported(const NetLayout& net, int32_t batch, const float* p
 cudaError_t launch_breed_eval_u8(const BreedArgs& b, const NetLayout& net, const float* parents, const int32_t* par1,
                                  const int32_t* par2, const int32_t* kind, float* children, const uint8_t* x,
                                  float x_div, const int32_t* y, int32_t batch, float alpha, const float* f_inh,
-                                 float* f_raw, float* f_adj, int32_t* correct, unsigned int* status,
+                                 float* f_raw, float* f_adj, int32_t* correct, bool x_ready, unsigned int* status,
                                  cudaStream_t stream);
 // One generation (ranking, selection, breeding, evaluation of 8-bit or FP32
 // inputs) in a single launch for small FP32 populations of d_0-h-d_out nets: one CTA

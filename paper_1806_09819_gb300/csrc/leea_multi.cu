@@ -272,18 +272,21 @@ leea_status set_x_div(leea_multi* m, float x_div)
     return LEEA_OK;
 }
 
+// The evaluation of table `which` (0: of the initial populations, the first kernel
+// on the stream since the caller's; a step's comes behind its own first kernel).
 cudaError_t launch_eval(leea_multi* m, int which, unsigned int* status, cudaStream_t stream)
 {
+    const bool x_ready = which != 0;
     if (m->grouped) {
-        cudaError_t err = launch_stage_xop_tiles(m->xtiles, m->n_xtiles, m->d_in, m->prm.precision, stream);
+        cudaError_t err = launch_stage_xop_tiles(m->xtiles, m->n_xtiles, m->d_in, m->prm.precision, x_ready, stream);
         if (err != cudaSuccess) return err;
         return launch_eval_shadow_group(m->d_in, m->d_out, m->prm.precision, m->n_max, m->eval_tab[which], m->n_runs,
                                         m->pop_max, m->any_tiles, m->units, m->n_units, m->sched, m->eval_grid, status,
                                         stream);
     }
     return launch_eval_shadow_runs(m->d_in, m->d_out, m->prm.precision, m->h_max, m->cw_max, m->n_runs, m->pop_max,
-                                   m->any_tiles, m->eval_tab[which], m->segs, m->seg_off, m->eval_grid, status,
-                                   stream);
+                                   m->any_tiles, m->eval_tab[which], m->segs, m->seg_off, m->eval_grid, x_ready,
+                                   status, stream);
 }
 
 // One breeding generation from buffer c: the generation counter, then the
@@ -911,7 +914,7 @@ leea_status leea_tune_group_eval(int32_t precision, int32_t d_in, int32_t hidden
         if (err == cudaSuccess) err = cudaGetDevice(&dev);
         if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         auto once = [&]() {
-            cudaError_t e = launch_stage_xop_tiles(tiles_dev, m_tiles, d_in, precision, nullptr);
+            cudaError_t e = launch_stage_xop_tiles(tiles_dev, m_tiles, d_in, precision, false, nullptr);
             if (e != cudaSuccess) return e;
             return launch_eval_shadow_group(d_in, d_out, precision, group * hidden, run_dev, 1, pop, m_tiles > 1,
                                             units_dev, static_cast<int32_t>(units.size()), sched, sms, status,

@@ -47,9 +47,10 @@ def late_copy(gpu, tmp_path_factory):
     fn = ctypes.CDLL(str(lib)).launch_late_copy
     fn.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_longlong, ctypes.c_void_p]
 
-    def run(src_t, dst_t):
+    def run(src_t, dst):
         n = src_t.numel() * src_t.element_size()
-        assert fn(src_t.data_ptr(), dst_t.data_ptr(), n, torch.cuda.current_stream().cuda_stream) == 0
+        dst = dst if isinstance(dst, int) else dst.data_ptr()
+        assert fn(src_t.data_ptr(), dst, n, torch.cuda.current_stream().cuda_stream) == 0
 
     return run
 
@@ -132,3 +133,67 @@ def test_generation_waits_for_its_batch(gpu, late_copy, kind, h, pop, batch):
             st.close()
     np.testing.assert_array_equal(out[0][0], out[1][0])
     np.testing.assert_array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("kind,h,pop,batch", [("fused", 64, 200, 100), ("bf16", 64, 60, 100), ("fp8", 160, 60, 200)])
+def test_kernels_that_load_the_batch_themselves(gpu, late_copy, kind, h, pop, batch):
+    """The fused breed + evaluate step and the chunked shadow evaluation."""
+    import torch
+    dims = [784, h, 10]
+    c, cp = gpu.leea_layout_num_params(dims), gpu.leea_padded_params(dims)
+    popv = torch.zeros((pop, cp), device="cuda")
+    popv[:, :c] = torch.from_numpy(synthetic.random_population(pop, c, seed=3, scale=0.1)).cuda()
+    x, y = _batch(batch, 784, False)
+    late = torch.zeros_like(x)
+    cor = torch.empty(pop, dtype=torch.int32, device="cuda")
+    prec = {"bf16": 1, "fp8": 2}.get(kind, 0)
+    if prec:
+        sh = torch.empty((pop, gpu.leea_shadow_stride(dims, prec)), dtype=torch.uint8, device="cuda")
+        se, am = torch.zeros(pop, dtype=torch.int32, device="cuda"), torch.empty(pop, device="cuda")
+        gpu.leea_make_shadow(pop, dims, prec, popv, sh, se, am)
+    par = torch.arange(pop, dtype=torch.int32, device="cuda")
+    two = torch.full((pop,), 2, dtype=torch.int32, device="cuda")
+    kids = torch.zeros_like(popv)
+
+    def call(xd, f):
+        if kind == "fused":
+            gpu.leea_breed_evaluate_u8(pop, dims, gpu.Params(mut_rate=0.1), 4, 1, popv, par, par, two, kids, xd, 255.0, y,
+                                       batch, 1.0, None, f, None, None)
+        else:
+            gpu.leea_evaluate_shadow_u8_noalloc(pop, dims, popv, prec, sh, se, xd, 255.0, y, batch, 1.0, None, f, None, cor)
+
+    want, got = torch.empty(pop, device="cuda"), torch.empty(pop, device="cuda")
+    call(x, want)
+    call(late, got)
+    torch.cuda.synchronize()
+    assert not torch.equal(want, got)
+    late_copy(x, late)
+    call(late, got)
+    assert gpu.leea_device_status() == 0
+    assert torch.equal(want, got)
+
+
+def test_runs_wait_for_their_first_batch(gpu, late_copy):
+    """The batching form reads its first minibatch where the caller writes it, in the object's own buffers."""
+    import torch
+    specs = [gpu.RunSpec(60, 32, 64, seed=1), gpu.RunSpec(50, 48, 40, seed=2)]
+    out = []
+    for is_late in (False, True):
+        m = gpu.MultiRun(specs, 784, 10, gpu.Params(precision=1, n_elite=1))
+        try:
+            rows = m.total_rows
+            g = torch.Generator(device="cuda").manual_seed(1)
+            x = torch.randint(0, 256, (rows, 784), device="cuda", dtype=torch.uint8, generator=g)
+            y = torch.randint(0, 10, (rows,), device="cuda", dtype=torch.int32, generator=g)
+            xb, yb = m.batch_buffers()
+            late_copy(torch.zeros_like(x), xb)
+            late_copy(y, yb)
+            torch.cuda.synchronize()
+            late_copy(x, xb)
+            if not is_late:
+                torch.cuda.synchronize()
+            assert m.lib.leea_multi_generation_u8(m._h, xb, 255.0, yb) == 0
+            out.append(np.asarray(m.fitness()))
+        finally:
+            m.close()
+    np.testing.assert_array_equal(out[0], out[1])
