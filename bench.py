@@ -110,11 +110,11 @@ STAGES = ("select", "breed", "evaluate")
 # dram__bytes_write.sum), valid only while the kernel source is unchanged.
 TRAFFIC = {
     "breed": {"bytes_per_launch": 467.92e6, "src_sha": "7ef2dd3ff5ab01c5", "capture": "P=1000 plain workload"},
-    "evaluate": {"bytes_per_launch": 369.01e6, "src_sha": "12869056f17ba4e8", "capture": "P=1000 plain workload"},
-    "breed_evaluate": {"bytes_per_launch": 738.19e6, "src_sha": "23e25d83744d9797", "capture": "P=1000 plain workload"},
+    "evaluate": {"bytes_per_launch": 369.13e6, "src_sha": "d2b37ca7d1cb24d2", "capture": "P=1000 plain workload"},
+    "breed_evaluate": {"bytes_per_launch": 740.24e6, "src_sha": "d58d8e60dd08e07b", "capture": "P=1000 plain workload"},
     # eval_mlp_tc_kernel alone (each individual's weight pieces read once from
     # DRAM, the other tiles from L2); the stage also splits the weights
-    "evaluate_paper_net": {"bytes_per_launch": 1059.44e6, "src_sha": "98b4baf63d0ccc97",
+    "evaluate_paper_net": {"bytes_per_launch": 986.13e6, "src_sha": "056ef0adac7455ee",
                            "capture": "paper-net workload, eval_mlp_tc_kernel"},
 }
 
@@ -692,8 +692,8 @@ def run_paper_net(args, rank: int, world: int, local_rank: int):
                        "kernel_timing": f"CUDA events around each kernel of every {PROFILE_EVERY}th generation "
                                         "inside the timed region",
                        "input": "uint8 levels k of 28x28 images, x = k/255, pooled on the GPU each step",
-                       "eval_kernel": ("tcgen05, FP16 operand pieces (FP32-class) in all four layers, FP32 accumulation "
-                                       "in TMEM; the loss in FP32" if tensor else
+                       "eval_kernel": ("tcgen05, FP16 operand pieces (FP32-class) in the hidden layers, FP32 accumulation "
+                                       "in TMEM; the last layer and the loss in FP32" if tensor else
                                        "CUDA-core FP32, layers chained in shared memory (64-sample tiles)"),
                        "l2": f"inputs larger than L2 (2 population buffers of "
                              f"{pop * leea.leea_padded_params(dims) * 4 / 1e6:.0f} MB), no flush"},

@@ -131,7 +131,12 @@ enum { LEEA_SIGMA_CONST = 0, LEEA_SIGMA_DECAY = 1, LEEA_SIGMA_SELF = 2 };
  * small a call does not pay for the staging, TENSOR's kernel or SIMT's.  SIMT:
  * exact FP32 FFMA on the CUDA cores.  TENSOR: tcgen05 tensor cores with a three-term TF32 split
  * (X_hi W_hi + X_hi W_lo + X_lo W_hi, FP32 accumulation), which is within
- * ~1e-6 relative of FP32; LEEA_EINVAL if the shape does not allow it.
+ * ~1e-6 relative of FP32; LEEA_EINVAL if the shape does not allow it.  The tensor
+ * cores truncate as they accumulate.  RMS error of a fitness against 64 bits,
+ * 784-h-10 nets: on initial weights (N(0, 1/d_0), images) 4e-8 to 7e-8 relative on
+ * the tensor cores and 5e-8 with SIMT; on weights twice as large 4e-7 (8-bit
+ * levels) and 6e-7 (floats; TENSOR 1.4e-6), four times as large 1e-6 and 2e-6
+ * (TENSOR 4e-6), while SIMT stays at 6e-8.
  * FUSED (state object, 8-bit generation calls, precision 0): every breeding
  * generation makes and evaluates each child in one kernel
  * (leea_breed_evaluate_u8), so the evaluation does not read the new

@@ -37,7 +37,7 @@
 //               per individual rather than four: the epilogue is bound by
 //               instruction latency (shared-memory loads feeding FMA chains),
 //               not by any pipe, so it needs the warps to hide it.
-// Measured, 2048 nets 784-112-10 on 256 samples: FP8 84 us (92 with the staging's
+// Measured, 2048 nets 784-112-10 on 256 samples: FP8 85 us (92 with the staging's
 // indices computed per unit, checks between the columns of a chain and 64-bit
 // descriptors built per MMA).  A pair takes about 9.5k cycles per tile, 7k of them
 // the epilogue's layer 2.
