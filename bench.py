@@ -110,11 +110,11 @@ STAGES = ("select", "breed", "evaluate")
 # dram__bytes_write.sum), valid only while the kernel source is unchanged.
 TRAFFIC = {
     "breed": {"bytes_per_launch": 467.92e6, "src_sha": "7ef2dd3ff5ab01c5", "capture": "P=1000 plain workload"},
-    "evaluate": {"bytes_per_launch": 369.13e6, "src_sha": "d2b37ca7d1cb24d2", "capture": "P=1000 plain workload"},
+    "evaluate": {"bytes_per_launch": 369.13e6, "src_sha": "32180b7ab715c5f7", "capture": "P=1000 plain workload"},
     "breed_evaluate": {"bytes_per_launch": 740.24e6, "src_sha": "d58d8e60dd08e07b", "capture": "P=1000 plain workload"},
     # eval_mlp_tc_kernel alone (each individual's weight pieces read once from
     # DRAM, the other tiles from L2); the stage also splits the weights
-    "evaluate_paper_net": {"bytes_per_launch": 986.13e6, "src_sha": "056ef0adac7455ee",
+    "evaluate_paper_net": {"bytes_per_launch": 986.13e6, "src_sha": "307e48e74b9a71f0",
                            "capture": "paper-net workload, eval_mlp_tc_kernel"},
 }
 

@@ -659,8 +659,8 @@ leea_status leea_breed_evaluate_u8(int32_t pop, const int32_t* dims, int32_t n_d
     unsigned int* status = device_status_ptr();
     if (!status) return fail(LEEA_ECUDA, "device status word unavailable");
     LEEA_CUDA_TRY(launch_breed_eval_u8(a, net, parents_dev, par1_dev, par2_dev, kind_dev, children_dev, x_u8_dev,
-                                       x_div, y_dev, batch, alpha, f_inh_dev, f_raw_dev, f_adj_dev, correct_dev, false, status,
-                                       static_cast<cudaStream_t>(stream)),
+                                       x_div, y_dev, batch, alpha, f_inh_dev, f_raw_dev, f_adj_dev, correct_dev, false,
+                                       status, static_cast<cudaStream_t>(stream)),
                   "breed + evaluate kernel");
     return LEEA_OK;
 }

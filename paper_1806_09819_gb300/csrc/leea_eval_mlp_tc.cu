@@ -723,7 +723,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                     a.flagged[seg.p] = 1;
             }
         } else {
-            // -------------------------------------------------------- layer 4 and the loss, one sample per thread
+            // -------------------------------------------------------- layer 4 and the loss
             for (Segments seg(a, blockIdx.x); ok && seg.valid(); seg.step(a), ++k) {
                 const float* b3 = s.param + (k & 1u) * param_floats(a.dims, a.wst) + d1 + d2;
                 const float *b4 = b3 + d3, *w4t = b4 + kMaxOutTc;
@@ -740,8 +740,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) eval_mlp_tc_kernel(const __grid
                     constexpr float kInv = 1.0f / kPieceScale;
                     const float scale[4] = { kInv, kInv, kInv, kInv };
                     float z[kMaxOutTc];
-                    quad_logits(a.no4, tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(a.col[2]), d3,
-                                scale, b3, w4t, a.wst, z);
+                    const uint32_t lanes = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
+                    quad_logits(a.no4, lanes + static_cast<uint32_t>(a.col[2]), d3, scale, b3, w4t, a.wst, z);
                     ptx::tc_fence_before();
                     arrive(s.d3_read);
                     double loss = 0.0;
@@ -830,7 +830,8 @@ __global__ void __launch_bounds__(256) combine_mlp_parts_kernel(const MlpTcArgs 
     int32_t good = 0;
     int t = 0;
     for (int c = c0; c <= c1; ++c) {
-        const int64_t end = static_cast<int64_t>(c + 1) * a.per_cta + min(c + 1, a.extra) - first;  // the CTA's last tile + 1
+        // One past the CTA's last tile, counted from the individual's first.
+        const int64_t end = static_cast<int64_t>(c + 1) * a.per_cta + min(c + 1, a.extra) - first;
         const int64_t e = (2 * static_cast<int64_t>(c) + (c == c0 ? 1 : 0)) * a.n_tiles;
         for (; t < a.n_tiles && t < end; ++t) {
             sum += a.part_loss[e + t];

@@ -237,7 +237,8 @@ uint32_t u8_stage_bytes(const U8Shape& u, int32_t batch)
 
 size_t u8_smem_bytes(const U8Shape& u, int32_t d_out, int32_t batch)
 {
-    return 1024 + static_cast<size_t>(u.n_stages) * u8_stage_bytes(u, batch) + u8_tail_bytes(u.hp, quad_row_floats(d_out), u.n_stages);
+    return 1024 + static_cast<size_t>(u.n_stages) * u8_stage_bytes(u, batch) +
+           u8_tail_bytes(u.hp, quad_row_floats(d_out), u.n_stages);
 }
 
 // K stage and ring depth: 64 inputs when at least kMinStages such stages fit in
@@ -880,7 +881,8 @@ __global__ void __launch_bounds__(256) stage_x16_kernel(const uint8_t* __restric
 // stage_x16_kernel.
 __global__ void __launch_bounds__(256) stage_xf_kernel(const float* __restrict__ x, int32_t batch, int32_t k, int32_t kp,
                                                        __half* __restrict__ x16, float* __restrict__ x_scale,
-                                                       float2* __restrict__ x_err, int32_t* __restrict__ flagged, int32_t pop, bool x_ready)
+                                                       float2* __restrict__ x_err, int32_t* __restrict__ flagged,
+                                                       int32_t pop, bool x_ready)
 {
     __shared__ uint32_t top[8];
     __shared__ float part_sq[8];
